@@ -1988,24 +1988,29 @@ __device__ __forceinline__ int mcv_bin(const double* t, int d, const int* m) {
 }
 
 // Mean bins of every fold: subject i adds to slice fold[i] (cnt, w, v, v2 are F x P).
+// MCV_LANES threads share a subject's observations: one thread each left 20 000
+// subjects' scatters (12.5 observations of four dependent-issue atomics) on 157
+// blocks (66 us at 64 x 64).
+constexpr int MCV_LANES = 8;
 __global__ void k_bin_mean_folds(int n, long long N, int d, int m0, int m1, int m2, int P,
                                  const int64_t* __restrict__ offs, const double* __restrict__ t,
                                  const double* __restrict__ y, const int32_t* __restrict__ fold,
                                  int nfold, int32_t* cnt, double* w, double* v, double* v2,
                                  int* __restrict__ err) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int i = (int)(g / MCV_LANES), part = (int)(g % MCV_LANES);
   if (i >= n) return;
   const int m[3] = {m0, m1, m2};
   const int64_t lo = offs[i], hi = offs[i + 1];
   const int f = fold[i];
   if (lo < 0 || hi < lo || hi > N || f < 0 || f >= nfold) {
-    atomicExch(err, DERR_BOUNDS);
+    if (part == 0) atomicExch(err, DERR_BOUNDS);
     return;
   }
   if (hi == lo) return;
   const double wi = 1.0 / (double)(hi - lo);
   const size_t base = (size_t)f * P;
-  for (int64_t j = lo; j < hi; ++j) {
+  for (int64_t j = lo + part; j < hi; j += MCV_LANES) {
     const size_t b = base + mcv_bin(t + j * d, d, m);
     const double yy = y[j];
     atomicAdd(cnt + b, 1);
@@ -2015,12 +2020,13 @@ __global__ void k_bin_mean_folds(int n, long long N, int d, int m0, int m1, int 
   }
 }
 
-// Training bins of fold f: the sums over all folds minus fold f's.
-__global__ void k_mean_train(int P, int F, int f, const int32_t* __restrict__ cnt,
+// Training bins of fold f0 + blockIdx.y: the sums over all folds minus that fold's
+// (slice blockIdx.y of ct, wt, vt).
+__global__ void k_mean_train(int P, int F, int f0, const int32_t* __restrict__ cnt,
                              const double* __restrict__ w, const double* __restrict__ v,
                              int32_t* __restrict__ ct, double* __restrict__ wt,
                              double* __restrict__ vt) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  const int p = blockIdx.x * blockDim.x + threadIdx.x, f = f0 + blockIdx.y;
   if (p >= P) return;
   int c = 0;
   double sw = 0.0, sv = 0.0;
@@ -2029,9 +2035,215 @@ __global__ void k_mean_train(int P, int F, int f, const int32_t* __restrict__ cn
     sw += w[(size_t)q * P + p];
     sv += v[(size_t)q * P + p];
   }
-  ct[p] = c - cnt[(size_t)f * P + p];
-  wt[p] = sw - w[(size_t)f * P + p];
-  vt[p] = sv - v[(size_t)f * P + p];
+  const size_t o = (size_t)blockIdx.y * P + p;
+  ct[o] = c - cnt[(size_t)f * P + p];
+  wt[o] = sw - w[(size_t)f * P + p];
+  vt[o] = sv - v[(size_t)f * P + p];
+}
+
+// Natural-order elimination of a (d+1) x (d+1) mean fit under the rules of fit_point:
+// the pivot test by multiplication and the pivots' reciprocals reused, so a regular
+// point costs D divisions in place of 3 D + 1 (an FP64 division is some 15 FP64
+// instructions, and this GPU issues those at 1/64 of the FP32 rate).
+template <int D>
+__device__ __forceinline__ double mcv_fit(double (&A)[D][D], double (&r)[D], int nonempty,
+                                          bool& empty) {
+  empty = !(A[0][0] > 0.0);
+  if (empty) return 0.0;
+  const double a00 = A[0][0], r0 = r[0];
+  bool ok = nonempty >= D;
+  double diag[D], inv[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) diag[k] = A[k][k];
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    ok = ok && A[k][k] > PIVOT_RTOL_F64 * diag[k];  // false for a diagonal <= 0 too
+    inv[k] = ok ? 1.0 / A[k][k] : 0.0;
+#pragma unroll
+    for (int i = k + 1; i < D; ++i) {
+      const double l = A[k][i] * inv[k];
+#pragma unroll
+      for (int j = i; j < D; ++j) A[i][j] -= l * A[k][j];
+      r[i] -= l * r[k];
+    }
+  }
+  if (!ok) return r0 / a00;
+  double x[D];
+#pragma unroll
+  for (int k = D - 1; k >= 0; --k) {
+    double s = r[k];
+#pragma unroll
+    for (int j = k + 1; j < D; ++j) s -= A[k][j] * x[j];
+    x[k] = s * inv[k];
+  }
+  return x[0];
+}
+
+// Bandwidths of one launch of the batched mean CV, widest windows first (so that the
+// long blocks start first and the short ones fill the tail).
+constexpr int MCV_MAXH = 64;
+struct McvH {
+  double h[MCV_MAXH][2];
+  int T[MCV_MAXH][2];
+  int ih[MCV_MAXH];
+};
+
+// All (bandwidth, fold) items of the mean smoother's CV, d <= 2, one launch: block
+// (row block, fold, bandwidth) fits HR rows of the R x C grid on the training bins of
+// its fold and adds the held-out terms to the item's accumulators.
+//   phase A  sums down the columns (axis 0) of W (K, K u, K u^2), V (K, K u) and the
+//            non-empty indicator (an integer), straight from the L2-resident bins;
+//   phase B  sums along the rows (axis 1) from shared memory: the 10 moments of a
+//            node stay in registers; the solve and the CV terms follow there.
+// Axis 0 first keeps the second pass inside the block's own rows (no halo is summed
+// twice).  The FP64 FMAs bound it: 64 x 64, 16 bandwidths of 0.03-0.3, 5 folds:
+// 14 x 2 FP64 flops per tap and node = 0.13 ms at the measured FP64 rate.  One launch
+// sequence per item (6 launches, 2-10 us each) took 2.9 ms for that call; it takes 0.235 ms.
+template <int DIM>
+__global__ void __launch_bounds__(256)
+    k_mean_cv_items(McvH hs, int R, int C, int HR, int F, const int32_t* __restrict__ ct,
+                    const double* __restrict__ wt, const double* __restrict__ vt,
+                    const double* __restrict__ wf, const double* __restrict__ vf,
+                    const double* __restrict__ v2f, double* __restrict__ acc) {
+  constexpr int D = DIM + 1;
+  extern __shared__ __align__(16) unsigned char mcv_sm[];
+  double* wr = reinterpret_cast<double*>(mcv_sm);  // [3][TW] axis 0 (d = 2)
+  double* wc = wr + 3 * TW;                        // [3][TW] last axis
+  double* mid = wc + 3 * TW;                       // [5][HR * C]
+  int* midn = reinterpret_cast<int*>(mid + 5 * (size_t)HR * C);  // [HR * C]
+  __shared__ double red[3][8];
+  const int q = blockIdx.z, f = blockIdx.y, P = R * C;
+  const int Tr = DIM == 2 ? hs.T[q][0] : 0, Tc = hs.T[q][DIM - 1];
+  const int a0 = blockIdx.x * HR, th = min(HR, R - a0), npts = th * C;
+  for (int e = threadIdx.x; e < DIM * TW; e += blockDim.x) {
+    const int ax = e / TW, t = e - ax * TW, off = t - TMAX;
+    const int M = (DIM == 2 && ax == 0) ? R : C;
+    // the weights of k_taps
+    const double hm = __dmul_rn(hs.h[q][ax], (double)M);
+    const double u = __ddiv_rn((double)off, hm);
+    const bool in = fabs(u) < 1.0 && abs(off) < M;
+    const double K = in ? __dmul_rn(0.75, __dsub_rn(1.0, __dmul_rn(u, u))) : 0.0;
+    double* w = (DIM == 2 && ax == 0) ? wr : wc;
+    w[t] = K;
+    w[TW + t] = __dmul_rn(K, u);
+    w[2 * TW + t] = __dmul_rn(K, __dmul_rn(u, u));
+  }
+  __syncthreads();
+  const size_t fo = (size_t)f * P;
+  const double *W = wt + fo, *V = vt + fo;
+  const int32_t* N = ct + fo;
+  for (int e = threadIdx.x; e < npts; e += blockDim.x) {
+    const int i = e / C, c = e - i * C, r = a0 + i;
+    if constexpr (DIM == 2) {
+      const int lo = max(-Tr, -r), hi = min(Tr, R - 1 - r);
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0, t0 = 0.0, t1 = 0.0;
+      int nn = 0;
+      const double* k0 = wr + TMAX;
+      int p = (r + lo) * C + c;
+#pragma unroll 4
+      for (int k = lo; k <= hi; ++k, p += C) {
+        const double w = W[p], v = V[p];
+        nn += N[p] > 0;
+        s0 = fma(k0[k], w, s0);
+        s1 = fma(k0[TW + k], w, s1);
+        s2 = fma(k0[2 * TW + k], w, s2);
+        t0 = fma(k0[k], v, t0);
+        t1 = fma(k0[TW + k], v, t1);
+      }
+      const int hc = HR * C;
+      mid[e] = s0;
+      mid[hc + e] = s1;
+      mid[2 * hc + e] = s2;
+      mid[3 * hc + e] = t0;
+      mid[4 * hc + e] = t1;
+      midn[e] = nn;
+    } else {
+      mid[e] = W[e];
+      mid[HR * C + e] = V[e];
+      midn[e] = N[e] > 0;
+    }
+  }
+  __syncthreads();
+  double ce = 0.0, win = 0.0, wout = 0.0;
+  for (int e = threadIdx.x; e < npts; e += blockDim.x) {
+    const int c = e % C, hc = HR * C;
+    const int lo = max(-Tc, -c), hi = min(Tc, C - 1 - c);
+    const double* k0 = wc + TMAX;
+    const double* x = mid + e;
+    int nn = 0;
+    double A[D][D], r[D];
+    if constexpr (DIM == 2) {
+      double s00 = 0.0, s01 = 0.0, s02 = 0.0, s10 = 0.0, s11 = 0.0, s20 = 0.0;
+      double t00 = 0.0, t01 = 0.0, t10 = 0.0;
+#pragma unroll 2
+      for (int k = lo; k <= hi; ++k) {
+        const double w0 = k0[k], w1 = k0[TW + k], w2 = k0[2 * TW + k];
+        const double x0 = x[k], x1 = x[hc + k], x3 = x[3 * hc + k];
+        nn += midn[e + k];
+        s00 = fma(w0, x0, s00);
+        s01 = fma(w1, x0, s01);
+        s02 = fma(w2, x0, s02);
+        s10 = fma(w0, x1, s10);
+        s11 = fma(w1, x1, s11);
+        s20 = fma(w0, x[2 * hc + k], s20);
+        t00 = fma(w0, x3, t00);
+        t01 = fma(w1, x3, t01);
+        t10 = fma(w0, x[4 * hc + k], t10);
+      }
+      A[0][0] = s00;
+      A[0][1] = A[1][0] = s10;
+      A[0][2] = A[2][0] = s01;
+      A[1][1] = s20;
+      A[1][2] = A[2][1] = s11;
+      A[2][2] = s02;
+      r[0] = t00;
+      r[1] = t10;
+      r[2] = t01;
+    } else {
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0, t0 = 0.0, t1 = 0.0;
+#pragma unroll 2
+      for (int k = lo; k <= hi; ++k) {
+        nn += midn[e + k];
+        s0 = fma(k0[k], x[k], s0);
+        s1 = fma(k0[TW + k], x[k], s1);
+        s2 = fma(k0[2 * TW + k], x[k], s2);
+        t0 = fma(k0[k], x[hc + k], t0);
+        t1 = fma(k0[TW + k], x[hc + k], t1);
+      }
+      A[0][0] = s0;
+      A[0][1] = A[1][0] = s1;
+      A[1][1] = s2;
+      r[0] = t0;
+      r[1] = t1;
+    }
+    bool empty;
+    const double g = mcv_fit<D>(A, r, nn, empty);
+    const size_t o = fo + (size_t)a0 * C + e;
+    if (empty) {
+      wout += wf[o];
+    } else {
+      ce += v2f[o] - 2.0 * g * vf[o] + g * g * wf[o];
+      win += wf[o];
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    ce += __shfl_xor_sync(0xffffffffu, ce, o);
+    win += __shfl_xor_sync(0xffffffffu, win, o);
+    wout += __shfl_xor_sync(0xffffffffu, wout, o);
+  }
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  if (lane == 0) {
+    red[0][wp] = ce;
+    red[1][wp] = win;
+    red[2][wp] = wout;
+  }
+  __syncthreads();
+  if (threadIdx.x < 24) {  // term threadIdx.x / 8, its 8 warps' sums
+    double s = red[threadIdx.x >> 3][threadIdx.x & 7];
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0x00ffffffu, s, o);
+    if ((threadIdx.x & 7) == 0)
+      atomicAdd(acc + 3 * ((size_t)hs.ih[q] * F + f) + (threadIdx.x >> 3), s);
+  }
 }
 
 // Held-out terms of fold f against the fit mu (status st): acc[0] += error,
@@ -2075,11 +2287,15 @@ fpca_status mean_cv_run(fpca_ctx* ctx, const fpca_grid* g, int n, const int64_t*
           cudaSuccess ||
       cudaStreamSynchronize(ctx->stream) != cudaSuccess)
     return fpca_check_launch(ctx, "mean_cv: offsets");
+  // d <= 2: one launch over all items, from the training bins of every fold; d = 3: the
+  // smoother's own passes, item by item, from one fold's training bins at a time
+  const int FT = d <= 2 ? F : 1;
   const size_t need = WsCarve::round(smooth_mean_scratch_bytes(P)) +
                       WsCarve::round(sizeof(int32_t) * (size_t)F * P) +
                       3 * WsCarve::round(sizeof(double) * (size_t)F * P) +
-                      WsCarve::round(sizeof(int32_t) * P) + 3 * WsCarve::round(sizeof(double) * P) +
-                      WsCarve::round(P) + WsCarve::round(sizeof(double) * 3 * (size_t)nh * F) + 4096;
+                      WsCarve::round(sizeof(int32_t) * (size_t)FT * P) +
+                      2 * WsCarve::round(sizeof(double) * (size_t)FT * P) +
+                      WsCarve::round(sizeof(double) * P) + WsCarve::round(P) + WsCarve::round(sizeof(double) * 3 * (size_t)nh * F) + 4096;
   void* ws = fpca_workspace(ctx, need);
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace (%zu bytes)", need);
   WsCarve c(ws);
@@ -2088,9 +2304,9 @@ fpca_status mean_cv_run(fpca_ctx* ctx, const fpca_grid* g, int n, const int64_t*
   double* fw = c.take<double>((size_t)F * P);
   double* fv = c.take<double>((size_t)F * P);
   double* fv2 = c.take<double>((size_t)F * P);
-  int32_t* ct = c.take<int32_t>(P);
-  double* wt = c.take<double>(P);
-  double* vt = c.take<double>(P);
+  int32_t* ct = c.take<int32_t>((size_t)FT * P);
+  double* wt = c.take<double>((size_t)FT * P);
+  double* vt = c.take<double>((size_t)FT * P);
   double* mu = c.take<double>(P);
   uint8_t* st = c.take<uint8_t>(P);
   double* acc = c.take<double>((size_t)3 * nh * F);
@@ -2099,12 +2315,46 @@ fpca_status mean_cv_run(fpca_ctx* ctx, const fpca_grid* g, int n, const int64_t*
   cudaMemsetAsync(fv, 0, sizeof(double) * (size_t)F * P, ctx->stream);
   cudaMemsetAsync(fv2, 0, sizeof(double) * (size_t)F * P, ctx->stream);
   cudaMemsetAsync(acc, 0, sizeof(double) * 3 * (size_t)nh * F, ctx->stream);
-  k_bin_mean_folds<<<(n + 127) / 128, 128, 0, ctx->stream>>>(
+  k_bin_mean_folds<<<(int)(((long long)n * MCV_LANES + 255) / 256), 256, 0, ctx->stream>>>(
       n, Nobs, d, g->m[0], d > 1 ? g->m[1] : 1, d > 2 ? g->m[2] : 1, P, offs, t, y, fold, F, fc,
       fw, fv, fv2, ctx->d_err);
   FPCA_LAUNCHED(ctx, "bin_mean_folds");
   const int nb = (P + 255) / 256;
-  for (int f = 0; f < F; ++f) {
+  if (d <= 2) {
+    k_mean_train<<<dim3(nb, F), 256, 0, ctx->stream>>>(P, F, 0, fc, fw, fv, ct, wt, vt);
+    FPCA_LAUNCHED(ctx, "mean_train");
+    const int R = d == 2 ? g->m[0] : 1, C = g->m[d - 1];
+    const int HR = std::min(R, std::max(1, 256 / C));  // about one node per thread
+    const size_t sm = sizeof(double) * (6 * TW + 5 * (size_t)HR * C) + sizeof(int) * (size_t)HR * C;
+    std::vector<int> by(nh);
+    for (int i = 0; i < nh; ++i) by[i] = i;
+    auto work = [&](int ih) {
+      int s = 0;
+      for (int k = 0; k < d; ++k) s += host_taps(h[(size_t)ih * d + k], g->m[k]);
+      return s;
+    };
+    std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return work(a) > work(b); });
+    for (int h0 = 0; h0 < nh; h0 += MCV_MAXH) {
+      const int nq = std::min(MCV_MAXH, nh - h0);
+      McvH hs{};
+      for (int q = 0; q < nq; ++q) {
+        hs.ih[q] = by[h0 + q];
+        for (int k = 0; k < d; ++k) {
+          hs.h[q][k] = h[(size_t)hs.ih[q] * d + k];
+          hs.T[q][k] = host_taps(hs.h[q][k], g->m[k]);
+        }
+      }
+      const dim3 grid((R + HR - 1) / HR, F, nq);
+      if (d == 2)
+        k_mean_cv_items<2><<<grid, 256, sm, ctx->stream>>>(hs, R, C, HR, F, ct, wt, vt, fw, fv, fv2,
+                                                           acc);
+      else
+        k_mean_cv_items<1><<<grid, 256, sm, ctx->stream>>>(hs, R, C, HR, F, ct, wt, vt, fw, fv, fv2,
+                                                           acc);
+      FPCA_LAUNCHED(ctx, "mean_cv_items");
+    }
+  }
+  for (int f = 0; d > 2 && f < F; ++f) {
     k_mean_train<<<nb, 256, 0, ctx->stream>>>(P, F, f, fc, fw, fv, ct, wt, vt);
     FPCA_LAUNCHED(ctx, "mean_train");
     for (int ih = 0; ih < nh; ++ih) {
