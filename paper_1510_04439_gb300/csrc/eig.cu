@@ -13,9 +13,12 @@
 
 #include "fpca_internal.cuh"
 #include "ff.cuh"
+#include "jacobi.cuh"
 #include "ptx.cuh"
 
 namespace {
+
+using namespace fpca_jacobi;
 
 template <typename TG>
 __device__ __forceinline__ double gval(const TG* G, long long idx) {
@@ -637,47 +640,6 @@ __global__ void __launch_bounds__(256) k_apply_ff(int P, int l, const TX* __rest
   Q[e] = (TX)ff::to_double(acc);
 }
 
-// Pair (p, q), p < q, of position i (0 <= i < ne / 2) at step `step` of a sweep of
-// the round-robin (circle) schedule: ne / 2 disjoint pairs per step, ne - 1 steps
-// (ne even; q == n marks the dummy of odd n).
-__device__ __forceinline__ void rr_pair(int ne, int step, int i, int& p, int& q) {
-  const int m = ne - 1;
-  if (i == 0) {
-    p = m;
-    q = step;
-  } else {
-    p = step + i;
-    if (p >= m) p -= m;
-    q = step - i;
-    if (q < 0) q += m;
-  }
-  if (p > q) {
-    const int t = p;
-    p = q;
-    q = t;
-  }
-}
-
-// The rotation (c, s) that annihilates a_pq: tau = (a_qq - a_pp) / (2 a_pq),
-// t = sign(tau) / (|tau| + sqrt(1 + tau^2)), c = 1 / sqrt(1 + t^2), s = t c.
-// The quotients and 1 / sqrt(1 + t^2) (argument in [1, 2]) use the fast
-// approximate forms: c^2 + s^2 = 1 then holds to a few FP32 ulps, and the
-// refinement that follows the FP32 Jacobi restores orthogonality anyway.  The
-// square root of 1 + tau^2 stays exact so that tau^2 = inf still gives t = 0.
-__device__ __forceinline__ void rr_rot(const float* A, int ld, int n, int p, int q, float& c,
-                                       float& sn) {
-  c = 1.f;
-  sn = 0.f;
-  if (q >= n) return;
-  const float apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
-  if (fabsf(apq) > 1e-30f && fabsf(apq) > 1e-18f * sqrtf(fabsf(app) * fabsf(aqq))) {
-    const float tau = __fdividef(aqq - app, 2.f * apq);
-    const float t = __fdividef(tau >= 0.f ? 1.f : -1.f, fabsf(tau) + sqrtf(1.f + tau * tau));
-    c = rsqrtf(1.f + t * t);
-    sn = t * c;
-  }
-}
-
 // Cyclic parallel Jacobi in FP32 on the n x n matrix in Acur (ld = n + 1), V
 // accumulating the rotations, until off(A)^2 <= tol diag(A)^2 or max_sweeps.
 // Every step applies ne / 2 disjoint rotations as one two-sided update:
@@ -1210,23 +1172,21 @@ fpca_status launch_jacobi_rr(fpca_ctx* ctx, int l, double* A, double* V, double*
 }
 
 // ---------------------------------------------------------------------------
-// Dense symmetric eigensolver (n <= 1024): block Jacobi in FP32, then the
-// Ogita-Aishima refinement in FP64.
+// Dense symmetric eigensolver (n <= 1024; n <= 256 has its own, eig_dense.cu): block
+// Jacobi in FP32, then the Ogita-Aishima refinement in FP64.
 // ---------------------------------------------------------------------------
 // A one-block cyclic Jacobi keeps every rotation step of an n x n matrix on one
 // SM, and one SM's FP64 rate and its round trips to memory make that take
 // hundreds of milliseconds at n = 256.  The two-sided block Jacobi method spreads
 // it: the indices are cut into blocks of BJ_S, and each round pairs the blocks
-// (round-robin, nb - 1 rounds per sweep); per pair (I, J) one CTA diagonalises the
-// 2 BJ_S x 2 BJ_S subproblem A[I u J, I u J] in shared memory (rr_jacobi_f32, a few
-// sweeps) into an orthogonal J_IJ; then A <- J' A J (a J_a' A[P_a, P_b] J_b product
+// (round-robin, nb - 1 rounds per sweep); per pair (I, J) one CTA turns the
+// 2 BJ_S x 2 BJ_S subproblem A[I u J, I u J] by one sweep of rotations in shared memory
+// (bj_sweep) into an orthogonal J_IJ; then A <- J' A J (a J_a' A[P_a, P_b] J_b product
 // per pair of pairs) and V <- V J spread over the whole GPU.  All of it in FP32;
 // the eigenvectors X = V then go through the FP64 refinement steps of Ogita and
 // Aishima (as launch_jacobi_rr), each of which squares the error, on the original
 // FP64 matrix.  n is padded to a multiple of 2 BJ_S with zero rows and columns,
 // which no rotation mixes with the real indices (their coupling is exactly zero).
-constexpr int BJ_S = 16;
-constexpr int BJ_W = 2 * BJ_S;  // subproblem width
 constexpr int BJ_SWEEPS = 12;   // sweeps at most (each ends with the convergence test)
 // The FP32 sweeps stop once the off-diagonal mass is at most this fraction of the
 // diagonal mass (off-diagonal norm 1e-4 of the diagonal's; FP32 round-off alone
@@ -1235,11 +1195,6 @@ constexpr int BJ_SWEEPS = 12;   // sweeps at most (each ends with the convergenc
 constexpr double BJ_TOL = 1e-8;
 
 inline int bj_ne(int n) { return (n + BJ_W - 1) / BJ_W * BJ_W; }
-
-// local index i of the subproblem of pair (I, J) -> global index
-__device__ __forceinline__ int bj_index(int I, int J, int i) {
-  return i < BJ_S ? I * BJ_S + i : J * BJ_S + (i - BJ_S);
-}
 
 __global__ void k_bj_init(int n, int ne, const double* __restrict__ A64, float* __restrict__ A,
                           float* __restrict__ V, int* __restrict__ done) {
@@ -1252,30 +1207,27 @@ __global__ void k_bj_init(int n, int ne, const double* __restrict__ A64, float* 
   if (blockIdx.x == 0 && threadIdx.x == 0) *done = 0;
 }
 
-// One CTA per block pair of the round: diagonalise the subproblem, write its
+// One CTA per block pair of the round: one sweep of rotations over the subproblem, its
 // rotation J (BJ_W x BJ_W, row-major) to Jg[pair].
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(BJ_NT)
     k_bj_sub(int ne, int round, const float* __restrict__ A, float* __restrict__ Jg,
              const int* __restrict__ done) {
-  __shared__ float a0[BJ_W * (BJ_W + 1)], a1[BJ_W * (BJ_W + 1)], vs[BJ_W * (BJ_W + 1)];
-  __shared__ float red[64], cs[64];
-  __shared__ int sdone;
+  __shared__ float a0[BJ_W * (BJ_W + 1)], a1[BJ_W * (BJ_W + 1)], js[BJ_W * (BJ_W + 1)];
+  __shared__ float cs[32];
   if (*done) return;
   const int nb = ne / BJ_S;
   int I, J;
   rr_pair(nb, round, blockIdx.x, I, J);
   constexpr int ld = BJ_W + 1;
-  for (int e = threadIdx.x; e < BJ_W * BJ_W; e += blockDim.x) {
-    const int i = e / BJ_W, j = e - (e / BJ_W) * BJ_W;
+  for (int e = threadIdx.x; e < BJ_W * BJ_W; e += BJ_NT) {
+    const int i = e / BJ_W, j = e % BJ_W;
     a0[i * ld + j] = A[(long long)bj_index(I, J, i) * ne + bj_index(I, J, j)];
-    vs[i * ld + j] = i == j ? 1.f : 0.f;
+    js[i * ld + j] = i == j ? 1.f : 0.f;
   }
   __syncthreads();
-  rr_jacobi_f32<1>(BJ_W, a0, a1, vs, 1, 1e-12f, red, cs, &sdone);
-  __syncthreads();
+  bj_sweep(a0, a1, js, ld, cs, round == 0);
   float* out = Jg + (size_t)blockIdx.x * BJ_W * BJ_W;
-  for (int e = threadIdx.x; e < BJ_W * BJ_W; e += blockDim.x)
-    out[e] = vs[(e / BJ_W) * ld + e % BJ_W];
+  for (int e = threadIdx.x; e < BJ_W * BJ_W; e += BJ_NT) out[e] = js[(e / BJ_W) * ld + e % BJ_W];
 }
 
 // One launch per round applies the round's rotations:
@@ -1363,33 +1315,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// V[rows, P_b] <- V[rows, P_b] J_b (the single-subproblem case): BJ_W rows
-// (blockIdx.x) of pair b = blockIdx.y.
-__global__ void __launch_bounds__(256)
-    k_bj_apply_v(int ne, int round, float* __restrict__ V, const float* __restrict__ Jg,
-                 const int* __restrict__ done) {
-  __shared__ float jb[BJ_W][BJ_W + 1], m[BJ_W][BJ_W + 1];
-  if (*done) return;
-  const int nb = ne / BJ_S;
-  int Ib, Jb;
-  rr_pair(nb, round, blockIdx.y, Ib, Jb);
-  const float* JB = Jg + (size_t)blockIdx.y * BJ_W * BJ_W;
-  const int r0 = blockIdx.x * BJ_W;
-  for (int e = threadIdx.x; e < BJ_W * BJ_W; e += blockDim.x) {
-    const int i = e / BJ_W, j = e - (e / BJ_W) * BJ_W;
-    jb[i][j] = JB[e];
-    m[i][j] = V[(long long)(r0 + i) * ne + bj_index(Ib, Jb, j)];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < BJ_W * BJ_W; e += blockDim.x) {
-    const int i = e / BJ_W, j = e - (e / BJ_W) * BJ_W;
-    float s = 0.f;
-#pragma unroll 8
-    for (int k = 0; k < BJ_W; ++k) s = fmaf(m[i][k], jb[k][j], s);
-    V[(long long)(r0 + i) * ne + bj_index(Ib, Jb, j)] = s;
-  }
-}
-
 // done = 1 once the off-diagonal mass of the sweep's last round (mass[0], summed
 // by k_bj_apply) is at most tol of the diagonal mass (mass[1]).
 __global__ void k_bj_check(const double* __restrict__ mass, double tol, int* __restrict__ done) {
@@ -1449,24 +1374,37 @@ __global__ void __launch_bounds__(256)
 }
 
 // Row i per block of the correction E: eigenvalues closer than
-// delta = 2 (||offdiag S|| + ||A|| ||R||) are treated as one cluster.
+// delta = 2 (||offdiag S|| + ||A|| ||R||) are treated as one cluster.  emax (zeroed) takes
+// the largest correction, 1 where a cluster still couples by more than 1e-13 ||A||.
 __global__ void __launch_bounds__(256)
     k_oa_correction(int n, const double* __restrict__ R, const double* __restrict__ S,
                     const double* __restrict__ lam, const double* __restrict__ acc,
-                    double* __restrict__ E) {
+                    double* __restrict__ E, float* __restrict__ emax) {
   const int i = blockIdx.x;
   const long long o = (long long)i * n;
   const double delta = 2.0 * (sqrt(acc[0]) + sqrt(acc[1]) * sqrt(acc[2]));
   const double li = lam[i];
+  float mag = 0.f;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
-    const double gap = lam[j] - li;
-    E[o + j] = (j == i || fabs(gap) <= delta) ? 0.5 * R[o + j] : (S[o + j] + lam[j] * R[o + j]) / gap;
+    const double gap = lam[j] - li, couple = S[o + j] + lam[j] * R[o + j];
+    const bool close = fabs(gap) <= delta;
+    const double e = (j == i || close) ? 0.5 * R[o + j] : couple / gap;
+    E[o + j] = e;
+    mag = fmaxf(mag, fabsf((float)e));
+    if (close && j != i && fabs(couple) > 1e-13 * sqrt(acc[1])) mag = 1.f;
   }
+  for (int k = 16; k > 0; k >>= 1) mag = fmaxf(mag, __shfl_xor_sync(0xffffffffu, mag, k));
+  if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(emax), __float_as_int(mag));
 }
 
-// X <- X + X E (row i per block; the row is staged before it is written).
-__global__ void k_oa_update(int n, double* __restrict__ X, const double* __restrict__ E) {
+constexpr float OA_BAD = 1e-8f;  // a correction this small leaves an error of its square
+
+// X <- X + X E (row i per block; the row is staged before it is written).  With `gate`
+// nothing is done unless *gate > OA_BAD.
+__global__ void k_oa_update(int n, double* __restrict__ X, const double* __restrict__ E,
+                            const float* __restrict__ gate = nullptr) {
   extern __shared__ double xrow[];
+  if (gate && !(*gate > OA_BAD)) return;
   const int i = blockIdx.x;
   for (int j = threadIdx.x; j < n; j += blockDim.x) xrow[j] = X[(long long)i * n + j];
   __syncthreads();
@@ -1483,8 +1421,11 @@ __global__ void k_oa_update(int n, double* __restrict__ X, const double* __restr
 }
 
 // Row i (block) of C = op(L) M (+ diag I): n up to 1024, two interleaved chains.
+// With `gate` nothing is done unless *gate > OA_BAD.
 __global__ void k_oa_rowmm(int n, const double* __restrict__ L, int tl, const double* __restrict__ M,
-                           double* __restrict__ C, double diag, double sign) {
+                           double* __restrict__ C, double diag, double sign,
+                           const float* __restrict__ gate = nullptr) {
+  if (gate && !(*gate > OA_BAD)) return;
   const int i = blockIdx.x;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     double s0 = 0.0, s1 = 0.0;
@@ -1505,7 +1446,8 @@ inline size_t dense_eig_bytes(int n) {
   return WsCarve::round(sizeof(float) * (size_t)ne * ne) * 2 +
          WsCarve::round(sizeof(float) * (size_t)npairs * BJ_W * BJ_W) + WsCarve::round(64) +
          WsCarve::round(sizeof(double) * (2 * BJ_SWEEPS + 4)) +
-         5 * WsCarve::round(sizeof(double) * (size_t)n * n) + WsCarve::round(sizeof(double) * n);
+         5 * WsCarve::round(sizeof(double) * (size_t)n * n) + WsCarve::round(sizeof(double) * n) +
+         WsCarve::round(sizeof(int) * rotate_ints(n));
 }
 
 // Eigenpairs of the symmetric n x n FP64 matrix A (n <= 1024): A <- diag(lambda),
@@ -1525,29 +1467,23 @@ fpca_status launch_dense_eig(fpca_ctx* ctx, int n, double* A, double* V, void* s
   double* U = c.take<double>(nn);
   double* S = c.take<double>(nn);
   double* lam = c.take<double>(n);
+  int* flag = c.take<int>(rotate_ints(n));
   double* E = U;  // U is dead once S is formed
+  float* emax = reinterpret_cast<float*>(done + 8);
   const int eb = (int)std::min<long long>(((long long)ne * ne + 255) / 256, 4096);
   k_bj_init<<<eb, 256, 0, ctx->stream>>>(n, ne, A, Af, Vf, done);
   FPCA_LAUNCHED(ctx, "eig_bj_init");
   cudaMemsetAsync(mass, 0, sizeof(double) * (2 * BJ_SWEEPS + 4), ctx->stream);
-  if (nb > 1) {
-    for (int sweep = 0; sweep < BJ_SWEEPS; ++sweep) {
-      for (int r = 0; r < nb - 1; ++r) {
-        k_bj_sub<<<npairs, 768, 0, ctx->stream>>>(ne, r, Af, Jg, done);
-        FPCA_LAUNCHED(ctx, "eig_bj_sub");
-        k_bj_apply<<<dim3(npairs, npairs + ne / BJ_W), 256, 0, ctx->stream>>>(
-            ne, r, Af, Vf, Jg, done, r == nb - 2 ? mass + 2 * sweep : nullptr);
-        FPCA_LAUNCHED(ctx, "eig_bj_apply");
-      }
-      k_bj_check<<<1, 32, 0, ctx->stream>>>(mass + 2 * sweep, BJ_TOL, done);
-      FPCA_LAUNCHED(ctx, "eig_bj_check");
+  for (int sweep = 0; sweep < BJ_SWEEPS; ++sweep) {
+    for (int r = 0; r < nb - 1; ++r) {
+      k_bj_sub<<<npairs, BJ_NT, 0, ctx->stream>>>(ne, r, Af, Jg, done);
+      FPCA_LAUNCHED(ctx, "eig_bj_sub");
+      k_bj_apply<<<dim3(npairs, npairs + ne / BJ_W), 256, 0, ctx->stream>>>(
+          ne, r, Af, Vf, Jg, done, r == nb - 2 ? mass + 2 * sweep : nullptr);
+      FPCA_LAUNCHED(ctx, "eig_bj_apply");
     }
-  } else {
-    // a single subproblem holds the whole (padded) matrix
-    k_bj_sub<<<1, 768, 0, ctx->stream>>>(ne, 0, Af, Jg, done);
-    FPCA_LAUNCHED(ctx, "eig_bj_sub");
-    k_bj_apply_v<<<dim3(ne / BJ_W, 1), 256, 0, ctx->stream>>>(ne, 0, Vf, Jg, done);
-    FPCA_LAUNCHED(ctx, "eig_bj_apply_v");
+    k_bj_check<<<1, 32, 0, ctx->stream>>>(mass + 2 * sweep, BJ_TOL, done);
+    FPCA_LAUNCHED(ctx, "eig_bj_check");
   }
   const int xb = (int)std::min<long long>(((long long)nn + 255) / 256, 4096);
   k_bj_extract<<<xb, 256, 0, ctx->stream>>>(n, ne, Vf, A, X, As);
@@ -1562,13 +1498,30 @@ fpca_status launch_dense_eig(fpca_ctx* ctx, int n, double* A, double* V, void* s
     FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
     double* acc = mass + 2 * BJ_SWEEPS + 1;
     cudaMemsetAsync(acc, 0, sizeof(double) * 3, ctx->stream);
+    cudaMemsetAsync(emax, 0, sizeof(float), ctx->stream);
     k_oa_norms<<<n, 256, 0, ctx->stream>>>(n, As, R, S, lam, acc);
     FPCA_LAUNCHED(ctx, "eig_oa_norms");
-    k_oa_correction<<<n, 256, 0, ctx->stream>>>(n, R, S, lam, acc, E);
+    k_oa_correction<<<n, 256, 0, ctx->stream>>>(n, R, S, lam, acc, E, emax);
     FPCA_LAUNCHED(ctx, "eig_oa_correction");
     k_oa_update<<<n, tpb, sizeof(double) * n, ctx->stream>>>(n, X, E);
     FPCA_LAUNCHED(ctx, "eig_oa_update");
   }
+  // eigenvalues closer than the couplings that the FP32 sweeps left: X made orthonormal again
+  // (Newton-Schulz steps X <- X + X (I - X'X) / 2, from the 0.1 or so that corrections beyond
+  // their first order leave), S anew and FP64 Jacobi; nothing happens where the last step's
+  // corrections were small
+  for (int step = 0; step < 5; ++step) {
+    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, X, R, 0.5, -0.5, emax);
+    FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
+    k_oa_update<<<n, tpb, sizeof(double) * n, ctx->stream>>>(n, X, R, emax);
+    FPCA_LAUNCHED(ctx, "eig_oa_update");
+  }
+  k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, As, 0, X, U, 0.0, 1.0, emax);
+  FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
+  k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, U, S, 0.0, 1.0, emax);
+  FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
+  fpca_status cr = launch_rotate(ctx, n, emax, OA_BAD, S, lam, X, R, U, mass, flag);
+  if (cr != FPCA_OK) return cr;
   k_rr_out<<<xb, 256, 0, ctx->stream>>>(n, lam, X, A, V);
   FPCA_LAUNCHED(ctx, "eig_out");
   return FPCA_OK;
@@ -1646,6 +1599,7 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
   const long long PP = (long long)P * P;
   const double dv = 1.0 / (double)P;
   const int n = full ? P : l;
+  const size_t dense_bytes = !full ? 0 : lead_eig_takes(P) ? lead_eig_bytes(P, k) : dense_eig_bytes(n);
   const size_t need = WsCarve::round(sizeof(TS) * PP) + WsCarve::round(sizeof(double) * 4) +
                       4 * WsCarve::round(sizeof(TS) * (size_t)P * l) +
                       2 * WsCarve::round(sizeof(double) * (size_t)l * l) +
@@ -1654,7 +1608,7 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
                       WsCarve::round(sizeof(double) * gram_part_doubles(P, l, ctx->num_sms)) +
                       WsCarve::round(sizeof(double) * (5 * (size_t)l * l + l)) +
                       WsCarve::round(sizeof(float) * proj_part_floats(P, l, ctx->num_sms)) +
-                      (full ? WsCarve::round(dense_eig_bytes(n)) : 0) + 4096;
+                      (full ? WsCarve::round(dense_bytes) : 0) + 4096;
   void* ws = fpca_workspace(ctx, need);
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace (%zu bytes)", need);
   WsCarve carve(ws);
@@ -1672,15 +1626,24 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
   double* part = carve.take<double>(gram_part_doubles(P, l, ctx->num_sms));
   double* rrs = carve.take<double>(5 * (size_t)l * l + l);
   float* ppart = carve.take<float>(proj_part_floats(P, l, ctx->num_sms));
-  char* dense = full ? carve.take<char>(dense_eig_bytes(n)) : nullptr;
+  char* dense = full ? carve.take<char>(dense_bytes) : nullptr;
 
   cudaMemsetAsync(trace, 0, sizeof(double), ctx->stream);
   k_matrixize<TG, TS><<<dim3((P + 31) / 32, (P + 31) / 32), dim3(32, 8), 0, ctx->stream>>>(
       P, gamma, domain, S, trace);
   FPCA_LAUNCHED(ctx, "matrixize");
   if (full) {
-    // dense eigenpairs of Sigma (FP64 copy)
+    // dense eigenpairs of Sigma (FP64)
     if constexpr (sizeof(TS) == 8) {
+      if (lead_eig_takes(P)) {
+        // A: the eigenvalues as a vector (row stride 0 below), order: 0..k-1
+        fpca_status ls = launch_lead_eig(ctx, P, k, S, A, evecs, order, dense);
+        if (ls != FPCA_OK) return ls;
+        k_finish<<<k, 1024, 0, ctx->stream>>>(P, 0, k, dv, 1.0 / std::sqrt(dv), A, order, trace,
+                                              evals, evecs, fve);
+        FPCA_LAUNCHED(ctx, "eig_finish");
+        return FPCA_OK;
+      }
       cudaMemcpyAsync(A, S, sizeof(double) * PP, cudaMemcpyDeviceToDevice, ctx->stream);
     } else {
       return fpca_fail(ctx, FPCA_E_UNSUPPORTED, "dense eigensolver needs FP64 gamma");

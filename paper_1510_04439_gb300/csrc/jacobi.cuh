@@ -1,0 +1,125 @@
+// Jacobi building blocks shared by the eigensolvers (eig.cu, eig_dense.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace fpca_jacobi {
+
+// Pair (p, q), p < q, of position i (0 <= i < ne / 2) at step `step` of a sweep of
+// the round-robin (circle) schedule: ne / 2 disjoint pairs per step, ne - 1 steps
+// (ne even; q == n marks the dummy of odd n).
+__device__ __forceinline__ void rr_pair(int ne, int step, int i, int& p, int& q) {
+  const int m = ne - 1;
+  if (i == 0) {
+    p = m;
+    q = step;
+  } else {
+    p = step + i;
+    if (p >= m) p -= m;
+    q = step - i;
+    if (q < 0) q += m;
+  }
+  if (p > q) {
+    const int t = p;
+    p = q;
+    q = t;
+  }
+}
+
+// The rotation (c, s) that annihilates a_pq: tau = (a_qq - a_pp) / (2 a_pq),
+// t = sign(tau) / (|tau| + sqrt(1 + tau^2)), c = 1 / sqrt(1 + t^2), s = t c.
+// The quotients and 1 / sqrt(1 + t^2) (argument in [1, 2]) use the fast
+// approximate forms: c^2 + s^2 = 1 then holds to a few FP32 ulps, and the
+// refinement that follows the FP32 Jacobi restores orthogonality anyway.  The
+// square root of 1 + tau^2 stays exact so that tau^2 = inf still gives t = 0.
+__device__ __forceinline__ void rr_rot(const float* A, int ld, int n, int p, int q, float& c,
+                                       float& sn) {
+  c = 1.f;
+  sn = 0.f;
+  if (q >= n) return;
+  const float apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
+  if (fabsf(apq) > 1e-30f && fabsf(apq) > 1e-18f * sqrtf(fabsf(app) * fabsf(aqq))) {
+    const float tau = __fdividef(aqq - app, 2.f * apq);
+    const float t = __fdividef(tau >= 0.f ? 1.f : -1.f, fabsf(tau) + sqrtf(1.f + tau * tau));
+    c = rsqrtf(1.f + t * t);
+    sn = t * c;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// block Jacobi (dense symmetric eigensolver)
+// ---------------------------------------------------------------------------
+constexpr int BJ_S = 16;        // indices per block
+constexpr int BJ_W = 2 * BJ_S;  // subproblem width
+constexpr int BJ_NT = 256;      // threads of a subproblem sweep: one per 2 x 2 block
+
+// local index i of the subproblem of block pair (I, J) -> global index
+__device__ __forceinline__ int bj_index(int I, int J, int i) {
+  return i < BJ_S ? I * BJ_S + i : J * BJ_S + (i - BJ_S);
+}
+
+// The 16 disjoint pairs of step s of a subproblem sweep: `within` (s = 0..14) the pairs
+// inside either block, otherwise (s = 0..15) the pairs across the two blocks.
+__device__ __forceinline__ void bj_step_pair(bool within, int s, int i, int& p, int& q) {
+  if (within) {
+    rr_pair(BJ_S, s, i & 7, p, q);
+    p += (i >> 3) * BJ_S;
+    q += (i >> 3) * BJ_S;
+  } else {
+    p = i;
+    q = BJ_S + ((i + s) & (BJ_S - 1));
+  }
+}
+
+// One sweep of rotations over the 32 x 32 subproblem in `cur` (ld 33, double-buffered with
+// `nxt`), accumulated into J (32 x 32, leading dimension ldj, identity on entry).  The
+// pairs across the blocks meet once; those inside a block only when `within` is set
+// (once per sweep of the whole matrix is enough, since each block takes part in every
+// round).  Sixteen threads form a step's rotations, then each of the 256 threads turns one
+// 2 x 2 block of A and two entry pairs of J: about 0.17 us a step, where every thread
+// forming its own two rotations was bound by its instruction count (0.7 us with 768
+// threads).
+__device__ __forceinline__ void bj_sweep(float* cur, float* nxt, float* J, int ldj, float* cs,
+                                         bool within) {
+  constexpr int ld = BJ_W + 1;
+  const int bi = threadIdx.x >> 4, bj = threadIdx.x & 15;
+  const int nw = within ? BJ_S - 1 : 0;
+  for (int st = 0; st < nw + BJ_S; ++st) {
+    const bool in = st < nw;
+    const int s = in ? st : st - nw;
+    if (threadIdx.x < 16) {
+      int p, q;
+      float c, sn;
+      bj_step_pair(in, s, threadIdx.x, p, q);
+      rr_rot(cur, ld, BJ_W, p, q, c, sn);
+      cs[2 * threadIdx.x] = c;
+      cs[2 * threadIdx.x + 1] = sn;
+    }
+    int pi, qi, pj, qj;
+    bj_step_pair(in, s, bi, pi, qi);
+    bj_step_pair(in, s, bj, pj, qj);
+    __syncthreads();
+    const float ci = cs[2 * bi], si = cs[2 * bi + 1], cj = cs[2 * bj], sj = cs[2 * bj + 1];
+    const float m00 = cur[pi * ld + pj], m01 = cur[pi * ld + qj];
+    const float m10 = cur[qi * ld + pj], m11 = cur[qi * ld + qj];
+    const float c00 = cj * m00 - sj * m01, c01 = sj * m00 + cj * m01;
+    const float c10 = cj * m10 - sj * m11, c11 = sj * m10 + cj * m11;
+    nxt[pi * ld + pj] = ci * c00 - si * c10;
+    nxt[pi * ld + qj] = ci * c01 - si * c11;
+    nxt[qi * ld + pj] = si * c00 + ci * c10;
+    nxt[qi * ld + qj] = si * c01 + ci * c11;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float* row = J + (bi + 16 * h) * ldj;
+      const float vp = row[pj], vq = row[qj];
+      row[pj] = cj * vp - sj * vq;
+      row[qj] = sj * vp + cj * vq;
+    }
+    __syncthreads();
+    float* t = cur;
+    cur = nxt;
+    nxt = t;
+  }
+}
+
+}  // namespace fpca_jacobi
