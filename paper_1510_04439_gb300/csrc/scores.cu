@@ -4,10 +4,11 @@
 // By the push-through identity Lambda Phi' (Phi Lambda Phi' + sigma^2 I)^{-1} =
 // (sigma^2 Lambda^{-1} + Phi'Phi)^{-1} Phi', each subject needs only the L x L
 // system (sigma^2 Lambda^{-1} + Phi_i'Phi_i) A_i = Phi_i' Y_i^C instead of an
-// N_i x N_i one: one warp accumulates Phi_i'Phi_i and Phi_i'Y_i^C over the
-// subject's observations (in chunks of 32 staged in shared memory), one lane
-// solves by Cholesky in FP64.  Functions known on the grid are read at the bin
-// of each observation (Section 3.2 binning).
+// N_i x N_i one.  Scattered data: one warp accumulates both sums over the subject's
+// observations.  Gridded data: the Phi_i'Phi_i of all subjects are one integer
+// matrix product on the tensor cores (k_pace_gram).  The systems are solved in
+// float-float with one FP64 refinement (pace_solve).  Functions known on the grid
+// are read at the bin of each observation (Section 3.2 binning).
 //
 // Scores by integration (dense data): A_il = dV sum over observed nodes of
 // (Y_i - mu) phi_l; reconstruction X_i = mu + sum_l A_il phi_l at the nodes; the
@@ -18,9 +19,11 @@
 // compensated dot product of Ogita, Rump and Oishi, "Accurate sum and dot
 // product", 2005, on float-float inputs from ff.cuh): about FP64 accuracy at
 // FP32 cost, since FP64 throughput on this GPU is 1/64 of FP32.  mu and phi are
-// split into float-float once per call; the small L x L solves stay FP64.
+// split into float-float once per call.
 #include <algorithm>
 #include <cmath>
+
+#include <cuda_fp16.h>
 
 #include "fpca_internal.cuh"
 #include "ff.cuh"
@@ -69,172 +72,582 @@ __device__ __forceinline__ ff::F2 centred(const void* y, int yprec, long long e,
   return ff::fast_two_sum(t.hi, t.lo - m.lo);
 }
 
-// out[e] = float-float split of in[e]
-__global__ void k_split_ff(long long n, const double* __restrict__ in, float2* __restrict__ out) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-       e += (long long)gridDim.x * blockDim.x) {
+// mu (row 0) and the first L eigenfunctions (rows 1..L) as float-float; bmax (NULL or
+// L x gridDim.x): each block's largest |phi_l|, rounded up, infinity if one is not finite.
+__global__ void __launch_bounds__(256)
+    k_split_ff(int P, const double* __restrict__ mu, const double* __restrict__ phi,
+               float2* __restrict__ mu2, float2* __restrict__ phi2, float* __restrict__ bmax) {
+  __shared__ float wmax[8];
+  const int l = (int)blockIdx.y - 1;
+  const double* in = l < 0 ? mu : phi + (long long)l * P;
+  float2* out = l < 0 ? mu2 : phi2 + (long long)l * P;
+  float top = 0.f;
+  for (int e = blockIdx.x * 256 + threadIdx.x; e < P; e += gridDim.x * 256) {
     const ff::F2 v = split(in[e]);
     out[e] = make_float2(v.hi, v.lo);
+    const float a = __double2float_ru(fabs(in[e]));
+    top = isfinite(a) ? fmaxf(top, a) : INFINITY;
+  }
+  if (l < 0 || !bmax) return;
+  for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = top;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) top = fmaxf(top, wmax[w]);
+    bmax[(long long)l * gridDim.x + blockIdx.x] = top;
   }
 }
 
-// layout 0: dense y (n x P, FP32/FP64 per yprec) with mask (or NULL);
-// layout 1: scattered offs / t / y (FP64).  mu2 (P) and phi2 (L x P) float-float.
-// WPS warps share a subject (its observations in chunks of 32, dealt round-robin);
-// their partial sums are added in FP64 through shared memory before one thread
-// solves.  Gridded data use WPS = 8 (thousands of nodes per subject), scattered
-// data WPS = 1 with 4 subjects per block.
-template <int WPS>
-constexpr int pace_threads() { return WPS == 1 ? 128 : 256; }
+// ---------------------------------------------------------------------------
+// the L x L systems
+// ---------------------------------------------------------------------------
 
-template <int WPS>
-__global__ void __launch_bounds__(pace_threads<WPS>())
-    k_scores_pace(ScGrid g, int n, int layout, const void* __restrict__ y, int yprec,
-                  const uint8_t* __restrict__ mask, const int64_t* __restrict__ offs,
+// A a = b by Cholesky in FP64, in place; false if A is not positive definite.
+__device__ bool solve_serial(double (*A)[SC_LMAX + 1], double* bb, int L) {
+  for (int jj = 0; jj < L; ++jj) {
+    double dj = A[jj][jj];
+    for (int k = 0; k < jj; ++k) dj -= A[jj][k] * A[jj][k];
+    if (!(dj > 0.0)) return false;
+    const double ljj = sqrt(dj), il = 1.0 / ljj;
+    A[jj][jj] = ljj;
+    for (int r = jj + 1; r < L; ++r) {
+      double v = A[r][jj];
+      for (int k = 0; k < jj; ++k) v -= A[r][k] * A[jj][k];
+      A[r][jj] = v * il;
+    }
+  }
+  for (int r = 0; r < L; ++r) {
+    double v = bb[r];
+    for (int k = 0; k < r; ++k) v -= A[r][k] * bb[k];
+    bb[r] = v / A[r][r];
+  }
+  for (int r = L - 1; r >= 0; --r) {
+    double v = bb[r];
+    for (int k = r + 1; k < L; ++k) v -= A[k][r] * bb[k];
+    bb[r] = v / A[r][r];
+  }
+  return true;
+}
+
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+template <int W>
+__device__ __forceinline__ ff::F2 shfl_ff(ff::F2 a, int src) {
+  return {__shfl_sync(0xffffffffu, a.hi, src, W), __shfl_sync(0xffffffffu, a.lo, src, W)};
+}
+
+// Shared memory of one subject's system.
+struct PaceSys {
+  double A[SC_LMAX][SC_LMAX + 1];  // Phi'Phi, both triangles
+  double b[SC_LMAX];               // Phi'Y^C, then the scores
+  double x[SC_LMAX];
+  float2 low[SC_LMAX][SC_LMAX + 1];
+};
+
+// (A + diag(add)) a = b for 32 / RL subjects of a warp, RL lanes each (lane r owns row r),
+// the scores left in sys->b.  A chain of dependent FP64 operations is what one thread's
+// FP64 Cholesky would wait on (~135 ns each here), so the factor is taken in float-float of
+// the system scaled to a unit-size diagonal by powers of two, and the solution refined once
+// with the FP64 residual: its error is the square of the float-float solve's, below FP64's
+// own for what passes the test on the correction (2^-25 of the solution).  What does not
+// pass (near-singular, not finite, extreme scales) is solved by one lane in FP64.
+template <int RL>
+__device__ void pace_solve(PaceSys* sys, const double* add, int L, bool valid, bool active,
+                           int* err) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, r = lane % RL;
+  const unsigned seg = (RL == 32 ? full : ((1u << RL) - 1u)) << (lane / RL * RL);
+  const bool in = r < L;
+  if (active && in) sys->A[r][r] += add[r];
+  __syncwarp();
+  const double dg = in && active ? sys->A[r][r] : 1.0, br = in && active ? sys->b[r] : 0.0;
+  const int ex = ((__double2hiint(dg) >> 20) & 0x7ff) - 1023;
+  bool fast = valid && dg > 0.0 && ex > -500 && ex < 500;
+  const int sr = fast ? -(ex >> 1) : 0;  // 2^sr scales row and column r
+  int eb = __double2hiint(br) & 0x7fffffff;
+  for (int o = RL / 2; o > 0; o >>= 1) eb = max(eb, __shfl_xor_sync(full, eb, o, RL));
+  eb = eb == 0 ? 0 : (eb >> 20) - 1023;
+  if (eb < -500 || eb > 500) {
+    fast = false;
+    eb = 0;
+  }
+  ff::F2 a[RL];
+#pragma unroll
+  for (int c = 0; c < RL; ++c) {
+    const int sc = __shfl_sync(full, sr, c, RL);
+    a[c] = in && active && c < L ? split(sys->A[r][c] * pow2(sr + sc)) : ff::make(c == r ? 1.f : 0.f);
+  }
+  ff::F2 inv = ff::make(1.f);
+#pragma unroll
+  for (int j = 0; j < RL; ++j) {
+    const ff::F2 p = shfl_ff<RL>(a[j], j);
+    if (!(p.hi > 1e-7f)) fast = false;
+    // 1 / sqrt(p): the FP32 value and one Newton step
+    const float y0 = rsqrtf(fmaxf(p.hi, 1e-7f));
+    const ff::F2 e = ff::add(ff::make(1.f), ff::neg(ff::mul(p, ff::two_prod(y0, y0))));
+    const ff::F2 iv = ff::fast_two_sum(y0, 0.5f * y0 * e.hi);
+    if (r == j) inv = iv;
+    a[j] = ff::mul(a[j], iv);  // column j of the factor
+    if (active) sys->low[r][j] = make_float2(a[j].hi, a[j].lo);
+#pragma unroll
+    for (int c = j + 1; c < RL; ++c) a[c] = ff::sub_mul(a[c], a[j], shfl_ff<RL>(a[j], c));
+  }
+  __syncwarp();
+  auto solve = [&](ff::F2 v) {
+    ff::F2 z = v;
+#pragma unroll
+    for (int k = 0; k < RL; ++k) {
+      const ff::F2 xk = shfl_ff<RL>(ff::mul(z, inv), k);
+      if (r == k) z = xk;
+      if (r > k) z = ff::sub_mul(z, a[k], xk);
+    }
+#pragma unroll
+    for (int k = RL - 1; k >= 0; --k) {
+      const ff::F2 xk = shfl_ff<RL>(ff::mul(z, inv), k);
+      if (r == k) z = xk;
+      if (r < k) {
+        const float2 lo = sys->low[k][r];
+        z = ff::sub_mul(z, ff::F2{lo.x, lo.y}, xk);
+      }
+    }
+    return z;
+  };
+  const ff::F2 x0 = solve(split(br * pow2(sr - eb)));
+  if (active && in) sys->x[r] = ff::to_double(x0) * pow2(sr);
+  __syncwarp();
+  double r0 = br * pow2(-eb), r1 = 0.0;
+  if (active && in) {
+#pragma unroll
+    for (int c = 0; c < RL; c += 2) {
+      if (c < L) r0 = fma(-sys->A[r][c], sys->x[c], r0);
+      if (c + 1 < L) r1 = fma(-sys->A[r][c + 1], sys->x[c + 1], r1);
+    }
+  }
+  const ff::F2 dx = solve(split((r0 + r1) * pow2(sr)));
+  float mx = fabsf(x0.hi), md = fabsf(dx.hi);
+  if (!(mx < INFINITY) || !(md < INFINITY)) fast = false;
+  for (int o = RL / 2; o > 0; o >>= 1) {
+    mx = fmaxf(mx, __shfl_xor_sync(full, mx, o, RL));
+    md = fmaxf(md, __shfl_xor_sync(full, md, o, RL));
+  }
+  if (!(md <= 0x1p-25f * mx)) fast = false;
+  const bool good = (__ballot_sync(full, !fast) & seg) == 0;
+  if (active && good && in)
+    sys->b[r] = (ff::to_double(x0) + ff::to_double(dx)) * pow2(sr) * pow2(eb);
+  if (active && !good && r == 0) {
+    if (!valid || !solve_serial(sys->A, sys->b, L)) {
+      atomicExch(err, DERR_NUMERIC);
+      for (int k = 0; k < L; ++k) sys->b[k] = __longlong_as_double(0x7ff8000000000000ll);
+    }
+  }
+  __syncwarp();
+}
+
+// sigma^2 / lambda_l into add, by the first L threads of a block, and whether the prior is
+// one: sigma^2 >= 0 and every lambda > 0.  Ends in a __syncthreads.
+__device__ bool pace_prior(const double* lam, const double* sigma2p, int L, double* add) {
+  const double sigma2 = *sigma2p;
+  const bool bad = !(sigma2 >= 0.0) || ((int)threadIdx.x < L && !(lam[threadIdx.x] > 0.0));
+  if ((int)threadIdx.x < L) add[threadIdx.x] = sigma2 / lam[threadIdx.x];
+  return !__syncthreads_or(bad);
+}
+
+// Scattered data (offs / t / y in FP64), mu2 (P) and phi2 (L x P) float-float: a warp per
+// subject, its observations in chunks of 32 staged in shared memory, each lane a few of the
+// NE + L sums.  LM: 8 or 16 >= L; the four subjects of a block are solved together, LM
+// lanes each.  n = 20000, 5..20 points, 24 x 24, L = 8: see pace_solve for the solves, which
+// took most of the time when one lane of the warp ran them in FP64.
+template <int LM>
+__global__ void __launch_bounds__(128)
+    k_scores_pace(ScGrid g, int n, const void* __restrict__ y, const int64_t* __restrict__ offs,
                   const double* __restrict__ t, const float2* __restrict__ mu2,
                   const double* __restrict__ lam, const float2* __restrict__ phi2, int L,
                   const double* __restrict__ sigma2p, double* __restrict__ scores,
                   int* __restrict__ err) {
-  constexpr int PACE_THREADS = pace_threads<WPS>();
-  constexpr int NW = PACE_THREADS / 32;  // warps per block
-  constexpr int SPB = NW / WPS;          // subjects per block
-  constexpr int NEMAX = SC_LMAX * (SC_LMAX + 1) / 2 + SC_LMAX;
-  __shared__ float2 rows[NW][32][SC_LMAX + 1];  // phi rows, then the residual
-  __shared__ double part[NW][NEMAX];             // each warp's sums: G entries, then b
-  __shared__ double sysA[SPB][SC_LMAX][SC_LMAX + 1];
-  __shared__ double sysb[SPB][SC_LMAX];
+  constexpr int NS = (LM * (LM + 1) / 2 + LM + 31) / 32;  // sums per lane
+  __shared__ float2 rows[4][32][LM + 1];                   // phi rows, then the residual
+  __shared__ PaceSys sys[4];
+  __shared__ double add[SC_LMAX];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int slot = warp / WPS, wsub = warp % WPS;
   const int NE = L * (L + 1) / 2;
-  // Upper-triangle entries e = lane + 32 q (row-major) of Phi_i' Phi_i held by this lane.
-  int er[5], ec[5];
+  // Upper-triangle entries e = lane + 32 q (row-major) of Phi_i' Phi_i, then the L
+  // entries of Phi_i' Y_i^C, held by this lane; er == LM: none
+  int er[NS], ec[NS];
 #pragma unroll
-  for (int q = 0; q < 5; ++q) {
+  for (int q = 0; q < NS; ++q) {
     int r = 0, rem = lane + 32 * q;
-    while (r < L && rem >= L - r) {
+    if (rem >= NE) {
+      er[q] = rem - NE < L ? rem - NE : LM;
+      ec[q] = LM;
+      continue;
+    }
+    while (rem >= L - r) {
       rem -= L - r;
       ++r;
     }
-    er[q] = r;  // r == L: no entry
+    er[q] = r;
     ec[q] = r + rem;
   }
-  for (int i0 = blockIdx.x * SPB; i0 < n; i0 += gridDim.x * SPB) {
-    const int i = i0 + slot;
-    const bool active = i < n;
-    Acc accG[5];
-    Acc accb;  // entry lane (< L) of Phi_i' Y_i^C
-    long long j0 = 0, j1 = 0;
-    if (active) {
-      if (layout == 1) {
-        j0 = offs[i];
-        j1 = offs[i + 1];
-      } else {
-        j1 = g.P;
-      }
-    }
-    for (long long c0 = j0 + 32 * wsub; c0 < j1; c0 += 32 * WPS) {
+  const bool valid = pace_prior(lam, sigma2p, L, add);
+  const int i = blockIdx.x * 4 + warp;
+  if (i < n) {
+    Acc acc[NS];
+    const long long j0 = offs[i], j1 = offs[i + 1];
+    for (long long c0 = j0; c0 < j1; c0 += 32) {
       const long long j = c0 + lane;
-      int b = -1;
-      ff::F2 yc = ff::make(0.f);
-      if (j < j1) {
-        if (layout == 1) {
-          b = sc_bin(g, t + j * g.d);
-          const float2 m = mu2[b];
-          yc = split(static_cast<const double*>(y)[j] - ((double)m.x + (double)m.y));
-        } else if (!mask || mask[(long long)i * g.P + j]) {
-          b = (int)j;
-          const float2 m = mu2[b];
-          yc = centred(y, yprec, (long long)i * g.P + j, ff::F2{m.x, m.y});
-        }
+      const int cnt = (int)(j1 - c0 < 32 ? j1 - c0 : 32);
+      if (lane < cnt) {
+        const int b = sc_bin(g, t + j * g.d);
+        const float2 m = mu2[b];
+        const ff::F2 yc = split(static_cast<const double*>(y)[j] - ((double)m.x + (double)m.y));
+        for (int l = 0; l < L; ++l) rows[warp][lane][l] = phi2[(long long)l * g.P + b];
+        rows[warp][lane][LM] = make_float2(yc.hi, yc.lo);
       }
-      for (int l = 0; l < L; ++l)
-        rows[warp][lane][l] = b >= 0 ? phi2[(long long)l * g.P + b] : make_float2(0.f, 0.f);
-      rows[warp][lane][SC_LMAX] = make_float2(yc.hi, yc.lo);
       __syncwarp();
 #pragma unroll
-      for (int q = 0; q < 5; ++q) {
-        if (er[q] < L) {
-          for (int k = 0; k < 32; ++k) {
+      for (int q = 0; q < NS; ++q) {
+        if (er[q] < LM) {
+          for (int k = 0; k < cnt; ++k) {
             const float2 a = rows[warp][k][er[q]], c = rows[warp][k][ec[q]];
-            accG[q].add_prod(ff::F2{a.x, a.y}, ff::F2{c.x, c.y});
+            acc[q].add_prod(ff::F2{a.x, a.y}, ff::F2{c.x, c.y});
           }
         }
       }
-      if (lane < L) {
-        for (int k = 0; k < 32; ++k) {
-          const float2 a = rows[warp][k][lane], c = rows[warp][k][SC_LMAX];
-          accb.add_prod(ff::F2{a.x, a.y}, ff::F2{c.x, c.y});
-        }
-      }
       __syncwarp();
     }
 #pragma unroll
-    for (int q = 0; q < 5; ++q)
-      if (er[q] < L) part[warp][lane + 32 * q] = accG[q].value();
-    if (lane < L) part[warp][NE + lane] = accb.value();
-    __syncthreads();
-    // the subject's sums, warps added in a fixed order
-    for (int e = threadIdx.x; e < SPB * (NE + L); e += PACE_THREADS) {
-      const int sl = e / (NE + L), k = e - sl * (NE + L);
-      double v = 0.0;
-      for (int w = 0; w < WPS; ++w) v += part[sl * WPS + w][k];
-      if (k < NE) {
-        int r = 0, rem = k;
-        while (rem >= L - r) {
-          rem -= L - r;
-          ++r;
-        }
-        sysA[sl][r][r + rem] = v;
-        sysA[sl][r + rem][r] = v;
+    for (int q = 0; q < NS; ++q) {
+      if (er[q] == LM) continue;
+      const double v = acc[q].value();
+      if (ec[q] == LM) {
+        sys[warp].b[er[q]] = v;
       } else {
-        sysb[sl][k - NE] = v;
+        sys[warp].A[er[q]][ec[q]] = v;
+        sys[warp].A[ec[q]][er[q]] = v;
       }
     }
-    __syncthreads();
-    if (wsub == 0 && lane == 0 && active) {
-      // (sigma^2 Lambda^{-1} + G) a = b by Cholesky in FP64, solved in place in bb.
-      double (*A)[SC_LMAX + 1] = sysA[slot];
-      double* bb = sysb[slot];
-      const double sigma2 = *sigma2p;
-      bool ok = sigma2 >= 0.0;
-      for (int l = 0; l < L; ++l) {
-        if (!(lam[l] > 0.0)) ok = false;
-        A[l][l] += sigma2 / lam[l];
+  }
+  __syncthreads();
+  constexpr int SPW = 32 / LM;  // subjects per solving warp
+  if (warp < 4 / SPW) {
+    const int sl = warp * SPW + lane / LM;
+    pace_solve<LM>(&sys[sl], add, L, valid, blockIdx.x * 4 + sl < n, err);
+  }
+  __syncthreads();
+  if (i < n && lane < L) scores[(long long)i * L + lane] = sys[warp].b[lane];
+}
+
+// ---------------------------------------------------------------------------
+// gridded data
+// ---------------------------------------------------------------------------
+// (Phi_i'Phi_i)_ab = sum over nodes of mask_ip (phi_a phi_b)(p): a product of the 0/1 masks
+// (n x P) with a P x NE table that no subject changes.  The table's entries are rounded to
+// 54-bit fixed point relative to 2^(e_a + e_b) > max |phi_a| max |phi_b| and cut into five
+// digits of 11 bits, which FP16 holds exactly; sums of up to PG_NODES digits are integers
+// below 2^20, which the FP32 accumulators hold exactly, so the whole product is exact but for
+// the table's rounding, 2^-54 of the bound a node.  That is closer than the float-float sums
+// wherever a subject's mean phi_l^2 is above 2^-8 of the bound; a subject with a smaller one
+// is summed again in float-float (k_pace_final).
+constexpr int PG_DIG = 5;        // digits
+constexpr int PG_BITS = 11;
+constexpr int PG_FIX = 53;       // fixed-point bits
+constexpr int PG_EBAD = 1000;    // exponent of a function that the digits cannot hold
+constexpr int PG_EZERO = -1000;  // exponent of a function that is zero everywhere
+constexpr int PG_COUNT = PG_BITS * (PG_DIG - 1);  // a leading digit of 1, as a fixed-point value
+
+__host__ __device__ constexpr int pg_groups(int L) { return L * (L + 1) / 2 / 8 + 1; }
+
+// The table in the order in which the product's B fragments are read: 64 nodes are four
+// steps of 16; lane 4g + t of step j holds column g of the 8 and nodes 16 t + 4 j + {0..3},
+// so that a lane's four steps of mask bytes are 16 consecutive ones.  Columns NE: a one
+// (the subject's node count), beyond: zeros.  A block makes 64 nodes' worth.
+__global__ void __launch_bounds__(256)
+    k_pace_table(int P, int L, int nbx, const float* __restrict__ bmax,
+                 const double* __restrict__ phi, uint2* __restrict__ table,
+                 int* __restrict__ expo) {
+  __shared__ double ph[SC_LMAX][64];
+  __shared__ int ex[SC_LMAX];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int NE = L * (L + 1) / 2, ng = pg_groups(L), p0 = blockIdx.x * 64;
+  for (int l = warp; l < L; l += 8) {
+    float top = 0.f;
+    for (int b = lane; b < nbx; b += 32) top = fmaxf(top, bmax[(long long)l * nbx + b]);
+    for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if (lane == 0) {
+      int e = PG_EZERO;
+      if (top > 0.f) {
+        e = top < INFINITY ? ilogbf(top) + 1 : PG_EBAD;
+        if (e < -60 || e > 60) e = PG_EBAD;
       }
-      for (int jj = 0; jj < L && ok; ++jj) {
-        double dj = A[jj][jj];
-        for (int k = 0; k < jj; ++k) dj -= A[jj][k] * A[jj][k];
-        if (!(dj > 0.0)) {
-          ok = false;
-          break;
-        }
-        const double ljj = sqrt(dj), il = 1.0 / ljj;
-        A[jj][jj] = ljj;
-        for (int r = jj + 1; r < L; ++r) {
-          double v = A[r][jj];
-          for (int k = 0; k < jj; ++k) v -= A[r][k] * A[jj][k];
-          A[r][jj] = v * il;
-        }
+      ex[l] = e;
+      if (blockIdx.x == 0) expo[l] = e;
+    }
+  }
+  for (int e = threadIdx.x; e < L * 64; e += 256) {
+    const int l = e >> 6, p = p0 + (e & 63);
+    ph[l][e & 63] = p < P ? phi[(long long)l * P + p] : 0.0;
+  }
+  __syncthreads();
+  for (int it = threadIdx.x; it < ng * 128; it += 256) {
+    const int t = it & 3, gcol = (it >> 2) & 7, j = (it >> 5) & 3, grp = it >> 7;
+    const int e = grp * 8 + gcol;
+    int a = 0, rem = e;
+    while (a < L && rem >= L - a) {
+      rem -= L - a;
+      ++a;
+    }
+    const int b = a + rem;
+    unsigned short dig[PG_DIG][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int q = 16 * t + 4 * j + i;
+      long long x = 0;
+      if (e < NE) {
+        const int ea = ex[a], eb = ex[b];
+        if (ea > PG_EZERO && ea < PG_EBAD && eb > PG_EZERO && eb < PG_EBAD)
+          x = __double2ll_rn(ph[a][q] * ph[b][q] * pow2(PG_FIX - ea - eb));
+      } else if (e == NE && p0 + q < P) {
+        x = 1ll << PG_COUNT;
       }
-      if (ok) {
-        for (int r = 0; r < L; ++r) {
-          double v = bb[r];
-          for (int k = 0; k < r; ++k) v -= A[r][k] * bb[k];
-          bb[r] = v / A[r][r];
-        }
-        for (int r = L - 1; r >= 0; --r) {
-          double v = bb[r];
-          for (int k = r + 1; k < L; ++k) v -= A[k][r] * bb[k];
-          bb[r] = v / A[r][r];
-        }
-      } else {
-        atomicExch(err, DERR_NUMERIC);
-        for (int r = 0; r < L; ++r) bb[r] = __longlong_as_double(0x7ff8000000000000ll);
+#pragma unroll
+      for (int d = PG_DIG - 1; d >= 0; --d) {
+        const int half = 1 << (PG_BITS - 1);
+        const int dv = d ? (int)((x + half) & (2 * half - 1)) - half : (int)x;
+        x = (x - dv) >> PG_BITS;
+        dig[d][i] = __half_as_ushort(__int2half_rn(dv));
       }
     }
-    __syncthreads();
-    if (wsub == 0 && lane < L && active) scores[(long long)i * L + lane] = sysb[slot][lane];
-    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < PG_DIG; ++d)
+      table[((size_t)(blockIdx.x * 4 + j) * ng * PG_DIG + grp * PG_DIG + d) * 32 + gcol * 4 + t] =
+          make_uint2(dig[d][0] | (unsigned)dig[d][1] << 16, dig[d][2] | (unsigned)dig[d][3] << 16);
+  }
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const unsigned (&a)[4], uint2 b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+// 0xff for each nonzero byte of the mask's 16 nodes p..p+15 of a row (NULL: all observed),
+// zero beyond the grid
+__device__ __forceinline__ uint4 mask16(const uint8_t* __restrict__ row, int p, int P, int vec) {
+  uint4 w = make_uint4(0, 0, 0, 0);
+  if (vec && p < P) {
+    if (row) {
+      w = *reinterpret_cast<const uint4*>(row + p);
+      w.x = __vcmpne4(w.x, 0);
+      w.y = __vcmpne4(w.y, 0);
+      w.z = __vcmpne4(w.z, 0);
+      w.w = __vcmpne4(w.w, 0);
+    } else {
+      w = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+  } else if (!vec) {
+    unsigned u[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (p + i < P && (!row || row[p + i])) u[i >> 2] |= 0xffu << (8 * (i & 3));
+    w = make_uint4(u[0], u[1], u[2], u[3]);
+  }
+  return w;
+}
+
+// out[(split * nb + i) * 8 ng + e]: the fixed-point sums over the split's nodes.  A warp takes
+// 16 subjects (its A fragments come straight from the mask's bytes) and GP groups of 8
+// columns; blockIdx: x 128 subjects, y a split of `per` x 64 nodes, z GP groups.  1.5 GFLOP
+// at n = 1000, P = 4096, L = 8: bound by the table's reads from L1/L2, so the simpler
+// warp-level products are as good as tcgen05's here.
+template <int GP>
+__global__ void __launch_bounds__(256)
+    k_pace_gram(int nb, int i0, int P, int ng, int per, const uint8_t* __restrict__ mask,
+                const uint2* __restrict__ table, long long* __restrict__ out, int vec) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int gr = lane >> 2, t = lane & 3;
+  const int ra = blockIdx.x * 128 + warp * 16 + gr, rb = ra + 8;
+  if (ra - gr >= nb) return;
+  const int g0 = blockIdx.z * GP, gn = min(GP, ng - g0);
+  const int n64 = (P + 63) / 64, k0 = blockIdx.y * per, k1 = min(n64, k0 + per);
+  float acc[GP][PG_DIG][4] = {};
+  const bool oka = ra < nb, okb = rb < nb;
+  const uint8_t* rowa = mask ? mask + (size_t)(i0 + (oka ? ra : 0)) * P : nullptr;
+  const uint8_t* rowb = mask ? mask + (size_t)(i0 + (okb ? rb : 0)) * P : nullptr;
+  for (int k = k0; k < k1; ++k) {
+    const int p = k * 64 + t * 16;
+    uint4 wa = mask16(rowa, p, P, vec), wb = mask16(rowb, p, P, vec);
+    if (!oka) wa = make_uint4(0, 0, 0, 0);
+    if (!okb) wb = make_uint4(0, 0, 0, 0);
+    const unsigned ua[4] = {wa.x, wa.y, wa.z, wa.w}, ub[4] = {wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const unsigned one = 0x3c003c00u;  // 1.0 where the byte is set
+      const unsigned a[4] = {__byte_perm(ua[j], 0, 0x1404) & one, __byte_perm(ub[j], 0, 0x1404) & one,
+                             __byte_perm(ua[j], 0, 0x3424) & one, __byte_perm(ub[j], 0, 0x3424) & one};
+      const uint2* tb = table + ((size_t)(k * 4 + j) * ng + g0) * PG_DIG * 32 + lane;
+#pragma unroll
+      for (int q = 0; q < GP; ++q) {
+        if (q < gn) {
+#pragma unroll
+          for (int d = 0; d < PG_DIG; ++d) mma_f16(acc[q][d], a, tb[(q * PG_DIG + d) * 32]);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < GP; ++q) {
+    if (q >= gn) break;
+    long long v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      v[c] = 0;
+#pragma unroll
+      for (int d = 0; d < PG_DIG; ++d) v[c] = v[c] * (1 << PG_BITS) + (int)acc[q][d][c];
+    }
+    const size_t o = ((size_t)blockIdx.y * nb + ra) * (8 * ng) + (g0 + q) * 8 + 2 * t;
+    if (oka) *reinterpret_cast<longlong2*>(out + o) = make_longlong2(v[0], v[1]);
+    if (okb)
+      *reinterpret_cast<longlong2*>(out + o + (size_t)8 * 8 * ng) = make_longlong2(v[2], v[3]);
+  }
+}
+
+// Phi_i'Y_i^C of two subjects and their systems.  A thread keeps both subjects' L
+// compensated sums over every 256th node, so a phi value read serves two subjects; the
+// sums join by a halving butterfly of float-float adds (one add per sum instead of
+// five; FP64 adds there would take longer than the sums themselves), the warps in FP64.
+constexpr int PF_SUB = 2;
+template <int LM>
+__global__ void __launch_bounds__(256)
+    k_pace_final(int nb, int i0, int P, const void* __restrict__ y, int yprec,
+                 const uint8_t* __restrict__ mask, const float2* __restrict__ mu2,
+                 const double* __restrict__ lam, const float2* __restrict__ phi2, int L,
+                 const double* __restrict__ sigma2p, int nsplit, const int* __restrict__ expo,
+                 const long long* __restrict__ gsum, double* __restrict__ scores,
+                 int* __restrict__ err) {
+  constexpr int NV = PF_SUB * LM;
+  __shared__ PaceSys sys[PF_SUB];
+  __shared__ double add[SC_LMAX];
+  __shared__ float2 wsum[8][NV];
+  __shared__ double count[PF_SUB];
+  __shared__ int redo[PF_SUB];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L);
+  const int s0 = blockIdx.x * PF_SUB;
+  const bool valid = pace_prior(lam, sigma2p, L, add);
+  if (tid < PF_SUB) redo[tid] = 0;
+  for (int it = tid; it < PF_SUB * (NE + 1); it += 256) {
+    const int sl = it / (NE + 1), e = it - sl * (NE + 1);
+    if (s0 + sl >= nb) continue;
+    long long hi = 0, lo = 0;  // of the splits' fixed-point sums
+    for (int k = 0; k < nsplit; ++k) {
+      const long long v = gsum[((size_t)k * nb + s0 + sl) * ng8 + e];
+      hi += v >> 32;
+      lo += v & 0xffffffffll;
+    }
+    const double v = fma((double)hi, 4294967296.0, (double)lo);
+    if (e == NE) {
+      count[sl] = v * pow2(-PG_COUNT);
+      continue;
+    }
+    int a = 0, rem = e;
+    while (rem >= L - a) {
+      rem -= L - a;
+      ++a;
+    }
+    const int b = a + rem, es = expo[a] + expo[b];
+    const double ge = es > -200 && es < 200 ? v * pow2(es - PG_FIX) : 0.0;
+    sys[sl].A[a][b] = ge;
+    sys[sl].A[b][a] = ge;
+  }
+  Acc acc[PF_SUB][LM];
+  for (int p = tid; p < P; p += 256) {
+    const float2 m = mu2[p];
+    ff::F2 r[PF_SUB];
+    bool ok[PF_SUB], any = false;
+#pragma unroll
+    for (int u = 0; u < PF_SUB; ++u) {
+      const long long at = (long long)(i0 + s0 + u) * P + p;
+      ok[u] = s0 + u < nb && (!mask || mask[at]);
+      r[u] = ok[u] ? centred(y, yprec, at, ff::F2{m.x, m.y}) : ff::make(0.f);
+      any |= ok[u];
+    }
+    if (!any) continue;
+#pragma unroll
+    for (int l = 0; l < LM; ++l) {
+      if (l < L) {
+        const float2 f = phi2[(long long)l * P + p];
+#pragma unroll
+        for (int u = 0; u < PF_SUB; ++u)
+          acc[u][l].add_prod(r[u], ok[u] ? ff::F2{f.x, f.y} : ff::make(0.f));
+      }
+    }
+  }
+  ff::F2 v[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k)
+    v[k] = ff::fast_two_sum(acc[k / LM][k % LM].s, acc[k / LM][k % LM].c);
+  int at = 0;  // the sum that this lane ends with
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st, left = NV >> (st + 1);
+    const bool up = lane & o;
+    if (up) at += left;
+#pragma unroll
+    for (int k = 0; k < (left > 0 ? left : 1); ++k) {
+      const ff::F2 give = up || left == 0 ? v[k] : v[k + left];
+      const ff::F2 keep = up && left > 0 ? v[k + left] : v[k];
+      v[k] = ff::add(keep, ff::F2{__shfl_xor_sync(0xffffffffu, give.hi, o),
+                                  __shfl_xor_sync(0xffffffffu, give.lo, o)});
+    }
+  }
+  wsum[warp][at] = make_float2(v[0].hi, v[0].lo);
+  __syncthreads();
+  if (tid < NV && tid % LM < L) {
+    double sum = 0.0;
+    for (int w = 0; w < 8; ++w) sum += (double)wsum[w][tid].x + (double)wsum[w][tid].y;
+    sys[tid / LM].b[tid % LM] = sum;
+  }
+  if (tid < PF_SUB * L) {  // the bound of the table's rounding, see above
+    const int sl = tid / L, l = tid - sl * L, e = expo[l];
+    if (s0 + sl < nb && e > PG_EZERO &&
+        (e == PG_EBAD || !(sys[sl].A[l][l] >= count[sl] * pow2(2 * e - 8))))
+      redo[sl] = 1;
+  }
+  __syncthreads();
+  for (int sl = 0; sl < PF_SUB; ++sl) {
+    if (!redo[sl]) continue;
+    for (int a = 0; a < L; ++a) {
+      for (int b = a; b < L; ++b) {
+        Acc ac;
+        for (int p = tid; p < P; p += 256) {
+          if (mask && !mask[(long long)(i0 + s0 + sl) * P + p]) continue;
+          const float2 fa = phi2[(long long)a * P + p], fb = phi2[(long long)b * P + p];
+          ac.add_prod(ff::F2{fa.x, fa.y}, ff::F2{fb.x, fb.y});
+        }
+        ff::F2 sum = ff::fast_two_sum(ac.s, ac.c);
+        for (int o = 16; o > 0; o >>= 1)
+          sum = ff::add(sum, ff::F2{__shfl_xor_sync(0xffffffffu, sum.hi, o),
+                                    __shfl_xor_sync(0xffffffffu, sum.lo, o)});
+        if (lane == 0) wsum[warp][0] = make_float2(sum.hi, sum.lo);
+        __syncthreads();
+        if (tid == 0) {
+          double t = 0.0;
+          for (int w = 0; w < 8; ++w) t += (double)wsum[w][0].x + (double)wsum[w][0].y;
+          sys[sl].A[a][b] = t;
+          sys[sl].A[b][a] = t;
+        }
+        __syncthreads();
+      }
+    }
+  }
+  if (warp == 0) {
+    const int sl = lane / LM < PF_SUB ? lane / LM : PF_SUB - 1;
+    const bool active = lane / LM < PF_SUB && s0 + sl < nb;
+    pace_solve<LM>(&sys[sl], add, L, valid, active, err);
+    for (int e = lane; e < PF_SUB * L; e += 32)
+      if (s0 + e / L < nb) scores[(long long)(i0 + s0) * L + e] = sys[e / L].b[e % L];
   }
 }
 
@@ -384,20 +797,70 @@ bool sc_valid(fpca_ctx* ctx, const fpca_grid* g, int L) {
   return true;
 }
 
-// mu (P) and the first L eigenfunctions (L x P) as float-float in the workspace.
-fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double* evecs,
-                     float2** mu2, float2** phi2) {
-  const size_t nmu = (size_t)P, nphi = (size_t)L * P;
-  float2* ws = static_cast<float2*>(fpca_workspace(ctx, sizeof(float2) * (nmu + nphi)));
+// Gridded data in batches: the scratch of fpca_scores_pace does not grow with n, and the
+// other two calls ask for the same, so which of them ran first makes no difference to a
+// graph capture.
+constexpr int PG_BATCH = 16384;  // subjects x splits
+
+struct ScWork {
+  float2 *mu2, *phi2;  // mu (P) and the first L eigenfunctions (L x P) as float-float
+  float* bmax;         // L x nbx block maxima of |phi|
+  int* expo;           // L exponents
+  uint2* table;
+  long long* gsum;
+  const double* phi;
+  int nbx, nsplit, per, batch;
+};
+
+fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double* evecs, ScWork* w) {
+  const int n64 = (P + 63) / 64, ng = pg_groups(L);
+  w->phi = evecs;
+  w->nbx = std::min((P + 255) / 256, 64);
+  // 256 nodes a split, 512 on grids that make plenty of them: digit sums stay below 2^20,
+  // fixed-point sums below 2^63
+  w->per = n64 <= 64 ? 4 : 8;
+  w->nsplit = (n64 + w->per - 1) / w->per;
+  w->batch = std::max(128, PG_BATCH / w->nsplit / 128 * 128);
+  const size_t nt = (size_t)n64 * 4 * ng * PG_DIG * 32;
+  const size_t ns = (size_t)w->nsplit * w->batch * 8 * ng;
+  void* ws = fpca_workspace(ctx, WsCarve::round(sizeof(float2) * P) +
+                                     WsCarve::round(sizeof(float2) * (size_t)L * P) +
+                                     WsCarve::round(sizeof(float) * L * w->nbx) + 256 +
+                                     WsCarve::round(sizeof(uint2) * nt) +
+                                     WsCarve::round(sizeof(long long) * ns));
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
-  *mu2 = ws;
-  *phi2 = ws + nmu;
-  k_split_ff<<<(int)std::min<size_t>((nmu + 255) / 256, 4096), 256, 0, ctx->stream>>>(
-      (long long)nmu, mu, *mu2);
+  WsCarve c(ws);
+  w->mu2 = c.take<float2>(P);
+  w->phi2 = c.take<float2>((size_t)L * P);
+  w->bmax = c.take<float>((size_t)L * w->nbx);
+  w->expo = c.take<int>(SC_LMAX);
+  w->table = c.take<uint2>(nt);
+  w->gsum = c.take<long long>(ns);
+  k_split_ff<<<dim3(w->nbx, L + 1), 256, 0, ctx->stream>>>(P, mu, evecs, w->mu2, w->phi2, w->bmax);
   FPCA_LAUNCHED(ctx, "split_ff");
-  k_split_ff<<<(int)std::min<size_t>((nphi + 255) / 256, 4096), 256, 0, ctx->stream>>>(
-      (long long)nphi, evecs, *phi2);
-  FPCA_LAUNCHED(ctx, "split_ff");
+  return FPCA_OK;
+}
+
+fpca_status pace_dense(fpca_ctx* ctx, const fpca_data* data, int P, int L, const ScWork& w,
+                       const double* evals, const double* sigma2, double* scores) {
+  const int n64 = (P + 63) / 64, ng = pg_groups(L);
+  k_pace_table<<<n64, 256, 0, ctx->stream>>>(P, L, w.nbx, w.bmax, w.phi, w.table, w.expo);
+  FPCA_LAUNCHED(ctx, "pace_table");
+  // 16 mask bytes at once where rows are whole multiples of them
+  const int vec = P % 16 == 0 && (reinterpret_cast<uintptr_t>(data->mask) & 15) == 0;
+  for (int i0 = 0; i0 < data->n; i0 += w.batch) {
+    const int nb = std::min(w.batch, data->n - i0);
+    const int gp = ng <= 2 ? 2 : 5;
+    auto gram = gp == 2 ? k_pace_gram<2> : k_pace_gram<5>;
+    gram<<<dim3((nb + 127) / 128, w.nsplit, (ng + gp - 1) / gp), 256, 0, ctx->stream>>>(
+        nb, i0, P, ng, w.per, data->mask, w.table, w.gsum, vec);
+    FPCA_LAUNCHED(ctx, "pace_gram");
+    auto fin = L <= 8 ? k_pace_final<8> : k_pace_final<16>;
+    fin<<<(nb + PF_SUB - 1) / PF_SUB, 256, 0, ctx->stream>>>(
+        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, evals, w.phi2, L, sigma2, w.nsplit,
+        w.expo, w.gsum, scores, ctx->d_err);
+    FPCA_LAUNCHED(ctx, "scores_pace");
+  }
   return FPCA_OK;
 }
 
@@ -418,21 +881,17 @@ fpca_status fpca_scores_pace(fpca_ctx* ctx, const fpca_data* data, const fpca_gr
   if (data->layout == FPCA_SPARSE && (!data->offs || !data->t))
     return fpca_fail(ctx, FPCA_E_INVALID_ARG, "scattered data need offs and t");
   const ScGrid g = sc_grid(grid);
-  float2 *mu2 = nullptr, *phi2 = nullptr;
-  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &mu2, &phi2);
+  ScWork w;
+  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w);
   if (s != FPCA_OK) return s;
   if (data->layout == FPCA_SPARSE) {
-    const int blocks = (data->n + 3) / 4;
-    k_scores_pace<1><<<blocks, pace_threads<1>(), 0, ctx->stream>>>(
-        g, data->n, 1, data->y, data->y_prec, data->mask, data->offs, data->t, mu2, evals, phi2,
-        L, sigma2, scores, ctx->d_err);
-  } else {
-    k_scores_pace<8><<<data->n, pace_threads<8>(), 0, ctx->stream>>>(
-        g, data->n, 0, data->y, data->y_prec, data->mask, data->offs, data->t, mu2, evals, phi2,
-        L, sigma2, scores, ctx->d_err);
+    auto kern = L <= 8 ? k_scores_pace<8> : k_scores_pace<16>;
+    kern<<<(data->n + 3) / 4, 128, 0, ctx->stream>>>(g, data->n, data->y, data->offs, data->t, w.mu2,
+                                                     evals, w.phi2, L, sigma2, scores, ctx->d_err);
+    FPCA_LAUNCHED(ctx, "scores_pace");
+    return FPCA_OK;
   }
-  FPCA_LAUNCHED(ctx, "scores_pace");
-  return FPCA_OK;
+  return pace_dense(ctx, data, g.P, L, w, evals, sigma2, scores);
 }
 
 fpca_status fpca_scores_integral(fpca_ctx* ctx, const fpca_data* data, const fpca_grid* grid,
@@ -445,16 +904,16 @@ fpca_status fpca_scores_integral(fpca_ctx* ctx, const fpca_data* data, const fpc
   if (data->layout != FPCA_DENSE || !data->y || data->n < 1)
     return fpca_fail(ctx, FPCA_E_INVALID_ARG, "scores by integration need gridded (dense) data");
   const ScGrid g = sc_grid(grid);
-  float2 *mu2 = nullptr, *phi2 = nullptr;
-  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &mu2, &phi2);
+  ScWork w;
+  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w);
   if (s != FPCA_OK) return s;
   const double dv = 1.0 / (double)g.P;
   if (L <= 8)
     k_scores_integral<8><<<data->n, 256, 0, ctx->stream>>>(data->n, g.P, data->y, data->y_prec,
-                                                           data->mask, mu2, phi2, L, dv, scores);
+                                                           data->mask, w.mu2, w.phi2, L, dv, scores);
   else
     k_scores_integral<16><<<data->n, 256, 0, ctx->stream>>>(data->n, g.P, data->y, data->y_prec,
-                                                            data->mask, mu2, phi2, L, dv, scores);
+                                                            data->mask, w.mu2, w.phi2, L, dv, scores);
   FPCA_LAUNCHED(ctx, "scores_integral");
   return FPCA_OK;
 }
@@ -470,14 +929,14 @@ fpca_status fpca_reconstruct(fpca_ctx* ctx, const fpca_grid* grid, const double*
   const int nsub = (n + RC_SUB - 1) / RC_SUB;
   if (nsub > 65535) return fpca_fail(ctx, FPCA_E_UNSUPPORTED, "more than 2^20 subjects per call");
   const ScGrid g = sc_grid(grid);
-  float2 *mu2 = nullptr, *phi2 = nullptr;
-  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &mu2, &phi2);
+  ScWork w;
+  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w);
   if (s != FPCA_OK) return s;
   const dim3 grid2((g.P + 255) / 256, nsub);
   if (L <= 8)
-    k_reconstruct<8><<<grid2, 256, 0, ctx->stream>>>(n, g.P, mu2, phi2, L, scores, xhat);
+    k_reconstruct<8><<<grid2, 256, 0, ctx->stream>>>(n, g.P, w.mu2, w.phi2, L, scores, xhat);
   else
-    k_reconstruct<16><<<grid2, 256, 0, ctx->stream>>>(n, g.P, mu2, phi2, L, scores, xhat);
+    k_reconstruct<16><<<grid2, 256, 0, ctx->stream>>>(n, g.P, w.mu2, w.phi2, L, scores, xhat);
   FPCA_LAUNCHED(ctx, "reconstruct");
   return FPCA_OK;
 }
