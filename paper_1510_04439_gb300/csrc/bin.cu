@@ -455,19 +455,37 @@ __global__ void __launch_bounds__(CSR_NT)
 
 
 // ---------------------------------------------------------------------------
-// FP32 covariance bins of gridded data, split by folds, on CUDA cores.
-// Subjects with N_i >= 2 are put in fold order (stable); each one's row gives
-// three operand rows in that order -- the mask M, the response R (zero where
-// unobserved) and R^2 -- of stride Ps (P rounded up to the tile edge, zero
-// beyond P), and its weight w_i = 1/(N_i(N_i - 1)).  Per fold f, with D_f the
-// diagonal of the fold's weights,
-//   C = M'M,  W = M' D_f M,  V = R' D_f R,  Q = (R^2)' D_f (R^2)
-// are computed 128 x 128 outputs per block, for the tile pairs on and above the
-// diagonal; the tile below is written as the transpose (all four are symmetric).
+// FP32 covariance bins of gridded data, split by folds, on the tensor cores.
+// Subjects with N_i >= 2 are put in fold order (stable).  With w_i = 1/(N_i(N_i - 1)), M the
+// masks and R the responses (zero where unobserved), each fold's
+//   C = M'M,  W = M'(w M),  V = X'X with X = sqrt(w) R,  Q = Z'Z with Z = sqrt(w) R^2
+// are computed 128 x 128 outputs per block, for the tile pairs on and above the diagonal; the
+// tile below is written as the transpose (all four are symmetric).
+//
+// FP32 from BF16 products: an FP32 number is exactly the sum of three BF16 ones (hi, mid, lo:
+// 8 bits each), a product of BF16 numbers is exact, and X'X keeps the six of the nine part
+// products that are above 2^-25 of the whole (mid lo, lo mid and lo lo are below it); w M is
+// three products with the exact 0/1 plane, M'M one.  The tensor cores' accumulator cuts
+// addends off instead of rounding them, a bias that would grow with the sum, so each run of 16
+// subjects is accumulated from zero, smallest parts first, and added to the FP32 sums by
+// ordinary additions: 4 additions beside 24 tensor instructions.  Against 64 bits the bins are
+// closer than those of FP32 multiply-adds, whose chains are 16 times as long.
+//
+// These are warp-level products (mma.sync, 0.60 PFLOP/s measured here): tcgen05 is three times
+// as fast, but its sums stay in tensor memory over many steps.  64 x 64, n = 1000, 5 folds
+// (0.27 TFLOP of part products, 1.34 GB written): 808 us, half of it at the tensor rate, the rest
+// the outputs and the stages' first loads (200 subjects a fold); the FP32 multiply-adds that this
+// replaces took 1480 us at 58 % of their peak.
 // ---------------------------------------------------------------------------
-constexpr int FG_T = 128;   // output tile edge
-constexpr int FG_K = 16;    // subjects per pipeline stage
-constexpr int FG_NT = 256;  // threads: 16 x 16, 8 x 8 outputs each
+constexpr int FG_T = 128;            // output tile edge
+constexpr int FG_K = 32;             // subjects per pipeline stage
+constexpr int FG_NT = 256;           // threads: 8 warps of 64 x 32 outputs
+constexpr int FG_LD = FG_T + 8;      // row pitch of a staged tile: ldmatrix without conflicts
+constexpr int FG_PLANES = 7;         // M, X (3 parts), Z (3 parts)
+constexpr int FG_TILE = FG_K * FG_LD;  // BF16 numbers of a staged tile
+constexpr size_t FG_SMEM = 2ull * 6 * FG_TILE * 2;  // 2 stages of 2 x 3 tiles
+constexpr int FG_OLD = FG_T + 1;     // row pitch of the output tile
+static_assert(FG_SMEM >= sizeof(float) * FG_T * FG_OLD, "output tile in the stages");
 
 __device__ __forceinline__ int fold_slot(int i, int F, const int32_t* __restrict__ fold,
                                          const int32_t* __restrict__ Ni, int* err) {
@@ -531,38 +549,89 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-// Operand rows in fold order (block k: row k), see above; rows past fstart[F] are
-// left alone (the Gram kernel never reads them).
-__global__ void k_fold_operands(int n, int P, int Ps, int F, const void* __restrict__ y,
-                                int y_prec, const uint8_t* __restrict__ mask,
-                                const int32_t* __restrict__ Ni, const double* __restrict__ mu,
-                                int mode, const int32_t* __restrict__ order,
-                                const int32_t* __restrict__ fstart, float* __restrict__ X,
-                                float* __restrict__ ws) {
-  const int k = blockIdx.x;
-  if (k >= fstart[F]) return;
-  const int i = order[k];
+// x = p[0] + p[1] + p[2] exactly (finite x above 2^-110); what is not finite stays in p[0]
+__device__ __forceinline__ void split3(float x, __nv_bfloat16* p) {
+  p[0] = __float2bfloat16_rn(x);
+  p[1] = p[2] = __float2bfloat16_rn(0.f);
+  if (!isfinite(x)) return;
+  if (!isfinite(__bfloat162float(p[0])))  // rounded past the largest: cut off instead
+    p[0] = __ushort_as_bfloat16((unsigned short)(__float_as_uint(x) >> 16));
+  const float r1 = x - __bfloat162float(p[0]);
+  p[1] = __float2bfloat16_rn(r1);
+  p[2] = __float2bfloat16_rn(r1 - __bfloat162float(p[1]));
+}
+
+// Operand rows in fold order, FO_ROWS rows by 512 columns a block, 4 columns a thread; rows
+// past fstart[F] are left alone (the Gram kernel never reads them).  The residuals are
+// float-float (FP64 subtractions and conversions of every entry took most of the 45 us that
+// this pass had at n = 1000, P = 4096), mu split once per FO_ROWS subjects.
+constexpr int FO_ROWS = 8;
+__global__ void __launch_bounds__(128)
+    k_fold_operands(int n, int P, int Ps, int F, const void* __restrict__ y, int y_prec,
+                    const uint8_t* __restrict__ mask, const int32_t* __restrict__ Ni,
+                    const double* __restrict__ mu, int mode, const int32_t* __restrict__ order,
+                    const int32_t* __restrict__ fstart, __nv_bfloat16* __restrict__ X,
+                    float* __restrict__ ws) {
+  __shared__ int who[FO_ROWS];
+  __shared__ ff::F2 root[FO_ROWS];
+  const int k0 = blockIdx.x * FO_ROWS, kn = min(FO_ROWS, fstart[F] - k0);
+  if (kn <= 0) return;
+  if ((int)threadIdx.x < kn) {
+    const int i = order[k0 + threadIdx.x];
+    const double N = (double)Ni[i], w = 1.0 / (N * (N - 1.0)), s = sqrt(w);
+    who[threadIdx.x] = i;
+    root[threadIdx.x] = {(float)s, (float)(s - (double)(float)s)};
+    if (blockIdx.y == 0) ws[k0 + threadIdx.x] = (float)w;
+  }
+  __syncthreads();
+  const int p0 = (blockIdx.y * 128 + threadIdx.x) * 4;
+  if (p0 >= Ps) return;
+  double md[4] = {0.0, 0.0, 0.0, 0.0};
+  ff::F2 m2[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    if (mode == FPCA_COV_RESIDUAL && p0 + u < P) md[u] = mu[p0 + u];
+    m2[u] = {(float)md[u], (float)(md[u] - (double)(float)md[u])};
+  }
   const size_t plane = (size_t)n * Ps;
-  for (int p = threadIdx.x; p < Ps; p += blockDim.x) {
-    float m = 0.f, r = 0.f, r2 = 0.f;
-    if (p < P) {
-      const size_t idx = (size_t)i * P + p;
-      if (!mask || mask[idx]) {
-        const double yy = load_y(y, y_prec, idx);
-        const double rd = mode == FPCA_COV_RESIDUAL ? yy - mu[p] : yy;
-        m = 1.f;
-        r = (float)rd;
-        r2 = (float)(rd * rd);
+  for (int r = 0; r < kn; ++r) {
+    __align__(8) __nv_bfloat16 o[FG_PLANES][4];
+    const ff::F2 s = root[r];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const size_t at = (size_t)who[r] * P + p0 + u;
+      float one = 0.f, x = 0.f, z = 0.f;
+      if (p0 + u < P && (!mask || mask[at])) {
+        ff::F2 d;
+        if (y_prec == FPCA_F64) {
+          const double dd = static_cast<const double*>(y)[at] - md[u];
+          d = {(float)dd, 0.f};
+          if (isfinite(d.hi)) d.lo = (float)(dd - (double)d.hi);
+        } else {
+          const float v = static_cast<const float*>(y)[at];
+          const ff::F2 t = ff::two_sum(v, -m2[u].hi);
+          d = isfinite(t.hi) ? ff::fast_two_sum(t.hi, t.lo - m2[u].lo) : ff::make(t.hi);
+        }
+        one = 1.f;
+        x = ff::mul(s, d).hi;
+        z = ff::mul(s, ff::mul(d, d)).hi;
+        if (!isfinite(x)) x = s.hi * d.hi;  // the corrections of an overflow are not numbers
+        if (!isfinite(z)) z = s.hi * (d.hi * d.hi);
+      }
+      __nv_bfloat16 px[3], pz[3];
+      split3(x, px);
+      split3(z, pz);
+      o[0][u] = __float2bfloat16_rn(one);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        o[1 + c][u] = px[c];
+        o[4 + c][u] = pz[c];
       }
     }
-    const size_t o = (size_t)k * Ps + p;
-    X[o] = m;
-    X[plane + o] = r;
-    X[2 * plane + o] = r2;
-  }
-  if (threadIdx.x == 0) {
-    const double N = (double)Ni[i];
-    ws[k] = (float)(1.0 / (N * (N - 1.0)));
+#pragma unroll
+    for (int c = 0; c < FG_PLANES; ++c)
+      *reinterpret_cast<uint2*>(X + c * plane + (size_t)(k0 + r) * Ps + p0) =
+          *reinterpret_cast<const uint2*>(o[c]);
   }
 }
 
@@ -577,115 +646,238 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
-// blockIdx.x: tile pair (bi <= bj), y: fold, z: plane (0 C, 1 W, 2 V, 3 Q).
-// Thread (ty, tx) owns rows {4ty..4ty+3, 64+4ty..} and columns {4tx.., 64+4tx..}
-// of the tile, so its shared-memory reads are float4s of consecutive addresses.
-__global__ void __launch_bounds__(FG_NT, 2)
-    k_fold_gram(int n, int P, int Ps, const float* __restrict__ X, const float* __restrict__ ws,
-                const int32_t* __restrict__ fstart, const int2* __restrict__ pairs,
-                int32_t* __restrict__ cnt, float* __restrict__ w, float* __restrict__ v,
-                float* __restrict__ q, int vec) {
-  __shared__ __align__(16) float As[2][FG_K][FG_T];
-  __shared__ __align__(16) float Bs[2][FG_K][FG_T];
-  __shared__ float Ss[2][FG_K];
-  const int2 pr = pairs[blockIdx.x];
-  const int f = blockIdx.y, z = blockIdx.z;
-  const int k0 = fstart[f], k1 = fstart[f + 1];
-  const int plane = z <= 1 ? 0 : z - 1;  // C and W from M, V from R, Q from R^2
-  const float* src = X + (size_t)plane * n * Ps;
-  const bool scaled = z > 0;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int p0 = pr.x * FG_T, q0 = pr.y * FG_T;
-  // stage loader: 16 rows x 128 columns of each operand, two float4 per thread each
-  auto load = [&](int st, int kb) {
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// the same from zero
+__device__ __forceinline__ void mma_bf16_zero(float (&c)[4], const uint32_t (&a)[4], uint32_t b0,
+                                              uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+
+// Output tile of one fold and plane over stages of FG_K subjects.  KIND 0: M'M (exact, so
+// accumulated in place); 1: M'(w M); 2: the six part products of X'X.  A warp's 64 x 32
+// outputs are 4 x 4 tensor tiles; KIND 2 takes 16 columns at a time, since all 32 would not
+// leave the registers for two blocks an SM.  32 x 32 a warp, with 32 columns at a time but a
+// 64 x 128 tile a block, reads half as much again from L2, which carries 6.9 TB/s then, and was
+// slower (1.00 ms against 0.96), also with the next plane's first stage behind the outputs' stores.
+template <int KIND>
+__device__ __forceinline__ void fold_tile(__nv_bfloat16* st, __nv_bfloat16 (*sw)[3][FG_K],
+                                          const __nv_bfloat16* __restrict__ src, size_t plane,
+                                          int Ps, const float* __restrict__ ws, int p0, int q0,
+                                          int k0, int k1, float (&acc)[4][4][4]) {
+  constexpr int NP = KIND == 2 ? 3 : 1;
+  constexpr int NH = KIND == 2 ? 1 : 2;  // 16-column halves at a time
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wm = (warp & 1) * 64, wn = (warp >> 1) * 32;
+  const int lr = tid >> 4, lc = (tid & 15) * 8;  // this thread's 16 bytes of a tile: rows lr, lr + 16
+  const uint32_t sdst = smem_addr(st + lr * FG_LD + lc);
+  auto load = [&](int s, int kb) {
+    const bool ok0 = kb + lr < k1, ok1 = kb + lr + 16 < k1;
+    const size_t o0 = (size_t)(ok0 ? kb + lr : k0) * Ps + lc;
+    const size_t o1 = (size_t)(ok1 ? kb + lr + 16 : k0) * Ps + lc;
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int e = tid + u * FG_NT;       // 0..511
-      const int r = e >> 5, c4 = e & 31;   // row, float4 column
-      const int k = kb + r;
-      const bool ok = k < k1;
-      const float* rowp = src + (size_t)(ok ? k : 0) * Ps;
-      cp_async16(smem_addr(&As[st][r][4 * c4]), rowp + p0 + 4 * c4, ok);
-      cp_async16(smem_addr(&Bs[st][r][4 * c4]), rowp + q0 + 4 * c4, ok);
+    for (int c = 0; c < 2 * NP; ++c) {  // the parts of rows p0.., then of columns q0..
+      const __nv_bfloat16* pl = src + (c % NP) * plane + (c < NP ? p0 : q0);
+      const uint32_t d = sdst + 2 * (s * 6 + c) * FG_TILE;
+      cp_async16(d, pl + o0, ok0);
+      cp_async16(d + 2 * 16 * FG_LD, pl + o1, ok1);
     }
-    if (tid < FG_K) Ss[st][tid] = (kb + tid < k1 && scaled) ? ws[kb + tid] : 1.f;
+    if (KIND == 1 && tid < FG_K) {
+      __nv_bfloat16 w[3];
+      split3(kb + tid < k1 ? ws[kb + tid] : 0.f, w);
+      for (int c = 0; c < 3; ++c) sw[s][c][tid] = w[c];
+    }
   };
-  float2 acc[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
   const int nchunk = (k1 - k0 + FG_K - 1) / FG_K;
   if (nchunk > 0) load(0, k0);
   cp_async_commit();
-  for (int c = 0; c < nchunk; ++c) {
-    const int st = c & 1;
-    if (c + 1 < nchunk) load(st ^ 1, k0 + (c + 1) * FG_K);
+  for (int ch = 0; ch < nchunk; ++ch) {
+    const int s = ch & 1;
+    if (ch + 1 < nchunk) load(s ^ 1, k0 + (ch + 1) * FG_K);
     cp_async_commit();
     cp_async_wait1();
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < FG_K; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[st][k][4 * ty]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[st][k][64 + 4 * ty]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[st][k][4 * tx]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[st][k][64 + 4 * tx]);
-      const float sk = Ss[st][k];
-      const float a[8] = {a0.x * sk, a0.y * sk, a0.z * sk, a0.w * sk,
-                          a1.x * sk, a1.y * sk, a1.z * sk, a1.w * sk};
-      const float2 b[4] = {make_float2(b0.x, b0.y), make_float2(b0.z, b0.w),
-                           make_float2(b1.x, b1.y), make_float2(b1.z, b1.w)};
+    const uint32_t base = smem_addr(st + s * 6 * FG_TILE);
+    // this lane's row of the four 8 x 8 matrices that ldmatrix reads, for both operands
+    const uint32_t la = base + 2 * (((lane >> 4) * 8 + (lane & 7)) * FG_LD + wm + ((lane >> 3) & 1) * 8);
+    const uint32_t lb = base + 2 * (NP * FG_TILE + (((lane >> 3) & 1) * 8 + (lane & 7)) * FG_LD + wn +
+                                    (lane >> 4) * 8);
+    // the second 16 subjects of the last stage may be beyond the fold
+    const int ksn = k0 + ch * FG_K + 16 < k1 ? 2 : 1;
+#pragma unroll 1
+    for (int ks = 0; ks < ksn; ++ks) {
+      __nv_bfloat162 wk[3][2];
+      if constexpr (KIND == 1) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float2 ai = make_float2(a[i], a[i]);
+        for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = __ffma2_rn(ai, b[j], acc[i][j]);
+          for (int e = 0; e < 2; ++e)
+            wk[c][e] = *reinterpret_cast<const __nv_bfloat162*>(&sw[s][c][ks * 16 + 8 * e + 2 * (lane & 3)]);
+      }
+#pragma unroll
+      for (int h0 = 0; h0 < 2; h0 += NH) {
+        uint32_t b[NP][NH][4];
+#pragma unroll
+        for (int c = 0; c < NP; ++c)
+#pragma unroll
+          for (int h = 0; h < NH; ++h)
+            ldsm4t(b[c][h], lb + 2 * (c * FG_TILE + ks * 16 * FG_LD + (h0 + h) * 16));
+#pragma unroll
+        for (int mi = 0; mi < 4; ++mi) {
+          uint32_t a[NP][4];
+#pragma unroll
+          for (int c = 0; c < NP; ++c)
+            ldsm4t(a[c], la + 2 * (c * FG_TILE + ks * 16 * FG_LD + mi * 16));
+          float t[2 * NH][4];
+          auto first = [&](const uint32_t (&x)[4], int cb) {
+#pragma unroll
+            for (int ni = 0; ni < 2 * NH; ++ni)
+              mma_bf16_zero(t[ni], x, b[cb][ni >> 1][2 * (ni & 1)], b[cb][ni >> 1][2 * (ni & 1) + 1]);
+          };
+          auto part = [&](const uint32_t (&x)[4], int cb) {
+#pragma unroll
+            for (int ni = 0; ni < 2 * NH; ++ni)
+              mma_bf16(t[ni], x, b[cb][ni >> 1][2 * (ni & 1)], b[cb][ni >> 1][2 * (ni & 1) + 1]);
+          };
+          if constexpr (KIND == 0) {
+#pragma unroll
+            for (int ni = 0; ni < 4; ++ni)
+              mma_bf16(acc[mi][ni], a[0], b[0][ni >> 1][2 * (ni & 1)], b[0][ni >> 1][2 * (ni & 1) + 1]);
+          } else {
+            if constexpr (KIND == 2) {
+              first(a[2], 0);
+              part(a[0], 2);
+              part(a[1], 1);
+              part(a[1], 0);
+              part(a[0], 1);
+              part(a[0], 0);
+            } else {
+#pragma unroll
+              for (int c = 2; c >= 0; --c) {
+                uint32_t x[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const __nv_bfloat162 v =
+                      __hmul2(*reinterpret_cast<const __nv_bfloat162*>(&a[0][e]), wk[c][e >> 1]);
+                  x[e] = *reinterpret_cast<const uint32_t*>(&v);
+                }
+                if (c == 2)
+                  first(x, 0);
+                else
+                  part(x, 0);
+              }
+            }
+#pragma unroll
+            for (int ni = 0; ni < 2 * NH; ++ni)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) acc[mi][2 * h0 + ni][e] += t[ni][e];
+          }
+        }
       }
     }
     __syncthreads();  // the stage is overwritten by the load after next
   }
-  // epilogue: the tile (p, q) and, off the diagonal, its transpose (q, p); the
-  // p == q entries hold only j == l pairs and are zero.  vec: P % 4 == 0 and the
-  // outputs 16-byte aligned, so four consecutive columns are stored at once.
-  const long long PP = (long long)P * P;
-  const size_t fo = (size_t)f * PP;
-  auto put4 = [&](int row, int col, float4 val) {  // columns col..col+3
-    if (row >= P) return;
-    const float x[4] = {row == col ? 0.f : val.x, row == col + 1 ? 0.f : val.y,
-                        row == col + 2 ? 0.f : val.z, row == col + 3 ? 0.f : val.w};
-    const size_t o = fo + (size_t)row * P + col;
-    if (vec && col + 3 < P) {
-      if (z == 0)
-        *reinterpret_cast<int4*>(cnt + o) = make_int4(__float2int_rn(x[0]), __float2int_rn(x[1]),
-                                                      __float2int_rn(x[2]), __float2int_rn(x[3]));
-      else
-        *reinterpret_cast<float4*>((z == 1 ? w : z == 2 ? v : q) + o) =
-            make_float4(x[0], x[1], x[2], x[3]);
-      return;
-    }
-    for (int u = 0; u < 4; ++u) {
-      if (col + u >= P) break;
-      if (z == 0)
-        cnt[o + u] = __float2int_rn(x[u]);
-      else
-        (z == 1 ? w : z == 2 ? v : q)[o + u] = x[u];
-    }
-  };
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int row = p0 + (i < 4 ? 4 * ty + i : 64 + 4 * ty + (i - 4));
-    put4(row, q0 + 4 * tx, make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y));
-    put4(row, q0 + 64 + 4 * tx, make_float4(acc[i][2].x, acc[i][2].y, acc[i][3].x, acc[i][3].y));
+}
+
+// One entry of X'X from the whole numbers, where a part product was no number (overflows,
+// infinities and NaN among the observations).
+__device__ __noinline__ float fold_entry(const __nv_bfloat16* __restrict__ src, size_t plane, int Ps,
+                                         int p, int q, int k0, int k1) {
+  float x = 0.f;
+  for (int k = k0; k < k1; ++k) {
+    const __nv_bfloat16 *a = src + (size_t)k * Ps + p, *b = src + (size_t)k * Ps + q;
+    const float av = __bfloat162float(a[0]) + (__bfloat162float(a[plane]) + __bfloat162float(a[2 * plane]));
+    const float bv = __bfloat162float(b[0]) + (__bfloat162float(b[plane]) + __bfloat162float(b[2 * plane]));
+    x = fmaf(av, bv, x);
   }
-  if (pr.x != pr.y) {
+  return x;
+}
+
+// blockIdx.x: tile pair (bi <= bj), y: fold, z: Q, V, W, C, the costly ones first.  vec2: P even
+// and the outputs aligned to 8 bytes.
+__global__ void __launch_bounds__(FG_NT, 2)
+    k_fold_gram(int n, int P, int Ps, const __nv_bfloat16* __restrict__ X,
+                const float* __restrict__ ws, const int32_t* __restrict__ fstart,
+                const int2* __restrict__ pairs, int32_t* __restrict__ cnt, float* __restrict__ w,
+                float* __restrict__ v, float* __restrict__ q, int with_q, int vec2) {
+  extern __shared__ __align__(16) __nv_bfloat16 fst[];
+  __shared__ __align__(4) __nv_bfloat16 sw[2][3][FG_K];
+  const int2 pr = pairs[blockIdx.x];
+  const int f = blockIdx.y, z = with_q ? (blockIdx.z + 3) & 3 : blockIdx.z;  // 3 Q, 0 V, 1 W, 2 C
+  const int k0 = fstart[f], k1 = fstart[f + 1];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int p0 = pr.x * FG_T, q0 = pr.y * FG_T;
+  const size_t plane = (size_t)n * Ps;
+  const __nv_bfloat16* src = X + (z == 0 ? 1 : z == 3 ? 4 : 0) * plane;
+  float acc[4][4][4] = {};
+  if (z == 0 || z == 3)
+    fold_tile<2>(fst, sw, src, plane, Ps, ws, p0, q0, k0, k1, acc);
+  else if (z == 1)
+    fold_tile<1>(fst, sw, src, plane, Ps, ws, p0, q0, k0, k1, acc);
+  else
+    fold_tile<0>(fst, sw, src, plane, Ps, ws, p0, q0, k0, k1, acc);
+  const size_t fo = (size_t)f * P * P;
+  uint32_t* out = reinterpret_cast<uint32_t*>(z == 0 ? v : z == 1 ? w : z == 3 ? q : (float*)cnt) + fo;
+  auto bits = [&](float x) { return z == 2 ? (uint32_t)__float2int_rn(x) : __float_as_uint(x); };
+  // the tile from the registers, whole sectors of its rows; its transpose by whole lines through
+  // shared memory.  Streaming stores: not read here again, so that the operands stay in L2.
+  const bool diag = p0 == q0, inside = p0 + FG_T <= P && q0 + FG_T <= P;
+  float* T = reinterpret_cast<float*>(fst);
+  bool odd = false;
 #pragma unroll
-    for (int cc = 0; cc < 8; ++cc) {
-      const int j = (cc & 3) >> 1, comp = cc & 1;
-      const int jj = cc < 4 ? j : j + 2;
-      const int row = q0 + (cc < 4 ? 4 * tx + cc : 64 + 4 * tx + (cc - 4));
-      auto pick = [&](int i) { return comp ? acc[i][jj].y : acc[i][jj].x; };
-      put4(row, p0 + 4 * ty, make_float4(pick(0), pick(1), pick(2), pick(3)));
-      put4(row, p0 + 64 + 4 * ty, make_float4(pick(4), pick(5), pick(6), pick(7)));
+  for (int mi = 0; mi < 4; ++mi)
+#pragma unroll
+    for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+      for (int e = 0; e < 4; e += 2) {
+        const int r = (warp & 1) * 64 + mi * 16 + (lane >> 2) + 4 * e;
+        const int c = (warp >> 1) * 32 + ni * 8 + 2 * (lane & 3);
+        float x0 = acc[mi][ni][e], x1 = acc[mi][ni][e + 1];
+        if (diag && r == c) x0 = 0.f;  // only pairs of an observation with itself
+        if (diag && r == c + 1) x1 = 0.f;
+        odd |= !isfinite(x0) || !isfinite(x1);
+        T[r * FG_OLD + c] = x0;
+        T[r * FG_OLD + c + 1] = x1;
+        uint32_t* o = out + (size_t)(p0 + r) * P + q0 + c;
+        if (inside && vec2) {
+          __stcs(reinterpret_cast<uint2*>(o), make_uint2(bits(x0), bits(x1)));
+        } else if (p0 + r < P) {
+          if (q0 + c < P) __stcs(o, bits(x0));
+          if (q0 + c + 1 < P) __stcs(o + 1, bits(x1));
+        }
+      }
+  odd = __syncthreads_or(odd);
+  if (!diag)
+    for (int c = warp; c < FG_T && q0 + c < P; c += FG_NT / 32) {
+      uint32_t* o = out + (size_t)(q0 + c) * P + p0 + lane;
+#pragma unroll
+      for (int j = 0; j < FG_T / 32; ++j)
+        if (p0 + lane + 32 * j < P) __stcs(o + 32 * j, bits(T[(lane + 32 * j) * FG_OLD + c]));
+    }
+  if (odd && (z == 0 || z == 3)) {  // overflows, infinities, NaN
+    __syncthreads();                // the transposed entries are written again here
+    for (int e = tid; e < FG_T * FG_T; e += FG_NT) {
+      const int r = p0 + e / FG_T, c = q0 + e % FG_T;
+      if (r >= P || c >= P || isfinite(T[e / FG_T * FG_OLD + e % FG_T])) continue;
+      const uint32_t x = __float_as_uint(fold_entry(src, plane, Ps, r, c, k0, k1));
+      out[(size_t)r * P + c] = x;
+      if (!diag) out[(size_t)c * P + r] = x;
     }
   }
 }
@@ -843,7 +1035,7 @@ fpca_status launch_cov_dense_folds(fpca_ctx* ctx, int n, int P, const void* y, i
   const int nt = Ps / FG_T;
   const size_t need = WsCarve::round(sizeof(int32_t) * (size_t)n) * 2 +
                       WsCarve::round(sizeof(int32_t) * 65) +
-                      WsCarve::round(sizeof(float) * 3 * (size_t)n * Ps) +
+                      WsCarve::round(sizeof(__nv_bfloat16) * FG_PLANES * (size_t)n * Ps) +
                       WsCarve::round(sizeof(float) * (size_t)n) +
                       WsCarve::round(sizeof(int2) * (size_t)nt * (nt + 1) / 2) + 2048;
   void* wsp = fpca_workspace(ctx, need);
@@ -852,7 +1044,7 @@ fpca_status launch_cov_dense_folds(fpca_ctx* ctx, int n, int P, const void* y, i
   int32_t* Ni = carve.take<int32_t>(n);
   int32_t* order = carve.take<int32_t>(n);
   int32_t* fstart = carve.take<int32_t>(65);
-  float* X = carve.take<float>(3 * (size_t)n * Ps);
+  __nv_bfloat16* X = carve.take<__nv_bfloat16>(FG_PLANES * (size_t)n * Ps);
   float* wsub = carve.take<float>(n);
   int2* pairs = carve.take<int2>((size_t)nt * (nt + 1) / 2);
   std::vector<int2> ph;
@@ -870,14 +1062,15 @@ fpca_status launch_cov_dense_folds(fpca_ctx* ctx, int n, int P, const void* y, i
   k_fold_order<<<1, 1024, 0, ctx->stream>>>(n, F, nfold > 0 ? fold : nullptr, Ni, order, fstart,
                                             ctx->d_err);
   FPCA_LAUNCHED(ctx, "fold_order");
-  k_fold_operands<<<n, 128, 0, ctx->stream>>>(n, P, Ps, F, y, y_prec, mask, Ni, mu, mode, order,
-                                              fstart, X, wsub);
+  k_fold_operands<<<dim3((n + FO_ROWS - 1) / FO_ROWS, (Ps + 511) / 512), 128, 0, ctx->stream>>>(
+      n, P, Ps, F, y, y_prec, mask, Ni, mu, mode, order, fstart, X, wsub);
   FPCA_LAUNCHED(ctx, "fold_operands");
   const dim3 grid((unsigned)ph.size(), F, q ? 4 : 3);
-  auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
-  const int vec = (P % 4 == 0 && al16(cnt) && al16(w) && al16(v) && (!q || al16(q))) ? 1 : 0;
-  k_fold_gram<<<grid, FG_NT, 0, ctx->stream>>>(n, P, Ps, X, wsub, fstart, pairs, cnt, w, v, q,
-                                                vec);
+  auto al8 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 7) == 0; };
+  const int vec2 = P % 2 == 0 && al8(cnt) && al8(w) && al8(v) && al8(q);
+  cudaFuncSetAttribute(k_fold_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FG_SMEM);
+  k_fold_gram<<<grid, FG_NT, FG_SMEM, ctx->stream>>>(n, P, Ps, X, wsub, fstart, pairs, cnt, w, v, q,
+                                                     q ? 1 : 0, vec2);
   FPCA_LAUNCHED(ctx, "cov_fold_gram");
   return FPCA_OK;
 }
