@@ -64,20 +64,36 @@ __device__ __forceinline__ ff::F2 split(double x) {
   return {hi, (float)(x - (double)hi)};
 }
 
-// y[e] - m in float-float, y FP32 or FP64, m = mu as float-float
-__device__ __forceinline__ ff::F2 centred(const void* y, int yprec, long long e, ff::F2 m) {
-  if (yprec == FPCA_F64)
-    return split(static_cast<const double*>(y)[e] - ((double)m.hi + (double)m.lo));
-  const ff::F2 t = ff::two_sum(static_cast<const float*>(y)[e], -m.hi);
+// y - m in float-float, y FP32 or FP64, m = mu as float-float
+__device__ __forceinline__ ff::F2 centred(double y, ff::F2 m) {
+  return split(y - ((double)m.hi + (double)m.lo));
+}
+__device__ __forceinline__ ff::F2 centred(float y, ff::F2 m) {
+  const ff::F2 t = ff::two_sum(y, -m.hi);
   return ff::fast_two_sum(t.hi, t.lo - m.lo);
 }
+__device__ __forceinline__ ff::F2 centred(const void* y, int yprec, long long e, ff::F2 m) {
+  return yprec == FPCA_F64 ? centred(static_cast<const double*>(y)[e], m)
+                           : centred(static_cast<const float*>(y)[e], m);
+}
 
-// mu (row 0) and the first L eigenfunctions (rows 1..L) as float-float; bmax (NULL or
-// L x gridDim.x): each block's largest |phi_l|, rounded up, infinity if one is not finite.
+// mu (row 0) and the first L eigenfunctions (rows 1..L) as float-float; bmax (L x gridDim.x):
+// each block's largest |phi_l|, rounded up, infinity if one is not finite.  For PACE (lam not
+// NULL) prior[l] = sigma^2 / lambda_l, and prior[SC_LMAX] = 1 if sigma^2 >= 0 and every
+// lambda > 0, else 0 (an FP64 division in every block of the later kernels took 3 us there).
 __global__ void __launch_bounds__(256)
     k_split_ff(int P, const double* __restrict__ mu, const double* __restrict__ phi,
-               float2* __restrict__ mu2, float2* __restrict__ phi2, float* __restrict__ bmax) {
+               float2* __restrict__ mu2, float2* __restrict__ phi2, float* __restrict__ bmax, int L,
+               const double* __restrict__ lam, const double* __restrict__ sigma2p,
+               double* __restrict__ prior) {
   __shared__ float wmax[8];
+  if (lam && blockIdx.x == 0 && blockIdx.y == 0) {
+    const double s2 = *sigma2p;
+    const bool bad = !(s2 >= 0.0) || ((int)threadIdx.x < L && !(lam[threadIdx.x] > 0.0));
+    if ((int)threadIdx.x < L) prior[threadIdx.x] = s2 / lam[threadIdx.x];
+    const int any = __syncthreads_or(bad);
+    if (threadIdx.x == 0) prior[SC_LMAX] = any ? 0.0 : 1.0;
+  }
   const int l = (int)blockIdx.y - 1;
   const double* in = l < 0 ? mu : phi + (long long)l * P;
   float2* out = l < 0 ? mu2 : phi2 + (long long)l * P;
@@ -88,7 +104,7 @@ __global__ void __launch_bounds__(256)
     const float a = __double2float_ru(fabs(in[e]));
     top = isfinite(a) ? fmaxf(top, a) : INFINITY;
   }
-  if (l < 0 || !bmax) return;
+  if (l < 0) return;
   for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = top;
   __syncthreads();
@@ -144,7 +160,7 @@ struct PaceSys {
   float2 low[SC_LMAX][SC_LMAX + 1];
 };
 
-// (A + diag(add)) a = b for 32 / RL subjects of a warp, RL lanes each (lane r owns row r),
+// (A + diag(prior)) a = b for 32 / RL subjects of a warp, RL lanes each (lane r owns row r),
 // the scores left in sys->b.  A chain of dependent FP64 operations is what one thread's
 // FP64 Cholesky would wait on (~135 ns each here), so the factor is taken in float-float of
 // the system scaled to a unit-size diagonal by powers of two, and the solution refined once
@@ -152,13 +168,14 @@ struct PaceSys {
 // own for what passes the test on the correction (2^-25 of the solution).  What does not
 // pass (near-singular, not finite, extreme scales) is solved by one lane in FP64.
 template <int RL>
-__device__ void pace_solve(PaceSys* sys, const double* add, int L, bool valid, bool active,
+__device__ void pace_solve(PaceSys* sys, const double* __restrict__ prior, int L, bool active,
                            int* err) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31, r = lane % RL;
   const unsigned seg = (RL == 32 ? full : ((1u << RL) - 1u)) << (lane / RL * RL);
   const bool in = r < L;
-  if (active && in) sys->A[r][r] += add[r];
+  const bool valid = prior[SC_LMAX] != 0.0;
+  if (active && in) sys->A[r][r] += prior[r];
   __syncwarp();
   const double dg = in && active ? sys->A[r][r] : 1.0, br = in && active ? sys->b[r] : 0.0;
   const int ex = ((__double2hiint(dg) >> 20) & 0x7ff) - 1023;
@@ -243,31 +260,21 @@ __device__ void pace_solve(PaceSys* sys, const double* add, int L, bool valid, b
   __syncwarp();
 }
 
-// sigma^2 / lambda_l into add, by the first L threads of a block, and whether the prior is
-// one: sigma^2 >= 0 and every lambda > 0.  Ends in a __syncthreads.
-__device__ bool pace_prior(const double* lam, const double* sigma2p, int L, double* add) {
-  const double sigma2 = *sigma2p;
-  const bool bad = !(sigma2 >= 0.0) || ((int)threadIdx.x < L && !(lam[threadIdx.x] > 0.0));
-  if ((int)threadIdx.x < L) add[threadIdx.x] = sigma2 / lam[threadIdx.x];
-  return !__syncthreads_or(bad);
-}
 
 // Scattered data (offs / t / y in FP64), mu2 (P) and phi2 (L x P) float-float: a warp per
 // subject, its observations in chunks of 32 staged in shared memory, each lane a few of the
 // NE + L sums.  LM: 8 or 16 >= L; the four subjects of a block are solved together, LM
-// lanes each.  n = 20000, 5..20 points, 24 x 24, L = 8: see pace_solve for the solves, which
-// took most of the time when one lane of the warp ran them in FP64.
+// lanes each.  n = 20000, 5..20 points, 24 x 24, L = 8: 84 us; 617 us when one lane of each
+// warp solved in FP64 and the chunks of 32 were always walked to their end.
 template <int LM>
 __global__ void __launch_bounds__(128)
     k_scores_pace(ScGrid g, int n, const void* __restrict__ y, const int64_t* __restrict__ offs,
                   const double* __restrict__ t, const float2* __restrict__ mu2,
-                  const double* __restrict__ lam, const float2* __restrict__ phi2, int L,
-                  const double* __restrict__ sigma2p, double* __restrict__ scores,
-                  int* __restrict__ err) {
+                  const double* __restrict__ prior, const float2* __restrict__ phi2, int L,
+                  double* __restrict__ scores, int* __restrict__ err) {
   constexpr int NS = (LM * (LM + 1) / 2 + LM + 31) / 32;  // sums per lane
   __shared__ float2 rows[4][32][LM + 1];                   // phi rows, then the residual
   __shared__ PaceSys sys[4];
-  __shared__ double add[SC_LMAX];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int NE = L * (L + 1) / 2;
   // Upper-triangle entries e = lane + 32 q (row-major) of Phi_i' Phi_i, then the L
@@ -288,7 +295,6 @@ __global__ void __launch_bounds__(128)
     er[q] = r;
     ec[q] = r + rem;
   }
-  const bool valid = pace_prior(lam, sigma2p, L, add);
   const int i = blockIdx.x * 4 + warp;
   if (i < n) {
     Acc acc[NS];
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(128)
   constexpr int SPW = 32 / LM;  // subjects per solving warp
   if (warp < 4 / SPW) {
     const int sl = warp * SPW + lane / LM;
-    pace_solve<LM>(&sys[sl], add, L, valid, blockIdx.x * 4 + sl < n, err);
+    pace_solve<LM>(&sys[sl], prior, L, blockIdx.x * 4 + sl < n, err);
   }
   __syncthreads();
   if (i < n && lane < L) scores[(long long)i * L + lane] = sys[warp].b[lane];
@@ -425,7 +431,7 @@ __global__ void __launch_bounds__(256)
 }
 
 __device__ __forceinline__ void mma_f16(float (&c)[4], const unsigned (&a)[4], uint2 b) {
-  asm volatile(
+  asm(
       "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};"
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
@@ -459,7 +465,7 @@ __device__ __forceinline__ uint4 mask16(const uint8_t* __restrict__ row, int p, 
 // out[(split * nb + i) * 8 ng + e]: the fixed-point sums over the split's nodes.  A warp takes
 // 16 subjects (its A fragments come straight from the mask's bytes) and GP groups of 8
 // columns; blockIdx: x 128 subjects, y a split of `per` x 64 nodes, z GP groups.  1.5 GFLOP
-// at n = 1000, P = 4096, L = 8: bound by the table's reads from L1/L2, so the simpler
+// at n = 1000, P = 4096, L = 8 in 10 us: bound by the table's reads from L1/L2, so the simpler
 // warp-level products are as good as tcgen05's here.
 template <int GP>
 __global__ void __launch_bounds__(256)
@@ -475,23 +481,40 @@ __global__ void __launch_bounds__(256)
   const bool oka = ra < nb, okb = rb < nb;
   const uint8_t* rowa = mask ? mask + (size_t)(i0 + (oka ? ra : 0)) * P : nullptr;
   const uint8_t* rowb = mask ? mask + (size_t)(i0 + (okb ? rb : 0)) * P : nullptr;
+  // the fragments of the next 16 nodes are loaded while these are multiplied (the loads took
+  // 0.95 of the time when each was waited for)
+  const uint2* tb = table + ((size_t)k0 * 4 * ng + g0) * PG_DIG * 32 + lane;
+  const size_t tstep = (size_t)ng * PG_DIG * 32;
+  uint2 b[2][GP * PG_DIG];
+  auto fetch = [&](uint2 (&f)[GP * PG_DIG]) {
+#pragma unroll
+    for (int q = 0; q < GP; ++q)
+      if (q < gn) {
+#pragma unroll
+        for (int d = 0; d < PG_DIG; ++d) f[q * PG_DIG + d] = tb[(q * PG_DIG + d) * 32];
+      }
+    tb += tstep;
+  };
+  auto masks = [&](const uint8_t* row, bool ok, int k) {
+    return ok && k < k1 ? mask16(row, k * 64 + t * 16, P, vec) : make_uint4(0, 0, 0, 0);
+  };
+  uint4 wa = masks(rowa, oka, k0), wb = masks(rowb, okb, k0);
+  if (k0 < k1) fetch(b[0]);
   for (int k = k0; k < k1; ++k) {
-    const int p = k * 64 + t * 16;
-    uint4 wa = mask16(rowa, p, P, vec), wb = mask16(rowb, p, P, vec);
-    if (!oka) wa = make_uint4(0, 0, 0, 0);
-    if (!okb) wb = make_uint4(0, 0, 0, 0);
     const unsigned ua[4] = {wa.x, wa.y, wa.z, wa.w}, ub[4] = {wb.x, wb.y, wb.z, wb.w};
+    wa = masks(rowa, oka, k + 1);
+    wb = masks(rowb, okb, k + 1);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const unsigned one = 0x3c003c00u;  // 1.0 where the byte is set
       const unsigned a[4] = {__byte_perm(ua[j], 0, 0x1404) & one, __byte_perm(ub[j], 0, 0x1404) & one,
                              __byte_perm(ua[j], 0, 0x3424) & one, __byte_perm(ub[j], 0, 0x3424) & one};
-      const uint2* tb = table + ((size_t)(k * 4 + j) * ng + g0) * PG_DIG * 32 + lane;
+      if (j < 3 || k + 1 < k1) fetch(b[(j + 1) & 1]);
 #pragma unroll
       for (int q = 0; q < GP; ++q) {
         if (q < gn) {
 #pragma unroll
-          for (int d = 0; d < PG_DIG; ++d) mma_f16(acc[q][d], a, tb[(q * PG_DIG + d) * 32]);
+          for (int d = 0; d < PG_DIG; ++d) mma_f16(acc[q][d], a, b[j & 1][q * PG_DIG + d]);
         }
       }
     }
@@ -514,28 +537,27 @@ __global__ void __launch_bounds__(256)
 }
 
 // Phi_i'Y_i^C of two subjects and their systems.  A thread keeps both subjects' L
-// compensated sums over every 256th node, so a phi value read serves two subjects; the
+// compensated sums over every 256th node, so a phi value read serves two subjects (L2
+// latency bounds it: 53 us at n = 1000, P = 4096, L = 8, where one warp per 1/8 subject that
+// formed Phi'Phi too took 269; a node ahead in registers costs a block an SM: 67 us); the
 // sums join by a halving butterfly of float-float adds (one add per sum instead of
 // five; FP64 adds there would take longer than the sums themselves), the warps in FP64.
 constexpr int PF_SUB = 2;
 template <int LM>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
     k_pace_final(int nb, int i0, int P, const void* __restrict__ y, int yprec,
                  const uint8_t* __restrict__ mask, const float2* __restrict__ mu2,
-                 const double* __restrict__ lam, const float2* __restrict__ phi2, int L,
-                 const double* __restrict__ sigma2p, int nsplit, const int* __restrict__ expo,
+                 const double* __restrict__ prior, const float2* __restrict__ phi2, int L, int nsplit, const int* __restrict__ expo,
                  const long long* __restrict__ gsum, double* __restrict__ scores,
                  int* __restrict__ err) {
   constexpr int NV = PF_SUB * LM;
   __shared__ PaceSys sys[PF_SUB];
-  __shared__ double add[SC_LMAX];
   __shared__ float2 wsum[8][NV];
   __shared__ double count[PF_SUB];
   __shared__ int redo[PF_SUB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L);
   const int s0 = blockIdx.x * PF_SUB;
-  const bool valid = pace_prior(lam, sigma2p, L, add);
   if (tid < PF_SUB) redo[tid] = 0;
   for (int it = tid; it < PF_SUB * (NE + 1); it += 256) {
     const int sl = it / (NE + 1), e = it - sl * (NE + 1);
@@ -562,28 +584,28 @@ __global__ void __launch_bounds__(256)
     sys[sl].A[b][a] = ge;
   }
   Acc acc[PF_SUB][LM];
+  bool clean = true;  // no phi value that times a zero is not zero
+  for (int l = 0; l < L; ++l) clean &= expo[l] != PG_EBAD;
+  const size_t row0 = (size_t)(i0 + s0) * P, row1 = (size_t)(i0 + min(s0 + 1, nb - 1)) * P;
   for (int p = tid; p < P; p += 256) {
+    // unobserved responses are read and not used, so that no load waits for another
+    const bool ok0 = !mask || mask[row0 + p], ok1 = s0 + 1 < nb && (!mask || mask[row1 + p]);
     const float2 m = mu2[p];
-    ff::F2 r[PF_SUB];
-    bool ok[PF_SUB], any = false;
-#pragma unroll
-    for (int u = 0; u < PF_SUB; ++u) {
-      const long long at = (long long)(i0 + s0 + u) * P + p;
-      ok[u] = s0 + u < nb && (!mask || mask[at]);
-      r[u] = ok[u] ? centred(y, yprec, at, ff::F2{m.x, m.y}) : ff::make(0.f);
-      any |= ok[u];
-    }
-    if (!any) continue;
+    ff::F2 r0 = centred(y, yprec, row0 + p, ff::F2{m.x, m.y});
+    ff::F2 r1 = centred(y, yprec, row1 + p, ff::F2{m.x, m.y});
+    if (!ok0) r0 = ff::make(0.f);
+    if (!ok1) r1 = ff::make(0.f);
 #pragma unroll
     for (int l = 0; l < LM; ++l) {
       if (l < L) {
         const float2 f = phi2[(long long)l * P + p];
-#pragma unroll
-        for (int u = 0; u < PF_SUB; ++u)
-          acc[u][l].add_prod(r[u], ok[u] ? ff::F2{f.x, f.y} : ff::make(0.f));
+        const ff::F2 ph{f.x, f.y};
+        acc[0][l].add_prod(r0, clean || ok0 ? ph : ff::make(0.f));
+        acc[1][l].add_prod(r1, clean || ok1 ? ph : ff::make(0.f));
       }
     }
   }
+  static_assert(PF_SUB == 2, "two subjects above");
   ff::F2 v[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k)
@@ -645,7 +667,7 @@ __global__ void __launch_bounds__(256)
   if (warp == 0) {
     const int sl = lane / LM < PF_SUB ? lane / LM : PF_SUB - 1;
     const bool active = lane / LM < PF_SUB && s0 + sl < nb;
-    pace_solve<LM>(&sys[sl], add, L, valid, active, err);
+    pace_solve<LM>(&sys[sl], prior, L, active, err);
     for (int e = lane; e < PF_SUB * L; e += 32)
       if (s0 + e / L < nb) scores[(long long)(i0 + s0) * L + e] = sys[e / L].b[e % L];
   }
@@ -805,6 +827,7 @@ constexpr int PG_BATCH = 16384;  // subjects x splits
 struct ScWork {
   float2 *mu2, *phi2;  // mu (P) and the first L eigenfunctions (L x P) as float-float
   float* bmax;         // L x nbx block maxima of |phi|
+  double* prior;       // see k_split_ff
   int* expo;           // L exponents
   uint2* table;
   long long* gsum;
@@ -812,7 +835,8 @@ struct ScWork {
   int nbx, nsplit, per, batch;
 };
 
-fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double* evecs, ScWork* w) {
+fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double* evecs, ScWork* w,
+                     const double* lam = nullptr, const double* sigma2 = nullptr) {
   const int n64 = (P + 63) / 64, ng = pg_groups(L);
   w->phi = evecs;
   w->nbx = std::min((P + 255) / 256, 64);
@@ -825,7 +849,7 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   const size_t ns = (size_t)w->nsplit * w->batch * 8 * ng;
   void* ws = fpca_workspace(ctx, WsCarve::round(sizeof(float2) * P) +
                                      WsCarve::round(sizeof(float2) * (size_t)L * P) +
-                                     WsCarve::round(sizeof(float) * L * w->nbx) + 256 +
+                                     WsCarve::round(sizeof(float) * L * w->nbx) + 512 +
                                      WsCarve::round(sizeof(uint2) * nt) +
                                      WsCarve::round(sizeof(long long) * ns));
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
@@ -834,15 +858,17 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   w->phi2 = c.take<float2>((size_t)L * P);
   w->bmax = c.take<float>((size_t)L * w->nbx);
   w->expo = c.take<int>(SC_LMAX);
+  w->prior = c.take<double>(SC_LMAX + 1);
   w->table = c.take<uint2>(nt);
   w->gsum = c.take<long long>(ns);
-  k_split_ff<<<dim3(w->nbx, L + 1), 256, 0, ctx->stream>>>(P, mu, evecs, w->mu2, w->phi2, w->bmax);
+  k_split_ff<<<dim3(w->nbx, L + 1), 256, 0, ctx->stream>>>(P, mu, evecs, w->mu2, w->phi2, w->bmax, L,
+                                                                lam, sigma2, w->prior);
   FPCA_LAUNCHED(ctx, "split_ff");
   return FPCA_OK;
 }
 
 fpca_status pace_dense(fpca_ctx* ctx, const fpca_data* data, int P, int L, const ScWork& w,
-                       const double* evals, const double* sigma2, double* scores) {
+                       double* scores) {
   const int n64 = (P + 63) / 64, ng = pg_groups(L);
   k_pace_table<<<n64, 256, 0, ctx->stream>>>(P, L, w.nbx, w.bmax, w.phi, w.table, w.expo);
   FPCA_LAUNCHED(ctx, "pace_table");
@@ -857,7 +883,7 @@ fpca_status pace_dense(fpca_ctx* ctx, const fpca_data* data, int P, int L, const
     FPCA_LAUNCHED(ctx, "pace_gram");
     auto fin = L <= 8 ? k_pace_final<8> : k_pace_final<16>;
     fin<<<(nb + PF_SUB - 1) / PF_SUB, 256, 0, ctx->stream>>>(
-        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, evals, w.phi2, L, sigma2, w.nsplit,
+        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, w.prior, w.phi2, L, w.nsplit,
         w.expo, w.gsum, scores, ctx->d_err);
     FPCA_LAUNCHED(ctx, "scores_pace");
   }
@@ -882,16 +908,16 @@ fpca_status fpca_scores_pace(fpca_ctx* ctx, const fpca_data* data, const fpca_gr
     return fpca_fail(ctx, FPCA_E_INVALID_ARG, "scattered data need offs and t");
   const ScGrid g = sc_grid(grid);
   ScWork w;
-  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w);
+  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w, evals, sigma2);
   if (s != FPCA_OK) return s;
   if (data->layout == FPCA_SPARSE) {
     auto kern = L <= 8 ? k_scores_pace<8> : k_scores_pace<16>;
     kern<<<(data->n + 3) / 4, 128, 0, ctx->stream>>>(g, data->n, data->y, data->offs, data->t, w.mu2,
-                                                     evals, w.phi2, L, sigma2, scores, ctx->d_err);
+                                                     w.prior, w.phi2, L, scores, ctx->d_err);
     FPCA_LAUNCHED(ctx, "scores_pace");
     return FPCA_OK;
   }
-  return pace_dense(ctx, data, g.P, L, w, evals, sigma2, scores);
+  return pace_dense(ctx, data, g.P, L, w, scores);
 }
 
 fpca_status fpca_scores_integral(fpca_ctx* ctx, const fpca_data* data, const fpca_grid* grid,
