@@ -1212,8 +1212,7 @@ __global__ void k_bj_init(int n, int ne, const double* __restrict__ A64, float* 
 __global__ void __launch_bounds__(BJ_NT)
     k_bj_sub(int ne, int round, const float* __restrict__ A, float* __restrict__ Jg,
              const int* __restrict__ done) {
-  __shared__ float a0[BJ_W * (BJ_W + 1)], a1[BJ_W * (BJ_W + 1)], js[BJ_W * (BJ_W + 1)];
-  __shared__ float cs[32];
+  __shared__ float a0[BJ_W * BJ_LD], a1[BJ_W * BJ_LD], js[BJ_W * (BJ_W + 1)];
   if (*done) return;
   const int nb = ne / BJ_S;
   int I, J;
@@ -1221,11 +1220,11 @@ __global__ void __launch_bounds__(BJ_NT)
   constexpr int ld = BJ_W + 1;
   for (int e = threadIdx.x; e < BJ_W * BJ_W; e += BJ_NT) {
     const int i = e / BJ_W, j = e % BJ_W;
-    a0[i * ld + j] = A[(long long)bj_index(I, J, i) * ne + bj_index(I, J, j)];
+    a0[i * BJ_LD + j] = A[(long long)bj_index(I, J, i) * ne + bj_index(I, J, j)];
     js[i * ld + j] = i == j ? 1.f : 0.f;
   }
   __syncthreads();
-  bj_sweep(a0, a1, js, ld, cs, round == 0);
+  bj_sweep(a0, a1, js, ld, round == 0);
   float* out = Jg + (size_t)blockIdx.x * BJ_W * BJ_W;
   for (int e = threadIdx.x; e < BJ_W * BJ_W; e += BJ_NT) out[e] = js[(e / BJ_W) * ld + e % BJ_W];
 }

@@ -37,7 +37,8 @@ using namespace fpca_jacobi;
 constexpr int LE_MAXN = 256;    // 8 block pairs: a portable cluster of 8 CTAs
 constexpr int LE_SWEEPS = 12;
 constexpr int LE_EXTRA = 4;     // vectors refined beyond k
-constexpr int LE_ITERS = 4;
+constexpr int LE_ITERS = 8;
+constexpr float LE_APART = 0.02f;  // off-diagonal norm over the gap that the refinement is left
 constexpr int LE_JLD = BJ_W + 4;             // row stride of a J in shared memory (16-byte rows)
 constexpr int LE_JS = BJ_W * LE_JLD + 4;     // floats per J: the 4 shift the banks of the next
 
@@ -46,7 +47,7 @@ __host__ __device__ constexpr int le_ld(int ne) { return ne + ne / 4; }
 
 inline size_t le_smem(int ne) {
   return sizeof(float) * (2 * (size_t)BJ_W * le_ld(ne) + (size_t)BJ_W * ne +
-                          (size_t)(ne / BJ_W) * LE_JS + 2 * BJ_W * (BJ_W + 1) + 32 + 16 + 16);
+                          (size_t)(ne / BJ_W) * LE_JS + 2 * BJ_W * BJ_LD + LE_MAXN + 16 + 16);
 }
 
 // Two-sided block Jacobi, one CTA per block pair of a round, the CTAs of the matrix in one
@@ -57,8 +58,9 @@ inline size_t le_smem(int ne) {
 // the two launches per round of the large-n path.  Columns of the row tiles are stored in
 // groups of 16 spaced by 20 floats, so that eight blocks' columns fall in different banks.
 __global__ void __launch_bounds__(BJ_NT, 1)
-    k_bj_cluster(int n, int ne, const double* __restrict__ A64, float* __restrict__ A,
-                 double* __restrict__ X, double* __restrict__ X0, float* __restrict__ lam32) {
+    k_bj_cluster(int n, int ne, int lead, int kk, const double* __restrict__ A64, float* __restrict__ A,
+                 double* __restrict__ X, double* __restrict__ X0, float* __restrict__ lam32,
+                 int* __restrict__ nref) {
   extern __shared__ __align__(16) float bjc[];
   const cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), NC = (int)cl.num_blocks();
@@ -67,10 +69,10 @@ __global__ void __launch_bounds__(BJ_NT, 1)
   float* Vr = Ar + BJ_W * LD;             // [32][LD]
   float* T = Vr + BJ_W * LD;              // [32][ne]
   float* Jall = T + BJ_W * ne;            // [NC][LE_JS]
-  float* a0 = Jall + NC * LE_JS;          // [32][33]
-  float* a1 = a0 + BJ_W * (BJ_W + 1);
-  float* cs = a1 + BJ_W * (BJ_W + 1);     // [32]
-  float* mass = cs + 32;                  // [8][2]: every CTA's off-diagonal, diagonal mass
+  float* a0 = Jall + NC * LE_JS;          // [32][BJ_LD]
+  float* a1 = a0 + BJ_W * BJ_LD;
+  float* dg = a1 + BJ_W * BJ_LD;          // [256]: the diagonal after a sweep
+  float* mass = dg + LE_MAXN;             // [8][2]: every CTA's off-diagonal, diagonal mass
   float* red = mass + 16;                 // [8][2]
   for (int e = tid; e < BJ_W * ne; e += BJ_NT) {
     const int i = e / ne, c = e - i * ne, gi = rank * BJ_W + i;
@@ -82,10 +84,12 @@ __global__ void __launch_bounds__(BJ_NT, 1)
   const bool act = tid < ne;
   const int ncg = ne / 8, rg = act ? tid / ncg : 0, cgp = act ? tid - rg * ncg : 0;
   float prev = 3e38f;
+  int done = 0;
   for (int sweep = 0; sweep < LE_SWEEPS; ++sweep) {
     for (int r = 0; r < nb - 1; ++r) {
       int I, J;
       rr_pair(nb, r, rank, I, J);
+#pragma unroll 4
       for (int e = tid; e < BJ_W * (ne / 4); e += BJ_NT) {
         const int i = e / (ne / 4), c4 = e - i * (ne / 4);
         *reinterpret_cast<float4*>(Ar + i * LD + 4 * c4 + 4 * (c4 >> 2)) =
@@ -95,11 +99,11 @@ __global__ void __launch_bounds__(BJ_NT, 1)
       __syncthreads();
       for (int e = tid; e < BJ_W * BJ_W; e += BJ_NT) {
         const int i = e / BJ_W, j = e % BJ_W;
-        a0[i * (BJ_W + 1) + j] = Ar[i * LD + (j < BJ_S ? 20 * I + j : 20 * J + j - BJ_S)];
+        a0[i * BJ_LD + j] = Ar[i * LD + (j < BJ_S ? 20 * I + j : 20 * J + j - BJ_S)];
         Jl[i * LE_JLD + j] = i == j ? 1.f : 0.f;
       }
       __syncthreads();
-      bj_sweep(a0, a1, Jl, LE_JLD, cs, r == 0);
+      bj_sweep(a0, a1, Jl, LE_JLD, r == 0);
       for (int c = 0; c < NC; ++c) {
         if (c == rank) continue;
         float4* dst = reinterpret_cast<float4*>(cl.map_shared_rank(Jall, c) + rank * LE_JS);
@@ -121,19 +125,29 @@ __global__ void __launch_bounds__(BJ_NT, 1)
         for (int h = 0; h < 2; ++h) {
           const float* ac = Ar + 4 * rg * LD + 20 * (h ? Jb : Ib);
           const float* vc = Vr + 4 * rg * LD + 20 * (h ? Jb : Ib);
-#pragma unroll 4
-          for (int k = 0; k < BJ_S; ++k) {
-            const float4 j0 = *reinterpret_cast<const float4*>(jr + (h * BJ_S + k) * LE_JLD);
-            const float4 j1 = *reinterpret_cast<const float4*>(jr + (h * BJ_S + k) * LE_JLD + 4);
-            const float jv[8] = {j0.x, j0.y, j0.z, j0.w, j1.x, j1.y, j1.z, j1.w};
+#pragma unroll 1
+          for (int k = 0; k < BJ_S; k += 4) {
+            float a[4][4], w[4][4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-              const float a = ac[q * LD + k], w = vc[q * LD + k];
+              const float4 av = *reinterpret_cast<const float4*>(ac + q * LD + k);
+              const float4 wv = *reinterpret_cast<const float4*>(vc + q * LD + k);
+              a[q][0] = av.x, a[q][1] = av.y, a[q][2] = av.z, a[q][3] = av.w;
+              w[q][0] = wv.x, w[q][1] = wv.y, w[q][2] = wv.z, w[q][3] = wv.w;
+            }
 #pragma unroll
-              for (int x = 0; x < 8; ++x) {
-                t[q][x] = fmaf(a, jv[x], t[q][x]);
-                v[q][x] = fmaf(w, jv[x], v[q][x]);
-              }
+            for (int kk = 0; kk < 4; ++kk) {
+              const float* jp = jr + (h * BJ_S + k + kk) * LE_JLD;
+              const float4 j0 = *reinterpret_cast<const float4*>(jp);
+              const float4 j1 = *reinterpret_cast<const float4*>(jp + 4);
+              const float jv[8] = {j0.x, j0.y, j0.z, j0.w, j1.x, j1.y, j1.z, j1.w};
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                  t[q][x] = fmaf(a[q][kk], jv[x], t[q][x]);
+                  v[q][x] = fmaf(w[q][kk], jv[x], v[q][x]);
+                }
             }
           }
         }
@@ -161,7 +175,7 @@ __global__ void __launch_bounds__(BJ_NT, 1)
           for (int x = 0; x < 8; ++x) t[q][x] = 0.f;
         const float* ja = Jl + 4 * rg;
         const float* tc = T + 4 * cgp;
-#pragma unroll 4
+#pragma unroll 8
         for (int k = 0; k < BJ_W; ++k) {
           const float4 a = *reinterpret_cast<const float4*>(ja + k * LE_JLD);
           const float4 t0 = *reinterpret_cast<const float4*>(tc + k * ne);
@@ -220,6 +234,28 @@ __global__ void __launch_bounds__(BJ_NT, 1)
     // converged to an off-diagonal norm of 1e-5 of the diagonal's, or stalled below 1e-4
     if (off <= 1e-10f * dia || off == 0.f || (off <= 1e-8f * dia && off > 0.25f * prev)) break;
     prev = off;
+    // or the `lead` largest eigenvalues stand so far from all others that the refinement takes
+    // the rest: what is left of the off-diagonal bounds every eigenvalue's error (Weyl) and,
+    // over the nearest gap, the factor by which an iteration there shrinks the error.  Only
+    // those are refined then (*nref): the others may still be mixed with one another.
+    if (off <= 1e-4f * dia) {
+      __syncthreads();
+      if (tid < n) dg[tid] = __ldcg(A + (size_t)tid * ne + tid);
+      __syncthreads();
+      bool apart = true;
+      if (tid < n) {
+        const float d = dg[tid];
+        float gap = 3e38f;
+        int rank = 0;
+        for (int j = 0; j < n; ++j) {
+          rank += dg[j] > d || (dg[j] == d && j < tid);
+          if (j != tid) gap = fminf(gap, fabsf(dg[j] - d));
+        }
+        apart = rank >= lead || sqrtf(off) <= LE_APART * gap;
+      }
+      done = __syncthreads_and(apart);
+      if (done) break;
+    }
   }
   for (int e = tid; e < BJ_W * n; e += BJ_NT) {
     const int i = e / n, c = e - i * n, gi = rank * BJ_W + i;
@@ -229,6 +265,7 @@ __global__ void __launch_bounds__(BJ_NT, 1)
       X0[(size_t)gi * n + c] = v;  // the fall-back's basis
     }
   }
+  if (rank == 0 && tid == 0) *nref = done ? lead : kk;
   if (tid < BJ_W && rank * BJ_W + tid < n) {
     const int c = rank * BJ_W + tid;
     lam32[c] = __ldcg(A + (size_t)c * ne + c);
@@ -240,13 +277,13 @@ __global__ void __launch_bounds__(BJ_NT, 1)
 // (kk x n).  state: [0] the Frobenius norm of A, [1..] the largest correction of iteration
 // 0, 1, ... (as float bits).
 __global__ void __launch_bounds__(LE_MAXN)
-    k_lead_init(int n, int kk, const float* __restrict__ lam32, const double* __restrict__ X,
+    k_lead_init(int n, const int* __restrict__ nref, const float* __restrict__ lam32, const double* __restrict__ X,
                 int* __restrict__ pos, int* __restrict__ lead, double* __restrict__ Xk,
                 float* __restrict__ state) {
   __shared__ float lam[LE_MAXN];
   __shared__ int ld[LE_MAXN];
   __shared__ float red[LE_MAXN / 32];
-  const int i = threadIdx.x;
+  const int i = threadIdx.x, kk = *nref;
   if (i < n) lam[i] = lam32[i];
   __syncthreads();
   if (i < n) {
@@ -284,12 +321,12 @@ __device__ __forceinline__ bool lead_done(const float* state, int it) {
 
 // U = A Xk' by one warp per (row i, vector j); the refined vectors take their columns in X.
 __global__ void __launch_bounds__(256)
-    k_lead_u(int n, int kk, int it, const double* __restrict__ A, const double* __restrict__ Xk,
+    k_lead_u(int n, const int* __restrict__ nref, int it, const double* __restrict__ A, const double* __restrict__ Xk,
              const int* __restrict__ lead, const float* __restrict__ state,
              double* __restrict__ U, double* __restrict__ X) {
   if (lead_done(state, it)) return;
   const int w = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (w >= n * kk) return;
+  if (w >= n * *nref) return;
   const int j = w / n, i = w - j * n;
   double s = 0.0;
   for (int m = lane; m < n; m += 32) s = fma(A[(size_t)i * n + m], Xk[(size_t)j * n + m], s);
@@ -303,11 +340,11 @@ __global__ void __launch_bounds__(256)
 // S[j][i] = X_i' U_j and R[j][i] = delta - X_i' Xk_j: block (32 columns i, vector j), 32
 // warps over the rows m (short FP64 chains), their sums added in shared memory.
 __global__ void __launch_bounds__(1024)
-    k_lead_sr(int n, int it, const double* __restrict__ X, const double* __restrict__ Xk,
+    k_lead_sr(int n, const int* __restrict__ nref, int it, const double* __restrict__ X, const double* __restrict__ Xk,
               const double* __restrict__ U, const int* __restrict__ pos,
               const float* __restrict__ state, double* __restrict__ S, double* __restrict__ R) {
   __shared__ double ps[32][33], pr[32][33];
-  if (lead_done(state, it)) return;
+  if (lead_done(state, it) || (int)blockIdx.y >= *nref) return;
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane, j = blockIdx.y;
   double s = 0.0, r = 0.0;
@@ -339,11 +376,11 @@ __global__ void __launch_bounds__(1024)
 // where both are refined, else by x_j alone).  state[1 + it] takes the largest correction of
 // the k wanted vectors, 1 while a cluster still couples by more than 1e-13 |A|.
 __global__ void __launch_bounds__(LE_MAXN)
-    k_lead_e(int n, int k, int it, const float* __restrict__ lam32, const int* __restrict__ pos,
+    k_lead_e(int n, int k, const int* __restrict__ nref, int it, const float* __restrict__ lam32, const int* __restrict__ pos,
              const int* __restrict__ lead, double* __restrict__ S, const double* __restrict__ R,
              double* __restrict__ E, double* __restrict__ lamk, float* __restrict__ state) {
   __shared__ float red[LE_MAXN / 32][2];
-  if (lead_done(state, it)) return;
+  if (lead_done(state, it) || (int)blockIdx.x >= *nref) return;
   const int i = threadIdx.x, j = blockIdx.x, self = lead[j];
   const bool in = i < n;
   const double s = in ? S[(size_t)j * n + i] : 0.0, r = in ? R[(size_t)j * n + i] : 0.0;
@@ -388,11 +425,11 @@ __global__ void __launch_bounds__(LE_MAXN)
 
 // Xk_j += X E_j by one warp per (row m, vector j).
 __global__ void __launch_bounds__(256)
-    k_lead_x(int n, int kk, int it, const double* __restrict__ X, const double* __restrict__ E,
+    k_lead_x(int n, const int* __restrict__ nref, int it, const double* __restrict__ X, const double* __restrict__ E,
              const float* __restrict__ state, double* __restrict__ Xk) {
   if (lead_done(state, it)) return;
   const int w = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (w >= n * kk) return;
+  if (w >= n * *nref) return;
   const int j = w / n, m = w - j * n;
   double s = 0.0;
   for (int i = lane; i < n; i += 32) s = fma(X[(size_t)m * n + i], E[(size_t)j * n + i], s);
@@ -569,12 +606,12 @@ __global__ void __launch_bounds__(256)
 // The k largest eigenvalues in descending order (ties by place) and their vectors: of the kk
 // refined ones (blocks 0..kk-1), or of all n (columns of X) after the fall-back.
 __global__ void __launch_bounds__(LE_MAXN)
-    k_lead_out(int n, int kk, int k, const float* __restrict__ state,
+    k_lead_out(int n, const int* __restrict__ nref, int k, const float* __restrict__ state,
                const double* __restrict__ lamk, const double* __restrict__ Xk,
                const double* __restrict__ lam, const double* __restrict__ X,
                double* __restrict__ theta, double* __restrict__ psi, int* __restrict__ order) {
   const bool full = state[LE_ITERS] > LE_BAD;
-  const int j = blockIdx.x, t = threadIdx.x, nv = full ? n : kk;
+  const int j = blockIdx.x, t = threadIdx.x, nv = full ? n : *nref;
   if (j >= nv) return;
   const double* l = full ? lam : lamk;
   const double lj = l[j];
@@ -610,7 +647,7 @@ fpca_status launch_rotate(fpca_ctx* ctx, int n, const float* gate, float limit, 
 size_t lead_eig_bytes(int n, int k) {
   const size_t ne = le_ne(n), kk = std::min(n, k + LE_EXTRA);
   return WsCarve::round(sizeof(float) * ne * ne) + WsCarve::round(sizeof(double) * (size_t)n * n) +
-         WsCarve::round(sizeof(float) * n) + 2 * WsCarve::round(sizeof(int) * n) +
+         WsCarve::round(sizeof(float) * n) + 2 * WsCarve::round(sizeof(int) * n) + WsCarve::round(sizeof(int)) +
          WsCarve::round(sizeof(float) * (LE_ITERS + 1)) +
          5 * WsCarve::round(sizeof(double) * kk * n) + WsCarve::round(sizeof(double) * kk) +
          4 * WsCarve::round(sizeof(double) * (size_t)n * n) + WsCarve::round(sizeof(double) * n) +
@@ -626,6 +663,7 @@ fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double
   float* lam32 = c.take<float>(n);
   int* pos = c.take<int>(n);
   int* lead = c.take<int>(n);
+  int* nref = c.take<int>(1);
   float* state = c.take<float>(LE_ITERS + 1);
   double* Xk = c.take<double>((size_t)kk * n);
   double* U = c.take<double>((size_t)kk * n);
@@ -654,19 +692,19 @@ fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_bj_cluster, n, ne, S, Af, X, X0, lam32);
+  cudaLaunchKernelEx(&cfg, k_bj_cluster, n, ne, k, kk, S, Af, X, X0, lam32, nref);
   FPCA_LAUNCHED(ctx, "eig_bj_cluster");
-  k_lead_init<<<8, LE_MAXN, 0, ctx->stream>>>(n, kk, lam32, X, pos, lead, Xk, state);
+  k_lead_init<<<8, LE_MAXN, 0, ctx->stream>>>(n, nref, lam32, X, pos, lead, Xk, state);
   FPCA_LAUNCHED(ctx, "eig_lead_init");
   const int wb = (n * kk + 7) / 8;  // blocks of 8 warps, one warp per (row, vector)
   for (int it = 0; it < LE_ITERS; ++it) {
-    k_lead_u<<<wb, 256, 0, ctx->stream>>>(n, kk, it, S, Xk, lead, state, U, X);
+    k_lead_u<<<wb, 256, 0, ctx->stream>>>(n, nref, it, S, Xk, lead, state, U, X);
     FPCA_LAUNCHED(ctx, "eig_lead_u");
-    k_lead_sr<<<dim3((n + 31) / 32, kk), 1024, 0, ctx->stream>>>(n, it, X, Xk, U, pos, state, Sx, R);
+    k_lead_sr<<<dim3((n + 31) / 32, kk), 1024, 0, ctx->stream>>>(n, nref, it, X, Xk, U, pos, state, Sx, R);
     FPCA_LAUNCHED(ctx, "eig_lead_sr");
-    k_lead_e<<<kk, LE_MAXN, 0, ctx->stream>>>(n, k, it, lam32, pos, lead, Sx, R, E, lamk, state);
+    k_lead_e<<<kk, LE_MAXN, 0, ctx->stream>>>(n, k, nref, it, lam32, pos, lead, Sx, R, E, lamk, state);
     FPCA_LAUNCHED(ctx, "eig_lead_e");
-    k_lead_x<<<wb, 256, 0, ctx->stream>>>(n, kk, it, X, E, state, Xk);
+    k_lead_x<<<wb, 256, 0, ctx->stream>>>(n, nref, it, X, E, state, Xk);
     FPCA_LAUNCHED(ctx, "eig_lead_x");
   }
   {
@@ -679,7 +717,7 @@ fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double
   }
   fpca_status cs = launch_rotate(ctx, n, state + LE_ITERS, LE_BAD, Sf, lamf, X0, Mf, Uf, normsq, flag);
   if (cs != FPCA_OK) return cs;
-  k_lead_out<<<n, LE_MAXN, 0, ctx->stream>>>(n, kk, k, state, lamk, Xk, lamf, X0, theta, psi, order);
+  k_lead_out<<<n, LE_MAXN, 0, ctx->stream>>>(n, nref, k, state, lamk, Xk, lamf, X0, theta, psi, order);
   FPCA_LAUNCHED(ctx, "eig_lead_out");
   return FPCA_OK;
 }

@@ -52,6 +52,7 @@ __device__ __forceinline__ void rr_rot(const float* A, int ld, int n, int p, int
 constexpr int BJ_S = 16;        // indices per block
 constexpr int BJ_W = 2 * BJ_S;  // subproblem width
 constexpr int BJ_NT = 256;      // threads of a subproblem sweep: one per 2 x 2 block
+constexpr int BJ_LD = 48;       // leading dimension of a subproblem in shared memory
 
 // local index i of the subproblem of block pair (I, J) -> global index
 __device__ __forceinline__ int bj_index(int I, int J, int i) {
@@ -71,35 +72,35 @@ __device__ __forceinline__ void bj_step_pair(bool within, int s, int i, int& p, 
   }
 }
 
-// One sweep of rotations over the 32 x 32 subproblem in `cur` (ld 33, double-buffered with
-// `nxt`), accumulated into J (32 x 32, leading dimension ldj, identity on entry).  The
-// pairs across the blocks meet once; those inside a block only when `within` is set
-// (once per sweep of the whole matrix is enough, since each block takes part in every
-// round).  Sixteen threads form a step's rotations, then each of the 256 threads turns one
-// 2 x 2 block of A and two entry pairs of J: about 0.17 us a step, where every thread
-// forming its own two rotations was bound by its instruction count (0.7 us with 768
-// threads).
-__device__ __forceinline__ void bj_sweep(float* cur, float* nxt, float* J, int ldj, float* cs,
-                                         bool within) {
-  constexpr int ld = BJ_W + 1;
+// The rotation of rr_rot by the approximate reciprocal and square root only (both give 0 for
+// an infinite tau^2); c^2 + s^2 = 1 to a few FP32 ulps all the same.
+__device__ __forceinline__ void bj_rot(float app, float apq, float aqq, float& c, float& sn) {
+  const float tau = __fdividef(aqq - app, 2.f * apq);
+  float root;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(tau, tau, 1.f)));
+  const float t = __fdividef(copysignf(1.f, tau), fabsf(tau) + root);
+  const bool on = fabsf(apq) > 1e-30f && fabsf(apq) > 1e-18f * fmaxf(fabsf(app), fabsf(aqq));
+  c = on ? rsqrtf(fmaf(t, t, 1.f)) : 1.f;
+  sn = on ? t * c : 0.f;
+}
+
+// One sweep of rotations over the 32 x 32 subproblem in `cur` (leading dimension BJ_LD,
+// double-buffered with `nxt`), accumulated into J (32 x 32, leading dimension ldj, identity on
+// entry).  The pairs across the blocks meet once; those inside a block only when `within` is
+// set (once per sweep of the whole matrix is enough, since each block takes part in every
+// round).  A serial chain of 16 or 31 steps, so each of the 256 threads forms the two rotations
+// of its 2 x 2 block itself and a step has one barrier; the J entries of the pairs across the
+// blocks stay in registers, the column that a pair gives up going to the next lane.  BJ_LD: the
+// two rows of a warp in different banks.  (Sixteen threads forming a step's rotations for all,
+// with exact square roots, took 0.47 us a step: see k_bj_cluster.)
+__device__ __forceinline__ void bj_sweep(float* cur, float* nxt, float* J, int ldj, bool within) {
+  constexpr int ld = BJ_LD;
   const int bi = threadIdx.x >> 4, bj = threadIdx.x & 15;
-  const int nw = within ? BJ_S - 1 : 0;
-  for (int st = 0; st < nw + BJ_S; ++st) {
-    const bool in = st < nw;
-    const int s = in ? st : st - nw;
-    if (threadIdx.x < 16) {
-      int p, q;
-      float c, sn;
-      bj_step_pair(in, s, threadIdx.x, p, q);
-      rr_rot(cur, ld, BJ_W, p, q, c, sn);
-      cs[2 * threadIdx.x] = c;
-      cs[2 * threadIdx.x + 1] = sn;
-    }
-    int pi, qi, pj, qj;
-    bj_step_pair(in, s, bi, pi, qi);
-    bj_step_pair(in, s, bj, pj, qj);
-    __syncthreads();
-    const float ci = cs[2 * bi], si = cs[2 * bi + 1], cj = cs[2 * bj], sj = cs[2 * bj + 1];
+  float cj, sj;
+  auto turn = [&](int pi, int qi, int pj, int qj) {
+    float ci, si;
+    bj_rot(cur[pi * ld + pi], cur[pi * ld + qi], cur[qi * ld + qi], ci, si);
+    bj_rot(cur[pj * ld + pj], cur[pj * ld + qj], cur[qj * ld + qj], cj, sj);
     const float m00 = cur[pi * ld + pj], m01 = cur[pi * ld + qj];
     const float m10 = cur[qi * ld + pj], m11 = cur[qi * ld + qj];
     const float c00 = cj * m00 - sj * m01, c01 = sj * m00 + cj * m01;
@@ -108,18 +109,50 @@ __device__ __forceinline__ void bj_sweep(float* cur, float* nxt, float* J, int l
     nxt[pi * ld + qj] = ci * c01 - si * c11;
     nxt[qi * ld + pj] = si * c00 + ci * c10;
     nxt[qi * ld + qj] = si * c01 + ci * c11;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float* row = J + (bi + 16 * h) * ldj;
-      const float vp = row[pj], vq = row[qj];
-      row[pj] = cj * vp - sj * vq;
-      row[qj] = sj * vp + cj * vq;
-    }
-    __syncthreads();
     float* t = cur;
     cur = nxt;
     nxt = t;
+  };
+  if (within) {
+    for (int s = 0; s < BJ_S - 1; ++s) {
+      int pi, qi, pj, qj;
+      bj_step_pair(true, s, bi, pi, qi);
+      bj_step_pair(true, s, bj, pj, qj);
+      turn(pi, qi, pj, qj);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float* row = J + (bi + 16 * h) * ldj;
+        const float vp = row[pj], vq = row[qj];
+        row[pj] = cj * vp - sj * vq;
+        row[qj] = sj * vp + cj * vq;
+      }
+      __syncthreads();
+    }
   }
+  float vp[2], vq[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    vp[h] = J[(bi + 16 * h) * ldj + bj];
+    vq[h] = J[(bi + 16 * h) * ldj + BJ_S + bj];
+  }
+  const int next = (threadIdx.x & 16) | ((bj + 1) & 15);
+#pragma unroll 4
+  for (int s = 0; s < BJ_S; ++s) {
+    turn(bi, BJ_S + ((bi + s) & (BJ_S - 1)), bj, BJ_S + ((bj + s) & (BJ_S - 1)));
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float a = vp[h], b = vq[h];
+      vp[h] = cj * a - sj * b;
+      vq[h] = __shfl_sync(0xffffffffu, sj * a + cj * b, next);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    J[(bi + 16 * h) * ldj + bj] = vp[h];
+    J[(bi + 16 * h) * ldj + BJ_S + bj] = vq[h];
+  }
+  __syncthreads();
 }
 
 }  // namespace fpca_jacobi
