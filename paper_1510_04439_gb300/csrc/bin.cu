@@ -239,66 +239,87 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// FP64 covariance bins of gridded data on CUDA cores: a 16 x 16 output tile
-// per block, subjects streamed through shared memory in chunks of 16.
-__global__ void k_cov_dense_f64(int n, int P, const void* __restrict__ y, int y_prec,
-                                const uint8_t* __restrict__ mask, const int32_t* __restrict__ Ni,
-                                const double* __restrict__ mu, int mode, int32_t* __restrict__ cnt,
-                                double* __restrict__ w, double* __restrict__ v) {
-  __shared__ double rp[16][17], rq[16][17], mp[16][17], mq[16][17], wsub[16];
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int p = blockIdx.y * 16 + ty, q = blockIdx.x * 16 + tx;
+// FP64 covariance bins of gridded data: an 8 x 8 output tile a block, tiles on and above the
+// diagonal (the ones below are their transposes), subjects streamed through shared memory.
+// FP64 runs at two results a clock on an SM here, so the tiles are small enough to give every
+// SM some at 64 nodes, and a pair costs three FP64 operations: the weight enters a subject's
+// row once, and the pair's weight is selected, not multiplied.  16 x 16 tiles of the whole
+// matrix with six operations took 65 us at 64 nodes, n = 100, and 60 us at 256, n = 50; these
+// take 26 and 20.
+constexpr int CD_T = 8;     // tile edge
+constexpr int CD_K = 32;    // subjects at a time
+constexpr int CD_W = 256;   // subjects whose weights are formed at a time
+__global__ void __launch_bounds__(CD_T * CD_T)
+    k_cov_dense_f64(int n, int P, int nt, const void* __restrict__ y, int y_prec,
+                    const uint8_t* __restrict__ mask, const int32_t* __restrict__ Ni,
+                    const double* __restrict__ mu, int mode, int32_t* __restrict__ cnt,
+                    double* __restrict__ w, double* __restrict__ v) {
+  __shared__ double rp[CD_K][CD_T + 1], rq[CD_K][CD_T + 1], wsub[CD_W];
+  __shared__ uint8_t mp[CD_K][CD_T], mq[CD_K][CD_T];
+  // tile pair (bi <= bj): bj runs fastest
+  int bi = 0, bj = (int)blockIdx.x;
+  while (bj >= nt - bi) bj -= nt - bi++;
+  bj += bi;
+  const int tid = threadIdx.x, tx = tid % CD_T, ty = tid / CD_T;
   int c = 0;
   double sw = 0.0, sv = 0.0;
-  for (int i0 = 0; i0 < n; i0 += 16) {
-    // load subject chunk: rows i0..i0+15 for the 16 p and 16 q columns
-    {
-      const int i = i0 + ty;
-      const int pc = blockIdx.y * 16 + tx, qc = blockIdx.x * 16 + tx;
-      double obs_p = 0.0, obs_q = 0.0, r_p = 0.0, r_q = 0.0;
-      if (i < n) {
-        if (pc < P) {
-          const size_t idx = (size_t)i * P + pc;
-          obs_p = (mask ? mask[idx] != 0 : true) ? 1.0 : 0.0;
-          if (obs_p != 0.0) {
-            const double yy = load_y(y, y_prec, idx);
-            r_p = mode == FPCA_COV_RESIDUAL ? yy - mu[pc] : yy;
-          }
-        }
-        if (qc < P) {
-          const size_t idx = (size_t)i * P + qc;
-          obs_q = (mask ? mask[idx] != 0 : true) ? 1.0 : 0.0;
-          if (obs_q != 0.0) {
-            const double yy = load_y(y, y_prec, idx);
-            r_q = mode == FPCA_COV_RESIDUAL ? yy - mu[qc] : yy;
-          }
+  for (int i0 = 0; i0 < n; i0 += CD_K) {
+    if (i0 % CD_W == 0) {
+      for (int e = tid; e < CD_W && i0 + e < n; e += CD_T * CD_T) {
+        const double N = (double)Ni[i0 + e];
+        wsub[e] = N >= 2.0 ? 1.0 / (N * (N - 1.0)) : 0.0;
+      }
+      __syncthreads();
+    }
+    const int kmax = min(CD_K, n - i0);
+    const double* wc = wsub + i0 % CD_W;
+#pragma unroll
+    for (int u = 0; u < 2 * CD_K / CD_T; ++u) {  // both sides, CD_T subjects at a time
+      const bool rows = u < CD_K / CD_T;
+      const int k = (u % (CD_K / CD_T)) * CD_T + ty, at = (rows ? bi : bj) * CD_T + tx;
+      bool ob = false;
+      double r = 0.0;
+      if (k < kmax && at < P) {
+        const size_t idx = (size_t)(i0 + k) * P + at;
+        ob = !mask || mask[idx] != 0;
+        if (ob) {
+          const double yy = load_y(y, y_prec, idx);
+          r = mode == FPCA_COV_RESIDUAL ? yy - mu[at] : yy;
         }
       }
-      mp[ty][tx] = obs_p;
-      rp[ty][tx] = r_p;
-      mq[ty][tx] = obs_q;
-      rq[ty][tx] = r_q;
-      if (tx == 0) {
-        const int N = i < n ? Ni[i] : 0;
-        wsub[ty] = N >= 2 ? 1.0 / ((double)N * (double)(N - 1)) : 0.0;
+      if (rows) {
+        mp[k][tx] = ob;
+        rp[k][tx] = k < kmax ? wc[k] * r : 0.0;
+      } else {
+        mq[k][tx] = ob;
+        rq[k][tx] = r;
       }
     }
     __syncthreads();
-    const int kmax = min(16, n - i0);
+#pragma unroll 4
     for (int k = 0; k < kmax; ++k) {
-      const double both = mp[k][ty] * mq[k][tx];
-      c += both != 0.0;
-      sw = __dadd_rn(sw, __dmul_rn(wsub[k], both));
-      sv = __dadd_rn(sv, __dmul_rn(__dmul_rn(wsub[k], rp[k][ty]), rq[k][tx]));
+      const bool both = mp[k][ty] & mq[k][tx];
+      c += both;
+      sw = __dadd_rn(sw, both ? wc[k] : 0.0);
+      sv = __dadd_rn(sv, __dmul_rn(rp[k][ty], rq[k][tx]));
     }
     __syncthreads();
   }
+  const int p = bi * CD_T + ty, q = bj * CD_T + tx;
   if (p < P && q < P) {
-    const size_t o = (size_t)p * P + q;
-    const bool diag = p == q;
-    cnt[o] = diag ? 0 : c;
-    w[o] = diag ? 0.0 : sw;
-    v[o] = diag ? 0.0 : sv;
+    if (p == q) {  // only pairs of an observation with itself
+      c = 0;
+      sw = sv = 0.0;
+    }
+    const size_t o = (size_t)p * P + q, ot = (size_t)q * P + p;
+    cnt[o] = c;
+    w[o] = sw;
+    v[o] = sv;
+    if (bi != bj) {
+      cnt[ot] = c;
+      w[ot] = sw;
+      v[ot] = sv;
+    }
   }
 }
 
@@ -945,9 +966,9 @@ fpca_status launch_cov_operands_bf16(fpca_ctx* ctx, int n, int P, int Kpad, cons
 fpca_status launch_cov_dense_f64(fpca_ctx* ctx, int n, int P, const void* y, int y_prec,
                                  const uint8_t* mask, const int32_t* Ni, const double* mu,
                                  int mode, int32_t* cnt, double* w, double* v) {
-  dim3 grid((P + 15) / 16, (P + 15) / 16);
-  k_cov_dense_f64<<<grid, dim3(16, 16), 0, ctx->stream>>>(n, P, y, y_prec, mask, Ni, mu, mode,
-                                                          cnt, w, v);
+  const int nt = (P + CD_T - 1) / CD_T;
+  k_cov_dense_f64<<<(unsigned)((long long)nt * (nt + 1) / 2), CD_T * CD_T, 0, ctx->stream>>>(
+      n, P, nt, y, y_prec, mask, Ni, mu, mode, cnt, w, v);
   FPCA_LAUNCHED(ctx, "cov_dense_f64");
   return FPCA_OK;
 }

@@ -198,18 +198,25 @@ struct VJobs {
 constexpr int VCOLS = 128;
 
 // Line L holds rows base + a*stride, a = 0..Ma-1, base = (L/stride)*Ma*stride + L%stride.
+// blockIdx.x: column block and, njobs blocks deep in z, job + njobs x (part of `nx` outputs of
+// the line): the sums are FP64 chains, so a small grid's lines are cut until every SM has some
+// (64 nodes, 15 taps: three blocks of 64 outputs took 136 us, 48 of 4 take 16).
 template <typename T, bool COMP>
 __global__ void __launch_bounds__(VCOLS)
-    k_vpass(VJobs jobs, int P, int Ma, int stride, int taps, const double* __restrict__ tab) {
+    k_vpass(VJobs jobs, int njobs, int nx, int P, int Ma, int stride, int taps,
+            const double* __restrict__ tab) {
   extern __shared__ unsigned char vsm[];
   T* wt = reinterpret_cast<T*>(vsm);   // [TROWS][TW]
-  T* tile = wt + TROWS * TW;           // [Ma][VCOLS]
-  const VJob& jb = jobs.j[blockIdx.z];
+  T* tile = wt + TROWS * TW;           // [rows a0..a1][VCOLS]
+  const VJob& jb = jobs.j[blockIdx.z % njobs];
+  const int x0 = (int)(blockIdx.z / njobs) * nx, x1 = min(Ma, x0 + nx);
+  const int a0 = max(0, x0 - taps), a1 = min(Ma, x1 + taps);
   for (int i = threadIdx.x; i < TROWS * TW; i += VCOLS) wt[i] = (T)tab[i];
   const int col = blockIdx.x * VCOLS + threadIdx.x;
   const int L = blockIdx.y;
   const long long base = (long long)(L / stride) * Ma * stride + (L % stride);
-  for (int a = 0; a < Ma; ++a) {
+#pragma unroll 4
+  for (int a = a0; a < a1; ++a) {
     const long long row = base + (long long)a * stride;
     T val = T(0);
     if (col < P) {
@@ -223,11 +230,11 @@ __global__ void __launch_bounds__(VCOLS)
         if (jb.sub) val -= static_cast<const T*>(jb.sub)[e];
       }
     }
-    tile[a * VCOLS + threadIdx.x] = val;
+    tile[(a - a0) * VCOLS + threadIdx.x] = val;
   }
   __syncthreads();
   if (col >= P) return;
-  for (int x = 0; x < Ma; ++x) {
+  for (int x = x0; x < x1; ++x) {
     const int lo = max(-taps, -x), hi = min(taps, Ma - 1 - x);
     T s0 = 0, s1 = 0, s2 = 0, c0 = 0, c1 = 0, c2 = 0;
     const T* w0 = wt + jb.row[0] * TW + TMAX;
@@ -235,20 +242,20 @@ __global__ void __launch_bounds__(VCOLS)
     const T* w2 = wt + jb.row[jb.npow > 2 ? 2 : 0] * TW + TMAX;
     if (jb.npow == 3) {
       for (int k = lo; k <= hi; ++k) {
-        const T vv = tile[(x + k) * VCOLS + threadIdx.x];
+        const T vv = tile[(x - a0 + k) * VCOLS + threadIdx.x];
         kadd<T, COMP>(s0, c0, w0[k], vv);
         kadd<T, COMP>(s1, c1, w1[k], vv);
         kadd<T, COMP>(s2, c2, w2[k], vv);
       }
     } else if (jb.npow == 2) {
       for (int k = lo; k <= hi; ++k) {
-        const T vv = tile[(x + k) * VCOLS + threadIdx.x];
+        const T vv = tile[(x - a0 + k) * VCOLS + threadIdx.x];
         kadd<T, COMP>(s0, c0, w0[k], vv);
         kadd<T, COMP>(s1, c1, w1[k], vv);
       }
     } else {
       for (int k = lo; k <= hi; ++k) {
-        const T vv = tile[(x + k) * VCOLS + threadIdx.x];
+        const T vv = tile[(x - a0 + k) * VCOLS + threadIdx.x];
         kadd<T, COMP>(s0, c0, w0[k], vv);
       }
     }
@@ -1331,8 +1338,13 @@ bool launch_vpass(fpca_ctx* ctx, const VJobs& jobs, int njobs, int P, int Ma, in
                            (int)(sizeof(T) * (TROWS * TW + (size_t)64 * VCOLS)));
       attr = true;
     }
-    k_vpass<T, COMP><<<grid, VCOLS, sizeof(T) * (TROWS * TW + (size_t)Ma * VCOLS), ctx->stream>>>(
-        jobs, P, Ma, stride, taps, tab);
+    int nx = Ma;
+    while (nx > 4 && (long long)grid.x * lines * njobs * ((Ma + nx - 1) / nx) < 4 * ctx->num_sms)
+      nx = (nx + 1) / 2;
+    const int rows = std::min(Ma, nx + 2 * taps);
+    k_vpass<T, COMP><<<dim3(grid.x, lines, njobs * ((Ma + nx - 1) / nx)), VCOLS,
+                       sizeof(T) * (TROWS * TW + (size_t)rows * VCOLS), ctx->stream>>>(
+        jobs, njobs, nx, P, Ma, stride, taps, tab);
   }
   return true;
 }
