@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(NT2, 2)
   // CV terms of the current item gathered in shared memory, added to its accumulators
   // when the CTA moves on to another item (one flush per item, not a reduction per tile)
   __shared__ CvShared cvs;
-  if (threadIdx.x == 0) cvs.v[0] = cvs.v[1] = cvs.v[2] = 0.0;
+  cv_clear(&cvs);
   __syncthreads();
   auto flush = [&]() {
     if (cur >= 0) cv_flush(&cvs, items[cur].ep.cvacc);
@@ -816,179 +816,166 @@ __global__ void __launch_bounds__(NT2, 2)
   flush();
 }
 
-// NO outputs x NP powers along a line from one sliding window:
-// out[p][j] = sum_{k < nt} w_p[k] * x[(j + k) * stride].
-template <int NO, int NP, bool COMP>
-__device__ __forceinline__ void slide_sum_multi(const float* __restrict__ x, int stride,
-                                                const float4* const (&w4)[NP], int nt,
-                                                float (&out)[NP][NO]) {
-  float win[NO + 4];
-#pragma unroll
-  for (int j = 0; j < NO; ++j) win[j] = x[j * stride];
-  float nxt[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) nxt[u] = x[(NO + u) * stride];
-  float sum[NP][NO], cmp[NP][NO];
-#pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int j = 0; j < NO; ++j) {
-      sum[q][j] = 0.f;
-      cmp[q][j] = 0.f;
-    }
-#pragma unroll 2
-  for (int kc = 0; kc < nt; kc += 4) {
-#pragma unroll
-    for (int u = 0; u < 4; ++u) win[NO + u] = nxt[u];
-    if (kc + 4 < nt) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) nxt[u] = x[(NO + kc + 4 + u) * stride];
-    }
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const float4 w = w4[q][kc >> 2];
-      if constexpr (COMP) {
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          float pp = w.x * win[j];
-          pp = fmaf(w.y, win[j + 1], pp);
-          pp = fmaf(w.z, win[j + 2], pp);
-          pp = fmaf(w.w, win[j + 3], pp);
-          chunk_add<true>(sum[q][j], cmp[q][j], pp);
-        }
-      } else {
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          sum[q][j] = fmaf(w.x, win[j], sum[q][j]);
-          sum[q][j] = fmaf(w.y, win[j + 1], sum[q][j]);
-          sum[q][j] = fmaf(w.z, win[j + 2], sum[q][j]);
-          sum[q][j] = fmaf(w.w, win[j + 3], sum[q][j]);
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < NO; ++j) win[j] = win[j + 4];
-  }
-#pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int j = 0; j < NO; ++j) out[q][j] = sum[q][j];
-}
-
-// slide_sum_multi with NCH = nt / 4 fixed at compile time (12-tap partials with COMP).
-template <int NO, int NP, int NCH, bool COMP>
-__device__ __forceinline__ void slide_sum_multi_fixed(const float* __restrict__ x, int stride,
-                                                      const float4* const (&w4)[NP],
-                                                      float (&out)[NP][NO]) {
-  constexpr int NW = NO + 4 * NCH;
-  float win[NW];
-#pragma unroll
-  for (int j = 0; j < NW; ++j) win[j] = x[j * stride];
-  float sum[NP][NO], cmp[NP][NO];
-#pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int j = 0; j < NO; ++j) {
-      sum[q][j] = 0.f;
-      cmp[q][j] = 0.f;
-    }
-  if constexpr (COMP) {
-    // partials of up to 12 taps (three chunks), Kahan-added: one compensation step per
-    // output for windows up to 24 taps, where 8-tap partials need two from 17 taps on
-    // (these passes are bound by their instruction count)
-#pragma unroll
-    for (int kc = 0; kc < NCH; kc += 3) {
-      const int nch = NCH - kc < 3 ? NCH - kc : 3;
-#pragma unroll
-      for (int q = 0; q < NP; ++q) {
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          float p = 0.f;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            if (c >= nch) break;
-            const float4 w = w4[q][kc + c];
-            const int b = 4 * (kc + c) + j;
-            p = (c == 0) ? w.x * win[b] : fmaf(w.x, win[b], p);
-            p = fmaf(w.y, win[b + 1], p);
-            p = fmaf(w.z, win[b + 2], p);
-            p = fmaf(w.w, win[b + 3], p);
-          }
-          if (kc == 0) {
-            sum[q][j] = p;
-          } else {
-            chunk_add<true>(sum[q][j], cmp[q][j], p);
-          }
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int kc = 0; kc < NCH; ++kc) {
-    const int b = 4 * kc;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      const float4 w = w4[q][kc];
-      if constexpr (!COMP) {
-#pragma unroll
-        for (int j = 0; j < NO; ++j) {
-          sum[q][j] = fmaf(w.x, win[b + j], sum[q][j]);
-          sum[q][j] = fmaf(w.y, win[b + j + 1], sum[q][j]);
-          sum[q][j] = fmaf(w.z, win[b + j + 2], sum[q][j]);
-          sum[q][j] = fmaf(w.w, win[b + j + 3], sum[q][j]);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < NP; ++q)
-#pragma unroll
-    for (int j = 0; j < NO; ++j) out[q][j] = sum[q][j];
-}
-
-template <int NO, int NP, bool COMP>
-__device__ __forceinline__ void slide_sum_multi_any(const float* __restrict__ x, int stride,
-                                                    const float4* const (&w4)[NP], int nt,
-                                                    float (&out)[NP][NO]) {
-  switch (nt >> 2) {
-    case 1: slide_sum_multi_fixed<NO, NP, 1, COMP>(x, stride, w4, out); return;
-    case 2: slide_sum_multi_fixed<NO, NP, 2, COMP>(x, stride, w4, out); return;
-    case 3: slide_sum_multi_fixed<NO, NP, 3, COMP>(x, stride, w4, out); return;
-    case 4: slide_sum_multi_fixed<NO, NP, 4, COMP>(x, stride, w4, out); return;
-    case 5: slide_sum_multi_fixed<NO, NP, 5, COMP>(x, stride, w4, out); return;
-    case 6: slide_sum_multi_fixed<NO, NP, 6, COMP>(x, stride, w4, out); return;
-    case 7: slide_sum_multi_fixed<NO, NP, 7, COMP>(x, stride, w4, out); return;
-    case 8: slide_sum_multi_fixed<NO, NP, 8, COMP>(x, stride, w4, out); return;
-    case 9: slide_sum_multi_fixed<NO, NP, 9, COMP>(x, stride, w4, out); return;
-    case 10: slide_sum_multi_fixed<NO, NP, 10, COMP>(x, stride, w4, out); return;
-    default: slide_sum_multi<NO, NP, COMP>(x, stride, w4, nt, out); return;
-  }
-}
-
-// s-side pass (FP32): one block = one line (Ma rows along the pass axis) x
-// 128 columns of one input array; rows padded with zeros above and below.
+// s-side pass (FP32): one block = one line (Ma rows along the pass axis) x 128 columns of one
+// input array; rows padded with zeros above and below.  A thread takes two columns and every
+// second group of VROWS outputs, in packed arithmetic: the pass is bound by its instruction
+// count, and two columns of a tile row are a register pair as they lie (64 x 64, 19 taps: VP_OLD
+// with one column a thread, VP_NEW).
 constexpr int VROWS = 8;  // outputs per sliding window
-template <int NP, bool COMP>
-__device__ __forceinline__ void vpass2_line(const VJob& jb, const float* tile, const float* wp,
-                                            int ntp, int Ma, int stride, long long base, int P,
-                                            int col) {
-  // Ma: the rows of the line computed here (a prefix of it, see SBand)
-  const float4* w4[NP];
+
+// s + p with Kahan compensation, c the negated error: four packed operations.
+template <bool COMP>
+__device__ __forceinline__ void chunk_add2(float2& s, float2& c, float2 p) {
+  if constexpr (COMP) {
+    const float2 y = __fadd2_rn(p, c);
+    const float2 t = __fadd2_rn(s, y);
+    c = __fadd2_rn(y, __ffma2_rn(t, make_float2(-1.f, -1.f), s));  // y - (t - s)
+    s = t;
+  } else {
+    s = __fadd2_rn(s, p);
+  }
+}
+
+// out[j] = sum_{k < 4 NCH} w[k] * x[(j + k) * VCOLS] for each of the job's powers, from one
+// window in registers; wp: {w, w} per tap, two taps per float4, ntp taps a row.  Partials of
+// up to 12 taps, Kahan-added (without COMP one running sum).
+template <int NCH, bool COMP, typename Put>
+__device__ __forceinline__ void vline_fixed(const VJob& jb, const float2* __restrict__ x,
+                                            const float4* __restrict__ wp, int ntp, Put put) {
+  constexpr int NW = VROWS + 4 * NCH - 1, PART = COMP ? 12 : 4 * NCH;
+  float2 win[NW];
 #pragma unroll
-  for (int q = 0; q < NP; ++q) w4[q] = reinterpret_cast<const float4*>(wp + jb.row[q] * ntp);
-  for (int x0 = 0; x0 < Ma; x0 += VROWS) {
-    float out[NP][VROWS];
-    slide_sum_multi_any<VROWS, NP, COMP>(tile + (size_t)x0 * VCOLS + threadIdx.x, VCOLS, w4, ntp,
-                                         out);
+  for (int j = 0; j < NW; ++j) win[j] = x[j * (VCOLS / 2)];
+#pragma unroll 1
+  for (int q = 0; q < jb.npow; ++q) {
+    const float4* w4 = wp + jb.row[q] * (ntp / 2);
+    float2 sum[VROWS], cmp[VROWS];
+#pragma unroll
+    for (int k0 = 0; k0 < 4 * NCH; k0 += PART) {
+      float2 p[VROWS];
+#pragma unroll
+      for (int k = k0; k < (k0 + PART < 4 * NCH ? k0 + PART : 4 * NCH); k += 2) {
+        const float4 w = w4[k >> 1];
+        const float2 wa = make_float2(w.x, w.y), wb = make_float2(w.z, w.w);
+#pragma unroll
+        for (int j = 0; j < VROWS; ++j) {
+          p[j] = k == k0 ? __fmul2_rn(wa, win[j + k]) : __ffma2_rn(wa, win[j + k], p[j]);
+          p[j] = __ffma2_rn(wb, win[j + k + 1], p[j]);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < VROWS; ++j) {
+        if (k0 == 0) {
+          sum[j] = p[j];
+          cmp[j] = make_float2(0.f, 0.f);
+        } else {
+          chunk_add2<COMP>(sum[j], cmp[j], p[j]);
+        }
+      }
+    }
+    put(q, sum);
+  }
+}
+
+// The same for any ntp (more than 40 taps), a partial of 4 taps at a time.
+template <bool COMP, typename Put>
+__device__ __forceinline__ void vline_any(const VJob& jb, const float2* __restrict__ x,
+                                          const float4* __restrict__ wp, int ntp, Put put) {
+#pragma unroll 1
+  for (int q = 0; q < jb.npow; ++q) {
+    const float4* w4 = wp + jb.row[q] * (ntp / 2);
+    float2 sum[VROWS], cmp[VROWS], win[VROWS + 3];
 #pragma unroll
     for (int j = 0; j < VROWS; ++j) {
-      const int x = x0 + j;
-      if (x < Ma) {
-        const long long o = (base + (long long)x * stride) * P + col;
+      sum[j] = cmp[j] = make_float2(0.f, 0.f);
+      win[j] = x[j * (VCOLS / 2)];
+    }
+#pragma unroll 1
+    for (int k = 0; k < ntp; k += 4) {
 #pragma unroll
-        for (int q = 0; q < NP; ++q) static_cast<float*>(jb.out[q])[o] = out[q][j];
+      for (int u = 0; u < 3; ++u) win[VROWS + u] = x[(VROWS + k + u) * (VCOLS / 2)];
+      const float4 wa = w4[k >> 1], wb = w4[(k >> 1) + 1];
+#pragma unroll
+      for (int j = 0; j < VROWS; ++j) {
+        const float2 w0 = make_float2(wa.x, wa.y), w1 = make_float2(wa.z, wa.w);
+        const float2 w2 = make_float2(wb.x, wb.y), w3 = make_float2(wb.z, wb.w);
+        if constexpr (COMP) {
+          float2 p = __fmul2_rn(w0, win[j]);
+          p = __ffma2_rn(w1, win[j + 1], p);
+          p = __ffma2_rn(w2, win[j + 2], p);
+          chunk_add2<true>(sum[j], cmp[j], __ffma2_rn(w3, win[j + 3], p));
+        } else {
+          sum[j] = __ffma2_rn(w0, win[j], sum[j]);
+          sum[j] = __ffma2_rn(w1, win[j + 1], sum[j]);
+          sum[j] = __ffma2_rn(w2, win[j + 2], sum[j]);
+          sum[j] = __ffma2_rn(w3, win[j + 3], sum[j]);
+        }
+      }
+      if (k + 4 < ntp) {
+#pragma unroll
+        for (int j = 0; j < VROWS - 1; ++j) win[j] = win[j + 4];
+        win[VROWS - 1] = x[(VROWS + k + 3) * (VCOLS / 2)];
       }
     }
+    put(q, sum);
+  }
+}
+
+// Columns col, col + 1 of the line's outputs (a prefix of Ma rows of it, see SBand).
+template <bool COMP, bool WIDE>
+__device__ __forceinline__ void vpass2_line(const VJob& jb, const float* tile, const float* wp,
+                                            int ntp, int Ma, int stride, long long base, int P,
+                                            int col0) {
+  constexpr int PAIRS = VCOLS / 2, GROUPS = VCOLS / PAIRS;
+  const int cp = threadIdx.x % PAIRS, col = col0 + 2 * cp;
+  if (col >= P) return;
+  const bool two = col + 1 < P, even = P % 2 == 0;
+  for (int x0 = VROWS * (threadIdx.x / PAIRS); x0 < Ma; x0 += VROWS * GROUPS) {
+    const float2* x = reinterpret_cast<const float2*>(tile + (size_t)x0 * VCOLS) + cp;
+    const float4* w4 = reinterpret_cast<const float4*>(wp);
+    auto put = [&](int q, const float2 (&out)[VROWS]) {
+      float* o = static_cast<float*>(jb.out[q]) + (base + (long long)x0 * stride) * P + col;
+#pragma unroll
+      for (int j = 0; j < VROWS; ++j) {
+        if (x0 + j < Ma) {
+          if (even) {
+            *reinterpret_cast<float2*>(o) = out[j];
+          } else {
+            o[0] = out[j].x;
+            if (two) o[1] = out[j].y;
+          }
+        }
+        o += (long long)stride * P;
+      }
+    };
+    if constexpr (WIDE) {
+      switch (ntp >> 2) {
+        case 7: vline_fixed<7, COMP>(jb, x, w4, ntp, put); break;
+        case 8: vline_fixed<8, COMP>(jb, x, w4, ntp, put); break;
+        case 9: vline_fixed<9, COMP>(jb, x, w4, ntp, put); break;
+        case 10: vline_fixed<10, COMP>(jb, x, w4, ntp, put); break;
+        default: vline_any<COMP>(jb, x, w4, ntp, put); break;
+      }
+    } else {
+      switch (ntp >> 2) {
+        case 1: vline_fixed<1, COMP>(jb, x, w4, ntp, put); break;
+        case 2: vline_fixed<2, COMP>(jb, x, w4, ntp, put); break;
+        case 3: vline_fixed<3, COMP>(jb, x, w4, ntp, put); break;
+        case 4: vline_fixed<4, COMP>(jb, x, w4, ntp, put); break;
+        case 5: vline_fixed<5, COMP>(jb, x, w4, ntp, put); break;
+        default: vline_fixed<6, COMP>(jb, x, w4, ntp, put); break;
+      }
+    }
+  }
+}
+
+// weights {w, w} in padded form: wp[row][k], k = 0..nt-1 <-> offset k - T (zero beyond 2T)
+__device__ __forceinline__ void load_weight_pairs(const double* __restrict__ tab, int T, int nt,
+                                                  float2* __restrict__ wp) {
+  for (int e = threadIdx.x; e < TROWS * nt; e += blockDim.x) {
+    const int row = e / nt, k = e - (e / nt) * nt;
+    const float w = k <= 2 * T ? (float)tab[row * TW + TMAX + (k - T)] : 0.f;
+    wp[e] = make_float2(w, w);
   }
 }
 
@@ -1004,14 +991,16 @@ struct SBand {
   int R, C, T0;
 };
 
-template <bool COMP>
-__global__ void __launch_bounds__(VCOLS)
+// WIDE: more than VNARROW padded taps; the narrower windows leave registers for a fourth block.
+constexpr int VNARROW = 24;
+template <bool COMP, bool WIDE>
+__global__ void __launch_bounds__(VCOLS, WIDE ? 3 : 4)
     k_vpass2(VJobs jobs, int P, int Ma, int stride, int taps, int ntp,
              const double* __restrict__ tab, int bulk, SBand band, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char vsm2[];
   __shared__ __align__(8) uint64_t vbar;
-  float* wp = reinterpret_cast<float*>(vsm2);  // [TROWS][ntp]
-  float* tile = wp + TROWS * ntp;              // [Ma + ntp + VROWS][VCOLS], row r <-> x = r - taps
+  float* wp = reinterpret_cast<float*>(vsm2);  // [TROWS][ntp] pairs
+  float* tile = wp + 2 * TROWS * ntp;          // [Ma + ntp + VROWS][VCOLS], row r <-> x = r - taps
   const int nrow = ((Ma + VROWS - 1) / VROWS) * VROWS + ntp;
   float* subt = tile + (size_t)nrow * VCOLS;   // [Ma][VCOLS] when a job subtracts a fold
   const VJob& jb = jobs.j[blockIdx.z];
@@ -1053,25 +1042,29 @@ __global__ void __launch_bounds__(VCOLS)
                          static_cast<const float*>(jb.sub) + e, rbytes, bar);
       }
     }
-    load_padded_weights(tab, taps, ntp, wp);
+    load_weight_pairs(tab, taps, ntp, reinterpret_cast<float2*>(wp));
     for (int r = 0; r < nrow; ++r)
       if (r < taps || r >= taps + Mload) tile[(size_t)r * VCOLS + threadIdx.x] = 0.f;
     const bool landed = ptx::mbar_wait(bar, 0, err);
     if (__syncthreads_or(!landed)) return;
     if (jb.in_int || jb.sub) {
-      for (int x = 0; x < Mload; ++x) {
-        float* tv = tile + (size_t)(x + taps) * VCOLS + threadIdx.x;
+      for (int e = threadIdx.x; e < Mload * (VCOLS / 4); e += VCOLS) {
+        float4* tv = reinterpret_cast<float4*>(tile + (size_t)taps * VCOLS) + e;
+        float4 v = *tv, u = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (jb.sub) u = reinterpret_cast<const float4*>(subt)[e];
         if (jb.in_int) {
-          int c = __float_as_int(*tv);
-          if (jb.sub) c -= __float_as_int(subt[(size_t)x * VCOLS + threadIdx.x]);
-          *tv = c > 0 ? 1.f : 0.f;
+          auto filled = [](float a, float b) {
+            return __float_as_int(a) - __float_as_int(b) > 0 ? 1.f : 0.f;
+          };
+          v = make_float4(filled(v.x, u.x), filled(v.y, u.y), filled(v.z, u.z), filled(v.w, u.w));
         } else {
-          *tv -= subt[(size_t)x * VCOLS + threadIdx.x];
+          v = make_float4(v.x - u.x, v.y - u.y, v.z - u.z, v.w - u.w);
         }
+        *tv = v;
       }
     }
   } else {
-    load_padded_weights(tab, taps, ntp, wp);
+    load_weight_pairs(tab, taps, ntp, reinterpret_cast<float2*>(wp));
     // rows in batches of 8 so that eight global loads are in flight per thread
     for (int r0 = 0; r0 < nrow; r0 += 8) {
       float vals[8];
@@ -1098,18 +1091,12 @@ __global__ void __launch_bounds__(VCOLS)
     }
   }
   __syncthreads();
-  if (col >= P) return;
-  if (jb.npow == 3)
-    vpass2_line<3, COMP>(jb, tile, wp, ntp, Mcomp, stride, base, P, col);
-  else if (jb.npow == 2)
-    vpass2_line<2, COMP>(jb, tile, wp, ntp, Mcomp, stride, base, P, col);
-  else
-    vpass2_line<1, COMP>(jb, tile, wp, ntp, Mcomp, stride, base, P, col);
+  vpass2_line<COMP, WIDE>(jb, tile, wp, ntp, Mcomp, stride, base, P, col0);
 }
 
 size_t vpass2_smem(int Ma, int ntp, bool with_sub) {
   const int nrow = ((Ma + VROWS - 1) / VROWS) * VROWS + ntp;
-  return sizeof(float) * ((size_t)TROWS * ntp + (size_t)nrow * VCOLS +
+  return sizeof(float) * (2 * (size_t)TROWS * ntp + (size_t)nrow * VCOLS +
                           (with_sub ? (size_t)Ma * VCOLS : 0));
 }
 
@@ -1323,14 +1310,20 @@ bool launch_vpass(fpca_ctx* ctx, const VJobs& jobs, int njobs, int P, int Ma, in
     const size_t sm = vpass2_smem(Ma, ntp, with_sub);
     // bulk row copies need 16-byte aligned rows: P a multiple of 4
     const int bulk = (P % 4 == 0) ? 1 : 0;
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_vpass2<COMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)vpass2_smem(64, 128, true));
-      attr = true;
-    }
-    k_vpass2<COMP><<<grid, VCOLS, sm, ctx->stream>>>(jobs, P, Ma, stride, taps, ntp, tab, bulk,
-                                                     band, ctx->d_err);
+    auto launch = [&](auto kern, bool& attr) {
+      if (!attr) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)vpass2_smem(64, 128, true));
+        attr = true;
+      }
+      kern<<<grid, VCOLS, sm, ctx->stream>>>(jobs, P, Ma, stride, taps, ntp, tab, bulk, band,
+                                             ctx->d_err);
+    };
+    static bool attr[2] = {false, false};
+    if (ntp > VNARROW)
+      launch(k_vpass2<COMP, true>, attr[1]);
+    else
+      launch(k_vpass2<COMP, false>, attr[0]);
   } else {
     static bool attr = false;
     if (!attr) {

@@ -335,12 +335,17 @@ static __constant__ int8_t c_slot_pow[NSL] = {0, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0,
 
 
 // CV terms a persistent CTA gathers over its tiles (held-out error, scored weight,
-// weight of EMPTY points) in shared memory: each warp adds its tile's sums with one
-// atomic per term, and the CTA adds the totals to ep.cvacc once (cv_flush).  No
-// register is held across tiles and no block barrier is spent per tile.
+// weight of EMPTY points) in shared memory: each warp adds its tile's sums to its own
+// row, and the CTA adds the totals to ep.cvacc once (cv_flush).  No register is held
+// across tiles, no block barrier is spent per tile, and no warp waits for another
+// (one row for all meant eight warps' FP64 compare-and-swap loops on three words).
 struct CvShared {
-  double v[3];
+  double v[NT2 / 32][3];
 };
+
+__device__ __forceinline__ void cv_clear(CvShared* cvs) {
+  if (threadIdx.x < NT2 / 32 * 3) (&cvs->v[0][0])[threadIdx.x] = 0.0;
+}
 
 __device__ __forceinline__ void cv_warp_add(CvShared* cvs, float e, float i, float o) {
 #pragma unroll
@@ -350,9 +355,10 @@ __device__ __forceinline__ void cv_warp_add(CvShared* cvs, float e, float i, flo
     o += __shfl_xor_sync(0xffffffffu, o, k);
   }
   if ((threadIdx.x & 31) == 0) {
-    atomicAdd(&cvs->v[0], (double)e);
-    atomicAdd(&cvs->v[1], (double)i);
-    atomicAdd(&cvs->v[2], (double)o);
+    double* v = cvs->v[threadIdx.x >> 5];
+    v[0] += (double)e;
+    v[1] += (double)i;
+    v[2] += (double)o;
   }
 }
 
@@ -360,14 +366,13 @@ __device__ __forceinline__ void cv_warp_add(CvShared* cvs, float e, float i, flo
 // precedes it) and the shared sums cleared for the next item.
 __device__ __forceinline__ void cv_flush(CvShared* cvs, double* acc) {
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (acc) {
-      atomicAdd(acc + 0, cvs->v[0]);
-      atomicAdd(acc + 1, cvs->v[1]);
-      atomicAdd(acc + 2, cvs->v[2]);
-    }
-    cvs->v[0] = cvs->v[1] = cvs->v[2] = 0.0;
+  if (threadIdx.x < 3 && acc) {
+    double s = 0.0;
+    for (int w = 0; w < NT2 / 32; ++w) s += cvs->v[w][threadIdx.x];
+    atomicAdd(acc + threadIdx.x, s);
   }
+  __syncthreads();
+  cv_clear(cvs);
   __syncthreads();
 }
 
@@ -376,40 +381,47 @@ __device__ __forceinline__ void cv_flush(CvShared* cvs, double* acc) {
 // status, CV terms and the fused y = Gamma_hat Omega epilogue.  `mid` is shared
 // scratch of at least HT * C + NTH floats (the y epilogue reuses it).  With `cvs`
 // the CV terms go to the CTA's shared sums (the kernel flushes them); without, the
-// block adds this tile's terms to ep.cvacc.
-template <int C, int NTH>
+// block adds this tile's terms to ep.cvacc.  With LIST only the nlist <= LIST points of
+// `list` (tile-local i C + c), their slots in [NSL][LIST + 1], and their CV terms to `terms`
+// ([3][LIST]) instead of the sums.
+template <int C, int NTH, int LIST = 0>
 __device__ __forceinline__ void tside_phase3(const float* __restrict__ slots, int SC, int half,
                                              int P, int xs, int a0, int th,
                                              const double* __restrict__ mu_raw,
                                              float* __restrict__ gamma,
                                              uint8_t* __restrict__ status, const Epilogue<float>& ep,
-                                             double* red, float* mid, CvShared* cvs = nullptr) {
+                                             double* red, float* mid, CvShared* cvs = nullptr,
+                                             const uint16_t* list = nullptr, int nlist = 0,
+                                             float* terms = nullptr) {
   // phase 3: per-point solve, write, epilogue terms (FP32; escalated systems
   // are queued for the float-float kernel; FP64 for the block sums of the CV terms)
   float cv_err = 0.f, cv_in = 0.f, cv_out = 0.f;
-  constexpr int PPT3 = (HT * C + NTH - 1) / NTH;
+  constexpr int PPT3 = LIST ? (LIST + NTH - 1) / NTH : (HT * C + NTH - 1) / NTH;
+  const int sstr = LIST ? LIST + 1 : HT * SC;  // between the slots of a point
   float gval[PPT3];
   int xts[PPT3];
 #pragma unroll
   for (int j = 0; j < PPT3; ++j) {
-    const int e = threadIdx.x + j * NTH;
+    int e = threadIdx.x + j * NTH;
     gval[j] = 0.f;
     xts[j] = -1;
-    if (e >= th * C) continue;
+    if (LIST ? e >= nlist : e >= th * C) continue;
+    const int at = e;
+    if (LIST) e = list[at];
     const int i = e / C, c = e % C;
-    if (half && (a0 + i) * C + c < xs) continue;  // taken from the mirror (t, s)
-    const float* sl = slots + (size_t)i * SC + c;
+    if (!LIST && half && (a0 + i) * C + c < xs) continue;  // taken from the mirror (t, s)
+    const float* sl = LIST ? slots + at : slots + (size_t)i * SC + c;
     float A[5][5], rv[5];
 #pragma unroll
     for (int i2 = 0; i2 < 5; ++i2) {
-      rv[i2] = sl[(size_t)rslot(2, i2) * HT * SC];
+      rv[i2] = sl[rslot(2, i2) * sstr];
 #pragma unroll
       for (int j2 = i2; j2 < 5; ++j2) {
-        A[i2][j2] = sl[(size_t)aslot(2, i2, j2) * HT * SC];
+        A[i2][j2] = sl[aslot(2, i2, j2) * sstr];
         A[j2][i2] = A[i2][j2];
       }
     }
-    const float cnt = sl[(size_t)(NSL - 1) * HT * SC];
+    const float cnt = sl[(NSL - 1) * sstr];
     uint8_t st;
     float gv = fit_point_f32<5, false>(A, rv, cnt + 0.25f, st);
     const int xt = (a0 + i) * C + c;
@@ -417,7 +429,7 @@ __device__ __forceinline__ void tside_phase3(const float* __restrict__ slots, in
       const unsigned slot = ep.esc_count ? atomicAdd(ep.esc_count, 1u) : 0xffffffffu;
       if (slot < (unsigned)ep.esc_cap) {
         float* dst = ep.esc_slots + (size_t)slot * NSL;
-        for (int q = 0; q < NSL; ++q) dst[q] = sl[(size_t)q * HT * SC];
+        for (int q = 0; q < NSL; ++q) dst[q] = sl[q * sstr];
         ep.esc_idx[slot] = make_int2(xs, xt);
         if (ep.esc_idx_item) ep.esc_idx_item[slot] = ep.esc_item_id;
         continue;  // the escalation kernel writes this point and its epilogue terms
@@ -426,10 +438,10 @@ __device__ __forceinline__ void tside_phase3(const float* __restrict__ slots, in
       float A2[5][5], r2[5];
 #pragma unroll
       for (int i2 = 0; i2 < 5; ++i2) {
-        r2[i2] = sl[(size_t)rslot(2, i2) * HT * SC];
+        r2[i2] = sl[rslot(2, i2) * sstr];
 #pragma unroll
         for (int j2 = i2; j2 < 5; ++j2) {
-          A2[i2][j2] = sl[(size_t)aslot(2, i2, j2) * HT * SC];
+          A2[i2][j2] = sl[aslot(2, i2, j2) * sstr];
           A2[j2][i2] = A2[i2][j2];
         }
       }
@@ -453,7 +465,13 @@ __device__ __forceinline__ void tside_phase3(const float* __restrict__ slots, in
       }
     }
   }
-  if (ep.cvacc && cvs) {
+  if (LIST) {
+    if ((int)threadIdx.x < nlist) {
+      terms[threadIdx.x] = cv_err;
+      terms[LIST + threadIdx.x] = cv_in;
+      terms[2 * LIST + threadIdx.x] = cv_out;
+    }
+  } else if (ep.cvacc && cvs) {
     cv_warp_add(cvs, cv_err, cv_in, cv_out);
   } else if (ep.cvacc) {
     const double s0 = block_sum<NTH>((double)cv_err, red);
@@ -688,6 +706,46 @@ __device__ __forceinline__ void ts_phase2(const TsGeom& g, const float2* __restr
   }
 }
 
+// CV terms only: a point without held-out pairs adds nothing, and with scattered data most
+// points of a fold have none (4 % have, at 64 x 64 with 20000 subjects in 5 folds).  A tile
+// with at most TS_LIST such points forms the moments of those alone, point by point from the
+// mid rows (the same partials as ts_phase2, so the same numbers), and solves those alone; a
+// tile without any is left after its held-out bins are read.  Its slots lie apart from the
+// input rows, so that the next tile's rows come in meanwhile.  The terms are added by the
+// threads that would have formed them, in the same order, so the scores are the same.
+// TS_LIST: what shared memory leaves with two CTAs an SM at 9 taps.
+constexpr int TS_LIST = 48;
+constexpr int TS_LIST_F = NSL * (TS_LIST + 1) + 3 * TS_LIST;  // floats: slots, terms
+template <int C, int TC, bool COMP>
+__device__ __forceinline__ void ts_points(const TsGeom& g, const float2* __restrict__ mid2,
+                                          const float2* __restrict__ w2,
+                                          const uint16_t* __restrict__ list, int nlist,
+                                          float* __restrict__ slots) {
+  constexpr int NTAP = 2 * TC + 1;
+  constexpr int NTP = (2 * TC + 2) & ~1;
+  for (int it = threadIdx.x; it < TS_UNITS * nlist; it += TS_NT) {
+    const int un = it / nlist, pt = it - un * nlist, e = list[pt];
+    const int u = c_ts_unit[un][0], pw = c_ts_unit[un][1];
+    const int sx = c_ts_unit[un][2], sy = c_ts_unit[un][3];
+    const float2* x = mid2 + ((size_t)u * HT + e / C) * g.RS2 + (g.off - TC) + e % C;
+    const float2* w = w2 + pw * NTP;
+    float2 o, cmp = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k0 = 0; k0 < NTAP; k0 += TS_PART) {
+      float2 part;
+#pragma unroll
+      for (int k = k0; k < (k0 + TS_PART < NTAP ? k0 + TS_PART : NTAP); ++k)
+        part = k == k0 ? __fmul2_rn(w[k], x[k]) : __ffma2_rn(w[k], x[k], part);
+      if (k0 == 0)
+        o = part;
+      else
+        kahan2<COMP>(o, cmp, part);
+    }
+    slots[sx * (TS_LIST + 1) + pt] = o.x;
+    if (sy >= 0) slots[sy * (TS_LIST + 1) + pt] = o.y;
+  }
+}
+
 // Tile t -> (s-row xs, first t1-row a0); whether it has work in half mode.  Tiles
 // run s-row-major (the tiles of one s-row share input rows, which then stay in
 // L2); the grid size is odd, so that each CTA, taking every gridDim.x-th tile,
@@ -757,6 +815,9 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
   float2* mid2 = w2 + TROWS * NTPC;                           // [TS_PAIRS][HT][RS2]
   float* in = reinterpret_cast<float*>(mid2 + (size_t)TS_PAIRS * HT * g.RS2);  // [10][nrp][C]
   float* slots = in;                                          // [NSL][HT][SC] (after phase 1)
+  const int in_f = 10 * g.nrp * C, slot_f = NSL * HT * g.SC;
+  float* pslots = in + (in_f > slot_f ? in_f : slot_f);       // [NSL][TS_LIST + 1]
+  float* terms = pslots + NSL * (TS_LIST + 1);                // [3][TS_LIST]
   const uint32_t bar = ptx::smem_u32(&tile_bar);
   if (threadIdx.x == 0) {
     ptx::mbar_init(bar, 1);
@@ -779,18 +840,93 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
   if (blockIdx.x >= gridDim.x / 2) __nanosleep(3000);
   uint32_t parity = 0;
   __shared__ CvShared cvs;  // this CTA's CV terms over its tiles
-  if (threadIdx.x == 0) cvs.v[0] = cvs.v[1] = cvs.v[2] = 0.0;
+  cv_clear(&cvs);
+  bool fetched = false;  // the tile's rows are on their way
+  constexpr int PPT = (HT * C + TS_NT - 1) / TS_NT;
+  __shared__ uint8_t held[2][TS_NT / 32][PPT];  // points with held-out pairs, per warp
+  __shared__ uint16_t list[TS_LIST];
+  const bool cv_only = ep.cvacc && !gamma && !status && !ep.y;
   __syncthreads();
   for (int t = ts_next(g, blockIdx.x); t < g.ntiles; parity ^= 1u) {
     int xs, a0;
     ts_tile(g, t, xs, a0);
     const int th = min(HT, g.R - a0);
-    ts_fetch<C>(g, varr, t, in, bar);
+    if (!fetched) ts_fetch<C>(g, varr, t, in, bar);
+    fetched = false;
+    unsigned mine[PPT];
+    if (cv_only) {
+#pragma unroll
+      for (int j = 0; j < PPT; ++j) {
+        const int e = threadIdx.x + j * TS_NT, xt = a0 * C + e;
+        const long long o = (long long)xs * g.P + xt;
+        const bool hit = e < th * C && !(g.half && xt < xs) &&
+                         (ep.wf[o] != 0.f || ep.vf[o] != 0.f || ep.qf[o] != 0.f);
+        mine[j] = __ballot_sync(0xffffffffu, hit);
+        if ((threadIdx.x & 31) == 0) held[parity][threadIdx.x >> 5][j] = __popc(mine[j]);
+      }
+    }
     const bool landed = ptx::mbar_wait(bar, parity, err);
     if (__syncthreads_or(!landed)) return;
+    const int tn = ts_next(g, t + gridDim.x);
+    int nlist = TS_LIST + 1;
+    int first[PPT] = {};  // of this warp's points in the list
+    if (cv_only) {
+      nlist = 0;
+#pragma unroll
+      for (int w = 0; w < TS_NT / 32; ++w)
+#pragma unroll
+        for (int j = 0; j < PPT; ++j) {
+          if (w == (threadIdx.x >> 5)) first[j] = nlist;
+          nlist += held[parity][w][j];
+        }
+      if (nlist == 0) {  // (the next tile counts into the other half of `held`)
+        t = tn;
+        continue;
+      }
+      if (nlist <= TS_LIST) {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int j = 0; j < PPT; ++j)
+          if (mine[j] >> lane & 1)
+            list[first[j] + __popc(mine[j] & ((1u << lane) - 1u))] = threadIdx.x + j * TS_NT;
+      }
+    }
     ts_phase1<C, TR, COMP>(g, in, w1, mid2);
     __syncthreads();
-    const int tn = ts_next(g, t + gridDim.x);
+    if (nlist <= TS_LIST) {
+      if (tn < g.ntiles) {
+        ts_fetch<C>(g, varr, tn, in, bar);
+        fetched = true;
+        if (threadIdx.x < 3 * HT * C / 32) {  // and its held-out bins into L2, a line a thread
+          int xn, an;
+          ts_tile(g, tn, xn, an);
+          const int which = threadIdx.x / (HT * C / 32), e = threadIdx.x % (HT * C / 32) * 32;
+          const float* src = which == 0 ? ep.wf : which == 1 ? ep.vf : ep.qf;
+          if (an * C + e < g.P)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (long long)xn * g.P + an * C + e));
+        }
+      }
+      ts_points<C, TC, COMP>(g, mid2, w2, list, nlist, pslots);
+      __syncthreads();
+      tside_phase3<C, TS_NT, TS_LIST>(pslots, g.SC, g.half, g.P, xs, a0, th, mu_raw, nullptr,
+                                      nullptr, ep, red, nullptr, nullptr, list, nlist, terms);
+      __syncthreads();
+      unsigned any = 0;
+      float ce = 0.f, ci = 0.f, co = 0.f;
+#pragma unroll
+      for (int j = 0; j < PPT; ++j) {
+        any |= mine[j];
+        if (mine[j] >> (threadIdx.x & 31) & 1) {
+          const int at = first[j] + __popc(mine[j] & ((1u << (threadIdx.x & 31)) - 1u));
+          ce += terms[at];
+          ci += terms[TS_LIST + at];
+          co += terms[2 * TS_LIST + at];
+        }
+      }
+      if (any) cv_warp_add(&cvs, ce, ci, co);
+      t = tn;
+      continue;
+    }
     ts_phase2<C, TC, COMP>(g, mid2, w2, slots);
     __syncthreads();
     tside_phase3<C, TS_NT>(slots, g.SC, g.half, g.P, xs, a0, th, mu_raw, gamma, status, ep, red,
@@ -831,7 +967,7 @@ inline size_t ts_smem(const TsGeom& g) {
   const size_t slot_f = (size_t)NSL * HT * g.SC;
   return sizeof(float2) * ((size_t)TROWS * ts_ntp(g.Tr) + (size_t)TROWS * ts_ntp(g.Tc) +
                            (size_t)TS_PAIRS * HT * g.RS2) +
-         sizeof(float) * (in_f > slot_f ? in_f : slot_f);
+         sizeof(float) * ((in_f > slot_f ? in_f : slot_f) + TS_LIST_F);
 }
 
 // Launches k_tsweep for the half-width T: two CTAs per SM walk the tiles.
