@@ -631,10 +631,12 @@ __device__ __forceinline__ bool hsolve2_tile(const float* __restrict__ varr, con
   const int rlo = max(0, a0 - g.Tr), rhi = min(R, a0 - g.Tr + g.nrp);
   const int skip = rlo - (a0 - g.Tr);  // padding rows above the grid
   const uint32_t bytes = (uint32_t)((rhi - rlo) * C * sizeof(float));
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    ptx::mbar_arrive_expect_tx(bar, 10 * bytes);
-    for (int a = 0; a < 10; ++a)
+    if (threadIdx.x == 0) ptx::mbar_arrive_expect_tx(bar, 10 * bytes);
+    __syncwarp();
+    const int a = threadIdx.x;  // ten lanes, a copy each
+    if (a < 10)
       ptx::bulk_load(ptx::smem_u32(in + ((size_t)a * g.nrp + skip) * C),
                      varr + a * PP + (long long)xs * P + (long long)rlo * C, bytes, bar);
   }
@@ -819,8 +821,8 @@ __global__ void __launch_bounds__(NT2, 2)
 // s-side pass (FP32): one block = one line (Ma rows along the pass axis) x 128 columns of one
 // input array; rows padded with zeros above and below.  A thread takes two columns and every
 // second group of VROWS outputs, in packed arithmetic: the pass is bound by its instruction
-// count, and two columns of a tile row are a register pair as they lie (64 x 64, 19 taps: VP_OLD
-// with one column a thread, VP_NEW).
+// count, and two columns of a tile row are a register pair as they lie (64 x 64, 19 taps, both
+// passes: 0.338 ms with one column a thread, 0.272 with two).
 constexpr int VROWS = 8;  // outputs per sliding window
 
 // s + p with Kahan compensation, c the negated error: four packed operations.
@@ -1275,6 +1277,20 @@ __global__ void k_pool_counts(int F, long long PP, const int32_t* __restrict__ i
 
 // cv[h] = err / w_in over folds; +inf when EMPTY points hold > 1% of the
 // held-out weight or nothing was scored.
+// One fold's training bins: the pooled ones less the fold's, as k_vpass2 forms them.
+template <typename T>
+__global__ void k_train_bins(long long PP, const int32_t* __restrict__ cnt, const T* __restrict__ w,
+                             const T* __restrict__ v, const int32_t* __restrict__ cf,
+                             const T* __restrict__ wf, const T* __restrict__ vf,
+                             int32_t* __restrict__ ct, T* __restrict__ wt, T* __restrict__ vt) {
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < PP;
+       e += (long long)gridDim.x * blockDim.x) {
+    ct[e] = cnt[e] - cf[e];
+    wt[e] = w[e] - wf[e];
+    vt[e] = v[e] - vf[e];
+  }
+}
+
 __global__ void k_cv_finish(int nh, int F, const double* __restrict__ acc, double* __restrict__ cv) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= nh) return;
@@ -1609,6 +1625,11 @@ fpca_status smooth_cov_typed(fpca_ctx* ctx, const fpca_grid* g, const fpca_covbi
   const long long PP = (long long)P * P;
   const int F = bins->nfold > 0 ? bins->nfold : 1;
   const int nmid = d == 2 ? 6 : 0;
+  // With TRAIN_MIN bandwidths or more a fold's training bins are formed once for all of them;
+  // with fewer the s-side passes subtract as they read (the extra pass costs what two save).
+  constexpr int TRAIN_MIN = 3;
+  bool train = cv && F > 1 && nh >= TRAIN_MIN;
+  size_t need_t = train ? WsCarve::round(sizeof(T) * PP) * 2 + WsCarve::round(4 * PP) : 0;
   // queue of escalated FP32 fits (d = 2 FP32 kernel): up to 2^21 points
   const int esc_cap = (sizeof(T) == 4 && d == 2) ? (int)std::min<long long>(PP, 1ll << 21) : 0;
   const size_t need = WsCarve::round(sizeof(double) * 3 * TROWS * TW * (size_t)nh) +
@@ -1632,19 +1653,28 @@ fpca_status smooth_cov_typed(fpca_ctx* ctx, const fpca_grid* g, const fpca_covbi
                WsCarve::round(sizeof(CvGridItem) * (size_t)nitems) +
                WsCarve::round(sizeof(int) * (size_t)esc_cap) + 1024;
       size_t fr = 0, tot = 0;
-      if (batched && need + need_b > ctx->ws_bytes) {
+      if (batched && need + need_t + need_b > ctx->ws_bytes) {
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
           cudaGetLastError();
           fr = 0;
         }
         // leave room: grow only into at most 80% of what is free
-        batched = need + need_b <= ctx->ws_bytes + (size_t)(0.8 * (double)fr);
+        batched = need + need_t + need_b <= ctx->ws_bytes + (size_t)(0.8 * (double)fr);
       }
     }
   }
-  void* ws = fpca_workspace(ctx, need + (batched ? need_b : 0));
+  // what a graph capture or the device has no room for is done without
+  if (train && ctx->capturing && need + need_t + (batched ? need_b : 0) > ctx->ws_bytes) {
+    train = false;
+    need_t = 0;
+  }
+  void* ws = fpca_workspace(ctx, need + need_t + (batched ? need_b : 0));
   if (!ws && batched) {
     batched = false;
+    ws = fpca_workspace(ctx, need + need_t);
+  }
+  if (!ws && train) {
+    train = false;
     ws = fpca_workspace(ctx, need);
   }
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace (%zu bytes)", need);
@@ -1693,6 +1723,13 @@ fpca_status smooth_cov_typed(fpca_ctx* ctx, const fpca_grid* g, const fpca_covbi
     v = vp;
     cnt = cp;
   }
+  T *wt = nullptr, *vt = nullptr;
+  int32_t* ct = nullptr;
+  if (train) {
+    wt = carve.take<T>(PP);
+    vt = carve.take<T>(PP);
+    ct = carve.take<int32_t>(PP);
+  }
   if (y) cudaMemsetAsync(y, 0, sizeof(float) * (size_t)nh * P * l, ctx->stream);
   for (int ih = 0; ih < nh; ++ih) {
     const double* hh = h + (size_t)ih * d;
@@ -1728,18 +1765,29 @@ fpca_status smooth_cov_typed(fpca_ctx* ctx, const fpca_grid* g, const fpca_covbi
     const T* fw = static_cast<const T*>(bins->w);
     const T* fv = static_cast<const T*>(bins->v);
     const T* fq = static_cast<const T*>(bins->q);
-    for (int ih = 0; ih < nh; ++ih) {
-      for (int f = 0; f < F; ++f) {
-        Epilogue<T> ep{};
-        with_queue(ep);
-        ep.wf = fw + (size_t)f * PP;
-        ep.vf = fv + (size_t)f * PP;
-        ep.qf = fq + (size_t)f * PP;
-        ep.cvacc = cvacc + 3 * ((size_t)ih * F + f);
-        fpca_status s = cov_smooth_one<T, COMP>(
-            ctx, g, cnt, w, v, bins->cnt + (size_t)f * PP, fw + (size_t)f * PP,
-            fv + (size_t)f * PP, h + (size_t)ih * d, tab_all + (size_t)ih * 3 * TROWS * TW, mids,
-            varr, mu_raw, nullptr, nullptr, ep, bins->asym == 0);
+    auto item = [&](int ih, int f) -> fpca_status {
+      Epilogue<T> ep{};
+      with_queue(ep);
+      ep.wf = fw + (size_t)f * PP;
+      ep.vf = fv + (size_t)f * PP;
+      ep.qf = fq + (size_t)f * PP;
+      ep.cvacc = cvacc + 3 * ((size_t)ih * F + f);
+      return cov_smooth_one<T, COMP>(
+          ctx, g, train ? ct : cnt, train ? wt : w, train ? vt : v,
+          train ? nullptr : bins->cnt + (size_t)f * PP, train ? nullptr : fw + (size_t)f * PP,
+          train ? nullptr : fv + (size_t)f * PP, h + (size_t)ih * d,
+          tab_all + (size_t)ih * 3 * TROWS * TW, mids, varr, mu_raw, nullptr, nullptr, ep,
+          bins->asym == 0);
+    };
+    for (int f = 0; f < F; ++f) {
+      if (train) {
+        k_train_bins<T><<<ctx->num_sms * 8, 256, 0, ctx->stream>>>(
+            PP, cnt, w, v, bins->cnt + (size_t)f * PP, fw + (size_t)f * PP, fv + (size_t)f * PP, ct,
+            wt, vt);
+        FPCA_LAUNCHED(ctx, "train_bins");
+      }
+      for (int ih = 0; ih < nh; ++ih) {
+        fpca_status s = item(ih, f);
         if (s != FPCA_OK) return s;
       }
     }

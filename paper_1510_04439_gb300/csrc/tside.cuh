@@ -765,8 +765,41 @@ __device__ __forceinline__ int ts_next(const TsGeom& g, int t) {
   return g.ntiles;
 }
 
-// Issue the bulk copies of tile t's in-grid input rows (thread 0) and zero its
-// padding rows (all threads; disjoint from the copied rows).
+// The held-out bins of this thread's points of tile t (point threadIdx.x + j TS_NT), zero for
+// those that the tile does not evaluate; every load is on its way before the first is used.
+template <int C>
+struct TsHeld {
+  static constexpr int PPT = (HT * C + TS_NT - 1) / TS_NT;
+  float x[PPT][3];
+  __device__ __forceinline__ void load(const TsGeom& g, const Epilogue<float>& ep, int t);
+  __device__ __forceinline__ unsigned bits() const {  // bit j: point j has held-out pairs
+    unsigned b = 0;
+#pragma unroll
+    for (int j = 0; j < PPT; ++j)
+      b |= (unsigned)(x[j][0] != 0.f || x[j][1] != 0.f || x[j][2] != 0.f) << j;
+    return b;
+  }
+};
+
+template <int C>
+__device__ __forceinline__ void TsHeld<C>::load(const TsGeom& g, const Epilogue<float>& ep, int t) {
+  int xs, a0;
+  ts_tile(g, t, xs, a0);
+  const int th = min(HT, g.R - a0);
+#pragma unroll
+  for (int j = 0; j < PPT; ++j) {
+    const int e = threadIdx.x + j * TS_NT, xt = a0 * C + e;
+    const long long o = (long long)xs * g.P + xt;
+    const bool in = e < th * C && !(g.half && xt < xs);
+    x[j][0] = in ? ep.wf[o] : 0.f;
+    x[j][1] = in ? ep.vf[o] : 0.f;
+    x[j][2] = in ? ep.qf[o] : 0.f;
+  }
+}
+
+// Issue the bulk copies of tile t's in-grid input rows (ten lanes of warp 0: one thread
+// takes 170 cycles a copy) and zero its padding rows (all threads; disjoint from the
+// copied rows).
 template <int C>
 __device__ __forceinline__ void ts_fetch(const TsGeom& g, const float* __restrict__ varr, int t,
                                          float* __restrict__ in, uint32_t bar) {
@@ -777,13 +810,14 @@ __device__ __forceinline__ void ts_fetch(const TsGeom& g, const float* __restric
   const int skip = rlo - (a0 - g.Tr);
   const int nrow = max(0, rhi - rlo);
   const uint32_t bytes = (uint32_t)(nrow * C * sizeof(float));
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    ptx::mbar_arrive_expect_tx(bar, 10 * bytes);
-    if (bytes > 0)
-      for (int a = 0; a < 10; ++a)
-        ptx::bulk_load(ptx::smem_u32(in + ((size_t)a * g.nrp + skip) * C),
-                       varr + a * PP + (long long)xs * g.P + (long long)rlo * C, bytes, bar);
+    if (threadIdx.x == 0) ptx::mbar_arrive_expect_tx(bar, 10 * bytes);
+    __syncwarp();
+    const int a = threadIdx.x;
+    if (bytes > 0 && a < 10)
+      ptx::bulk_load(ptx::smem_u32(in + ((size_t)a * g.nrp + skip) * C),
+                     varr + a * PP + (long long)xs * g.P + (long long)rlo * C, bytes, bar);
   }
   constexpr int C4 = C / 4;
   const int padrows = g.nrp - nrow;
@@ -799,7 +833,9 @@ __device__ __forceinline__ void ts_fetch(const TsGeom& g, const float* __restric
 
 // Two CTAs fit an SM up to 9 taps each side (shared memory); wider windows run one
 // CTA per SM and may use every register.
-template <bool COMP, int C, int TR, int TC>
+// CV: the sums of ep.cvacc and no other output; not CV: no such sums (a kernel for both
+// spilled at 9 taps, 0.51 against 0.49 ms).
+template <bool COMP, int C, int TR, int TC, bool CV>
 __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
     k_tsweep(const float* __restrict__ varr, TsGeom g, const double* __restrict__ tabr,
              const double* __restrict__ tabc, const double* __restrict__ mu_raw,
@@ -843,9 +879,11 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
   cv_clear(&cvs);
   bool fetched = false;  // the tile's rows are on their way
   constexpr int PPT = (HT * C + TS_NT - 1) / TS_NT;
-  __shared__ uint8_t held[2][TS_NT / 32][PPT];  // points with held-out pairs, per warp
+  static_assert(TS_NT / 32 * PPT % 4 == 0, "counts in whole words");
+  __shared__ __align__(4) uint8_t held[2][TS_NT / 32 * PPT];  // points with held-out pairs
+  int heldt = -1;      // the tile that `bits` is of
+  unsigned bits = 0;
   __shared__ uint16_t list[TS_LIST];
-  const bool cv_only = ep.cvacc && !gamma && !status && !ep.y;
   __syncthreads();
   for (int t = ts_next(g, blockIdx.x); t < g.ntiles; parity ^= 1u) {
     int xs, a0;
@@ -854,15 +892,16 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
     if (!fetched) ts_fetch<C>(g, varr, t, in, bar);
     fetched = false;
     unsigned mine[PPT];
-    if (cv_only) {
+    if constexpr (CV) {
+      if (heldt != t) {
+        TsHeld<C> hv;
+        hv.load(g, ep, t);
+        bits = hv.bits();
+      }
 #pragma unroll
       for (int j = 0; j < PPT; ++j) {
-        const int e = threadIdx.x + j * TS_NT, xt = a0 * C + e;
-        const long long o = (long long)xs * g.P + xt;
-        const bool hit = e < th * C && !(g.half && xt < xs) &&
-                         (ep.wf[o] != 0.f || ep.vf[o] != 0.f || ep.qf[o] != 0.f);
-        mine[j] = __ballot_sync(0xffffffffu, hit);
-        if ((threadIdx.x & 31) == 0) held[parity][threadIdx.x >> 5][j] = __popc(mine[j]);
+        mine[j] = __ballot_sync(0xffffffffu, bits >> j & 1);
+        if ((threadIdx.x & 31) == 0) held[parity][(threadIdx.x >> 5) * PPT + j] = __popc(mine[j]);
       }
     }
     const bool landed = ptx::mbar_wait(bar, parity, err);
@@ -870,15 +909,21 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
     const int tn = ts_next(g, t + gridDim.x);
     int nlist = TS_LIST + 1;
     int first[PPT] = {};  // of this warp's points in the list
-    if (cv_only) {
+    if constexpr (CV) {
+      // counts are bytes (at most 32 each), summed four at a time
+      const uint32_t* hw = reinterpret_cast<const uint32_t*>(held[parity]);
       nlist = 0;
 #pragma unroll
-      for (int w = 0; w < TS_NT / 32; ++w)
+      for (int k = 0; k < TS_NT / 32 * PPT / 4; ++k) {
+        const uint32_t word = hw[k];
 #pragma unroll
         for (int j = 0; j < PPT; ++j) {
-          if (w == (threadIdx.x >> 5)) first[j] = nlist;
-          nlist += held[parity][w][j];
+          const int before = (int)(threadIdx.x >> 5) * PPT + j - 4 * k;  // its bytes in front
+          const uint32_t m = before >= 4 ? 0xffffffffu : before > 0 ? (1u << 8 * before) - 1u : 0u;
+          first[j] = __dp4a(word & m, 0x01010101u, (unsigned)first[j]);
         }
+        nlist = __dp4a(word, 0x01010101u, (unsigned)nlist);
+      }
       if (nlist == 0) {  // (the next tile counts into the other half of `held`)
         t = tn;
         continue;
@@ -893,20 +938,18 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
     }
     ts_phase1<C, TR, COMP>(g, in, w1, mid2);
     __syncthreads();
-    if (nlist <= TS_LIST) {
+    if (CV && nlist <= TS_LIST) {
+      TsHeld<C> hv;
       if (tn < g.ntiles) {
         ts_fetch<C>(g, varr, tn, in, bar);
         fetched = true;
-        if (threadIdx.x < 3 * HT * C / 32) {  // and its held-out bins into L2, a line a thread
-          int xn, an;
-          ts_tile(g, tn, xn, an);
-          const int which = threadIdx.x / (HT * C / 32), e = threadIdx.x % (HT * C / 32) * 32;
-          const float* src = which == 0 ? ep.wf : which == 1 ? ep.vf : ep.qf;
-          if (an * C + e < g.P)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(src + (long long)xn * g.P + an * C + e));
-        }
+        hv.load(g, ep, tn);
       }
       ts_points<C, TC, COMP>(g, mid2, w2, list, nlist, pslots);
+      if (tn < g.ntiles) {
+        heldt = tn;
+        bits = hv.bits();
+      }
       __syncthreads();
       tside_phase3<C, TS_NT, TS_LIST>(pslots, g.SC, g.half, g.P, xs, a0, th, mu_raw, nullptr,
                                       nullptr, ep, red, nullptr, nullptr, list, nlist, terms);
@@ -929,10 +972,19 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
     }
     ts_phase2<C, TC, COMP>(g, mid2, w2, slots);
     __syncthreads();
-    tside_phase3<C, TS_NT>(slots, g.SC, g.half, g.P, xs, a0, th, mu_raw, gamma, status, ep, red,
-                           reinterpret_cast<float*>(mid2), &cvs);
+    if constexpr (CV) {
+      Epilogue<float> e = ep;
+      e.y = nullptr;
+      tside_phase3<C, TS_NT>(slots, g.SC, g.half, g.P, xs, a0, th, mu_raw, nullptr, nullptr, e, red,
+                             reinterpret_cast<float*>(mid2), &cvs);
+    } else {
+      Epilogue<float> e = ep;
+      e.cvacc = nullptr;
+      tside_phase3<C, TS_NT>(slots, g.SC, g.half, g.P, xs, a0, th, mu_raw, gamma, status, e, red,
+                             reinterpret_cast<float*>(mid2));
+    }
     // the y epilogue used the mid rows as scratch: restore their zero halo
-    if (ep.y) {
+    if (!CV && ep.y) {
       __syncthreads();
       const int padw = g.RS2 - C;
       for (int e = threadIdx.x; e < TS_PAIRS * HT * padw; e += TS_NT) {
@@ -944,7 +996,7 @@ __global__ void __launch_bounds__(TS_NT, (TR <= 9 && TC <= 9) ? 2 : 1)
     __syncthreads();  // phase 3 read the slots, which alias the next tile's input rows
     t = tn;
   }
-  if (ep.cvacc) cv_flush(&cvs, ep.cvacc);
+  if constexpr (CV) cv_flush(&cvs, ep.cvacc);
 }
 
 inline TsGeom ts_geometry(int P, int M1, int M2, int Tr, int Tc) {
@@ -975,15 +1027,20 @@ template <bool COMP, int C, int T>
 void tsweep_launch_t(fpca_ctx* ctx, size_t smem, const float* varr, const TsGeom& g,
                      const double* tabr, const double* tabc, const double* mu_raw, float* gamma,
                      uint8_t* status, const Epilogue<float>& ep) {
-  static int attr = 0;  // dynamic shared memory the kernel is configured for
-  if ((int)smem > attr) {
-    cudaFuncSetAttribute(k_tsweep<COMP, C, T, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    attr = (int)smem;
-  }
+  static int attr[2] = {0, 0};  // dynamic shared memory the kernels are configured for
   const int nb = g.ntiles < 2 * ctx->num_sms - 1 ? g.ntiles : 2 * ctx->num_sms - 1;
-  k_tsweep<COMP, C, T, T><<<nb > 0 ? nb : 1, TS_NT, smem, ctx->stream>>>(
-      varr, g, tabr, tabc, mu_raw, gamma, status, ep, ctx->d_err);
+  auto launch = [&](auto kern, int& have) {
+    if ((int)smem > have) {
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      have = (int)smem;
+    }
+    kern<<<nb > 0 ? nb : 1, TS_NT, smem, ctx->stream>>>(varr, g, tabr, tabc, mu_raw, gamma, status,
+                                                        ep, ctx->d_err);
+  };
+  if (ep.cvacc && !gamma && !status && !ep.y)
+    launch(k_tsweep<COMP, C, T, T, true>, attr[1]);
+  else
+    launch(k_tsweep<COMP, C, T, T, false>, attr[0]);
 }
 
 #define FPCA_TSWEEP_PARAMS                                                                     \
