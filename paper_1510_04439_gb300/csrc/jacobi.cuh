@@ -28,21 +28,27 @@ __device__ __forceinline__ void rr_pair(int ne, int step, int i, int& p, int& q)
 
 // The rotation (c, s) that annihilates a_pq: tau = (a_qq - a_pp) / (2 a_pq),
 // t = sign(tau) / (|tau| + sqrt(1 + tau^2)), c = 1 / sqrt(1 + t^2), s = t c.
-// The quotients and 1 / sqrt(1 + t^2) (argument in [1, 2]) use the fast
-// approximate forms: c^2 + s^2 = 1 then holds to a few FP32 ulps, and the
-// refinement that follows the FP32 Jacobi restores orthogonality anyway.  The
-// square root of 1 + tau^2 stays exact so that tau^2 = inf still gives t = 0.
+// Approximate reciprocals and square roots (each gives 0 for an infinite tau^2): a serial
+// chain of rotations waits on them, c^2 + s^2 = 1 holds to a few FP32 ulps all the same, and
+// the refinement that follows every FP32 Jacobi restores orthogonality.
+__device__ __forceinline__ void bj_rot(float app, float apq, float aqq, float& c, float& sn) {
+  const float tau = __fdividef(aqq - app, 2.f * apq);
+  float root;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(tau, tau, 1.f)));
+  const float t = __fdividef(copysignf(1.f, tau), fabsf(tau) + root);
+  const bool on = fabsf(apq) > 1e-30f && fabsf(apq) > 1e-18f * fmaxf(fabsf(app), fabsf(aqq));
+  c = on ? rsqrtf(fmaf(t, t, 1.f)) : 1.f;
+  sn = on ? t * c : 0.f;
+}
+
+// The same from the matrix A (n x n, leading dimension ld); q >= n: none.
 __device__ __forceinline__ void rr_rot(const float* A, int ld, int n, int p, int q, float& c,
                                        float& sn) {
-  c = 1.f;
-  sn = 0.f;
-  if (q >= n) return;
-  const float apq = A[p * ld + q], app = A[p * ld + p], aqq = A[q * ld + q];
-  if (fabsf(apq) > 1e-30f && fabsf(apq) > 1e-18f * sqrtf(fabsf(app) * fabsf(aqq))) {
-    const float tau = __fdividef(aqq - app, 2.f * apq);
-    const float t = __fdividef(tau >= 0.f ? 1.f : -1.f, fabsf(tau) + sqrtf(1.f + tau * tau));
-    c = rsqrtf(1.f + t * t);
-    sn = t * c;
+  if (q < n) {
+    bj_rot(A[p * ld + p], A[p * ld + q], A[q * ld + q], c, sn);
+  } else {
+    c = 1.f;
+    sn = 0.f;
   }
 }
 
@@ -70,18 +76,6 @@ __device__ __forceinline__ void bj_step_pair(bool within, int s, int i, int& p, 
     p = i;
     q = BJ_S + ((i + s) & (BJ_S - 1));
   }
-}
-
-// The rotation of rr_rot by the approximate reciprocal and square root only (both give 0 for
-// an infinite tau^2); c^2 + s^2 = 1 to a few FP32 ulps all the same.
-__device__ __forceinline__ void bj_rot(float app, float apq, float aqq, float& c, float& sn) {
-  const float tau = __fdividef(aqq - app, 2.f * apq);
-  float root;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(tau, tau, 1.f)));
-  const float t = __fdividef(copysignf(1.f, tau), fabsf(tau) + root);
-  const bool on = fabsf(apq) > 1e-30f && fabsf(apq) > 1e-18f * fmaxf(fabsf(app), fabsf(aqq));
-  c = on ? rsqrtf(fmaf(t, t, 1.f)) : 1.f;
-  sn = on ? t * c : 0.f;
 }
 
 // One sweep of rotations over the 32 x 32 subproblem in `cur` (leading dimension BJ_LD,

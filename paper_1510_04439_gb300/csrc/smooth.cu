@@ -825,19 +825,6 @@ __global__ void __launch_bounds__(NT2, 2)
 // passes: 0.338 ms with one column a thread, 0.272 with two).
 constexpr int VROWS = 8;  // outputs per sliding window
 
-// s + p with Kahan compensation, c the negated error: four packed operations.
-template <bool COMP>
-__device__ __forceinline__ void chunk_add2(float2& s, float2& c, float2 p) {
-  if constexpr (COMP) {
-    const float2 y = __fadd2_rn(p, c);
-    const float2 t = __fadd2_rn(s, y);
-    c = __fadd2_rn(y, __ffma2_rn(t, make_float2(-1.f, -1.f), s));  // y - (t - s)
-    s = t;
-  } else {
-    s = __fadd2_rn(s, p);
-  }
-}
-
 // out[j] = sum_{k < 4 NCH} w[k] * x[(j + k) * VCOLS] for each of the job's powers, from one
 // window in registers; wp: {w, w} per tap, two taps per float4, ntp taps a row.  Partials of
 // up to 12 taps, Kahan-added (without COMP one running sum).
@@ -871,7 +858,7 @@ __device__ __forceinline__ void vline_fixed(const VJob& jb, const float2* __rest
           sum[j] = p[j];
           cmp[j] = make_float2(0.f, 0.f);
         } else {
-          chunk_add2<COMP>(sum[j], cmp[j], p[j]);
+          kahan2<COMP>(sum[j], cmp[j], p[j]);
         }
       }
     }
@@ -905,7 +892,7 @@ __device__ __forceinline__ void vline_any(const VJob& jb, const float2* __restri
           float2 p = __fmul2_rn(w0, win[j]);
           p = __ffma2_rn(w1, win[j + 1], p);
           p = __ffma2_rn(w2, win[j + 2], p);
-          chunk_add2<true>(sum[j], cmp[j], __ffma2_rn(w3, win[j + 3], p));
+          kahan2<true>(sum[j], cmp[j], __ffma2_rn(w3, win[j + 3], p));
         } else {
           sum[j] = __ffma2_rn(w0, win[j], sum[j]);
           sum[j] = __ffma2_rn(w1, win[j + 1], sum[j]);

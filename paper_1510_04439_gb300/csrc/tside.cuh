@@ -568,14 +568,13 @@ struct TsGeom {
   int ntiles;      // t1 blocks x P s-rows
 };
 
-__device__ __forceinline__ float2 f2neg(float2 a) { return make_float2(-a.x, -a.y); }
-
+// s + p with Kahan compensation, c the negated error: four packed operations.
 template <bool COMP>
 __device__ __forceinline__ void kahan2(float2& s, float2& c, float2 p) {
   if constexpr (COMP) {
-    const float2 y = __fadd2_rn(p, f2neg(c));
+    const float2 y = __fadd2_rn(p, c);
     const float2 t = __fadd2_rn(s, y);
-    c = __fadd2_rn(__fadd2_rn(t, f2neg(s)), f2neg(y));
+    c = __fadd2_rn(y, __ffma2_rn(t, make_float2(-1.f, -1.f), s));  // y - (t - s)
     s = t;
   } else {
     s = __fadd2_rn(s, p);
