@@ -371,15 +371,20 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-// Corrections of vector j (block): E[j][i].  Pairs closer than
-// 2 (|off-diagonal S_j| + |A| |R_j|) are a cluster: only made orthogonal (by both vectors
-// where both are refined, else by x_j alone).  state[1 + it] takes the largest correction of
-// the k wanted vectors, 1 while a cluster still couples by more than 1e-13 |A|.
+// Corrections e_i of vector j (blockIdx.x; each of its blocks forms them all, which takes less
+// than a launch of their own), then Xk_j += X e on the rows of blockIdx.y, a warp a row.
+// Pairs closer than 2 (|off-diagonal S_j| + |A| |R_j|) are a cluster: only made orthogonal (by
+// both vectors where both are refined, else by x_j alone).  state[1 + it] takes the largest
+// correction of the k wanted vectors, 1 while a cluster still couples by more than 1e-13 |A|.
+constexpr int LX_BLOCKS = 8;  // row blocks of a vector
 __global__ void __launch_bounds__(LE_MAXN)
-    k_lead_e(int n, int k, const int* __restrict__ nref, int it, const float* __restrict__ lam32, const int* __restrict__ pos,
-             const int* __restrict__ lead, double* __restrict__ S, const double* __restrict__ R,
-             double* __restrict__ E, double* __restrict__ lamk, float* __restrict__ state) {
+    k_lead_ex(int n, int k, const int* __restrict__ nref, int it, const float* __restrict__ lam32,
+              const int* __restrict__ pos, const int* __restrict__ lead,
+              const double* __restrict__ S, const double* __restrict__ R,
+              const double* __restrict__ X, double* __restrict__ Xk, double* __restrict__ lamk,
+              float* __restrict__ state) {
   __shared__ float red[LE_MAXN / 32][2];
+  __shared__ double es[LE_MAXN];
   if (lead_done(state, it) || (int)blockIdx.x >= *nref) return;
   const int i = threadIdx.x, j = blockIdx.x, self = lead[j];
   const bool in = i < n;
@@ -412,29 +417,25 @@ __global__ void __launch_bounds__(LE_MAXN)
     const double couple = s + lj * r;
     const bool close = fabs(gap) <= (double)delta;
     const double e = i == self ? 0.5 * r : close ? (pos[i] >= 0 ? 0.5 * r : r) : couple / gap;
-    E[(size_t)j * n + i] = e;
+    es[i] = e;
     mag = fabsf((float)e);
     if (close && i != self && fabs(couple) > 1e-13 * (double)state[0]) mag = 1.f;
   }
-  for (int o = 16; o > 0; o >>= 1) mag = fmaxf(mag, __shfl_xor_sync(0xffffffffu, mag, o));
-  // (a NaN compares as larger than any number here: not converged)
-  if ((i & 31) == 0 && j < k)
-    atomicMax(reinterpret_cast<int*>(state + 1 + it), __float_as_int(mag) & 0x7fffffff);
-  if (i == 0) lamk[j] = lj;
-}
-
-// Xk_j += X E_j by one warp per (row m, vector j).
-__global__ void __launch_bounds__(256)
-    k_lead_x(int n, const int* __restrict__ nref, int it, const double* __restrict__ X, const double* __restrict__ E,
-             const float* __restrict__ state, double* __restrict__ Xk) {
-  if (lead_done(state, it)) return;
-  const int w = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (w >= n * *nref) return;
-  const int j = w / n, m = w - j * n;
-  double s = 0.0;
-  for (int i = lane; i < n; i += 32) s = fma(X[(size_t)m * n + i], E[(size_t)j * n + i], s);
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) Xk[(size_t)j * n + m] += s;
+  if (blockIdx.y == 0) {
+    for (int o = 16; o > 0; o >>= 1) mag = fmaxf(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+    // (a NaN compares as larger than any number here: not converged)
+    if ((i & 31) == 0 && j < k)
+      atomicMax(reinterpret_cast<int*>(state + 1 + it), __float_as_int(mag) & 0x7fffffff);
+    if (i == 0) lamk[j] = lj;
+  }
+  __syncthreads();
+  const int lane = i & 31;
+  for (int m = blockIdx.y * (LE_MAXN / 32) + (i >> 5); m < n; m += LX_BLOCKS * (LE_MAXN / 32)) {
+    double a = 0.0;
+    for (int c = lane; c < n; c += 32) a = fma(X[(size_t)m * n + c], es[c], a);
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane == 0) Xk[(size_t)j * n + m] += a;
+  }
 }
 
 // The FP64 fall-back's first half, when the last iteration over the leading vectors left a
@@ -649,7 +650,7 @@ size_t lead_eig_bytes(int n, int k) {
   return WsCarve::round(sizeof(float) * ne * ne) + WsCarve::round(sizeof(double) * (size_t)n * n) +
          WsCarve::round(sizeof(float) * n) + 2 * WsCarve::round(sizeof(int) * n) + WsCarve::round(sizeof(int)) +
          WsCarve::round(sizeof(float) * (LE_ITERS + 1)) +
-         5 * WsCarve::round(sizeof(double) * kk * n) + WsCarve::round(sizeof(double) * kk) +
+         4 * WsCarve::round(sizeof(double) * kk * n) + WsCarve::round(sizeof(double) * kk) +
          4 * WsCarve::round(sizeof(double) * (size_t)n * n) + WsCarve::round(sizeof(double) * n) +
          WsCarve::round(sizeof(double)) + WsCarve::round(sizeof(int) * rotate_ints(n)) + 4096;
 }
@@ -669,7 +670,6 @@ fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double
   double* U = c.take<double>((size_t)kk * n);
   double* Sx = c.take<double>((size_t)kk * n);
   double* R = c.take<double>((size_t)kk * n);
-  double* E = c.take<double>((size_t)kk * n);
   double* lamk = c.take<double>(kk);
   double* X0 = c.take<double>((size_t)n * n);
   double* Uf = c.take<double>((size_t)n * n);
@@ -702,9 +702,8 @@ fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double
     FPCA_LAUNCHED(ctx, "eig_lead_u");
     k_lead_sr<<<dim3((n + 31) / 32, kk), 1024, 0, ctx->stream>>>(n, nref, it, X, Xk, U, pos, state, Sx, R);
     FPCA_LAUNCHED(ctx, "eig_lead_sr");
-    k_lead_e<<<kk, LE_MAXN, 0, ctx->stream>>>(n, k, nref, it, lam32, pos, lead, Sx, R, E, lamk, state);
-    FPCA_LAUNCHED(ctx, "eig_lead_e");
-    k_lead_x<<<wb, 256, 0, ctx->stream>>>(n, nref, it, X, E, state, Xk);
+    k_lead_ex<<<dim3(kk, LX_BLOCKS), LE_MAXN, 0, ctx->stream>>>(n, k, nref, it, lam32, pos, lead, Sx, R,
+                                                               X, Xk, lamk, state);
     FPCA_LAUNCHED(ctx, "eig_lead_x");
   }
   {
