@@ -317,13 +317,29 @@ __global__ void __launch_bounds__(NT)
         const int xr = a0 + i;
         const int lo = max(-Tr, -xr), hi = min(Tr, R - 1 - xr);
         const T* col = ina + (size_t)(xr - r0) * C + c;
+        if constexpr (COMP) {
+          // one by one: side by side the compiler's compensated sums end in other last bits,
+          // and a point's status near the fall-back threshold hangs on them
 #pragma unroll
-        for (int a1 = 0; a1 < 3; ++a1) {
-          if (a1 > md) break;
-          const T* w = wr + (box ? 3 : a1) * TW + TMAX;
-          T s = 0, cmp = 0;
-          for (int k = lo; k <= hi; ++k) kadd<T, COMP>(s, cmp, w[k], col[k * C]);
-          mid[(size_t)a1 * npts + e] = s;
+          for (int a1 = 0; a1 < 3; ++a1) {
+            if (a1 > md) break;
+            const T* w = wr + (box ? 3 : a1) * TW + TMAX;
+            T s = 0, cmp = 0;
+            for (int k = lo; k <= hi; ++k) kadd<T, COMP>(s, cmp, w[k], col[k * C]);
+            mid[(size_t)a1 * npts + e] = s;
+          }
+        } else {
+          // the powers side by side: each sum is a chain of dependent operations
+          T s[3] = {};
+          for (int k = lo; k <= hi; ++k) {
+            const T x = col[k * C];
+#pragma unroll
+            for (int a1 = 0; a1 < 3; ++a1)
+              if (a1 <= md) s[a1] = fma(wr[(box ? 3 : a1) * TW + TMAX + k], x, s[a1]);
+          }
+#pragma unroll
+          for (int a1 = 0; a1 < 3; ++a1)
+            if (a1 <= md) mid[(size_t)a1 * npts + e] = s[a1];
         }
       }
       __syncthreads();
@@ -335,20 +351,45 @@ __global__ void __launch_bounds__(NT)
       if (e < npts) {
         const int i = e / C, c = e - (e / C) * C;
         const int lo = max(-Tc, -c), hi = min(Tc, C - 1 - c);
+        if constexpr (COMP) {
 #pragma unroll
-        for (int a1 = 0; a1 < 3; ++a1) {
+          for (int a1 = 0; a1 < 3; ++a1) {
 #pragma unroll
-          for (int a2 = 0; a2 < 3; ++a2) {
-            const int slot = slot_of(d, a, a1, a2);
-            if (slot < 0) continue;
-            const T* rowp = (d == 2) ? mid + (size_t)a1 * npts + (size_t)i * C
-                                     : ina + (size_t)(a0 + i - r0) * C;
-            const T* w = wc + (box ? 3 : a2) * TW + TMAX;
-            T s = 0, cmp = 0;
-            for (int k = lo; k <= hi; ++k) kadd<T, COMP>(s, cmp, w[k], rowp[c + k]);
-            acc[j][slot] = s;
+            for (int a2 = 0; a2 < 3; ++a2) {
+              const int slot = slot_of(d, a, a1, a2);
+              if (slot < 0) continue;
+              const T* rowp = (d == 2) ? mid + (size_t)a1 * npts + (size_t)i * C
+                                       : ina + (size_t)(a0 + i - r0) * C;
+              const T* w = wc + (box ? 3 : a2) * TW + TMAX;
+              T s = 0, cmp = 0;
+              for (int k = lo; k <= hi; ++k) kadd<T, COMP>(s, cmp, w[k], rowp[c + k]);
+              acc[j][slot] = s;
+            }
+          }
+          continue;
+        }
+        // every sum of this array side by side (at most six), the weights read once a tap
+        T s[3][3] = {};
+        for (int k = lo; k <= hi; ++k) {
+          T w[3];
+#pragma unroll
+          for (int a2 = 0; a2 < 3; ++a2)
+            if (a2 <= md) w[a2] = wc[(box ? 3 : a2) * TW + TMAX + k];
+#pragma unroll
+          for (int a1 = 0; a1 < 3; ++a1) {
+            if (slot_of(d, a, a1, 0) < 0) continue;
+            const T x = (d == 2) ? mid[(size_t)a1 * npts + (size_t)i * C + c + k]
+                                 : ina[(size_t)(a0 + i - r0) * C + c + k];
+#pragma unroll
+            for (int a2 = 0; a2 < 3; ++a2)
+              if (slot_of(d, a, a1, a2) >= 0) s[a1][a2] = fma(w[a2], x, s[a1][a2]);
           }
         }
+#pragma unroll
+        for (int a1 = 0; a1 < 3; ++a1)
+#pragma unroll
+          for (int a2 = 0; a2 < 3; ++a2)
+            if (slot_of(d, a, a1, a2) >= 0) acc[j][slot_of(d, a, a1, a2)] = s[a1][a2];
       }
     }
     if constexpr (d == 2) __syncthreads();
@@ -365,6 +406,11 @@ __global__ void __launch_bounds__(NT)
     xts[j] = -1;
     if (e >= npts) continue;
     const int xt = a0 * C + e;  // flat t index: (a0 + i) * C + c
+    const long long o = (long long)xs * P + xt;
+    // CV terms only: a point without held-out pairs adds nothing
+    if (ep.cvacc && !gamma && !status && !ep.y && ep.wf[o] == T(0) && ep.vf[o] == T(0) &&
+        ep.qf[o] == T(0))
+      continue;
     T A[D][D], rv[D];
 #pragma unroll
     for (int i2 = 0; i2 < D; ++i2) {
@@ -378,7 +424,6 @@ __global__ void __launch_bounds__(NT)
     uint8_t st;
     double g = fit_point<D, T>(A, rv, (double)acc[j][NS - 1] + 0.25, st);
     if (mu_raw && st != FPCA_PT_EMPTY) g -= mu_raw[xs] * mu_raw[xt];
-    const long long o = (long long)xs * P + xt;
     if (gamma) gamma[o] = (T)g;
     if (status) status[o] = st;
     xts[j] = xt;

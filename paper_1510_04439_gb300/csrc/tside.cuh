@@ -62,8 +62,42 @@ __device__ __forceinline__ T elim_solve(T (&A)[D][D], T (&r)[D], double& minrati
   return x[0];
 }
 
+// elim_solve's value (the same operations in the same order) without its FP64 pivot ratios:
+// clear = every pivot is above 1.01 ESCALATE_F32 of its diagonal, so that the smallest ratio
+// is known to need no second solve.
+template <int D>
+__device__ __forceinline__ float elim_clear(float (&A)[D][D], float (&r)[D], bool& clear) {
+  float diag[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) diag[i] = A[i][i];
+  clear = true;
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    const float piv = A[k][k];
+    if (!(piv > 0.f && piv > (float)(1.01 * ESCALATE_F32) * diag[k])) clear = false;
+    const float inv = 1.f / piv;
+#pragma unroll
+    for (int i = k + 1; i < D; ++i) {
+      const float l = A[k][i] * inv;
+#pragma unroll
+      for (int j = i; j < D; ++j) A[i][j] -= l * A[k][j];
+      r[i] -= l * r[k];
+    }
+  }
+  float x[D];
+#pragma unroll
+  for (int k = D - 1; k >= 0; --k) {
+    float s = r[k];
+#pragma unroll
+    for (int j = k + 1; j < D; ++j) s -= A[k][j] * x[j];
+    x[k] = s / A[k][k];
+  }
+  return x[0];
+}
+
 // Status and value of one local fit from its normal equations (in T) and the
-// number of non-empty bins in the window.
+// number of non-empty bins in the window.  In FP32 a clear system takes no FP64
+// operation (six divisions before, at 1/64 of the FP32 rate).
 template <int D, typename T>
 __device__ __forceinline__ double fit_point(T (&A)[D][D], T (&r)[D], double nonempty,
                                             uint8_t& st) {
@@ -71,17 +105,18 @@ __device__ __forceinline__ double fit_point(T (&A)[D][D], T (&r)[D], double none
     st = FPCA_PT_EMPTY;
     return __longlong_as_double(0x7ff8000000000000ll);
   }
-  const double lc = (double)r[0] / (double)A[0][0];
+  // the local constant fit (the elimination leaves r[0] and A[0][0] as they are)
+  auto constant = [&]() { return (double)r[0] / (double)A[0][0]; };
   if (nonempty < (double)D) {
     st = FPCA_PT_FALLBACK;
-    return lc;
+    return constant();
   }
   if constexpr (sizeof(T) == 8) {
     double ratio;
     const double b = elim_solve<D, T>(A, r, ratio);
     if (ratio <= PIVOT_RTOL_F64) {
       st = FPCA_PT_FALLBACK;
-      return lc;
+      return constant();
     }
     st = FPCA_PT_OK;
     return b;
@@ -92,6 +127,18 @@ __device__ __forceinline__ double fit_point(T (&A)[D][D], T (&r)[D], double none
       rc[i] = r[i];
 #pragma unroll
       for (int j = 0; j < D; ++j) Ac[i][j] = A[i][j];
+    }
+    bool clear;
+    const T bc = elim_clear<D>(A, r, clear);
+    if (clear) {
+      st = FPCA_PT_OK;
+      return (double)bc;
+    }
+#pragma unroll
+    for (int i = 0; i < D; ++i) {
+      r[i] = rc[i];
+#pragma unroll
+      for (int j = 0; j < D; ++j) A[i][j] = Ac[i][j];
     }
     double ratio;
     const T b = elim_solve<D, T>(A, r, ratio);
@@ -109,7 +156,7 @@ __device__ __forceinline__ double fit_point(T (&A)[D][D], T (&r)[D], double none
     const double bd = elim_solve<D, double>(Ad, rd, ratio);
     if (ratio <= PIVOT_RTOL_F32) {
       st = FPCA_PT_FALLBACK;
-      return lc;
+      return constant();
     }
     st = FPCA_PT_OK;
     return bd;
