@@ -536,33 +536,114 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Phi_i'Y_i^C of two subjects and their systems.  A thread keeps both subjects' L
-// compensated sums over every 256th node, so a phi value read serves two subjects (L2
-// latency bounds it: 53 us at n = 1000, P = 4096, L = 8, where one warp per 1/8 subject that
-// formed Phi'Phi too took 269; a node ahead in registers costs a block an SM: 67 us); the
-// sums join by a halving butterfly of float-float adds (one add per sum instead of
-// five; FP64 adds there would take longer than the sums themselves), the warps in FP64.
-constexpr int PF_SUB = 2;
+// Phi_i'Y_i^C over a chunk of nodes: the chunk's phi in shared memory, two subjects a warp,
+// each lane both subjects' L compensated sums over every 32nd node (a phi value read serves
+// both); the sums join by a halving butterfly of float-float adds (one add a sum instead of
+// five; FP64 adds there would take longer than the sums themselves).  blockIdx: x chunk,
+// y 16 subjects; bpart[(chunk * nb + i) * L + l].  n = 1000, P = 4096, L = 8: 38 us, bound by
+// its FP32 instructions, and 16 for the systems; n = 1500, P = 1320, L = 13: 38 and 30.  With
+// phi from L2 and a block taking two whole subjects and their systems: 53 and 131 (one warp
+// per 1/8 subject, forming Phi'Phi too: 269 and 293).
+template <int LM>
+constexpr int pd_chunk() { return LM == 8 ? 512 : 256; }
 template <int LM>
 __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
-    k_pace_final(int nb, int i0, int P, const void* __restrict__ y, int yprec,
-                 const uint8_t* __restrict__ mask, const float2* __restrict__ mu2,
-                 const double* __restrict__ prior, const float2* __restrict__ phi2, int L, int nsplit, const int* __restrict__ expo,
-                 const long long* __restrict__ gsum, double* __restrict__ scores,
+    k_pace_dots(int nb, int i0, int P, const void* __restrict__ y, int yprec,
+                const uint8_t* __restrict__ mask, const float2* __restrict__ mu2,
+                const float2* __restrict__ phi2, int L, const int* __restrict__ expo,
+                float2* __restrict__ bpart) {
+  constexpr int NV = 2 * LM, CH = pd_chunk<LM>();
+  __shared__ float2 ph[LM][CH];
+  __shared__ float2 mus[CH];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int p0 = blockIdx.x * CH, pn = min(CH, P - p0);
+  for (int e = tid; e < LM * CH; e += 256) {
+    const int l = e / CH, c = e % CH;
+    ph[l][c] = l < L && c < pn ? phi2[(long long)l * P + p0 + c] : make_float2(0.f, 0.f);
+  }
+  for (int c = tid; c < pn; c += 256) mus[c] = mu2[p0 + c];
+  bool clean = true;  // no phi value that times a zero is not zero
+  for (int l = 0; l < L; ++l) clean &= expo[l] != PG_EBAD;
+  __syncthreads();
+  const int s0 = blockIdx.y * 16 + warp * 2;
+  if (s0 >= nb) return;
+  const size_t row0 = (size_t)(i0 + s0) * P + p0, row1 = (size_t)(i0 + min(s0 + 1, nb - 1)) * P + p0;
+  Acc acc[2][LM];
+#pragma unroll 2
+  for (int c = lane; c < pn; c += 32) {
+    // unobserved responses are read and not used, so that no load waits for another
+    const bool ok0 = !mask || mask[row0 + c], ok1 = s0 + 1 < nb && (!mask || mask[row1 + c]);
+    const float2 m = mus[c];
+    ff::F2 r0 = centred(y, yprec, row0 + c, ff::F2{m.x, m.y});
+    ff::F2 r1 = centred(y, yprec, row1 + c, ff::F2{m.x, m.y});
+    if (!ok0) r0 = ff::make(0.f);
+    if (!ok1) r1 = ff::make(0.f);
+#pragma unroll
+    for (int l = 0; l < LM; ++l) {
+      if (l < L) {
+        const ff::F2 f{ph[l][c].x, ph[l][c].y};
+        acc[0][l].add_prod(r0, clean || ok0 ? f : ff::make(0.f));
+        acc[1][l].add_prod(r1, clean || ok1 ? f : ff::make(0.f));
+      }
+    }
+  }
+  ff::F2 v[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k)
+    v[k] = ff::fast_two_sum(acc[k / LM][k % LM].s, acc[k / LM][k % LM].c);
+  int at = 0;  // the sum that this lane ends with
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st, left = NV >> (st + 1);
+    const bool up = lane & o;
+    if (up) at += left;
+#pragma unroll
+    for (int k = 0; k < (left > 0 ? left : 1); ++k) {
+      const ff::F2 give = up || left == 0 ? v[k] : v[k + left];
+      const ff::F2 keep = up && left > 0 ? v[k + left] : v[k];
+      v[k] = ff::add(keep, ff::F2{__shfl_xor_sync(0xffffffffu, give.hi, o),
+                                  __shfl_xor_sync(0xffffffffu, give.lo, o)});
+    }
+  }
+  const int sl = s0 + at / LM, l = at % LM;  // (with 16 sums two lanes hold the same one)
+  if (sl < nb && l < L)
+    bpart[((size_t)blockIdx.x * nb + sl) * L + l] = make_float2(v[0].hi, v[0].lo);
+}
+
+// The systems of 32 / LM subjects: the sums of the node splits and chunks, the test of the
+// table's bound (Phi'Phi again in float-float where it fails), and the solves.
+template <int LM>
+__global__ void __launch_bounds__(128)
+    k_pace_final(int nb, int i0, int P, const uint8_t* __restrict__ mask,
+                 const double* __restrict__ prior, const float2* __restrict__ phi2, int L, int nsplit,
+                 int nchunk, const int* __restrict__ expo, const long long* __restrict__ gsum,
+                 const float2* __restrict__ bpart, double* __restrict__ scores,
                  int* __restrict__ err) {
-  constexpr int NV = PF_SUB * LM;
-  __shared__ PaceSys sys[PF_SUB];
-  __shared__ float2 wsum[8][NV];
-  __shared__ double count[PF_SUB];
-  __shared__ int redo[PF_SUB];
+  constexpr int SUB = 32 / LM;
+  __shared__ PaceSys sys[SUB];
+  __shared__ float2 wsum[4];
+  __shared__ double count[SUB];
+  __shared__ int redo[SUB];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L);
-  const int s0 = blockIdx.x * PF_SUB;
-  if (tid < PF_SUB) redo[tid] = 0;
-  for (int it = tid; it < PF_SUB * (NE + 1); it += 256) {
-    const int sl = it / (NE + 1), e = it - sl * (NE + 1);
+  const int s0 = blockIdx.x * SUB;
+  if (tid < SUB) redo[tid] = 0;
+  for (int it = tid; it < SUB * (NE + 1 + L); it += 128) {
+    const int sl = it / (NE + 1 + L), e = it - sl * (NE + 1 + L);
     if (s0 + sl >= nb) continue;
+    if (e > NE) {
+      const int l = e - NE - 1;
+      double b0 = 0.0, b1 = 0.0;
+      for (int k = 0; k < nchunk; ++k) {
+        const float2 v = bpart[((size_t)k * nb + s0 + sl) * L + l];
+        b0 += (double)v.x;
+        b1 += (double)v.y;
+      }
+      sys[sl].b[l] = b0 + b1;
+      continue;
+    }
     long long hi = 0, lo = 0;  // of the splits' fixed-point sums
+#pragma unroll 4
     for (int k = 0; k < nsplit; ++k) {
       const long long v = gsum[((size_t)k * nb + s0 + sl) * ng8 + e];
       hi += v >> 32;
@@ -583,67 +664,20 @@ __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
     sys[sl].A[a][b] = ge;
     sys[sl].A[b][a] = ge;
   }
-  Acc acc[PF_SUB][LM];
-  bool clean = true;  // no phi value that times a zero is not zero
-  for (int l = 0; l < L; ++l) clean &= expo[l] != PG_EBAD;
-  const size_t row0 = (size_t)(i0 + s0) * P, row1 = (size_t)(i0 + min(s0 + 1, nb - 1)) * P;
-  for (int p = tid; p < P; p += 256) {
-    // unobserved responses are read and not used, so that no load waits for another
-    const bool ok0 = !mask || mask[row0 + p], ok1 = s0 + 1 < nb && (!mask || mask[row1 + p]);
-    const float2 m = mu2[p];
-    ff::F2 r0 = centred(y, yprec, row0 + p, ff::F2{m.x, m.y});
-    ff::F2 r1 = centred(y, yprec, row1 + p, ff::F2{m.x, m.y});
-    if (!ok0) r0 = ff::make(0.f);
-    if (!ok1) r1 = ff::make(0.f);
-#pragma unroll
-    for (int l = 0; l < LM; ++l) {
-      if (l < L) {
-        const float2 f = phi2[(long long)l * P + p];
-        const ff::F2 ph{f.x, f.y};
-        acc[0][l].add_prod(r0, clean || ok0 ? ph : ff::make(0.f));
-        acc[1][l].add_prod(r1, clean || ok1 ? ph : ff::make(0.f));
-      }
-    }
-  }
-  static_assert(PF_SUB == 2, "two subjects above");
-  ff::F2 v[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k)
-    v[k] = ff::fast_two_sum(acc[k / LM][k % LM].s, acc[k / LM][k % LM].c);
-  int at = 0;  // the sum that this lane ends with
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int o = 16 >> st, left = NV >> (st + 1);
-    const bool up = lane & o;
-    if (up) at += left;
-#pragma unroll
-    for (int k = 0; k < (left > 0 ? left : 1); ++k) {
-      const ff::F2 give = up || left == 0 ? v[k] : v[k + left];
-      const ff::F2 keep = up && left > 0 ? v[k + left] : v[k];
-      v[k] = ff::add(keep, ff::F2{__shfl_xor_sync(0xffffffffu, give.hi, o),
-                                  __shfl_xor_sync(0xffffffffu, give.lo, o)});
-    }
-  }
-  wsum[warp][at] = make_float2(v[0].hi, v[0].lo);
   __syncthreads();
-  if (tid < NV && tid % LM < L) {
-    double sum = 0.0;
-    for (int w = 0; w < 8; ++w) sum += (double)wsum[w][tid].x + (double)wsum[w][tid].y;
-    sys[tid / LM].b[tid % LM] = sum;
-  }
-  if (tid < PF_SUB * L) {  // the bound of the table's rounding, see above
+  if (tid < SUB * L) {  // the bound of the table's rounding, see above
     const int sl = tid / L, l = tid - sl * L, e = expo[l];
     if (s0 + sl < nb && e > PG_EZERO &&
         (e == PG_EBAD || !(sys[sl].A[l][l] >= count[sl] * pow2(2 * e - 8))))
       redo[sl] = 1;
   }
   __syncthreads();
-  for (int sl = 0; sl < PF_SUB; ++sl) {
+  for (int sl = 0; sl < SUB; ++sl) {
     if (!redo[sl]) continue;
     for (int a = 0; a < L; ++a) {
       for (int b = a; b < L; ++b) {
         Acc ac;
-        for (int p = tid; p < P; p += 256) {
+        for (int p = tid; p < P; p += 128) {
           if (mask && !mask[(long long)(i0 + s0 + sl) * P + p]) continue;
           const float2 fa = phi2[(long long)a * P + p], fb = phi2[(long long)b * P + p];
           ac.add_prod(ff::F2{fa.x, fa.y}, ff::F2{fb.x, fb.y});
@@ -652,11 +686,11 @@ __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
         for (int o = 16; o > 0; o >>= 1)
           sum = ff::add(sum, ff::F2{__shfl_xor_sync(0xffffffffu, sum.hi, o),
                                     __shfl_xor_sync(0xffffffffu, sum.lo, o)});
-        if (lane == 0) wsum[warp][0] = make_float2(sum.hi, sum.lo);
+        if (lane == 0) wsum[warp] = make_float2(sum.hi, sum.lo);
         __syncthreads();
         if (tid == 0) {
           double t = 0.0;
-          for (int w = 0; w < 8; ++w) t += (double)wsum[w][0].x + (double)wsum[w][0].y;
+          for (int w = 0; w < 4; ++w) t += (double)wsum[w].x + (double)wsum[w].y;
           sys[sl].A[a][b] = t;
           sys[sl].A[b][a] = t;
         }
@@ -665,10 +699,9 @@ __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
     }
   }
   if (warp == 0) {
-    const int sl = lane / LM < PF_SUB ? lane / LM : PF_SUB - 1;
-    const bool active = lane / LM < PF_SUB && s0 + sl < nb;
-    pace_solve<LM>(&sys[sl], prior, L, active, err);
-    for (int e = lane; e < PF_SUB * L; e += 32)
+    const int sl = lane / LM;
+    pace_solve<LM>(&sys[sl], prior, L, s0 + sl < nb, err);
+    for (int e = lane; e < SUB * L; e += 32)
       if (s0 + e / L < nb) scores[(long long)(i0 + s0) * L + e] = sys[e / L].b[e % L];
   }
 }
@@ -831,8 +864,9 @@ struct ScWork {
   int* expo;           // L exponents
   uint2* table;
   long long* gsum;
+  float2* bpart;       // partial Phi'Y^C of the node chunks
   const double* phi;
-  int nbx, nsplit, per, batch;
+  int nbx, nsplit, per, batch, nchunk;
 };
 
 fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double* evecs, ScWork* w,
@@ -845,13 +879,16 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   w->per = n64 <= 64 ? 4 : 8;
   w->nsplit = (n64 + w->per - 1) / w->per;
   w->batch = std::max(128, PG_BATCH / w->nsplit / 128 * 128);
+  const int chunk = L <= 8 ? pd_chunk<8>() : pd_chunk<16>();
+  w->nchunk = (P + chunk - 1) / chunk;
   const size_t nt = (size_t)n64 * 4 * ng * PG_DIG * 32;
   const size_t ns = (size_t)w->nsplit * w->batch * 8 * ng;
   void* ws = fpca_workspace(ctx, WsCarve::round(sizeof(float2) * P) +
                                      WsCarve::round(sizeof(float2) * (size_t)L * P) +
                                      WsCarve::round(sizeof(float) * L * w->nbx) + 512 +
                                      WsCarve::round(sizeof(uint2) * nt) +
-                                     WsCarve::round(sizeof(long long) * ns));
+                                     WsCarve::round(sizeof(long long) * ns) +
+                                     WsCarve::round(sizeof(float2) * w->nchunk * w->batch * L));
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
   WsCarve c(ws);
   w->mu2 = c.take<float2>(P);
@@ -861,6 +898,7 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   w->prior = c.take<double>(SC_LMAX + 1);
   w->table = c.take<uint2>(nt);
   w->gsum = c.take<long long>(ns);
+  w->bpart = c.take<float2>((size_t)w->nchunk * w->batch * L);
   k_split_ff<<<dim3(w->nbx, L + 1), 256, 0, ctx->stream>>>(P, mu, evecs, w->mu2, w->phi2, w->bmax, L,
                                                                 lam, sigma2, w->prior);
   FPCA_LAUNCHED(ctx, "split_ff");
@@ -881,10 +919,15 @@ fpca_status pace_dense(fpca_ctx* ctx, const fpca_data* data, int P, int L, const
     gram<<<dim3((nb + 127) / 128, w.nsplit, (ng + gp - 1) / gp), 256, 0, ctx->stream>>>(
         nb, i0, P, ng, w.per, data->mask, w.table, w.gsum, vec);
     FPCA_LAUNCHED(ctx, "pace_gram");
+    auto dots = L <= 8 ? k_pace_dots<8> : k_pace_dots<16>;
+    dots<<<dim3(w.nchunk, (nb + 15) / 16), 256, 0, ctx->stream>>>(
+        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, w.phi2, L, w.expo, w.bpart);
+    FPCA_LAUNCHED(ctx, "pace_dots");
     auto fin = L <= 8 ? k_pace_final<8> : k_pace_final<16>;
-    fin<<<(nb + PF_SUB - 1) / PF_SUB, 256, 0, ctx->stream>>>(
-        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, w.prior, w.phi2, L, w.nsplit,
-        w.expo, w.gsum, scores, ctx->d_err);
+    const int sub = L <= 8 ? 4 : 2;
+    fin<<<(nb + sub - 1) / sub, 128, 0, ctx->stream>>>(nb, i0, P, data->mask, w.prior, w.phi2, L,
+                                                      w.nsplit, w.nchunk, w.expo, w.gsum, w.bpart,
+                                                      scores, ctx->d_err);
     FPCA_LAUNCHED(ctx, "scores_pace");
   }
   return FPCA_OK;
