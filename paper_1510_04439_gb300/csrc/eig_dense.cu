@@ -1,9 +1,11 @@
 // Leading eigenpairs of a symmetric FP64 matrix with n <= 256 (the dense path of
 // fpca_rproj_eig on small grids).
 //
-// A serial chain bounds it: some 90 rounds of dependent rotations at 256 x 256.  The whole
-// FP64 fit of a 16 x 16 grid takes 2.8 ms with it and took 4.9 ms through launch_dense_eig
-// (180 launches of each round's two kernels among them); of a 64-node curve 0.75 ms, from 1.16.
+// A serial chain bounds it: some 75 rounds of dependent rotations at 256 x 256 (1.2 ms; 2.6
+// with two barriers and exact square roots in a rotation step, and sweeps until every
+// off-diagonal was small).  The whole FP64 fit of a 16 x 16 grid takes 1.3 to 1.4 ms with it and
+// took 4.9 ms through launch_dense_eig (180 launches of each round's two kernels among them);
+// of a 64-node curve 0.43 ms, from 1.16.
 //
 //  1. Block Jacobi in FP32 on one thread-block cluster (k_bj_cluster): all eigenvectors to
 //     about 1e-5 or better.
