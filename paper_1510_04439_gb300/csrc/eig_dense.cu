@@ -8,7 +8,7 @@
 // of a 64-node curve 0.43 ms, from 1.16.
 //
 //  1. Block Jacobi in FP32 on one thread-block cluster (k_bj_cluster): all eigenvectors to
-//     about 1e-5 or better.
+//     about 1e-5 or better, or until the off-diagonal norm is LE_APART of the wanted gaps.
 //  2. The k leading vectors (and a few more, so that nearly equal eigenvalues at the edge
 //     are ordered by their refined values) are refined in FP64 against the FP32 basis X:
 //     for vector x_j,  s_ij = x_i' A x_j,  r_ij = delta_ij - x_i' x_j,
