@@ -340,6 +340,10 @@ constexpr int OBS_LANES = 8;  // threads per subject
 // no pairs or is skipped) and the rows' observation counts.  Offsets outside
 // 0 <= offs[i] <= offs[i+1] <= N and folds outside 0..nfold-1 are reported (DERR_BOUNDS)
 // and the subject is skipped.  row is set to -1 by the caller.
+// A skipped subject's neighbours can overlap (offsets 0, 10, 5, 12: the first and the third
+// both hold observations 5..9).  An observation goes to the subject that claims its row first,
+// and only that one writes the record and counts it: the counts add up to at most N and equal
+// what k_row_fill places, and a record's lo and ni are one checked subject's.
 __global__ void k_obs_rows(int n, long long N, int d, int m0, int m1, int m2, int P,
                            const int64_t* __restrict__ offs, const double* __restrict__ t,
                            const double* __restrict__ y, const double* __restrict__ mu, int mode,
@@ -366,10 +370,10 @@ __global__ void k_obs_rows(int n, long long N, int d, int m0, int m1, int m2, in
   const int m[3] = {m0, m1, m2};
   for (int64_t j = lo + part; j < hi; j += OBS_LANES) {
     const int b = bin_index(t + j * d, d, m);
+    if (atomicCAS(row + j, -1, f * P + b) != -1) continue;  // another subject's (see above)
     ob[j] = b;
     rec[j] = ObsRec{mode == FPCA_COV_RESIDUAL ? y[j] - mu[b] : y[j], (int32_t)lo,
                     (int32_t)(hi - lo)};
-    row[j] = f * P + b;
     atomicAdd(rowcount + f * P + b, 1);
   }
 }
