@@ -34,7 +34,8 @@ __device__ __forceinline__ void tile_pair(int L, int& bi, int& bj) {
   bi = L - (int)((long long)bj * (bj + 1) / 2);
 }
 
-// Sigma = sym(G) with NaN and out-of-domain entries zeroed; trace accumulated.
+// Sigma = sym(G) with NaN and out-of-domain entries zeroed; trace accumulated; of an FP64 Sigma
+// (the dense eigensolvers') also the bits of its largest magnitude into *top.
 // The arithmetic is done in the type of Sigma (FP32 for the projected path).
 // A block takes the pair of 32 x 32 tiles (I, J) and (J, I), I <= J, so G is read once and
 // Sigma written once: s = (g_pq + g_qp) / 2 is formed for (p, q) in (I, J) and written there
@@ -45,8 +46,9 @@ constexpr int MX_T = 32, MX_R = 8, MX_U = MX_T / MX_R;  // tile, block rows, row
 template <typename TG, typename TS>
 __global__ void __launch_bounds__(MX_T * MX_R)
     k_matrixize(int P, const TG* __restrict__ G, const int32_t* __restrict__ dom,
-                TS* __restrict__ S, double* __restrict__ trace) {
+                TS* __restrict__ S, double* __restrict__ trace, unsigned long long* __restrict__ top) {
   __shared__ TS tile[MX_T][MX_T + 1];
+  unsigned long long big = 0;
   __shared__ double dsum;  // this block's part of the trace (diagonal blocks only)
   int bi, bj;
   tile_pair((int)blockIdx.x, bi, bj);
@@ -81,8 +83,14 @@ __global__ void __launch_bounds__(MX_T * MX_R)
       if (dp[u] <= 0 || dq <= 0) sv = TS(0);
       S[(long long)p * P + q] = sv;
       if (p == q) atomicAdd(&dsum, (double)sv);
+      if constexpr (sizeof(TS) == 8)
+        big = max(big, (unsigned long long)__double_as_longlong(sv) & 0x7fffffffffffffffull);
     }
     tile[tx][r] = sv;
+  }
+  if constexpr (sizeof(TS) == 8) {
+    for (int o = 16; o > 0; o >>= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if (tx == 0) atomicMax(top, big);
   }
   __syncthreads();
   if (i0 == j0) {
@@ -900,14 +908,22 @@ __global__ void k_rr_out(int n, const double* __restrict__ lam, const double* __
   }
 }
 
-// Rank of each eigenvalue (descending; ties by index) -> order[rank] = index.
+// out = in 2^-e (eig_exponent), element by element
+__global__ void k_scale(long long n, const double* __restrict__ in,
+                        const unsigned long long* __restrict__ top, double* __restrict__ out) {
+  const int ex = eig_exponent(*top);
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
+       e += (long long)gridDim.x * blockDim.x)
+    out[e] = eig_scaled(in[e], ex);
+}
+
+// Rank of each eigenvalue (descending; ties by index; NaN last) -> order[rank] = index.
 __global__ void k_eig_order(int n, const double* __restrict__ A, int* __restrict__ order) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
     const double ti = A[(long long)i * n + i];
     int rank = 0;
     for (int j = 0; j < n; ++j) {
-      const double tj = A[(long long)j * n + j];
-      rank += (tj > ti) || (tj == ti && j < i);
+      rank += eig_before(A[(long long)j * n + j], j, ti, i);
     }
     order[rank] = i;
   }
@@ -949,7 +965,9 @@ __global__ void k_dense_vectors(int P, int k, const double* __restrict__ V,
 // phi = psi / sqrt(dV) (inv_sqrt_dv = 1 / sqrt(dV) from the host), lambda = theta
 // dV, FVE = cumulative theta / trace.  One block per eigenvector.  The magnitudes
 // are compared through their bit patterns (non-negative doubles order as their
-// 64-bit integers), keyed with the index so that ties take the first entry.
+// 64-bit integers), keyed with the index so that ties take the first entry.  top (or NULL):
+// the eigenvalues are those of the scaled matrix (eig_exponent) and are scaled back; a matrix
+// that is not finite has NaN eigenpairs.
 __device__ __forceinline__ unsigned long long fin_better(unsigned long long a, int ia,
                                                          unsigned long long b, int ib) {
   return (b > a || (b == a && ib < ia)) ? 1ull : 0ull;
@@ -958,8 +976,10 @@ __device__ __forceinline__ unsigned long long fin_better(unsigned long long a, i
 __global__ void __launch_bounds__(1024)
     k_finish(int P, int n, int k, double dv, double inv_sqrt_dv, const double* __restrict__ Aeig,
              const int* __restrict__ order, const double* __restrict__ trace,
-             double* __restrict__ evals, double* __restrict__ evecs, double* __restrict__ fve) {
-  const int j = blockIdx.x;
+             double* __restrict__ evals, double* __restrict__ evecs, double* __restrict__ fve,
+             const unsigned long long* __restrict__ top = nullptr) {
+  const int j = blockIdx.x, ex = top ? eig_exponent(*top) : 0;
+  const bool finite = !top || *top < EIG_INF;
   double* v = evecs + (long long)j * P;
   __shared__ unsigned long long wb[32];
   __shared__ int wi[32];
@@ -1001,14 +1021,17 @@ __global__ void __launch_bounds__(1024)
     if (lane == 0) sgn = (bidx != 0x7fffffff && v[bidx] < 0.0) ? -inv_sqrt_dv : inv_sqrt_dv;
   }
   __syncthreads();
-  const double scale = sgn;
+  const double scale = finite ? sgn : __longlong_as_double(0x7ff8000000000000ll);
   for (int r = threadIdx.x; r < P; r += blockDim.x) v[r] *= scale;
   if (threadIdx.x == 0) {
-    const double th = Aeig[(long long)order[j] * n + order[j]];
-    evals[j] = th * dv;
+    auto theta = [&](int i) {
+      const double th = eig_scaled(Aeig[(long long)order[i] * n + order[i]], -ex);
+      return finite ? th : __longlong_as_double(0x7ff8000000000000ll);
+    };
+    evals[j] = theta(j) * dv;
     if (fve) {
       double cum = 0.0;
-      for (int i = 0; i <= j; ++i) cum += Aeig[(long long)order[i] * n + order[i]];
+      for (int i = 0; i <= j; ++i) cum += theta(i);
       fve[j] = cum / trace[0];
     }
   }
@@ -1467,7 +1490,7 @@ inline size_t dense_eig_bytes(int n) {
          WsCarve::round(sizeof(int) * rotate_ints(n));
 }
 
-// Eigenpairs of the symmetric n x n FP64 matrix A (n <= 1024): A <- diag(lambda),
+// Eigenpairs of the symmetric n x n FP64 matrix A (n <= 1024, entries below 1): A <- diag(lambda),
 // V <- eigenvectors (columns), like launch_jacobi_rr.
 fpca_status launch_dense_eig(fpca_ctx* ctx, int n, double* A, double* V, void* scratch) {
   const int ne = bj_ne(n), nb = ne / BJ_S, npairs = ne / BJ_W;
@@ -1645,24 +1668,26 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
   float* ppart = carve.take<float>(proj_part_floats(P, l, ctx->num_sms));
   char* dense = full ? carve.take<char>(dense_bytes) : nullptr;
 
-  cudaMemsetAsync(trace, 0, sizeof(double), ctx->stream);
+  unsigned long long* top = reinterpret_cast<unsigned long long*>(trace + 1);
+  cudaMemsetAsync(trace, 0, 2 * sizeof(double), ctx->stream);
   const long long mt = (P + MX_T - 1) / MX_T;
   k_matrixize<TG, TS><<<(unsigned)(mt * (mt + 1) / 2), dim3(MX_T, MX_R), 0, ctx->stream>>>(
-      P, gamma, domain, S, trace);
+      P, gamma, domain, S, trace, top);
   FPCA_LAUNCHED(ctx, "matrixize");
   if (full) {
     // dense eigenpairs of Sigma (FP64)
     if constexpr (sizeof(TS) == 8) {
       if (lead_eig_takes(P)) {
         // A: the eigenvalues as a vector (row stride 0 below), order: 0..k-1
-        fpca_status ls = launch_lead_eig(ctx, P, k, S, A, evecs, order, dense);
+        fpca_status ls = launch_lead_eig(ctx, P, k, S, top, A, evecs, order, dense);
         if (ls != FPCA_OK) return ls;
         k_finish<<<k, 1024, 0, ctx->stream>>>(P, 0, k, dv, 1.0 / std::sqrt(dv), A, order, trace,
-                                              evals, evecs, fve);
+                                              evals, evecs, fve, top);
         FPCA_LAUNCHED(ctx, "eig_finish");
         return FPCA_OK;
       }
-      cudaMemcpyAsync(A, S, sizeof(double) * PP, cudaMemcpyDeviceToDevice, ctx->stream);
+      k_scale<<<(int)std::min<long long>((PP + 255) / 256, 4096), 256, 0, ctx->stream>>>(PP, S, top, A);
+      FPCA_LAUNCHED(ctx, "eig_scale");
     } else {
       return fpca_fail(ctx, FPCA_E_UNSUPPORTED, "dense eigensolver needs FP64 gamma");
     }
@@ -1674,7 +1699,7 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
                                                                                     evecs);
     FPCA_LAUNCHED(ctx, "dense_vectors");
     k_finish<<<k, 1024, 0, ctx->stream>>>(P, P, k, dv, 1.0 / std::sqrt(dv), A, order, trace,
-                                          evals, evecs, fve);
+                                          evals, evecs, fve, top);
     FPCA_LAUNCHED(ctx, "eig_finish");
     return FPCA_OK;
   }

@@ -5,6 +5,43 @@
 
 namespace fpca_jacobi {
 
+// Integers that order as the numbers do, NaN below all (and 64-bit comparisons are slow here).
+__device__ __forceinline__ int eig_key(float x) {
+  const int b = __float_as_int(x);
+  if (isnan(x)) return (int)0x80000000;
+  return b >= 0 ? b : (b << 1) == 0 ? 0 : b ^ 0x7fffffff;
+}
+__device__ __forceinline__ long long eig_key(double x) {
+  const long long b = __double_as_longlong(x), m = b & 0x7fffffffffffffffll;
+  if (m > 0x7ff0000000000000ll) return (long long)0x8000000000000000ull;
+  return b >= 0 ? b : m == 0 ? 0 : b ^ 0x7fffffffffffffffll;
+}
+
+// Eigenvalue a (place i) comes before b (place j): descending, ties by place, NaN last.  A total
+// order, so that ranks are a permutation and every rank's entry is written.
+template <typename T>
+__device__ __forceinline__ bool eig_before(T a, int i, T b, int j) {
+  const auto ka = eig_key(a), kb = eig_key(b);
+  return ka > kb || (ka == kb && i < j);
+}
+
+// The dense eigensolvers work on A 2^-e, e the exponent for which the largest entry lies in
+// [1/2, 1): their FP32 copies, squares and thresholds then neither overflow nor vanish whatever
+// the scale of the data (from 1.8e19 on a square of FP32 is infinite), and the scaling is exact.
+// `top`: the bits of the largest |entry|, which order as the numbers do; not finite: e = 0.
+constexpr unsigned long long EIG_INF = 0x7ff0000000000000ull;
+__device__ __forceinline__ int eig_exponent(unsigned long long top) {
+  if (top == 0 || top >= EIG_INF) return 0;
+  return ilogb(__longlong_as_double((long long)top)) + 1;
+}
+// x 2^-e, by the exponent bits where both are normal numbers (FP64 operations are slow here)
+__device__ __forceinline__ double eig_scaled(double x, int e) {
+  const int hi = __double2hiint(x), ex = (hi >> 20) & 0x7ff;
+  if (ex > 0 && ex < 0x7ff && ex - e > 0 && ex - e < 0x7ff)
+    return __hiloint2double(hi - e * (1 << 20), __double2loint(x));
+  return scalbn(x, -e);
+}
+
 // Pair (p, q), p < q, of position i (0 <= i < ne / 2) at step `step` of a sweep of
 // the round-robin (circle) schedule: ne / 2 disjoint pairs per step, ne - 1 steps
 // (ne even; q == n marks the dummy of odd n).
