@@ -1372,13 +1372,21 @@ __global__ void k_bj_extract(int n, int ne, const float* __restrict__ V, const d
   }
 }
 
+constexpr int OA_STEPS = 5;
+constexpr float OA_BAD = 1e-8f;  // a correction this small leaves an error of its square
+
+// Nothing left for a step to do: the last one's largest correction (NULL: take the step).
+__device__ __forceinline__ bool oa_done(const float* gate) { return gate && !(*gate > OA_BAD); }
+
 // Refinement pieces for n up to 1024 (one thread per column, lambda in global).
 // Row i per block: lam[i] = S_ii / (1 - R_ii) and the squared norms of the
 // off-diagonal of S, of A and of R added to acc[0..2] (zeroed by the caller).
 __global__ void __launch_bounds__(256)
     k_oa_norms(int n, const double* __restrict__ A, const double* __restrict__ R,
-               const double* __restrict__ S, double* __restrict__ lam, double* __restrict__ acc) {
+               const double* __restrict__ S, double* __restrict__ lam, double* __restrict__ acc,
+               const float* __restrict__ gate) {
   __shared__ double red[8][3];
+  if (oa_done(gate)) return;
   const int i = blockIdx.x;
   const long long o = (long long)i * n;
   double so = 0.0, an = 0.0, rn = 0.0;
@@ -1413,13 +1421,31 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// wanted[i] = 1 where eigenvalue i is among the k largest (a warp per eigenvalue).
+__global__ void __launch_bounds__(256)
+    k_oa_wanted(int n, int k, const double* __restrict__ lam, int* __restrict__ wanted,
+                const float* __restrict__ gate) {
+  const int i = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (oa_done(gate) || i >= n) return;
+  const double li = lam[i];
+  int rank = 0;
+  for (int j = lane; j < n; j += 32) rank += eig_before(lam[j], j, li, i);
+  for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+  if (lane == 0) wanted[i] = rank < k;
+}
+
 // Row i per block of the correction E: eigenvalues closer than
-// delta = 2 (||offdiag S|| + ||A|| ||R||) are treated as one cluster.  emax (zeroed) takes
-// the largest correction, 1 where a cluster still couples by more than 1e-13 ||A||.
+// delta = 2 (||offdiag S|| + ||A|| ||R||) are treated as one cluster.  emax (zeroed; NULL on the
+// steps that are always taken) gets the largest correction of a wanted vector, 1 where one still
+// couples within a cluster by more than 1e-13 ||A||.  The others do not count: the trailing
+// eigenvalues of a smoothed covariance lie below the FP32 couplings of the sweeps, so that some
+// pair of them always would.
 __global__ void __launch_bounds__(256)
     k_oa_correction(int n, const double* __restrict__ R, const double* __restrict__ S,
                     const double* __restrict__ lam, const double* __restrict__ acc,
-                    double* __restrict__ E, float* __restrict__ emax) {
+                    double* __restrict__ E, const int* __restrict__ wanted,
+                    float* __restrict__ emax, const float* __restrict__ gate) {
+  if (oa_done(gate)) return;
   const int i = blockIdx.x;
   const long long o = (long long)i * n;
   const double delta = 2.0 * (sqrt(acc[0]) + sqrt(acc[1]) * sqrt(acc[2]));
@@ -1430,21 +1456,20 @@ __global__ void __launch_bounds__(256)
     const bool close = fabs(gap) <= delta;
     const double e = (j == i || close) ? 0.5 * R[o + j] : couple / gap;
     E[o + j] = e;
+    if (!emax || !wanted[j]) continue;
     mag = fmaxf(mag, fabsf((float)e));
     if (close && j != i && fabs(couple) > 1e-13 * sqrt(acc[1])) mag = 1.f;
   }
+  if (!emax) return;
   for (int k = 16; k > 0; k >>= 1) mag = fmaxf(mag, __shfl_xor_sync(0xffffffffu, mag, k));
   if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<int*>(emax), __float_as_int(mag));
 }
 
-constexpr float OA_BAD = 1e-8f;  // a correction this small leaves an error of its square
-
-// X <- X + X E (row i per block; the row is staged before it is written).  With `gate`
-// nothing is done unless *gate > OA_BAD.
+// X <- X + X E (row i per block; the row is staged before it is written).
 __global__ void k_oa_update(int n, double* __restrict__ X, const double* __restrict__ E,
                             const float* __restrict__ gate = nullptr) {
   extern __shared__ double xrow[];
-  if (gate && !(*gate > OA_BAD)) return;
+  if (oa_done(gate)) return;
   const int i = blockIdx.x;
   for (int j = threadIdx.x; j < n; j += blockDim.x) xrow[j] = X[(long long)i * n + j];
   __syncthreads();
@@ -1461,11 +1486,10 @@ __global__ void k_oa_update(int n, double* __restrict__ X, const double* __restr
 }
 
 // Row i (block) of C = op(L) M (+ diag I): n up to 1024, two interleaved chains.
-// With `gate` nothing is done unless *gate > OA_BAD.
 __global__ void k_oa_rowmm(int n, const double* __restrict__ L, int tl, const double* __restrict__ M,
                            double* __restrict__ C, double diag, double sign,
                            const float* __restrict__ gate = nullptr) {
-  if (gate && !(*gate > OA_BAD)) return;
+  if (oa_done(gate)) return;
   const int i = blockIdx.x;
   for (int j = threadIdx.x; j < n; j += blockDim.x) {
     double s0 = 0.0, s1 = 0.0;
@@ -1487,12 +1511,15 @@ inline size_t dense_eig_bytes(int n) {
          WsCarve::round(sizeof(float) * (size_t)npairs * BJ_W * BJ_W) + WsCarve::round(64) +
          WsCarve::round(sizeof(double) * (2 * BJ_SWEEPS + 4)) +
          5 * WsCarve::round(sizeof(double) * (size_t)n * n) + WsCarve::round(sizeof(double) * n) +
-         WsCarve::round(sizeof(int) * rotate_ints(n));
+         WsCarve::round(sizeof(int) * rotate_ints(n)) + WsCarve::round(sizeof(int) * n);
 }
 
 // Eigenpairs of the symmetric n x n FP64 matrix A (n <= 1024, entries below 1): A <- diag(lambda),
-// V <- eigenvectors (columns), like launch_jacobi_rr.
-fpca_status launch_dense_eig(fpca_ctx* ctx, int n, double* A, double* V, void* scratch) {
+// V <- eigenvectors (columns), like launch_jacobi_rr; of the k largest also those of close
+// eigenvalues.  What these need in FP64 is gated by their own corrections: gated by all n, a
+// smoothed covariance (18 x 18 nodes, 4 eigenpairs) took the FP64 Jacobi for its trailing
+// eigenvalues: 21.8 ms for the whole fit, 4.8 now.  Bound by the FP32 rounds' launches and the steps' FP64 products.
+fpca_status launch_dense_eig(fpca_ctx* ctx, int n, int k, double* A, double* V, void* scratch) {
   const int ne = bj_ne(n), nb = ne / BJ_S, npairs = ne / BJ_W;
   WsCarve c(scratch);
   float* Af = c.take<float>((size_t)ne * ne);
@@ -1508,6 +1535,7 @@ fpca_status launch_dense_eig(fpca_ctx* ctx, int n, double* A, double* V, void* s
   double* S = c.take<double>(nn);
   double* lam = c.take<double>(n);
   int* flag = c.take<int>(rotate_ints(n));
+  int* wanted = c.take<int>(n);
   double* E = U;  // U is dead once S is formed
   float* emax = reinterpret_cast<float*>(done + 8);
   const int eb = (int)std::min<long long>(((long long)ne * ne + 255) / 256, 4096);
@@ -1529,38 +1557,47 @@ fpca_status launch_dense_eig(fpca_ctx* ctx, int n, double* A, double* V, void* s
   k_bj_extract<<<xb, 256, 0, ctx->stream>>>(n, ne, Vf, A, X, As);
   FPCA_LAUNCHED(ctx, "eig_bj_extract");
   const int tpb = std::min(1024, ((n + 31) / 32) * 32);
-  for (int step = 0; step < 3; ++step) {
-    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, X, R, 1.0, -1.0);   // R = I - X'X
+  // three steps, and up to two more while a wanted vector's correction is not small (each step
+  // squares the error; a relative gap of 1e-2 needs a fourth)
+  cudaMemsetAsync(emax, 0, sizeof(float) * OA_STEPS, ctx->stream);
+  for (int step = 0; step < OA_STEPS; ++step) {
+    const float* gate = step < 3 ? nullptr : emax + step - 1;
+    float* em = step < 2 ? nullptr : emax + step;
+    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, X, R, 1.0, -1.0, gate);   // R = I - X'X
     FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
-    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, As, 0, X, U, 0.0, 1.0);   // U = A X
+    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, As, 0, X, U, 0.0, 1.0, gate);   // U = A X
     FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
-    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, U, S, 0.0, 1.0);    // S = X' A X
+    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, U, S, 0.0, 1.0, gate);    // S = X' A X
     FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
     double* acc = mass + 2 * BJ_SWEEPS + 1;
     cudaMemsetAsync(acc, 0, sizeof(double) * 3, ctx->stream);
-    cudaMemsetAsync(emax, 0, sizeof(float), ctx->stream);
-    k_oa_norms<<<n, 256, 0, ctx->stream>>>(n, As, R, S, lam, acc);
+    k_oa_norms<<<n, 256, 0, ctx->stream>>>(n, As, R, S, lam, acc, gate);
     FPCA_LAUNCHED(ctx, "eig_oa_norms");
-    k_oa_correction<<<n, 256, 0, ctx->stream>>>(n, R, S, lam, acc, E, emax);
+    if (em) {
+      k_oa_wanted<<<(n + 7) / 8, 256, 0, ctx->stream>>>(n, k, lam, wanted, gate);
+      FPCA_LAUNCHED(ctx, "eig_oa_wanted");
+    }
+    k_oa_correction<<<n, 256, 0, ctx->stream>>>(n, R, S, lam, acc, E, wanted, em, gate);
     FPCA_LAUNCHED(ctx, "eig_oa_correction");
-    k_oa_update<<<n, tpb, sizeof(double) * n, ctx->stream>>>(n, X, E);
+    k_oa_update<<<n, tpb, sizeof(double) * n, ctx->stream>>>(n, X, E, gate);
     FPCA_LAUNCHED(ctx, "eig_oa_update");
   }
-  // eigenvalues closer than the couplings that the FP32 sweeps left: X made orthonormal again
+  const float* bad = emax + OA_STEPS - 1;  // zero where the last step was not taken
+  // wanted eigenvalues closer than the couplings that the FP32 sweeps left: X made orthonormal again
   // (Newton-Schulz steps X <- X + X (I - X'X) / 2, from the 0.1 or so that corrections beyond
   // their first order leave), S anew and FP64 Jacobi; nothing happens where the last step's
   // corrections were small
   for (int step = 0; step < 5; ++step) {
-    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, X, R, 0.5, -0.5, emax);
+    k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, X, R, 0.5, -0.5, bad);
     FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
-    k_oa_update<<<n, tpb, sizeof(double) * n, ctx->stream>>>(n, X, R, emax);
+    k_oa_update<<<n, tpb, sizeof(double) * n, ctx->stream>>>(n, X, R, bad);
     FPCA_LAUNCHED(ctx, "eig_oa_update");
   }
-  k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, As, 0, X, U, 0.0, 1.0, emax);
+  k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, As, 0, X, U, 0.0, 1.0, bad);
   FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
-  k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, U, S, 0.0, 1.0, emax);
+  k_oa_rowmm<<<n, tpb, 0, ctx->stream>>>(n, X, 1, U, S, 0.0, 1.0, bad);
   FPCA_LAUNCHED(ctx, "eig_oa_rowmm");
-  fpca_status cr = launch_rotate(ctx, n, emax, OA_BAD, S, lam, X, R, U, mass, flag);
+  fpca_status cr = launch_rotate(ctx, n, bad, OA_BAD, S, lam, X, R, U, mass, flag);
   if (cr != FPCA_OK) return cr;
   k_rr_out<<<xb, 256, 0, ctx->stream>>>(n, lam, X, A, V);
   FPCA_LAUNCHED(ctx, "eig_out");
@@ -1691,7 +1728,7 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
     } else {
       return fpca_fail(ctx, FPCA_E_UNSUPPORTED, "dense eigensolver needs FP64 gamma");
     }
-    fpca_status ds = launch_dense_eig(ctx, P, A, V, dense);
+    fpca_status ds = launch_dense_eig(ctx, P, k, A, V, dense);
     if (ds != FPCA_OK) return ds;
     k_eig_order<<<1, 1024, 0, ctx->stream>>>(P, A, order);
     FPCA_LAUNCHED(ctx, "eig_order");
