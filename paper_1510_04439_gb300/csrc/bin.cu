@@ -327,29 +327,36 @@ __global__ void __launch_bounds__(CD_T * CD_T)
 // Covariance bins of scattered data, row by row.  The observations are grouped by
 // (fold, bin): one row of the output arrays holds exactly the pairs whose first
 // observation lies in that bin, so a CTA sums a row in shared memory and writes every
-// entry once.
+// entry once.  Rows of more than `chunk` observations are cut into chunks, a CTA each, which
+// add their sums to the cleared row.
 // ---------------------------------------------------------------------------
 struct ObsRec {
   double r;        // response (residual or raw)
   int32_t lo, ni;  // first observation and observation count of its subject
 };
+// Chunk of a long row: its row and place there (1, 2, ...; a row's first chunk is not listed).
+struct RowChunk {
+  int32_t row, place;
+};
 
 constexpr int OBS_LANES = 8;  // threads per subject
 
-// Per observation: its bin, its record, its row (fold * P + bin; -1 where the subject has
-// no pairs or is skipped) and the rows' observation counts.  Offsets outside
-// 0 <= offs[i] <= offs[i+1] <= N and folds outside 0..nfold-1 are reported (DERR_BOUNDS)
-// and the subject is skipped.  row is set to -1 by the caller.
+// Per observation: its bin, its record, its weight and its row (fold * P + bin; -1 where the
+// subject has no pairs or is skipped).  Offsets outside 0 <= offs[i] <= offs[i+1] <= N and folds
+// outside 0..nfold-1 are reported (DERR_BOUNDS) and the subject is skipped.  row is set to -1 by
+// the caller.
 // A skipped subject's neighbours can overlap (offsets 0, 10, 5, 12: the first and the third
 // both hold observations 5..9).  An observation goes to the subject that claims its row first,
-// and only that one writes the record and counts it: the counts add up to at most N and equal
-// what k_row_fill places, and a record's lo and ni are one checked subject's.
+// and only that one writes the record, so that its lo and ni are one checked subject's; it is
+// counted and listed by its row, once.  With `rank` the rows are counted here, each observation
+// taking its rank in its row; else by k_row_count.
 __global__ void k_obs_rows(int n, long long N, int d, int m0, int m1, int m2, int P,
                            const int64_t* __restrict__ offs, const double* __restrict__ t,
                            const double* __restrict__ y, const double* __restrict__ mu, int mode,
                            const int32_t* __restrict__ fold, int nfold, int32_t* __restrict__ ob,
-                           ObsRec* __restrict__ rec, int32_t* __restrict__ row,
-                           int32_t* __restrict__ rowcount, int* __restrict__ err) {
+                           ObsRec* __restrict__ rec, double* __restrict__ wt,
+                           int32_t* __restrict__ row, int32_t* __restrict__ rowcount,
+                           int32_t* __restrict__ rank, int* __restrict__ err) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const int i = (int)(g / OBS_LANES), part = (int)(g % OBS_LANES);
   if (i >= n) return;
@@ -368,21 +375,51 @@ __global__ void k_obs_rows(int n, long long N, int d, int m0, int m1, int m2, in
     }
   }
   const int m[3] = {m0, m1, m2};
+  const double wi = 1.0 / ((double)(hi - lo) * (double)(hi - lo - 1));
   for (int64_t j = lo + part; j < hi; j += OBS_LANES) {
     const int b = bin_index(t + j * d, d, m);
     if (atomicCAS(row + j, -1, f * P + b) != -1) continue;  // another subject's (see above)
     ob[j] = b;
     rec[j] = ObsRec{mode == FPCA_COV_RESIDUAL ? y[j] - mu[b] : y[j], (int32_t)lo,
                     (int32_t)(hi - lo)};
-    atomicAdd(rowcount + f * P + b, 1);
+    wt[j] = wi;
+    if (rank) rank[j] = atomicAdd(rowcount + f * P + b, 1);
   }
 }
 
+// The observation counts of few, long rows and each observation's rank in its row, counted in
+// shared memory first: one atomic per block and row, where 250 000 on 64 counters took 60 us.
+constexpr int RC_NT = 1024, RC_PER = 4, RC_ROWS = 1024;
+__global__ void __launch_bounds__(RC_NT)
+    k_row_count(long long N, int rows, const int32_t* __restrict__ row,
+                int32_t* __restrict__ rowcount, int32_t* __restrict__ rank) {
+  __shared__ int32_t hist[RC_ROWS];
+  const long long j0 = blockIdx.x * (long long)(RC_NT * RC_PER) + threadIdx.x;
+  int32_t r[RC_PER], k[RC_PER];
+#pragma unroll
+  for (int u = 0; u < RC_PER; ++u) {
+    const long long j = j0 + u * RC_NT;
+    r[u] = j < N ? row[j] : -1;
+  }
+  for (int e = threadIdx.x; e < rows; e += RC_NT) hist[e] = 0;
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < RC_PER; ++u) k[u] = r[u] >= 0 ? atomicAdd(hist + r[u], 1) : 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < rows; e += RC_NT)
+    if (hist[e] > 0) hist[e] = atomicAdd(rowcount + e, hist[e]);
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < RC_PER; ++u)
+    if (r[u] >= 0) rank[j0 + u * RC_NT] = hist[r[u]] + k[u];
+}
+
 // Each row's place in the list of observations: the rows take consecutive runs in no
-// particular order (one atomic per warp), so no scan is needed.
-__global__ void k_row_starts(int rows, const int32_t* __restrict__ rowcount,
-                             int32_t* __restrict__ start, int32_t* __restrict__ cursor,
-                             int32_t* __restrict__ total) {
+// particular order (one atomic per warp), so no scan is needed.  Rows longer than `chunk` list
+// their further chunks: at most N / chunk in all.
+__global__ void k_row_starts(int rows, int chunk, const int32_t* __restrict__ rowcount,
+                             int32_t* __restrict__ start, int32_t* __restrict__ total,
+                             int32_t* __restrict__ nextra, RowChunk* __restrict__ extra) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   const int c = r < rows ? rowcount[r] : 0;
   int incl = c;
@@ -394,56 +431,114 @@ __global__ void k_row_starts(int rows, const int32_t* __restrict__ rowcount,
   int base = 0;
   if (lane == 31) base = atomicAdd(total, incl);
   base = __shfl_sync(0xffffffffu, base, 31);
-  if (r < rows) {
-    start[r] = base + incl - c;
-    cursor[r] = base + incl - c;
+  if (r < rows) start[r] = base + incl - c;
+  if (c > chunk) {
+    const int more = (c - 1) / chunk, at = atomicAdd(nextra, more);
+    for (int k = 0; k < more; ++k) extra[at + k] = RowChunk{r, k + 1};
   }
 }
 
-__global__ void k_row_fill(long long N, const int32_t* __restrict__ row,
-                           int32_t* __restrict__ cursor, int32_t* __restrict__ list) {
+// The lists, and (blocks from `fill` on, one per further chunk) zeros in the rows that are summed
+// in chunks; es: bytes of an entry of w, v and q.
+__global__ void k_row_fill(long long N, int fill, const int32_t* __restrict__ row,
+                           const int32_t* __restrict__ start, const int32_t* __restrict__ rank,
+                           int32_t* __restrict__ list, int P, int es, const int32_t* __restrict__ nextra, const RowChunk* __restrict__ extra,
+                           int32_t* __restrict__ cnt, void* __restrict__ w, void* __restrict__ v,
+                           void* __restrict__ q) {
+  if ((int)blockIdx.x >= fill) {
+    const int x = blockIdx.x - fill;
+    if (x >= *nextra || extra[x].place != 1) return;
+    const size_t o = (size_t)extra[x].row * P;
+    void* const dst[3] = {w, v, q};
+    for (int e = threadIdx.x; e < P; e += blockDim.x) cnt[o + e] = 0;
+    for (void* d : dst) {
+      if (!d) continue;
+      uint32_t* out = reinterpret_cast<uint32_t*>(static_cast<char*>(d) + o * es);
+      for (int e = threadIdx.x; e < P * (es / 4); e += blockDim.x) out[e] = 0u;
+    }
+    return;
+  }
   const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (j >= N || row[j] < 0) return;
-  list[atomicAdd(cursor + row[j], 1)] = (int32_t)j;
+  list[start[row[j]] + rank[j]] = (int32_t)j;
 }
 
-// One output row (blockIdx.x = fold * P + bin), columns [blockIdx.y * PC, + PC): each warp
-// takes an observation j of the row at a time, its lanes the other observations of j's
-// subject; terms as w_i, w_i r r', w_i (r r')^2 in FP64, rounded to T and added in shared
-// memory.  The finished row goes out by one bulk copy per array (or plain stores where
-// a row does not start on 16 bytes).
-// What bounds it is the write of the F x P x P arrays: 20 000 subjects of 5..20
-// observations on 64 x 64 bins, 5 folds (1.34 GB, 0.2 ms at 6.8 TB/s) take 0.38 ms for
-// the whole call.  The scatter it replaces took 0.74 ms: it cleared the arrays and added
-// each pair's four terms by global atomics, on lines already gone from L2.
+// One chunk of an output row (blockIdx.x < rows: the first chunk of row fold * P + bin, else an
+// entry of `extra`), columns [blockIdx.y * PC, + PC): each warp takes up to 32 observations of the
+// row at a time (fewer where the chunk would not give every warp some) and its lanes the pairs of
+// all of them with the other observations of their subjects; terms as w_i, w_i r r', w_i (r r')^2
+// in FP64, rounded to T and added in shared memory.  A row of one chunk goes out by
+// one bulk copy per array (or plain stores where a row does not start on 16 bytes); chunks of a
+// longer one add what is not zero to the cleared row.
+// Large outputs are bound by their write: 20 000 subjects of 5..20 observations on 64 x 64
+// bins, 5 folds (1.34 GB, 0.2 ms at 6.8 TB/s) take 0.34 ms for the whole call.  A scatter by global
+// atomics took 0.74 ms: it cleared the arrays and added each pair's four terms on lines already
+// gone from L2.  Small ones are bound by the FP64 terms (two results a clock and SM), so no lane
+// without a pair, and the weight's division once a subject: on 24 x 24 bins 0.28 ms with an
+// observation a warp and a division each, 0.11 now (the scatter: 0.12).
+// One CTA a row left SMs idle where rows are few, and one SM with a row that holds much of the
+// data: 64 bins without folds 0.82 ms, 0.10 now (the scatter: 0.21); half of all observations in
+// one bin of 64 x 64 7.5 ms, 0.57 now (the scatter: 1.0).
 constexpr int CSR_NT = 256;
+constexpr int CSR_CHUNK = 256;   // observations per chunk, at least: 32 a warp
 template <typename T>
 __global__ void __launch_bounds__(CSR_NT)
-    k_cov_rows(int P, int PC, const int32_t* __restrict__ rowcount,
+    k_cov_rows(int rows, int P, int PC, int chunk, const int32_t* __restrict__ rowcount,
                const int32_t* __restrict__ start, const int32_t* __restrict__ list,
                const int32_t* __restrict__ ob, const ObsRec* __restrict__ rec,
-               int32_t* __restrict__ cnt, T* __restrict__ w, T* __restrict__ v, T* __restrict__ q,
-               int bulk) {
+               const double* __restrict__ wt, const int32_t* __restrict__ nextra,
+               const RowChunk* __restrict__ extra, int32_t* __restrict__ cnt, T* __restrict__ w,
+               T* __restrict__ v, T* __restrict__ q, int bulk) {
   extern __shared__ __align__(128) unsigned char csr_sm[];
   T* sw = reinterpret_cast<T*>(csr_sm);  // [PC] each, PC a multiple of 4
   T* sv = sw + PC;
   T* sq = sv + PC;
   int32_t* sc = reinterpret_cast<int32_t*>(q ? sq + PC : sq);
-  const int r = blockIdx.x, c0 = blockIdx.y * PC, nc = min(PC, P - c0);
+  int r = blockIdx.x, first = 0;
+  if (r >= rows) {
+    const int x = r - rows;
+    if (x >= *nextra) return;
+    r = extra[x].row;
+    first = extra[x].place * chunk;
+  }
+  const int c0 = blockIdx.y * PC, nc = min(PC, P - c0);
   const int words = ((q ? 3 : 2) * (int)sizeof(T) + 4) * PC / 16;
   for (int e = threadIdx.x; e < words; e += CSR_NT)
     reinterpret_cast<int4*>(csr_sm)[e] = make_int4(0, 0, 0, 0);
-  const int n = rowcount[r], lane = threadIdx.x & 31;
+  constexpr int NW = CSR_NT / 32;
+  const int all = rowcount[r], last = first + min(chunk, all - first);
+  const int lane = threadIdx.x & 31, take = min(32, (last - first + NW - 1) / NW);
   const int32_t* lst = list + start[r];
   __syncthreads();
-  for (int e = threadIdx.x >> 5; e < n; e += CSR_NT / 32) {
-    const int j = lst[e];
-    const ObsRec o = rec[j];
-    const double wi = 1.0 / ((double)o.ni * (double)(o.ni - 1));
-    for (int k = lane; k < o.ni; k += 32) {
-      const int l = o.lo + k, c = ob[l] - c0;
-      if (l == j || c < 0 || c >= nc) continue;
-      const double prod = o.r * rec[l].r;
+  for (int b = first + (int)(threadIdx.x >> 5) * take; b < last; b += NW * take) {
+    int j = -1, lo = 0, ni = 0;
+    double rj = 0.0, wj = 0.0;
+    if (lane < take && b + lane < last) {
+      j = lst[b + lane];
+      const ObsRec o = rec[j];
+      rj = o.r, lo = o.lo, ni = o.ni;
+      wj = wt[j];
+    }
+    int end = ni;  // of the lane's pairs among the warp's
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, end, o);
+      if (lane >= o) end += x;
+    }
+    const int total = __shfl_sync(0xffffffffu, end, 31);
+    for (int p0 = 0; p0 < total; p0 += 32) {
+      const int p = p0 + lane;
+      int i = 0;  // pair p's observation: as many as end at or before p
+#pragma unroll
+      for (int step = 16; step > 0; step >>= 1)
+        if (__shfl_sync(0xffffffffu, end, i + step - 1) <= p) i += step;
+      const int l = __shfl_sync(0xffffffffu, lo + ni - end, i) + p;
+      const int self = __shfl_sync(0xffffffffu, j, i);
+      const double ri = __shfl_sync(0xffffffffu, rj, i), wi = __shfl_sync(0xffffffffu, wj, i);
+      if (p >= total || l == self) continue;
+      const int c = ob[l] - c0;
+      if (c < 0 || c >= nc) continue;
+      const double prod = ri * rec[l].r;
       atomicAdd(sc + c, 1);
       atomicAdd(sw + c, (T)wi);
       atomicAdd(sv + c, (T)(wi * prod));
@@ -451,6 +546,17 @@ __global__ void __launch_bounds__(CSR_NT)
     }
   }
   const size_t o = (size_t)r * P + c0;
+  if (all > chunk) {
+    __syncthreads();
+    for (int c = threadIdx.x; c < nc; c += CSR_NT) {
+      if (sc[c] == 0) continue;
+      atomicAdd(cnt + o + c, sc[c]);
+      atomicAdd(w + o + c, sw[c]);
+      atomicAdd(v + o + c, sv[c]);
+      if (q) atomicAdd(q + o + c, sq[c]);
+    }
+    return;
+  }
   if (bulk) {  // every thread's sums visible to the copies, which one thread issues
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -996,43 +1102,64 @@ fpca_status launch_cov_sparse(fpca_ctx* ctx, int n, const fpca_grid* g, const in
     return fpca_fail(ctx, FPCA_E_UNSUPPORTED, "%d bins x %d folds", P, F);
   const int rows = P * F;
   const size_t N = (size_t)Nobs;
-  void* ws = fpca_workspace(ctx, WsCarve::round(4 * N) * 3 + WsCarve::round(sizeof(ObsRec) * N) +
-                                     WsCarve::round(4 * (size_t)rows) * 3 + 4096);
+  // columns per CTA: at most 64 KB (FP32) or 56 KB (FP64) of sums, so that three CTAs share
+  // an SM and one's copies out overlap the others' sums
+  const int PC = std::min(prec == FPCA_F64 ? 2048 : 4096, (P + 3) / 4 * 4);
+  const int ncol = (P + PC - 1) / PC;
+  // chunks: no row is longer than what gives every SM a dozen (fewer, and the last to start hold
+  // up the call; many more, and rows that would not need it are cleared and added)
+  const int chunk = (int)std::max<long long>(CSR_CHUNK, Nobs * ncol / (12ll * ctx->num_sms));
+  const int nx = (int)(Nobs / chunk);  // further chunks at most
+  // a launch of its own for the counts pays where a counter would take many atomics
+  const bool count = rows <= RC_ROWS && Nobs > 64ll * rows;
+  void* ws = fpca_workspace(ctx, WsCarve::round(4 * N) * 4 + WsCarve::round(sizeof(ObsRec) * N) +
+                                     WsCarve::round(sizeof(double) * N) +
+                                     WsCarve::round(sizeof(RowChunk) * (size_t)nx) +
+                                     WsCarve::round(4 * (size_t)rows) * 2 + 4096);
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
   WsCarve carve(ws);
   int32_t* ob = carve.take<int32_t>(N);
   int32_t* row = carve.take<int32_t>(N);
+  int32_t* rank = carve.take<int32_t>(N);
   int32_t* list = carve.take<int32_t>(N);
   ObsRec* rec = carve.take<ObsRec>(N);
-  int32_t* rowcount = carve.take<int32_t>((size_t)rows + 1);  // [rows]: the list's length
+  double* wt = carve.take<double>(N);
+  RowChunk* extra = carve.take<RowChunk>(nx);
+  int32_t* rowcount = carve.take<int32_t>((size_t)rows + 2);  // [rows]: the list's length
+  int32_t* nextra = rowcount + rows + 1;
   int32_t* start = carve.take<int32_t>(rows);
-  int32_t* cursor = carve.take<int32_t>(rows);
-  cudaMemsetAsync(rowcount, 0, sizeof(int32_t) * ((size_t)rows + 1), ctx->stream);
+  cudaMemsetAsync(rowcount, 0, sizeof(int32_t) * ((size_t)rows + 2), ctx->stream);
   if (Nobs > 0) {
     cudaMemsetAsync(row, 0xff, sizeof(int32_t) * N, ctx->stream);  // -1: no pairs
     k_obs_rows<<<(int)(((long long)n * OBS_LANES + 255) / 256), 256, 0, ctx->stream>>>(
         n, Nobs, g->d, g->m[0], g->d > 1 ? g->m[1] : 1, g->d > 2 ? g->m[2] : 1, P, offs, t, y, mu,
-        mode, fold, nfold, ob, rec, row, rowcount, ctx->d_err);
+        mode, fold, nfold, ob, rec, wt, row, rowcount, count ? nullptr : rank, ctx->d_err);
     FPCA_LAUNCHED(ctx, "obs_rows");
+    if (count) {
+      const long long per = RC_NT * RC_PER;
+      k_row_count<<<(int)((Nobs + per - 1) / per), RC_NT, 0, ctx->stream>>>(Nobs, rows, row,
+                                                                            rowcount, rank);
+      FPCA_LAUNCHED(ctx, "row_count");
+    }
   }
-  k_row_starts<<<(rows + 255) / 256, 256, 0, ctx->stream>>>(rows, rowcount, start, cursor,
-                                                            rowcount + rows);
+  k_row_starts<<<(rows + 255) / 256, 256, 0, ctx->stream>>>(rows, chunk, rowcount, start,
+                                                            rowcount + rows, nextra, extra);
   FPCA_LAUNCHED(ctx, "row_starts");
   if (Nobs > 0) {
-    k_row_fill<<<(int)((Nobs + 255) / 256), 256, 0, ctx->stream>>>(Nobs, row, cursor, list);
+    const int fill = (int)((Nobs + 255) / 256);
+    k_row_fill<<<fill + nx, 256, 0, ctx->stream>>>(Nobs, fill, row, start, rank, list, P,
+                                                   prec == FPCA_F64 ? 8 : 4, nextra, extra, cnt, w,
+                                                   v, q);
     FPCA_LAUNCHED(ctx, "row_fill");
   }
-  // columns per CTA: at most 64 KB (FP32) or 56 KB (FP64) of sums, so that three CTAs share
-  // an SM and one's copies out overlap the others' sums
   auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   const int bulk = (P % 4 == 0 && al16(cnt) && al16(w) && al16(v) && (!q || al16(q))) ? 1 : 0;
   auto launch = [&](auto kern, auto* pw, auto* pv, auto* pq) -> fpca_status {
-    const int cap = sizeof(*pw) == 8 ? 2048 : 4096;
-    const int PC = std::min(cap, (P + 3) / 4 * 4);
     const size_t sm = (size_t)PC * ((pq ? 3 : 2) * sizeof(*pw) + 4);
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    kern<<<dim3(rows, (P + PC - 1) / PC), CSR_NT, sm, ctx->stream>>>(
-        P, PC, rowcount, start, list, ob, rec, cnt, pw, pv, pq, bulk);
+    kern<<<dim3(rows + nx, ncol), CSR_NT, sm, ctx->stream>>>(rows, P, PC, chunk, rowcount, start,
+                                                             list, ob, rec, wt, nextra, extra, cnt,
+                                                             pw, pv, pq, bulk);
     FPCA_LAUNCHED(ctx, "cov_rows");
     return FPCA_OK;
   };
