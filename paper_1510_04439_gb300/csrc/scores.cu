@@ -352,8 +352,8 @@ __global__ void __launch_bounds__(128)
 // digits of 11 bits, which FP16 holds exactly; sums of up to PG_NODES digits are integers
 // below 2^20, which the FP32 accumulators hold exactly, so the whole product is exact but for
 // the table's rounding, 2^-54 of the bound a node.  That is closer than the float-float sums
-// wherever a subject's mean phi_l^2 is above 2^-8 of the bound; a subject with a smaller one
-// is summed again in float-float (k_pace_final).
+// wherever a subject's mean phi_l^2 is above 2^-8 of the bound; the row of a function whose mean
+// is smaller is summed in float-float (pace_rows).
 constexpr int PG_DIG = 5;        // digits
 constexpr int PG_BITS = 11;
 constexpr int PG_FIX = 53;       // fixed-point bits
@@ -536,25 +536,137 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// The table's bound does not hold for a function (exponent e) of a subject: its mean square is
+// below 2^-8 of 2^(2e).  all, nodes: the upper 32 bits of the fixed-point sums of phi_l^2 (units
+// of 2^(2e - PG_FIX)) and of the node count (2^-PG_COUNT), so that the exponents cancel.
+__device__ __forceinline__ bool pace_small(long long all, long long nodes, int e) {
+  return e > PG_EZERO && (e == PG_EBAD || all < 2 * nodes);
+}
+static_assert(PG_FIX - 8 == PG_COUNT + 1, "pace_small");
+// Place of entry (a, b), a <= b, in the upper triangle.
+__device__ __forceinline__ int pace_entry(int L, int a, int b) { return a * L - a * (a - 1) / 2 + b - a; }
+
+// The warp's sums of NV lane values each: a halving butterfly (one add a sum instead of five),
+// v[0] <- sum number `at` (returned; with NV < 32 several lanes hold the same one).
+template <int NV>
+__device__ __forceinline__ int warp_halve(ff::F2 (&v)[NV]) {
+  const int lane = threadIdx.x & 31;
+  int at = 0;
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int o = 16 >> st, left = NV >> (st + 1);
+    const bool up = lane & o;
+    if (up) at += left;
+#pragma unroll
+    for (int k = 0; k < (left > 0 ? left : 1); ++k) {
+      const ff::F2 give = up || left == 0 ? v[k] : v[k + left];
+      const ff::F2 keep = up && left > 0 ? v[k + left] : v[k];
+      v[k] = ff::add(keep, ff::F2{__shfl_xor_sync(0xffffffffu, give.hi, o),
+                                  __shfl_xor_sync(0xffffffffu, give.lo, o)});
+    }
+  }
+  return at;
+}
+
+// Rows `small` (a bit each) of one subject's Phi'Phi over a chunk's pn nodes, in float-float, by
+// one warp; out: the chunk's entries of the subject.  Each row serves all its entries, so that a
+// localised function costs L sums of the L (L + 1) / 2.
+template <int LM, int CH>
+__device__ __forceinline__ void pace_rows(unsigned small, const float2 (*ph)[CH], int pn,
+                                          const uint8_t* __restrict__ row, int L, bool clean,
+                                          float2* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  for (unsigned left = small; left; left &= left - 1) {
+    const int l = __ffs(left) - 1;
+    const unsigned done = small & ((1u << l) - 1u);  // entries of an earlier row
+    Acc acc[LM];
+#pragma unroll 2
+    for (int c = lane; c < pn; c += 32) {
+      const bool ok = !row || row[c];
+      const float2 x = ph[l][c];
+      const ff::F2 fl = ok ? ff::F2{x.x, x.y} : ff::make(0.f);
+#pragma unroll
+      for (int b = 0; b < LM; ++b) {
+        if (b < L && !(done >> b & 1)) {
+          const ff::F2 f{ph[b][c].x, ph[b][c].y};
+          acc[b].add_prod(fl, clean || ok ? f : ff::make(0.f));
+        }
+      }
+    }
+    ff::F2 v[LM];
+#pragma unroll
+    for (int b = 0; b < LM; ++b) v[b] = ff::fast_two_sum(acc[b].s, acc[b].c);
+    const int b = warp_halve<LM>(v);
+    if (b < L && !(done >> b & 1))
+      out[pace_entry(L, min(l, b), max(l, b))] = make_float2(v[0].hi, v[0].lo);
+  }
+}
+
+// All rows at once, where most are wanted: rows A0..A1 - 1 of the triangle (at most NV entries,
+// which is what the registers hold), ordered by column.
+template <int LM, int CH, int A0, int A1, int NV>
+__device__ __forceinline__ void pace_triangle(const float2 (*ph)[CH], int pn,
+                                              const uint8_t* __restrict__ row, int L, bool clean,
+                                              float2* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  if (A0 >= L) return;
+  Acc acc[NV];
+#pragma unroll 1
+  for (int c = lane; c < pn; c += 32) {
+    const bool ok = !row || row[c];
+    ff::F2 fa[A1 - A0];
+#pragma unroll
+    for (int a = A0; a < A1; ++a) fa[a - A0] = ok ? ff::F2{ph[a][c].x, ph[a][c].y} : ff::make(0.f);
+    int k = 0;
+#pragma unroll
+    for (int b = A0; b < LM; ++b) {
+      if (b < L) {
+        const ff::F2 f{ph[b][c].x, ph[b][c].y};
+#pragma unroll
+        for (int a = A0; a < A1; ++a)
+          if (a <= b) acc[k + a - A0].add_prod(fa[a - A0], clean || ok ? f : ff::make(0.f));
+      }
+      k += (b < A1 ? b + 1 : A1) - A0;
+    }
+  }
+  ff::F2 v[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = ff::fast_two_sum(acc[k].s, acc[k].c);
+  int k = warp_halve<NV>(v);
+  for (int b = A0; b < L; ++b) {
+    const int rows = (b < A1 ? b + 1 : A1) - A0;
+    if (k < rows) {
+      out[pace_entry(L, A0 + k, b)] = make_float2(v[0].hi, v[0].lo);
+      break;
+    }
+    k -= rows;
+  }
+}
+
 // Phi_i'Y_i^C over a chunk of nodes: the chunk's phi in shared memory, two subjects a warp,
 // each lane both subjects' L compensated sums over every 32nd node (a phi value read serves
-// both); the sums join by a halving butterfly of float-float adds (one add a sum instead of
-// five; FP64 adds there would take longer than the sums themselves).  blockIdx: x chunk,
-// y 16 subjects; bpart[(chunk * nb + i) * L + l].  n = 1000, P = 4096, L = 8: 38 us, bound by
-// its FP32 instructions, and 16 for the systems; n = 1500, P = 1320, L = 13: 38 and 30.  With
-// phi from L2 and a block taking two whole subjects and their systems: 53 and 131 (one warp
-// per 1/8 subject, forming Phi'Phi too: 269 and 293).
-template <int LM>
-constexpr int pd_chunk() { return LM == 8 ? 512 : 256; }
+// both); the sums join in float-float (FP64 adds there would take longer than the sums
+// themselves).  The same warp then forms the rows of its subjects' Phi'Phi that the table does
+// not hold.  n = 1000, P = 4096, whole call: L = 8 83 us, 114 with one localised function, 197 with
+// all of them; L = 13 142, 204 and 462 (all entries of such a subject one after the other, in the
+// solving block: 604 and 742; all subjects' entries in float-float, before there was a table: 280
+// and 404, which is still the better one where more than eight functions are all localised).
+// blockIdx: x chunk, y 16 subjects; bpart[(chunk * nb + i) * L + l], rpart[(chunk * nb + i) * NE +
+// entry].  This kernel, bound by its FP32 instructions, takes 38 us of the 83 and the systems 16
+// (n = 1500, P = 1320, L = 13: 38 and 30); with phi from L2 and a block taking two whole subjects
+// and their systems 53 and 131, one warp per 1/8 subject, forming Phi'Phi too, 269 and 293.
+constexpr int PD_CHUNK = 512;  // nodes (256 with 16 functions: 155 us for L = 13)
 template <int LM>
 __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
     k_pace_dots(int nb, int i0, int P, const void* __restrict__ y, int yprec,
                 const uint8_t* __restrict__ mask, const float2* __restrict__ mu2,
-                const float2* __restrict__ phi2, int L, const int* __restrict__ expo,
-                float2* __restrict__ bpart) {
-  constexpr int NV = 2 * LM, CH = pd_chunk<LM>();
-  __shared__ float2 ph[LM][CH];
-  __shared__ float2 mus[CH];
+                const float2* __restrict__ phi2, int L, const int* __restrict__ expo, int nsplit,
+                const long long* __restrict__ gsum, float2* __restrict__ bpart,
+                float2* __restrict__ rpart) {
+  constexpr int NV = 2 * LM, CH = PD_CHUNK;
+  extern __shared__ __align__(16) float2 pds[];
+  float2(*ph)[CH] = reinterpret_cast<float2(*)[CH]>(pds);
+  float2* mus = pds + LM * CH;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int p0 = blockIdx.x * CH, pn = min(CH, P - p0);
   for (int e = tid; e < LM * CH; e += 256) {
@@ -591,43 +703,63 @@ __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
 #pragma unroll
   for (int k = 0; k < NV; ++k)
     v[k] = ff::fast_two_sum(acc[k / LM][k % LM].s, acc[k / LM][k % LM].c);
-  int at = 0;  // the sum that this lane ends with
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int o = 16 >> st, left = NV >> (st + 1);
-    const bool up = lane & o;
-    if (up) at += left;
-#pragma unroll
-    for (int k = 0; k < (left > 0 ? left : 1); ++k) {
-      const ff::F2 give = up || left == 0 ? v[k] : v[k + left];
-      const ff::F2 keep = up && left > 0 ? v[k + left] : v[k];
-      v[k] = ff::add(keep, ff::F2{__shfl_xor_sync(0xffffffffu, give.hi, o),
-                                  __shfl_xor_sync(0xffffffffu, give.lo, o)});
-    }
-  }
+  const int at = warp_halve<NV>(v);
   const int sl = s0 + at / LM, l = at % LM;  // (with 16 sums two lanes hold the same one)
   if (sl < nb && l < L)
     bpart[((size_t)blockIdx.x * nb + sl) * L + l] = make_float2(v[0].hi, v[0].lo);
+  // the table's bound: lanes 0..15 the functions of subject s0, 16..31 those of the next
+  const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L), f = lane & 15, si = s0 + (lane >> 4);
+  bool small = false;
+  if (f < L && si < nb) {
+    const int e = expo[f];
+    const long long* g = gsum + (size_t)si * ng8;
+    const int ff = pace_entry(L, f, f);
+    long long all = 0, nodes = 0;
+#pragma unroll 8
+    for (int k = 0; k < nsplit; ++k, g += (size_t)nb * ng8) {
+      all += g[ff] >> 32;
+      nodes += g[NE] >> 32;
+    }
+    small = pace_small(all, nodes, e);
+  }
+  const unsigned which = __ballot_sync(0xffffffffu, small);
+  if (!which) return;
+  for (int h = 0; h < 2; ++h) {
+    const unsigned rows = which >> (16 * h) & 0xffffu;
+    const uint8_t* row = mask ? mask + (h ? row1 : row0) : nullptr;
+    float2* out = rpart + ((size_t)blockIdx.x * nb + s0 + h) * NE;
+    if (2 * __popc(rows) <= L) {
+      pace_rows<LM, CH>(rows, ph, pn, row, L, clean, out);
+    } else if constexpr (LM == 8) {
+      pace_triangle<LM, CH, 0, 2, 16>(ph, pn, row, L, clean, out);
+      pace_triangle<LM, CH, 2, 4, 16>(ph, pn, row, L, clean, out);
+      pace_triangle<LM, CH, 4, 8, 16>(ph, pn, row, L, clean, out);
+    } else {
+      pace_triangle<LM, CH, 0, 2, 32>(ph, pn, row, L, clean, out);
+      pace_triangle<LM, CH, 2, 4, 32>(ph, pn, row, L, clean, out);
+      pace_triangle<LM, CH, 4, 6, 32>(ph, pn, row, L, clean, out);
+      pace_triangle<LM, CH, 6, 9, 32>(ph, pn, row, L, clean, out);
+      pace_triangle<LM, CH, 9, 16, 32>(ph, pn, row, L, clean, out);
+    }
+  }
 }
 
-// The systems of 32 / LM subjects: the sums of the node splits and chunks, the test of the
-// table's bound (Phi'Phi again in float-float where it fails), and the solves.
+// The systems of 32 / LM subjects: the sums of the node splits and chunks (the chunks' rows where
+// the table's bound does not hold), and the solves.
 template <int LM>
 __global__ void __launch_bounds__(128)
-    k_pace_final(int nb, int i0, int P, const uint8_t* __restrict__ mask,
-                 const double* __restrict__ prior, const float2* __restrict__ phi2, int L, int nsplit,
-                 int nchunk, const int* __restrict__ expo, const long long* __restrict__ gsum,
-                 const float2* __restrict__ bpart, double* __restrict__ scores,
-                 int* __restrict__ err) {
+    k_pace_final(int nb, int i0, const double* __restrict__ prior, int L, int nsplit, int nchunk,
+                 const int* __restrict__ expo, const long long* __restrict__ gsum,
+                 const float2* __restrict__ bpart, const float2* __restrict__ rpart,
+                 double* __restrict__ scores, int* __restrict__ err) {
   constexpr int SUB = 32 / LM;
   __shared__ PaceSys sys[SUB];
-  __shared__ float2 wsum[4];
-  __shared__ double count[SUB];
-  __shared__ int redo[SUB];
+  __shared__ long long top[SUB][SC_LMAX + 1];  // upper halves of the diagonal's sums, the count's
+  __shared__ unsigned small[SUB];              // a bit per row from rpart
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L);
   const int s0 = blockIdx.x * SUB;
-  if (tid < SUB) redo[tid] = 0;
+  if (tid < SUB) small[tid] = 0;
   for (int it = tid; it < SUB * (NE + 1 + L); it += 128) {
     const int sl = it / (NE + 1 + L), e = it - sl * (NE + 1 + L);
     if (s0 + sl >= nb) continue;
@@ -649,9 +781,8 @@ __global__ void __launch_bounds__(128)
       hi += v >> 32;
       lo += v & 0xffffffffll;
     }
-    const double v = fma((double)hi, 4294967296.0, (double)lo);
     if (e == NE) {
-      count[sl] = v * pow2(-PG_COUNT);
+      top[sl][SC_LMAX] = hi;
       continue;
     }
     int a = 0, rem = e;
@@ -660,43 +791,37 @@ __global__ void __launch_bounds__(128)
       ++a;
     }
     const int b = a + rem, es = expo[a] + expo[b];
+    if (a == b) top[sl][a] = hi;
+    const double v = fma((double)hi, 4294967296.0, (double)lo);
     const double ge = es > -200 && es < 200 ? v * pow2(es - PG_FIX) : 0.0;
     sys[sl].A[a][b] = ge;
     sys[sl].A[b][a] = ge;
   }
   __syncthreads();
-  if (tid < SUB * L) {  // the bound of the table's rounding, see above
-    const int sl = tid / L, l = tid - sl * L, e = expo[l];
-    if (s0 + sl < nb && e > PG_EZERO &&
-        (e == PG_EBAD || !(sys[sl].A[l][l] >= count[sl] * pow2(2 * e - 8))))
-      redo[sl] = 1;
+  bool any = false;
+  if (tid < SUB * L) {
+    const int sl = tid / L, l = tid - sl * L;
+    any = s0 + sl < nb && pace_small(top[sl][l], top[sl][SC_LMAX], expo[l]);
+    if (any) atomicOr(&small[sl], 1u << l);
   }
-  __syncthreads();
-  for (int sl = 0; sl < SUB; ++sl) {
-    if (!redo[sl]) continue;
-    for (int a = 0; a < L; ++a) {
-      for (int b = a; b < L; ++b) {
-        Acc ac;
-        for (int p = tid; p < P; p += 128) {
-          if (mask && !mask[(long long)(i0 + s0 + sl) * P + p]) continue;
-          const float2 fa = phi2[(long long)a * P + p], fb = phi2[(long long)b * P + p];
-          ac.add_prod(ff::F2{fa.x, fa.y}, ff::F2{fb.x, fb.y});
-        }
-        ff::F2 sum = ff::fast_two_sum(ac.s, ac.c);
-        for (int o = 16; o > 0; o >>= 1)
-          sum = ff::add(sum, ff::F2{__shfl_xor_sync(0xffffffffu, sum.hi, o),
-                                    __shfl_xor_sync(0xffffffffu, sum.lo, o)});
-        if (lane == 0) wsum[warp] = make_float2(sum.hi, sum.lo);
-        __syncthreads();
-        if (tid == 0) {
-          double t = 0.0;
-          for (int w = 0; w < 4; ++w) t += (double)wsum[w].x + (double)wsum[w].y;
-          sys[sl].A[a][b] = t;
-          sys[sl].A[b][a] = t;
-        }
-        __syncthreads();
+  if (__syncthreads_or(any)) {
+    for (int it = tid; it < SUB * NE; it += 128) {
+      const int sl = it / NE, e = it - sl * NE;
+      int a = 0, rem = e;
+      while (rem >= L - a) {
+        rem -= L - a;
+        ++a;
       }
+      if (!((small[sl] >> a | small[sl] >> (a + rem)) & 1)) continue;
+      double t = 0.0;
+      for (int k = 0; k < nchunk; ++k) {
+        const float2 v = rpart[((size_t)k * nb + s0 + sl) * NE + e];
+        t += (double)v.x + (double)v.y;
+      }
+      sys[sl].A[a][a + rem] = t;
+      sys[sl].A[a + rem][a] = t;
     }
+    __syncthreads();
   }
   if (warp == 0) {
     const int sl = lane / LM;
@@ -864,7 +989,7 @@ struct ScWork {
   int* expo;           // L exponents
   uint2* table;
   long long* gsum;
-  float2* bpart;       // partial Phi'Y^C of the node chunks
+  float2 *bpart, *rpart;  // partial Phi'Y^C and rows of Phi'Phi of the node chunks
   const double* phi;
   int nbx, nsplit, per, batch, nchunk;
 };
@@ -879,8 +1004,8 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   w->per = n64 <= 64 ? 4 : 8;
   w->nsplit = (n64 + w->per - 1) / w->per;
   w->batch = std::max(128, PG_BATCH / w->nsplit / 128 * 128);
-  const int chunk = L <= 8 ? pd_chunk<8>() : pd_chunk<16>();
-  w->nchunk = (P + chunk - 1) / chunk;
+  w->nchunk = (P + PD_CHUNK - 1) / PD_CHUNK;
+  const size_t NE = (size_t)L * (L + 1) / 2;
   const size_t nt = (size_t)n64 * 4 * ng * PG_DIG * 32;
   const size_t ns = (size_t)w->nsplit * w->batch * 8 * ng;
   void* ws = fpca_workspace(ctx, WsCarve::round(sizeof(float2) * P) +
@@ -888,7 +1013,8 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
                                      WsCarve::round(sizeof(float) * L * w->nbx) + 512 +
                                      WsCarve::round(sizeof(uint2) * nt) +
                                      WsCarve::round(sizeof(long long) * ns) +
-                                     WsCarve::round(sizeof(float2) * w->nchunk * w->batch * L));
+                                     WsCarve::round(sizeof(float2) * w->nchunk * w->batch * L) +
+                                     WsCarve::round(sizeof(float2) * w->nchunk * w->batch * NE));
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
   WsCarve c(ws);
   w->mu2 = c.take<float2>(P);
@@ -899,6 +1025,7 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   w->table = c.take<uint2>(nt);
   w->gsum = c.take<long long>(ns);
   w->bpart = c.take<float2>((size_t)w->nchunk * w->batch * L);
+  w->rpart = c.take<float2>((size_t)w->nchunk * w->batch * NE);
   k_split_ff<<<dim3(w->nbx, L + 1), 256, 0, ctx->stream>>>(P, mu, evecs, w->mu2, w->phi2, w->bmax, L,
                                                                 lam, sigma2, w->prior);
   FPCA_LAUNCHED(ctx, "split_ff");
@@ -920,14 +1047,17 @@ fpca_status pace_dense(fpca_ctx* ctx, const fpca_data* data, int P, int L, const
         nb, i0, P, ng, w.per, data->mask, w.table, w.gsum, vec);
     FPCA_LAUNCHED(ctx, "pace_gram");
     auto dots = L <= 8 ? k_pace_dots<8> : k_pace_dots<16>;
-    dots<<<dim3(w.nchunk, (nb + 15) / 16), 256, 0, ctx->stream>>>(
-        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, w.phi2, L, w.expo, w.bpart);
+    const int dsm = (int)sizeof(float2) * PD_CHUNK * (L <= 8 ? 9 : 17);
+    cudaFuncSetAttribute(dots, cudaFuncAttributeMaxDynamicSharedMemorySize, dsm);
+    dots<<<dim3(w.nchunk, (nb + 15) / 16), 256, dsm, ctx->stream>>>(
+        nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, w.phi2, L, w.expo,
+        w.nsplit, w.gsum, w.bpart, w.rpart);
     FPCA_LAUNCHED(ctx, "pace_dots");
     auto fin = L <= 8 ? k_pace_final<8> : k_pace_final<16>;
     const int sub = L <= 8 ? 4 : 2;
-    fin<<<(nb + sub - 1) / sub, 128, 0, ctx->stream>>>(nb, i0, P, data->mask, w.prior, w.phi2, L,
-                                                      w.nsplit, w.nchunk, w.expo, w.gsum, w.bpart,
-                                                      scores, ctx->d_err);
+    fin<<<(nb + sub - 1) / sub, 128, 0, ctx->stream>>>(nb, i0, w.prior, L, w.nsplit, w.nchunk,
+                                                      w.expo, w.gsum, w.bpart, w.rpart, scores,
+                                                      ctx->d_err);
     FPCA_LAUNCHED(ctx, "scores_pace");
   }
   return FPCA_OK;
