@@ -77,8 +77,8 @@ __device__ __forceinline__ ff::F2 centred(const void* y, int yprec, long long e,
                            : centred(static_cast<const float*>(y)[e], m);
 }
 
-// mu (row 0) and the first L eigenfunctions (rows 1..L) as float-float; bmax (L x gridDim.x):
-// each block's largest |phi_l|, rounded up, infinity if one is not finite.  For PACE (lam not
+// mu (row 0) and the first L eigenfunctions (rows 1..L) as float-float; bmax (L x gridDim.x, or
+// NULL): each block's largest |phi_l|, rounded up, infinity if one is not finite.  For PACE (lam not
 // NULL) prior[l] = sigma^2 / lambda_l, and prior[SC_LMAX] = 1 if sigma^2 >= 0 and every
 // lambda > 0, else 0 (an FP64 division in every block of the later kernels took 3 us there).
 __global__ void __launch_bounds__(256)
@@ -98,13 +98,13 @@ __global__ void __launch_bounds__(256)
   const double* in = l < 0 ? mu : phi + (long long)l * P;
   float2* out = l < 0 ? mu2 : phi2 + (long long)l * P;
   float top = 0.f;
-  for (int e = blockIdx.x * 256 + threadIdx.x; e < P; e += gridDim.x * 256) {
+  for (long long e = blockIdx.x * 256 + threadIdx.x; e < P; e += gridDim.x * 256) {
     const ff::F2 v = split(in[e]);
     out[e] = make_float2(v.hi, v.lo);
     const float a = __double2float_ru(fabs(in[e]));
     top = isfinite(a) ? fmaxf(top, a) : INFINITY;
   }
-  if (l < 0) return;
+  if (l < 0 || !bmax) return;
   for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = top;
   __syncthreads();
@@ -977,15 +977,14 @@ bool sc_valid(fpca_ctx* ctx, const fpca_grid* g, int L) {
   return true;
 }
 
-// Gridded data in batches: the scratch of fpca_scores_pace does not grow with n, and the
-// other two calls ask for the same, so which of them ran first makes no difference to a
-// graph capture.
+// Gridded data in batches: the scratch of fpca_scores_pace does not grow with n.
 constexpr int PG_BATCH = 16384;  // subjects x splits
 
 struct ScWork {
   float2 *mu2, *phi2;  // mu (P) and the first L eigenfunctions (L x P) as float-float
-  float* bmax;         // L x nbx block maxima of |phi|
   double* prior;       // see k_split_ff
+  // PACE of gridded data
+  float* bmax;         // L x nbx block maxima of |phi|
   int* expo;           // L exponents
   uint2* table;
   long long* gsum;
@@ -994,38 +993,43 @@ struct ScWork {
   int nbx, nsplit, per, batch, nchunk;
 };
 
+// mu and phi in float-float; with `grid` also what PACE of gridded data works with.  The other
+// calls take none of that: at 2^20 nodes and L = 16 it is 2.4 GB beside their 0.14.
 fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double* evecs, ScWork* w,
-                     const double* lam = nullptr, const double* sigma2 = nullptr) {
+                     const double* lam = nullptr, const double* sigma2 = nullptr, bool grid = false) {
   const int n64 = (P + 63) / 64, ng = pg_groups(L);
+  *w = ScWork{};
   w->phi = evecs;
-  w->nbx = std::min((P + 255) / 256, 64);
+  w->nbx = std::min((P + 255) / 256, grid ? 64 : 4096);
   // 256 nodes a split, 512 on grids that make plenty of them: digit sums stay below 2^20,
   // fixed-point sums below 2^63
   w->per = n64 <= 64 ? 4 : 8;
   w->nsplit = (n64 + w->per - 1) / w->per;
   w->batch = std::max(128, PG_BATCH / w->nsplit / 128 * 128);
   w->nchunk = (P + PD_CHUNK - 1) / PD_CHUNK;
-  const size_t NE = (size_t)L * (L + 1) / 2;
   const size_t nt = (size_t)n64 * 4 * ng * PG_DIG * 32;
   const size_t ns = (size_t)w->nsplit * w->batch * 8 * ng;
-  void* ws = fpca_workspace(ctx, WsCarve::round(sizeof(float2) * P) +
-                                     WsCarve::round(sizeof(float2) * (size_t)L * P) +
-                                     WsCarve::round(sizeof(float) * L * w->nbx) + 512 +
-                                     WsCarve::round(sizeof(uint2) * nt) +
-                                     WsCarve::round(sizeof(long long) * ns) +
-                                     WsCarve::round(sizeof(float2) * w->nchunk * w->batch * L) +
-                                     WsCarve::round(sizeof(float2) * w->nchunk * w->batch * NE));
-  if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
+  const size_t nc = (size_t)w->nchunk * w->batch;
+  const size_t nr = (size_t)L * (L + 1) / 2;
+  size_t need = WsCarve::round(sizeof(float2) * P) + WsCarve::round(sizeof(float2) * (size_t)L * P) + 512;
+  if (grid)
+    need += WsCarve::round(sizeof(float) * L * w->nbx) + 512 + WsCarve::round(sizeof(uint2) * nt) +
+            WsCarve::round(sizeof(long long) * ns) + WsCarve::round(sizeof(float2) * nc * L) +
+            WsCarve::round(sizeof(float2) * nc * nr);
+  void* ws = fpca_workspace(ctx, need);
+  if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace (%zu bytes)", need);
   WsCarve c(ws);
   w->mu2 = c.take<float2>(P);
   w->phi2 = c.take<float2>((size_t)L * P);
-  w->bmax = c.take<float>((size_t)L * w->nbx);
-  w->expo = c.take<int>(SC_LMAX);
   w->prior = c.take<double>(SC_LMAX + 1);
-  w->table = c.take<uint2>(nt);
-  w->gsum = c.take<long long>(ns);
-  w->bpart = c.take<float2>((size_t)w->nchunk * w->batch * L);
-  w->rpart = c.take<float2>((size_t)w->nchunk * w->batch * NE);
+  if (grid) {
+    w->bmax = c.take<float>((size_t)L * w->nbx);
+    w->expo = c.take<int>(SC_LMAX);
+    w->table = c.take<uint2>(nt);
+    w->gsum = c.take<long long>(ns);
+    w->bpart = c.take<float2>(nc * L);
+    w->rpart = c.take<float2>(nc * nr);
+  }
   k_split_ff<<<dim3(w->nbx, L + 1), 256, 0, ctx->stream>>>(P, mu, evecs, w->mu2, w->phi2, w->bmax, L,
                                                                 lam, sigma2, w->prior);
   FPCA_LAUNCHED(ctx, "split_ff");
@@ -1081,7 +1085,7 @@ fpca_status fpca_scores_pace(fpca_ctx* ctx, const fpca_data* data, const fpca_gr
     return fpca_fail(ctx, FPCA_E_INVALID_ARG, "scattered data need offs and t");
   const ScGrid g = sc_grid(grid);
   ScWork w;
-  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w, evals, sigma2);
+  fpca_status s = sc_split(ctx, g.P, L, mu, evecs, &w, evals, sigma2, data->layout != FPCA_SPARSE);
   if (s != FPCA_OK) return s;
   if (data->layout == FPCA_SPARSE) {
     auto kern = L <= 8 ? k_scores_pace<8> : k_scores_pace<16>;
