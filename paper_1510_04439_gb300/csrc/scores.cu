@@ -366,15 +366,16 @@ __host__ __device__ constexpr int pg_groups(int L) { return L * (L + 1) / 2 / 8 
 // The table in the order in which the product's B fragments are read: 64 nodes are four
 // steps of 16; lane 4g + t of step j holds column g of the 8 and nodes 16 t + 4 j + {0..3},
 // so that a lane's four steps of mask bytes are 16 consecutive ones.  Columns NE: a one
-// (the subject's node count), beyond: zeros.  A block makes 64 nodes' worth.
+// (the subject's node count), beyond: zeros.  A block makes 64 nodes' worth, of the 64s from
+// `first` on.
 __global__ void __launch_bounds__(256)
-    k_pace_table(int P, int L, int nbx, const float* __restrict__ bmax,
+    k_pace_table(int P, int first, int L, int nbx, const float* __restrict__ bmax,
                  const double* __restrict__ phi, uint2* __restrict__ table,
                  int* __restrict__ expo) {
   __shared__ double ph[SC_LMAX][64];
   __shared__ int ex[SC_LMAX];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int NE = L * (L + 1) / 2, ng = pg_groups(L), p0 = blockIdx.x * 64;
+  const int NE = L * (L + 1) / 2, ng = pg_groups(L), p0 = (first + blockIdx.x) * 64;
   for (int l = warp; l < L; l += 8) {
     float top = 0.f;
     for (int b = lane; b < nbx; b += 32) top = fmaxf(top, bmax[(long long)l * nbx + b]);
@@ -464,26 +465,27 @@ __device__ __forceinline__ uint4 mask16(const uint8_t* __restrict__ row, int p, 
 
 // out[(split * nb + i) * 8 ng + e]: the fixed-point sums over the split's nodes.  A warp takes
 // 16 subjects (its A fragments come straight from the mask's bytes) and GP groups of 8
-// columns; blockIdx: x 128 subjects, y a split of `per` x 64 nodes, z GP groups.  1.5 GFLOP
+// columns; blockIdx: x 128 subjects, y a split of `per` x 64 nodes, from the 64s `first` on, of
+// which the table holds `have`, z GP groups.  1.5 GFLOP
 // at n = 1000, P = 4096, L = 8 in 10 us: bound by the table's reads from L1/L2, so the simpler
 // warp-level products are as good as tcgen05's here.
 template <int GP>
 __global__ void __launch_bounds__(256)
-    k_pace_gram(int nb, int i0, int P, int ng, int per, const uint8_t* __restrict__ mask,
-                const uint2* __restrict__ table, long long* __restrict__ out, int vec) {
+    k_pace_gram(int nb, int i0, int P, int first, int have, int ng, int per,
+                const uint8_t* __restrict__ mask, const uint2* __restrict__ table, long long* __restrict__ out, int vec) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gr = lane >> 2, t = lane & 3;
   const int ra = blockIdx.x * 128 + warp * 16 + gr, rb = ra + 8;
   if (ra - gr >= nb) return;
   const int g0 = blockIdx.z * GP, gn = min(GP, ng - g0);
-  const int n64 = (P + 63) / 64, k0 = blockIdx.y * per, k1 = min(n64, k0 + per);
+  const int k0 = first + blockIdx.y * per, k1 = min(first + have, k0 + per);
   float acc[GP][PG_DIG][4] = {};
   const bool oka = ra < nb, okb = rb < nb;
   const uint8_t* rowa = mask ? mask + (size_t)(i0 + (oka ? ra : 0)) * P : nullptr;
   const uint8_t* rowb = mask ? mask + (size_t)(i0 + (okb ? rb : 0)) * P : nullptr;
   // the fragments of the next 16 nodes are loaded while these are multiplied (the loads took
   // 0.95 of the time when each was waited for)
-  const uint2* tb = table + ((size_t)k0 * 4 * ng + g0) * PG_DIG * 32 + lane;
+  const uint2* tb = table + ((size_t)(k0 - first) * 4 * ng + g0) * PG_DIG * 32 + lane;
   const size_t tstep = (size_t)ng * PG_DIG * 32;
   uint2 b[2][GP * PG_DIG];
   auto fetch = [&](uint2 (&f)[GP * PG_DIG]) {
@@ -602,6 +604,29 @@ __device__ __forceinline__ void pace_rows(unsigned small, const float2 (*ph)[CH]
   }
 }
 
+// which[i]: the functions of subject i that the table does not hold, a bit each; a warp a subject.
+// On grids of many splits, where k_pace_dots does not go through all of them in every block.
+__global__ void __launch_bounds__(256)
+    k_pace_check(int nb, int L, int nsplit, const int* __restrict__ expo,
+                 const long long* __restrict__ gsum, unsigned* __restrict__ which) {
+  const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (s >= nb) return;
+  const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L);
+  long long nodes = 0;
+  unsigned bits = 0;
+  for (int f = -1; f < L; ++f) {
+    const long long* g = gsum + (size_t)s * ng8 + (f < 0 ? NE : pace_entry(L, f, f));
+    long long all = 0;
+    for (int k = lane; k < nsplit; k += 32) all += g[(size_t)k * nb * ng8] >> 32;
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+    if (f < 0)
+      nodes = all;
+    else if (pace_small(all, nodes, expo[f]))
+      bits |= 1u << f;
+  }
+  if (lane == 0) which[s] = bits;
+}
+
 // All rows at once, where most are wanted: rows A0..A1 - 1 of the triangle (at most NV entries,
 // which is what the registers hold), ordered by column.
 template <int LM, int CH, int A0, int A1, int NV>
@@ -661,8 +686,8 @@ __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
     k_pace_dots(int nb, int i0, int P, const void* __restrict__ y, int yprec,
                 const uint8_t* __restrict__ mask, const float2* __restrict__ mu2,
                 const float2* __restrict__ phi2, int L, const int* __restrict__ expo, int nsplit,
-                const long long* __restrict__ gsum, float2* __restrict__ bpart,
-                float2* __restrict__ rpart) {
+                const long long* __restrict__ gsum, const unsigned* __restrict__ checked,
+                float2* __restrict__ bpart, float2* __restrict__ rpart) {
   constexpr int NV = 2 * LM, CH = PD_CHUNK;
   extern __shared__ __align__(16) float2 pds[];
   float2(*ph)[CH] = reinterpret_cast<float2(*)[CH]>(pds);
@@ -707,10 +732,13 @@ __global__ void __launch_bounds__(256, LM == 8 ? 4 : 2)
   const int sl = s0 + at / LM, l = at % LM;  // (with 16 sums two lanes hold the same one)
   if (sl < nb && l < L)
     bpart[((size_t)blockIdx.x * nb + sl) * L + l] = make_float2(v[0].hi, v[0].lo);
-  // the table's bound: lanes 0..15 the functions of subject s0, 16..31 those of the next
+  // the table's bound: lanes 0..15 the functions of subject s0, 16..31 those of the next (from
+  // k_pace_check where it ran)
   const int NE = L * (L + 1) / 2, ng8 = 8 * pg_groups(L), f = lane & 15, si = s0 + (lane >> 4);
   bool small = false;
-  if (f < L && si < nb) {
+  if (f < L && si < nb && checked) {
+    small = checked[si] >> f & 1;
+  } else if (f < L && si < nb) {
     const int e = expo[f];
     const long long* g = gsum + (size_t)si * ng8;
     const int ff = pace_entry(L, f, f);
@@ -977,8 +1005,15 @@ bool sc_valid(fpca_ctx* ctx, const fpca_grid* g, int L) {
   return true;
 }
 
-// Gridded data in batches: the scratch of fpca_scores_pace does not grow with n.
-constexpr int PG_BATCH = 16384;  // subjects x splits
+// Gridded data in batches of subjects and slabs of nodes: the scratch of fpca_scores_pace does
+// not grow with n, and on the largest grids it stays below that of the functions' copies.
+constexpr int PG_BATCH = 16384;   // subjects x splits ...
+constexpr int PG_MOST = 65536;    // ... and beyond 512 splits, where 128 subjects are more
+constexpr int PG_SLAB = 4096;     // 64s of nodes whose table is held at a time (2^18 nodes)
+static_assert(PG_SLAB % 8 == 0, "whole splits in a slab");
+// Splits up to which k_pace_dots tests the table's bound itself (32 splits, 128 x 128 nodes,
+// n = 500: 132 us, 138 with k_pace_check; 512 splits, n = 100: 920 and 716).
+constexpr int PG_INLINE = 64;
 
 struct ScWork {
   float2 *mu2, *phi2;  // mu (P) and the first L eigenfunctions (L x P) as float-float
@@ -988,6 +1023,7 @@ struct ScWork {
   int* expo;           // L exponents
   uint2* table;
   long long* gsum;
+  unsigned* which;        // k_pace_check
   float2 *bpart, *rpart;  // partial Phi'Y^C and rows of Phi'Phi of the node chunks
   const double* phi;
   int nbx, nsplit, per, batch, nchunk;
@@ -1005,16 +1041,18 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
   // fixed-point sums below 2^63
   w->per = n64 <= 64 ? 4 : 8;
   w->nsplit = (n64 + w->per - 1) / w->per;
-  w->batch = std::max(128, PG_BATCH / w->nsplit / 128 * 128);
+  w->batch = w->nsplit <= PG_MOST / 128 ? std::max(128, PG_BATCH / w->nsplit / 128 * 128)
+                                        : std::max(16, PG_MOST / w->nsplit / 16 * 16);
   w->nchunk = (P + PD_CHUNK - 1) / PD_CHUNK;
-  const size_t nt = (size_t)n64 * 4 * ng * PG_DIG * 32;
+  const size_t nt = (size_t)std::min(n64, PG_SLAB) * 4 * ng * PG_DIG * 32;
   const size_t ns = (size_t)w->nsplit * w->batch * 8 * ng;
   const size_t nc = (size_t)w->nchunk * w->batch;
   const size_t nr = (size_t)L * (L + 1) / 2;
   size_t need = WsCarve::round(sizeof(float2) * P) + WsCarve::round(sizeof(float2) * (size_t)L * P) + 512;
   if (grid)
     need += WsCarve::round(sizeof(float) * L * w->nbx) + 512 + WsCarve::round(sizeof(uint2) * nt) +
-            WsCarve::round(sizeof(long long) * ns) + WsCarve::round(sizeof(float2) * nc * L) +
+            WsCarve::round(sizeof(long long) * ns) + WsCarve::round(sizeof(unsigned) * w->batch) +
+            WsCarve::round(sizeof(float2) * nc * L) +
             WsCarve::round(sizeof(float2) * nc * nr);
   void* ws = fpca_workspace(ctx, need);
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace (%zu bytes)", need);
@@ -1027,6 +1065,7 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
     w->expo = c.take<int>(SC_LMAX);
     w->table = c.take<uint2>(nt);
     w->gsum = c.take<long long>(ns);
+    w->which = c.take<unsigned>(w->batch);
     w->bpart = c.take<float2>(nc * L);
     w->rpart = c.take<float2>(nc * nr);
   }
@@ -1038,24 +1077,34 @@ fpca_status sc_split(fpca_ctx* ctx, int P, int L, const double* mu, const double
 
 fpca_status pace_dense(fpca_ctx* ctx, const fpca_data* data, int P, int L, const ScWork& w,
                        double* scores) {
-  const int n64 = (P + 63) / 64, ng = pg_groups(L);
-  k_pace_table<<<n64, 256, 0, ctx->stream>>>(P, L, w.nbx, w.bmax, w.phi, w.table, w.expo);
-  FPCA_LAUNCHED(ctx, "pace_table");
+  const int n64 = (P + 63) / 64, ng = pg_groups(L), gp = ng <= 2 ? 2 : 5;
   // 16 mask bytes at once where rows are whole multiples of them
   const int vec = P % 16 == 0 && (reinterpret_cast<uintptr_t>(data->mask) & 15) == 0;
+  auto gram = gp == 2 ? k_pace_gram<2> : k_pace_gram<5>;
   for (int i0 = 0; i0 < data->n; i0 += w.batch) {
     const int nb = std::min(w.batch, data->n - i0);
-    const int gp = ng <= 2 ? 2 : 5;
-    auto gram = gp == 2 ? k_pace_gram<2> : k_pace_gram<5>;
-    gram<<<dim3((nb + 127) / 128, w.nsplit, (ng + gp - 1) / gp), 256, 0, ctx->stream>>>(
-        nb, i0, P, ng, w.per, data->mask, w.table, w.gsum, vec);
-    FPCA_LAUNCHED(ctx, "pace_gram");
+    for (int first = 0; first < n64; first += PG_SLAB) {  // (whole splits)
+      const int have = std::min(PG_SLAB, n64 - first);
+      if (i0 == 0 || n64 > PG_SLAB) {
+        k_pace_table<<<have, 256, 0, ctx->stream>>>(P, first, L, w.nbx, w.bmax, w.phi, w.table, w.expo);
+        FPCA_LAUNCHED(ctx, "pace_table");
+      }
+      gram<<<dim3((nb + 127) / 128, (have + w.per - 1) / w.per, (ng + gp - 1) / gp), 256, 0,
+             ctx->stream>>>(nb, i0, P, first, have, ng, w.per, data->mask, w.table,
+                            w.gsum + (size_t)(first / w.per) * nb * 8 * ng, vec);
+      FPCA_LAUNCHED(ctx, "pace_gram");
+    }
+    const bool check = w.nsplit > PG_INLINE;
+    if (check) {
+      k_pace_check<<<(nb + 7) / 8, 256, 0, ctx->stream>>>(nb, L, w.nsplit, w.expo, w.gsum, w.which);
+      FPCA_LAUNCHED(ctx, "pace_check");
+    }
     auto dots = L <= 8 ? k_pace_dots<8> : k_pace_dots<16>;
     const int dsm = (int)sizeof(float2) * PD_CHUNK * (L <= 8 ? 9 : 17);
     cudaFuncSetAttribute(dots, cudaFuncAttributeMaxDynamicSharedMemorySize, dsm);
     dots<<<dim3(w.nchunk, (nb + 15) / 16), 256, dsm, ctx->stream>>>(
         nb, i0, P, data->y, data->y_prec, data->mask, w.mu2, w.phi2, L, w.expo,
-        w.nsplit, w.gsum, w.bpart, w.rpart);
+        w.nsplit, w.gsum, check ? w.which : nullptr, w.bpart, w.rpart);
     FPCA_LAUNCHED(ctx, "pace_dots");
     auto fin = L <= 8 ? k_pace_final<8> : k_pace_final<16>;
     const int sub = L <= 8 ? 4 : 2;
