@@ -43,10 +43,10 @@ struct fpca_ctx {
   int f3_ncta = 0, f3_nitems = 0, f3_npairs = 0;
   // t-side sweep kernel of the FP32 d = 2 covariance smoother: 0 = automatic,
   // 1 = the scalar sweep (k_hsolve2), 2 = the packed-pair sweep where built;
-  // the automatic choice per (M1, M2, T1, T2, compensated, half) once timed:
+  // the automatic choice per (M1, M2, T1, T2, compensated, half, CV terms alone) once timed:
   // 1 or 2 as above
   int tside_kernel = 0;
-  std::map<std::array<int, 6>, int> tside_choice;
+  std::map<std::array<int, 7>, int> tside_choice;
   // schedule of the K-fold CV grid of the FP32 d = 2 smoother: 0 item by item,
   // 1 batched (one persistent t-side launch), 2 automatic; the automatic choice
   // per (M1, M2, folds, compensated, taps of every bandwidth) once timed: 0 or 1

@@ -1472,14 +1472,24 @@ fpca_status cov_smooth_one(fpca_ctx* ctx, const fpca_grid* g, const int32_t* cnt
         bool packed = use_ts;
         if (use_ts && hs_ok && ctx->tside_kernel == 0) {
           // autotune: both sweeps built for this grid and these windows; time each
-          // once (twice, keeping the faster run) and remember the faster in the context
-          const std::array<int, 6> key = {M1, M2, Tax[0], Tax[1], COMP ? 1 : 0, tg.half};
+          // once (twice, keeping the faster run) and remember the faster in the context.
+          // CV terms alone are timed for themselves: the packed sweep solves only where
+          // held-out pairs are then (64 x 64, 16 bandwidths, gridded folds: 110 ms with the
+          // surfaces' choice, 89 with its own).  The choice does not depend on how many
+          // points that is: where the two are close (32 columns, 11 taps: 0.83..1.11) the
+          // scalar one is better on gridded and scattered folds alike.
+          const int cv_only = ef.cvacc && !gm && !status && !ef.y;
+          std::array<int, 7> key = {M1, M2, Tax[0], Tax[1], COMP ? 1 : 0, tg.half, cv_only};
           auto it = ctx->tside_choice.find(key);
+          if (it == ctx->tside_choice.end() && ctx->capturing) {
+            key[6] = !cv_only;  // inside a capture the other's choice will do
+            it = ctx->tside_choice.find(key);
+          }
           if (it == ctx->tside_choice.end()) {
             if (fpca_no_capture(ctx, "timing the t-side sweeps") != FPCA_OK)
               return FPCA_E_UNSUPPORTED;
-            Epilogue<float> e = ef;  // no accumulating epilogues, escalations solved in place
-            e.cvacc = nullptr;
+            Epilogue<float> e = ef;  // escalations solved in place
+            if (!cv_only) e.cvacc = nullptr;
             e.y = nullptr;
             e.esc_count = nullptr;
             cudaEvent_t ev[5];
@@ -1499,6 +1509,7 @@ fpca_status cov_smooth_one(fpca_ctx* ctx, const fpca_grid* g, const int32_t* cnt
             for (int q = 0; q < 4; ++q) cudaEventElapsedTime(&t[q], ev[q], ev[q + 1]);
             for (auto& x : ev) cudaEventDestroy(x);
             if (st != FPCA_OK) return st;
+            if (cv_only) cudaMemsetAsync(ef.cvacc, 0, 3 * sizeof(double), ctx->stream);  // as it was
             const float tts = std::min(t[0], t[2]), ths = std::min(t[1], t[3]);
             it = ctx->tside_choice.emplace(key, tts <= ths ? 2 : 1).first;
           }

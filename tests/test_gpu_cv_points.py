@@ -1,6 +1,6 @@
 """CV sweeps that solve only where held-out pairs are, point by point: the listed fold carries the
 score (its squared products, which no fit uses, are a million times the others'), so that one lost
-or misplaced point shows."""
+or misplaced point shows; and the sweep that CV runs is chosen by timing CV itself."""
 import numpy as np
 import pytest
 
@@ -73,3 +73,30 @@ def test_every_listed_point_counts(m, per_tile, nh):
     less = score(m, bins, hs, B.F64, 0)
     assert np.all(np.abs(less - ref) >= 5 * TOL * np.abs(ref))
 
+
+def test_cv_is_timed_as_cv():
+    from paper_1510_04439_gb300 import binding as B
+    m = (16, 32)
+    bins = problem(m, 3, 0)
+    hs = [[4.5 / 16, 4.5 / 32]]
+    ctx = B.Context(0)
+    ctx.set_cv_batch(0)
+    P = m[0] * m[1]
+    c, w, v, q = dev(bins[0]), *(dev(a.astype(np.float32)) for a in bins[1:])
+    pool = [c.sum(0).to(torch.int32), w.sum(0), v.sum(0)]
+    gamma = torch.empty(P, P, device="cuda:0")
+    out = torch.empty(3, 1, dtype=torch.float64, device="cuda:0")
+    ctx.smooth_cov_project(m, *pool, hs, B.F32C, gamma=gamma)    # the surface's choice is made
+    ctx.sync()
+    launched = []
+    for k in range(3):
+        before = ctx.launches
+        ctx.smooth_cov_project(m, c, w, v, hs, B.F32C, q=q, nfold=3, cv=out[k])
+        launched.append(ctx.launches - before)
+    ctx.sync()
+    # the first call times the sweeps on their CV terms, leaving no trace in the score
+    assert launched[0] > launched[1] == launched[2]
+    got = out.cpu().numpy()[:, 0]
+    assert np.all(np.abs(got - got[0]) <= 1e-12 * got[0])
+    ref = score(m, bins, hs, B.F64, 0)
+    assert np.all(np.abs(got - ref) <= TOL * ref)
