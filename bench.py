@@ -565,6 +565,18 @@ def taps(h, M):
     return 0
 
 
+def held_out_points(torch, w, v, q):
+    """Points that K-fold CV scores, over the folds: those whose held-out bins (each F x P x P)
+    are not empty, of the whole surfaces and of t >= s.  An item-by-item CV sweep solves the
+    latter alone (the packed one; a point without held-out pairs adds nothing to the score)."""
+    full = half = 0
+    for f in range(w.shape[0]):
+        on = (w[f] != 0) | (v[f] != 0) | (q[f] != 0)
+        full += int(on.sum())
+        half += int(torch.triu(on).sum())
+    return full, half
+
+
 def load_traffic(kernel):
     """Per-launch DRAM bytes of ``kernel`` from the committed ncu summary, if it
     was taken on the current source of that kernel; else None."""
@@ -871,14 +883,19 @@ def main():
             sched[name] = {"ms_per_grid": ms_s, "t_side_kernel": top,
                            "t_side_ms": t_side[0] / 3, "t_side_launches": t_side[1] // 3}
         ctx.set_cv_batch("auto")
-        # the t-side sweeps' FP32 work over the grid: per item and evaluated (t >= s)
-        # point, 2 (15 L1 + 21 L2) + 100 flops with L the mean in-grid window lengths
+        # the t-side sweeps' FP32 work over the grid: per item and solved (t >= s) point,
+        # 2 (15 L1 + 21 L2) + 100 flops with L the mean in-grid window lengths.  The packed
+        # sweep solves only points with held-out pairs (what it forms of their tiles' other
+        # points is not counted), the scalar and the batched one every point.
         Ms = Ds.m[0]
+        top_k = sched[chosen]["t_side_kernel"]
+        held_full, held_half = held_out_points(torch, sb.cw, sb.cv_, sb.cq)
+        if top_k != "cov_tsweep":
+            held_full, held_half = Ds.nfold * Ps * Ps, Ds.nfold * Ps * (Ps + 1) // 2
         cv_flops = 0.0
         for hh in hs:
             Th = taps(hh, Ms)
-            cv_flops += Ds.nfold * (2.0 * 36 * mean_window(Ms, Th) + 100.0) * Ps * (Ps + 1) / 2
-        top_k = sched[chosen]["t_side_kernel"]
+            cv_flops += (2.0 * 36 * mean_window(Ms, Th) + 100.0) * held_half
         t_ms = sched[chosen]["t_side_ms"]
         cv_roof = None
         if t_ms > 0 and peaks and peaks.get("fp32_tflops"):
@@ -887,7 +904,8 @@ def main():
                        "peak": peaks["fp32_tflops"], "unit": "TFLOP/s",
                        "frac": ach / peaks["fp32_tflops"], "ms_t_side_per_grid": t_ms,
                        "flops_basis": "sum over the 80 items of (2 (15 L1 + 21 L2) + 100) "
-                                      "flops x P (P + 1) / 2 evaluated points",
+                                      "flops x solved points (t >= s)",
+                       "points_solved_per_bandwidth": held_half,
                        "peak_basis": "measured FP32 FMA peak (alu_peaks_measured)"}
         scores = sb.scores.cpu().numpy()
         fits = len(hs) * Ds.nfold
@@ -900,7 +918,10 @@ def main():
         t_tr = time.perf_counter() - t0
         cvx = {"workload": f"sparse_2d_64x64_n{Ds.n}_5fold_16h", "ms_per_grid": ms_cv,
                "schedule_chosen": chosen, "schedules": sched, "roofline": cv_roof,
-               "fits": fits, "value": fits * float(Ps) * Ps / (ms_cv * 1e-3), "unit": UNIT,
+               "fits": fits, "value": len(hs) * float(held_full) / (ms_cv * 1e-3), "unit": UNIT,
+               "points": "points of the surfaces solved (with their mirrored ones): those with "
+                         "held-out pairs where the packed sweep runs, else all",
+               "points_per_bandwidth": held_full,
                "best_h": hs[int(np.argmin(scores))], "best_cv": float(np.min(scores)),
                "trust_region": {"h": list(h_tr), "cv": cv_tr, "evaluations": len(tr),
                                 "wall_ms": t_tr * 1e3,
