@@ -131,8 +131,8 @@ fpca_status fpca_alu_probe(fpca_ctx* ctx, int fp64, int blocks, int iters, doubl
 /* Choice of the t-side moment sweep of the FP32 d = 2 covariance smoother
  * (fpca_smooth_cov_project with FPCA_F32 / FPCA_F32C):
  *  0  automatic (default): the candidates built for the grid and windows are
- *     timed once per (grid, windows, precision) on the context's stream and the
- *     fastest is remembered in the context;
+ *     timed once per (grid, windows, precision, surfaces or CV scores) on the
+ *     context's stream and the fastest is remembered in the context;
  *  1  the scalar sweep (every t-plane layout and window);
  *  2  the packed-pair sweep where it is built (t-planes 32 or 64 wide, the
  *     same window on both t axes), else the scalar one.
@@ -156,8 +156,10 @@ fpca_status fpca_set_sweep_kernel(fpca_ctx* ctx, int kernel);
  *     remembered in the context.
  * Batched falls back to item by item when the items' arrays do not fit in 80%
  * of the free device memory, when the widest window's tile exceeds the shared
- * memory, or when sweep kernel 2 is forced.  Both compute the same fits and CV
- * terms (the same sums per point, FP32 tolerance). */
+ * memory, or when sweep kernel 2 is forced.  Both give the same CV terms (the
+ * same sums per point, FP32 tolerance); item by item, the packed sweep and the
+ * sweeps of other grids fit only points with held-out pairs, since the others
+ * add nothing to a score. */
 fpca_status fpca_set_cv_batch(fpca_ctx* ctx, int batch);
 
 /* Self-check of the device-side failure detection.  Launches one thread
@@ -245,13 +247,20 @@ fpca_status fpca_smooth_mean_cv(fpca_ctx* ctx, const fpca_data* data, const fpca
  *   entries (only j == l pairs) set to zero.  prec FPCA_F64 uses FP64
  *   CUDA-core products (w, v double); FPCA_BF16 uses tcgen05 tensor cores
  *   with BF16 operands and FP32 accumulation (w, v float); counts are exact
- *   for n < 2^24.  FPCA_F32 uses FP32 CUDA-core products (w, v, q float; the
- *   terms w_i R R and their sums rounded to FP32) and is the one dense
+ *   for n < 2^24.  FPCA_F32 forms FP32 sums (w, v, q float) on the tensor cores:
+ *   sqrt(w_i) R and sqrt(w_i) R^2 rounded to FP32 and cut into three BF16 parts,
+ *   the six of their nine products above 2^-25 of the whole added up to 16
+ *   subjects at a time, and those sums added in FP32 (closer to 64 bits than
+ *   FP32 multiply-adds); counts exact for n < 2^24.  It is the one dense
  *   precision that takes fold/nfold and q, with the meaning they have for
  *   sparse data; FPCA_F64 and FPCA_BF16 need fold = NULL, nfold = 0, q = NULL.
  *  Sparse data: integer-exact pair scatter; FPCA_F64 or FPCA_F32 sums.
  *   fold (length n, values 0..nfold-1) splits the pairs into nfold slices;
  *   q (may be NULL) receives sum w (R R)^2 for cross-validation.
+ *   A subject with offsets out of 0 <= offs[i] <= offs[i+1] <= offs[n], or a
+ *   fold out of range, is left out and the next fpca_sync() reports it; an
+ *   observation that two of its neighbours then both hold counts for one of
+ *   them (which one is not defined).
  * cnt, w, v, q are F x P x P (F = max(nfold, 1)) and are overwritten. */
 fpca_status fpca_bin_cov(fpca_ctx* ctx, const fpca_data* data, const fpca_grid* grid,
                          const double* mu, int prec, int mode,
@@ -298,11 +307,14 @@ fpca_status fpca_smooth_cov_project(fpca_ctx* ctx, const fpca_grid* grid,
  *  gamma: P x P, double (gamma_prec FPCA_F64) or float (FPCA_F32).
  *  domain: P int32 mean-bin counts from fpca_bin_mean (a node is inside
  *   Omega when its count is > 0), or NULL for the whole box.
- *  full = 1: all eigenpairs of Sigma itself (gamma FP64, P <= 1024), of which the
- *   leading k are returned: two-sided block Jacobi in FP32 (blocks of 16 indices,
- *   each round's block pairs diagonalised side by side, the rotations applied
- *   across the GPU), then three Ogita-Aishima refinement steps in FP64 on the
- *   FP64 matrix (each squares the error: eigenpairs to about FP64 accuracy).
+ *  full = 1: the leading k eigenpairs of Sigma itself (gamma FP64, P <= 1024) to
+ *   about FP64 accuracy: two-sided block Jacobi in FP32 (blocks of 16 indices,
+ *   each round's block pairs rotated side by side) on Sigma scaled by a power of
+ *   two to entries below 1, then Ogita-Aishima refinement in FP64 -- up to 256
+ *   nodes of the wanted vectors alone, up to eight steps; beyond, of all vectors,
+ *   three steps and up to two more while a wanted one is not converged -- and,
+ *   where wanted eigenvalues are closer than this resolves, FP64 Jacobi.  Any
+ *   scale of the surface will do; one with infinite entries has NaN eigenpairs.
  *  full = 0: random projection (Section 3.4) with the caller's Gaussian
  *   test matrix omega (P x l float, k < l <= 64): Y = Sigma Omega, power_iters
  *   rounds of Q = orth(Y), Y = Sigma Q, then Q = orth(Y), B = Q' Sigma Q and
@@ -475,10 +487,14 @@ fpca_status fpca_sigma2(fpca_ctx* ctx, const fpca_grid* grid, const int32_t* cnt
  *   A_i = Lambda Phi_i' (Phi_i Lambda Phi_i' + sigma^2 I)^{-1} (Y_i - mu(t_i)),
  * evaluated through the push-through identity as the L x L system
  *   (sigma^2 Lambda^{-1} + Phi_i' Phi_i) A_i = Phi_i' (Y_i - mu(t_i))
- * (sums in compensated FP32 -- error-free products and additions on
- * float-float inputs, about FP64 accuracy -- then an FP64 Cholesky).  Gridded
- * data (mask or all nodes) and
- * scattered data (offs, t) are both accepted.  A subject without observations
+ * (scattered data: sums in compensated FP32 -- error-free products and additions
+ * on float-float inputs, about FP64 accuracy; gridded data: Phi_i' Phi_i as an
+ * exact integer product of the masks with 54-bit fixed-point phi_a phi_b, except
+ * the rows of functions that are too small on a subject's nodes for that -- their
+ * mean square there below 2^-8 of 2^(2e) > max phi^2 -- and Phi_i' Y, in
+ * compensated FP32; then a Cholesky factor in float-float, about 48 bits, with one
+ * refinement by the FP64 residual, or in FP64 where the correction is not small).
+ * Gridded data (mask or all nodes) and scattered data (offs, t) are both accepted.  A subject without observations
  * gets A_i = 0 (the prior mean).  sigma2 is ONE device double (e.g. the output
  * of fpca_sigma2, so no host round trip separates the two calls); it must be
  * >= 0 and every evals[l] > 0 (with sigma2 == 0 the system is singular for a
@@ -495,7 +511,8 @@ fpca_status fpca_sigma2(fpca_ctx* ctx, const fpca_grid* grid, const int32_t* cnt
  *
  * Each of the three splits mu and the first L eigenfunctions into float-float
  * in the context's workspace first (which may synchronise the stream the first
- * time it grows). */
+ * time it grows).  PACE of gridded data takes more of it than the others (so
+ * run that call itself before capturing it). */
 fpca_status fpca_scores_pace(fpca_ctx* ctx, const fpca_data* data, const fpca_grid* grid,
                              const double* mu, const double* evals, const double* evecs, int L,
                              const double* sigma2, double* scores);

@@ -1307,8 +1307,6 @@ __global__ void k_pool_counts(int F, long long PP, const int32_t* __restrict__ i
   out[e] = s;
 }
 
-// cv[h] = err / w_in over folds; +inf when EMPTY points hold > 1% of the
-// held-out weight or nothing was scored.
 // One fold's training bins: the pooled ones less the fold's, as k_vpass2 forms them.
 template <typename T>
 __global__ void k_train_bins(long long PP, const int32_t* __restrict__ cnt, const T* __restrict__ w,
@@ -1323,6 +1321,8 @@ __global__ void k_train_bins(long long PP, const int32_t* __restrict__ cnt, cons
   }
 }
 
+// cv[h] = err / w_in over folds; +inf when EMPTY points hold > 1% of the
+// held-out weight or nothing was scored.
 __global__ void k_cv_finish(int nh, int F, const double* __restrict__ acc, double* __restrict__ cv) {
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   if (h >= nh) return;
