@@ -11,6 +11,7 @@
 // Parameter vector: for each layer, W (fan_in x fan_out, row-major) then b.
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -37,7 +38,7 @@ __device__ __forceinline__ float gelu_grad(float z) {
 // ---------------------------------------------------------------------------
 // The step in three launches:
 //   k_mlp_weights  FP16 copies of the hidden layers' weights, and transposes of those the
-//                  backward pass multiplies by; the batch's mask count, a part a block;
+//                  backward pass multiplies by; the batch's mask count, in parts;
 //   k_mlp_rows     a CTA takes R rows of the batch through the whole network and back:
 //                  the rows are independent between the loss and the weights, so nothing
 //                  but the weights (384 KB in FP16, from L2) is read between layers;
@@ -56,27 +57,30 @@ __host__ __device__ constexpr int w16_off(int copy) {
 }
 constexpr int W16_COUNT = 32 * HID + 4 * HID * HID;
 
-constexpr int MW_BLOCKS = 8 + 64 + 64;
+constexpr int MW_TILES = 8 + 64 + 64;
+constexpr int MC_MAX = 128;        // parts of the mask count
+constexpr int MC_BYTES = 256 * 32; // bytes of a part, unless that makes more than MC_MAX
 
-// A 32 x 32 tile per block: blocks 0..7 layer 0, then 64 each for layers 1 and 2.  With `mask`
-// (nm bytes) each block counts its share into mcount[block].
+// A 32 x 32 tile per block: blocks 0..7 layer 0, then 64 each for layers 1 and 2.  The blocks
+// beyond MW_TILES count a part of the mask (nm bytes) each, into mcount.
 __global__ void __launch_bounds__(256)
     k_mlp_weights(const float* __restrict__ th, __half* __restrict__ w16,
                   const uint8_t* __restrict__ mask, long long nm, int* __restrict__ mcount) {
   __shared__ __half t[32][33];
-  if (mask) {
-    const long long per = (nm + MW_BLOCKS - 1) / MW_BLOCKS, e0 = blockIdx.x * per;
-    const long long e1 = e0 + per < nm ? e0 + per : nm;
-    int c = 0;
-    for (long long e = e0 + threadIdx.x; e < e1; e += 256) c += mask[e] ? 1 : 0;
+  if (blockIdx.x >= MW_TILES) {
+    const int part = blockIdx.x - MW_TILES, parts = gridDim.x - MW_TILES;
     __shared__ int mc[8];
+    int c = 0;
+#pragma unroll 4
+    for (long long e = part * 256 + threadIdx.x; e < nm; e += parts * 256) c += mask[e] ? 1 : 0;
     for (int q = 16; q > 0; q >>= 1) c += __shfl_xor_sync(0xffffffffu, c, q);
     if ((threadIdx.x & 31) == 0) mc[threadIdx.x >> 5] = c;
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int q = 1; q < 8; ++q) c += mc[q];
-      mcount[blockIdx.x] = c;
+      mcount[part] = c;
     }
+    return;
   }
   const int b = blockIdx.x, l = b < 8 ? 0 : b < 72 ? 1 : 2, tile = b - (l == 0 ? 0 : l == 1 ? 8 : 72);
   const int r0 = (tile / 8) * 32, c0 = (tile % 8) * 32;
@@ -137,7 +141,8 @@ struct MlpBuf {
   float* D[3];     // gradients w.r.t. the hidden pre-activations, B x 256
   float* D3;       // gradient w.r.t. the output, B x 8 (two zero columns)
   float* losspart; // one per CTA
-  int* mcount;     // observed targets, one part per block of k_mlp_weights
+  int* mcount;     // observed targets, in `parts` parts
+  int parts;
   __half* w16;
 };
 
@@ -201,7 +206,7 @@ __global__ void __launch_bounds__(256)
   }
   // masked loss: its denominator is the whole batch's mask count (each CTA going through the
   // whole mask made the step quadratic in the batch: 2^20 rows 441 ms, 57 with the parts)
-  int cnt = t < MW_BLOCKS ? w.mcount[t] : 0;
+  int cnt = t < w.parts ? w.mcount[t] : 0;
   for (int q = 16; q > 0; q >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, q);
   if (lane == 0) rc[wp] = cnt;
   __syncthreads();
@@ -389,7 +394,7 @@ fpca_status mlp_buffers(fpca_ctx* ctx, int Bn, int R, int train, MlpBuf& w) {
   if (train)
     need += WsCarve::round(sizeof(float) * 32 * B) + 6 * WsCarve::round(sizeof(float) * HID * B) +
             WsCarve::round(sizeof(float) * 8 * B) + WsCarve::round(sizeof(float) * (B / R + 1)) +
-            WsCarve::round(sizeof(int) * MW_BLOCKS);
+            WsCarve::round(sizeof(int) * MC_MAX);
   void* ws = fpca_workspace(ctx, need);
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace (%zu bytes)", need);
   WsCarve c(ws);
@@ -403,7 +408,8 @@ fpca_status mlp_buffers(fpca_ctx* ctx, int Bn, int R, int train, MlpBuf& w) {
   }
   w.D3 = c.take<float>(8 * B);
   w.losspart = c.take<float>(B / R + 1);
-  w.mcount = c.take<int>(MW_BLOCKS);
+  w.mcount = c.take<int>(MC_MAX);
+  w.parts = (int)std::min<long long>(MC_MAX, (6ll * Bn + MC_BYTES - 1) / MC_BYTES);
   return FPCA_OK;
 }
 
@@ -420,8 +426,7 @@ fpca_status mlp_launch_rows(fpca_ctx* ctx, const float* th, const float* feat, c
 
 fpca_status mlp_rows(fpca_ctx* ctx, const float* th, const float* feat, const float* target,
                      const uint8_t* mask, int Bn, int R, const MlpBuf& w, float* out, int train) {
-  k_mlp_weights<<<MW_BLOCKS, 256, 0, ctx->stream>>>(th, w.w16, train ? mask : nullptr, 6ll * Bn,
-                                                    w.mcount);
+  k_mlp_weights<<<MW_TILES + w.parts, 256, 0, ctx->stream>>>(th, w.w16, mask, 6ll * Bn, w.mcount);
   FPCA_LAUNCHED(ctx, "mlp_weights");
   if (R == 2) return mlp_launch_rows<2>(ctx, th, feat, target, mask, Bn, w, out, train);
   if (R == 4) return mlp_launch_rows<4>(ctx, th, feat, target, mask, Bn, w, out, train);
