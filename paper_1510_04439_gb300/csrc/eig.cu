@@ -908,9 +908,10 @@ __global__ void k_rr_out(int n, const double* __restrict__ lam, const double* __
   }
 }
 
-// out = in 2^-e (eig_exponent), element by element
-__global__ void k_scale(long long n, const double* __restrict__ in,
-                        const unsigned long long* __restrict__ top, double* __restrict__ out) {
+// out = in 2^-e (eig_exponent), element by element; out may be in.  A launch of its own (3 to 5 us):
+// done by k_bj_cluster as it reads the matrix it took 4 to 10 at 64 nodes and 13 to 30 at 256.
+__global__ void k_scale(long long n, const double* in, const unsigned long long* __restrict__ top,
+                        double* out) {
   const int ex = eig_exponent(*top);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
        e += (long long)gridDim.x * blockDim.x)
@@ -920,11 +921,9 @@ __global__ void k_scale(long long n, const double* __restrict__ in,
 // Rank of each eigenvalue (descending; ties by index; NaN last) -> order[rank] = index.
 __global__ void k_eig_order(int n, const double* __restrict__ A, int* __restrict__ order) {
   for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const double ti = A[(long long)i * n + i];
+    const long long ti = eig_key(A[(long long)i * n + i]);
     int rank = 0;
-    for (int j = 0; j < n; ++j) {
-      rank += eig_before(A[(long long)j * n + j], j, ti, i);
-    }
+    for (int j = 0; j < n; ++j) rank += eig_before(eig_key(A[(long long)j * n + j]), j, ti, i);
     order[rank] = i;
   }
 }
@@ -1427,9 +1426,9 @@ __global__ void __launch_bounds__(256)
                 const float* __restrict__ gate) {
   const int i = (int)((blockIdx.x * 256u + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (oa_done(gate) || i >= n) return;
-  const double li = lam[i];
+  const long long ki = eig_key(lam[i]);
   int rank = 0;
-  for (int j = lane; j < n; j += 32) rank += eig_before(lam[j], j, li, i);
+  for (int j = lane; j < n; j += 32) rank += eig_before(eig_key(lam[j]), j, ki, i);
   for (int o = 16; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
   if (lane == 0) wanted[i] = rank < k;
 }
@@ -1714,17 +1713,19 @@ fpca_status rproj_typed(fpca_ctx* ctx, const fpca_grid* g, const TG* gamma, cons
   if (full) {
     // dense eigenpairs of Sigma (FP64)
     if constexpr (sizeof(TS) == 8) {
-      if (lead_eig_takes(P)) {
+      const bool lead = lead_eig_takes(P);
+      k_scale<<<(int)std::min<long long>((PP + 255) / 256, 4096), 256, 0, ctx->stream>>>(
+          PP, S, top, lead ? S : A);
+      FPCA_LAUNCHED(ctx, "eig_scale");
+      if (lead) {
         // A: the eigenvalues as a vector (row stride 0 below), order: 0..k-1
-        fpca_status ls = launch_lead_eig(ctx, P, k, S, top, A, evecs, order, dense);
+        fpca_status ls = launch_lead_eig(ctx, P, k, S, A, evecs, order, dense);
         if (ls != FPCA_OK) return ls;
         k_finish<<<k, 1024, 0, ctx->stream>>>(P, 0, k, dv, 1.0 / std::sqrt(dv), A, order, trace,
                                               evals, evecs, fve, top);
         FPCA_LAUNCHED(ctx, "eig_finish");
         return FPCA_OK;
       }
-      k_scale<<<(int)std::min<long long>((PP + 255) / 256, 4096), 256, 0, ctx->stream>>>(PP, S, top, A);
-      FPCA_LAUNCHED(ctx, "eig_scale");
     } else {
       return fpca_fail(ctx, FPCA_E_UNSUPPORTED, "dense eigensolver needs FP64 gamma");
     }

@@ -19,7 +19,7 @@
 //     error by the basis' own (1e-5 or better over the relative gap) instead of squaring it,
 //     and costs 3 n^2 k FP64 multiply-adds instead of 4 n^3: FP64 runs at 1/64 of the FP32
 //     rate here, and refining all n vectors took 0.47 ms of 256 x 256.
-//     All of it works on A scaled to entries below 1 (eig_exponent), in place.
+//     All of it works on a matrix scaled to entries below 1 (eig_exponent).
 //  3. Where this leaves a wanted vector unconverged (eigenvalues closer than the FP32
 //     couplings of the basis, a null space), the basis is made orthonormal in FP64 and
 //     X'AX, nearly diagonal, diagonalised by FP64 Jacobi (k_lead_full, k_rotate; both
@@ -61,8 +61,7 @@ inline size_t le_smem(int ne) {
 // the two launches per round of the large-n path.  Columns of the row tiles are stored in
 // groups of 16 spaced by 20 floats, so that eight blocks' columns fall in different banks.
 __global__ void __launch_bounds__(BJ_NT, 1)
-    k_bj_cluster(int n, int ne, int lead, int kk, const unsigned long long* __restrict__ top,
-                 double* __restrict__ A64, float* __restrict__ A,
+    k_bj_cluster(int n, int ne, int lead, int kk, const double* __restrict__ A64, float* __restrict__ A,
                  double* __restrict__ X, double* __restrict__ X0, float* __restrict__ lam32,
                  int* __restrict__ nref) {
   extern __shared__ __align__(16) float bjc[];
@@ -78,16 +77,9 @@ __global__ void __launch_bounds__(BJ_NT, 1)
   float* dg = a1 + BJ_W * BJ_LD;          // [256]: the diagonal after a sweep
   float* mass = dg + LE_MAXN;             // [8][2]: every CTA's off-diagonal, diagonal mass
   float* red = mass + 16;                 // [8][2]
-  const int ex = eig_exponent(*top);
   for (int e = tid; e < BJ_W * ne; e += BJ_NT) {
     const int i = e / ne, c = e - i * ne, gi = rank * BJ_W + i;
-    float a = 0.f;
-    if (gi < n && c < n) {
-      const double x = eig_scaled(A64[(size_t)gi * n + c], ex);
-      A64[(size_t)gi * n + c] = x;
-      a = (float)x;
-    }
-    __stcg(A + (size_t)gi * ne + c, a);
+    __stcg(A + (size_t)gi * ne + c, (gi < n && c < n) ? (float)A64[(size_t)gi * n + c] : 0.f);
     Vr[i * LD + c + 4 * (c >> 4)] = gi == c ? 1.f : 0.f;
   }
   cl.sync();
@@ -259,7 +251,7 @@ __global__ void __launch_bounds__(BJ_NT, 1)
         float gap = 3e38f;
         int rank = 0;
         for (int j = 0; j < n; ++j) {
-          rank += eig_before(dg[j], j, d, tid);
+          rank += dg[j] > d || (dg[j] == d && j < tid);
           if (j != tid) gap = fminf(gap, fabsf(dg[j] - d));
         }
         apart = rank >= lead || sqrtf(off) <= LE_APART * gap;
@@ -292,15 +284,18 @@ __global__ void __launch_bounds__(LE_MAXN)
                 int* __restrict__ pos, int* __restrict__ lead, double* __restrict__ Xk,
                 float* __restrict__ state) {
   __shared__ float lam[LE_MAXN];
-  __shared__ int ld[LE_MAXN];
+  __shared__ int key[LE_MAXN], ld[LE_MAXN];
   __shared__ float red[LE_MAXN / 32];
   const int i = threadIdx.x, kk = *nref;
-  if (i < n) lam[i] = lam32[i];
+  if (i < n) {
+    lam[i] = lam32[i];
+    key[i] = eig_key(lam[i]);
+  }
   __syncthreads();
   if (i < n) {
-    const float li = lam[i];
+    const int ki = key[i];
     int rank = 0;
-    for (int j = 0; j < n; ++j) rank += eig_before(lam[j], j, li, i);
+    for (int j = 0; j < n; ++j) rank += eig_before(key[j], j, ki, i);
     if (rank < kk) ld[rank] = i;
     if (blockIdx.x == 0) {
       pos[i] = rank < kk ? rank : -1;
@@ -627,7 +622,7 @@ __global__ void __launch_bounds__(LE_MAXN)
   if (j >= nv) return;
   const double* l = full ? lam : lamk;
   const double lj = l[j];
-  const int rank = __syncthreads_count(t < nv && eig_before(l[t], t, lj, j));
+  const int rank = __syncthreads_count(t < nv && eig_before(eig_key(l[t]), t, eig_key(lj), j));
   if (rank >= k) return;
   if (t < n) psi[(size_t)rank * n + t] = full ? X[(size_t)t * n + j] : Xk[(size_t)j * n + t];
   if (t == 0) {
@@ -666,8 +661,8 @@ size_t lead_eig_bytes(int n, int k) {
          WsCarve::round(sizeof(double)) + WsCarve::round(sizeof(int) * rotate_ints(n)) + 4096;
 }
 
-fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, double* S, const unsigned long long* top,
-                            double* theta, double* psi, int* order, void* scratch) {
+fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double* theta,
+                            double* psi, int* order, void* scratch) {
   const int ne = le_ne(n), kk = std::min(n, k + LE_EXTRA);
   WsCarve c(scratch);
   float* Af = c.take<float>((size_t)ne * ne);
@@ -703,7 +698,7 @@ fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, double* S, const unsign
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_bj_cluster, n, ne, k, kk, top, S, Af, X, X0, lam32, nref);
+  cudaLaunchKernelEx(&cfg, k_bj_cluster, n, ne, k, kk, S, Af, X, X0, lam32, nref);
   FPCA_LAUNCHED(ctx, "eig_bj_cluster");
   k_lead_init<<<8, LE_MAXN, 0, ctx->stream>>>(n, nref, lam32, X, pos, lead, Xk, state);
   FPCA_LAUNCHED(ctx, "eig_lead_init");

@@ -159,13 +159,12 @@ fpca_status smooth_cov_run(fpca_ctx* ctx, const fpca_grid* g, const fpca_covbins
                            const double* h, int nh, int prec, const double* mu_raw,
                            const float* omega, int l, void* gamma, uint8_t* status, float* y,
                            double* cv);
-// eig_dense.cu: leading k eigenpairs of a small symmetric FP64 matrix S (n x n; scaled in place
-// to entries below 1, *top the bits of its largest |entry|), the scaled matrix's eigenvalues
-// descending into theta[0..k), vectors into psi (row j = vector j), order[j] = j
+// eig_dense.cu: leading k eigenpairs of a small symmetric FP64 matrix S (n x n, entries below 1),
+// eigenvalues descending into theta[0..k), vectors into psi (row j = vector j), order[j] = j
 bool lead_eig_takes(int n);
 size_t lead_eig_bytes(int n, int k);
-fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, double* S, const unsigned long long* top,
-                            double* theta, double* psi, int* order, void* scratch);
+fpca_status launch_lead_eig(fpca_ctx* ctx, int n, int k, const double* S, double* theta,
+                            double* psi, int* order, void* scratch);
 // FP64 Jacobi on the nearly diagonal S = X'AX (n <= 1024), if *gate > limit: rotations into
 // the columns of X, eigenvalues into lam; Ma, Mb: n x n scratch, normsq: one double, flag:
 // rotate_ints(n) ints.

@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 namespace fpca_jacobi {
 
 // Integers that order as the numbers do, NaN below all (and 64-bit comparisons are slow here).
@@ -17,12 +19,13 @@ __device__ __forceinline__ long long eig_key(double x) {
   return b >= 0 ? b : m == 0 ? 0 : b ^ 0x7fffffffffffffffll;
 }
 
-// Eigenvalue a (place i) comes before b (place j): descending, ties by place, NaN last.  A total
-// order, so that ranks are a permutation and every rank's entry is written.
-template <typename T>
-__device__ __forceinline__ bool eig_before(T a, int i, T b, int j) {
-  const auto ka = eig_key(a), kb = eig_key(b);
-  return ka > kb || (ka == kb && i < j);
+// The eigenvalue of key a (place i) comes before that of key b (place j): descending, ties by
+// place, NaN last.  A total order, so that ranks are a permutation and every rank's entry is
+// written.
+template <typename K>
+__device__ __forceinline__ bool eig_before(K a, int i, K b, int j) {
+  static_assert(std::is_integral<K>::value, "keys");
+  return a > b || (a == b && i < j);
 }
 
 // The dense eigensolvers work on A 2^-e, e the exponent for which the largest entry lies in
