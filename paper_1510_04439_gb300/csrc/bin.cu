@@ -341,10 +341,10 @@ struct RowChunk {
 
 constexpr int OBS_LANES = 8;  // threads per subject
 
-// Per observation: its bin, its record, its weight and its row (fold * P + bin; -1 where the
-// subject has no pairs or is skipped).  Offsets outside 0 <= offs[i] <= offs[i+1] <= N and folds
-// outside 0..nfold-1 are reported (DERR_BOUNDS) and the subject is skipped.  row is set to -1 by
-// the caller.
+// Per observation: its bin, its record, its weight and its row + 1 (row = fold * P + bin; 0 where
+// the subject has no pairs or is skipped).  Offsets outside 0 <= offs[i] <= offs[i+1] <= N and folds
+// outside 0..nfold-1 are reported (DERR_BOUNDS) and the subject is skipped.  The caller
+// clears row.
 // A skipped subject's neighbours can overlap (offsets 0, 10, 5, 12: the first and the third
 // both hold observations 5..9).  An observation goes to the subject that claims its row first,
 // and only that one writes the record, so that its lo and ni are one checked subject's; it is
@@ -378,7 +378,7 @@ __global__ void k_obs_rows(int n, long long N, int d, int m0, int m1, int m2, in
   const double wi = 1.0 / ((double)(hi - lo) * (double)(hi - lo - 1));
   for (int64_t j = lo + part; j < hi; j += OBS_LANES) {
     const int b = bin_index(t + j * d, d, m);
-    if (atomicCAS(row + j, -1, f * P + b) != -1) continue;  // another subject's (see above)
+    if (atomicCAS(row + j, 0, f * P + b + 1) != 0) continue;  // another subject's (see above)
     ob[j] = b;
     rec[j] = ObsRec{mode == FPCA_COV_RESIDUAL ? y[j] - mu[b] : y[j], (int32_t)lo,
                     (int32_t)(hi - lo)};
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(RC_NT)
 #pragma unroll
   for (int u = 0; u < RC_PER; ++u) {
     const long long j = j0 + u * RC_NT;
-    r[u] = j < N ? row[j] : -1;
+    r[u] = j < N ? row[j] - 1 : -1;
   }
   for (int e = threadIdx.x; e < rows; e += RC_NT) hist[e] = 0;
   __syncthreads();
@@ -459,8 +459,9 @@ __global__ void k_row_fill(long long N, int fill, const int32_t* __restrict__ ro
     return;
   }
   const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (j >= N || row[j] < 0) return;
-  list[start[row[j]] + rank[j]] = (int32_t)j;
+  if (j >= N) return;
+  const int r = row[j] - 1;
+  if (r >= 0) list[start[r] + rank[j]] = (int32_t)j;
 }
 
 // One chunk of an output row (blockIdx.x < rows: the first chunk of row fold * P + bin, else an
@@ -1119,18 +1120,18 @@ fpca_status launch_cov_sparse(fpca_ctx* ctx, int n, const fpca_grid* g, const in
   if (!ws) return fpca_fail(ctx, FPCA_E_OOM, "workspace");
   WsCarve carve(ws);
   int32_t* ob = carve.take<int32_t>(N);
-  int32_t* row = carve.take<int32_t>(N);
+  // row, and the rows' counts behind it: cleared together ([rows]: the list's length)
+  int32_t* row = carve.take<int32_t>(N + (size_t)rows + 2);
+  int32_t* rowcount = row + N;
   int32_t* rank = carve.take<int32_t>(N);
   int32_t* list = carve.take<int32_t>(N);
   ObsRec* rec = carve.take<ObsRec>(N);
   double* wt = carve.take<double>(N);
   RowChunk* extra = carve.take<RowChunk>(nx);
-  int32_t* rowcount = carve.take<int32_t>((size_t)rows + 2);  // [rows]: the list's length
   int32_t* nextra = rowcount + rows + 1;
   int32_t* start = carve.take<int32_t>(rows);
-  cudaMemsetAsync(rowcount, 0, sizeof(int32_t) * ((size_t)rows + 2), ctx->stream);
+  cudaMemsetAsync(row, 0, sizeof(int32_t) * (N + (size_t)rows + 2), ctx->stream);
   if (Nobs > 0) {
-    cudaMemsetAsync(row, 0xff, sizeof(int32_t) * N, ctx->stream);  // -1: no pairs
     k_obs_rows<<<(int)(((long long)n * OBS_LANES + 255) / 256), 256, 0, ctx->stream>>>(
         n, Nobs, g->d, g->m[0], g->d > 1 ? g->m[1] : 1, g->d > 2 ? g->m[2] : 1, P, offs, t, y, mu,
         mode, fold, nfold, ob, rec, wt, row, rowcount, count ? nullptr : rank, ctx->d_err);
