@@ -442,7 +442,8 @@ __global__ void k_row_starts(int rows, int chunk, const int32_t* __restrict__ ro
 // in chunks; es: bytes of an entry of w, v and q.
 __global__ void k_row_fill(long long N, int fill, const int32_t* __restrict__ row,
                            const int32_t* __restrict__ start, const int32_t* __restrict__ rank,
-                           int32_t* __restrict__ list, int P, int es, const int32_t* __restrict__ nextra, const RowChunk* __restrict__ extra,
+                           int32_t* __restrict__ list, int P, int es,
+                           const int32_t* __restrict__ nextra, const RowChunk* __restrict__ extra,
                            int32_t* __restrict__ cnt, void* __restrict__ w, void* __restrict__ v,
                            void* __restrict__ q) {
   if ((int)blockIdx.x >= fill) {

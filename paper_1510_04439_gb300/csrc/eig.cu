@@ -1517,7 +1517,8 @@ inline size_t dense_eig_bytes(int n) {
 // V <- eigenvectors (columns), like launch_jacobi_rr; of the k largest also those of close
 // eigenvalues.  What these need in FP64 is gated by their own corrections: gated by all n, a
 // smoothed covariance (18 x 18 nodes, 4 eigenpairs) took the FP64 Jacobi for its trailing
-// eigenvalues: 21.8 ms for the whole fit, 4.8 now.  Bound by the FP32 rounds' launches and the steps' FP64 products.
+// eigenvalues: 21.8 ms for the whole fit, 4.8 now.  Bound by the FP32 rounds' launches and the
+// steps' FP64 products.
 fpca_status launch_dense_eig(fpca_ctx* ctx, int n, int k, double* A, double* V, void* scratch) {
   const int ne = bj_ne(n), nb = ne / BJ_S, npairs = ne / BJ_W;
   WsCarve c(scratch);

@@ -472,7 +472,8 @@ __device__ __forceinline__ uint4 mask16(const uint8_t* __restrict__ row, int p, 
 template <int GP>
 __global__ void __launch_bounds__(256)
     k_pace_gram(int nb, int i0, int P, int first, int have, int ng, int per,
-                const uint8_t* __restrict__ mask, const uint2* __restrict__ table, long long* __restrict__ out, int vec) {
+                const uint8_t* __restrict__ mask, const uint2* __restrict__ table,
+                long long* __restrict__ out, int vec) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int gr = lane >> 2, t = lane & 3;
   const int ra = blockIdx.x * 128 + warp * 16 + gr, rb = ra + 8;
